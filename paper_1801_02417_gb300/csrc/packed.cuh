@@ -57,6 +57,31 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
+// ---- thread-block clusters: the barrier of all threads of a cluster (release / acquire, so
+// shared memory written before it is seen after it), and loads from the shared memory of
+// the CTA of rank `r` at the address that `p` has in this CTA.
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, int r) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(r));
+  return a;
+}
+__device__ __forceinline__ int ld_cluster(const int* p, int r) {
+  int v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(cluster_addr(p, r)) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_cluster4(const float* p, int r) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(cluster_addr(p, r))
+               : "memory");
+  return v;
+}
+
 // Poll budget of the bounded waits. c_wait_polls (one copy per translation unit,
 // set by set_wait_polls_here) bounds the first wait on a barrier phase; a CTA
 // whose wait gave up drains its copies still in flight with the full budget

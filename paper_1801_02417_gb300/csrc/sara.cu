@@ -76,106 +76,6 @@ __device__ __forceinline__ u64 cdup(const float2& c) { return *reinterpret_cast<
     default: CALL(16); break;     \
   }
 
-__device__ __forceinline__ void sara_epilogue(int mode, float val, size_t idx, float* coef, float* thr, float scale,
-                                              float gamma, float delta) {
-  if (mode == SARA_DUAL) {
-    const float t = thr[idx];
-    const float a = fmaf(scale, val, coef[idx]);
-    coef[idx] = fminf(fmaxf(a, -t), t);
-  } else if (mode == SARA_APPLY) {
-    coef[idx] = scale * val;
-  } else {
-    thr[idx] = gamma * delta / (delta + fabsf(scale * val));
-  }
-}
-
-// One synthesis level: coefficients at level l (approximation from `approx_in`
-// or, at the coarsest level, from coef; details from coef) -> approximation at
-// level l-1 (m x m) into approx_out, or at level 1 the summed image
-// out = (A_dirac + sum_b synth_b) / 3.
-__global__ void __launch_bounds__(256) k_synthesis(const float* __restrict__ coef, const float* __restrict__ approx_in,
-                                                   int coarsest, int m, int TI, int n, int finest,
-                                                   float* __restrict__ approx_out, float* __restrict__ out) {
-  extern __shared__ float sm[];
-  const int map = blockIdx.z;
-  const int hm = m >> 1;
-  const int tilesx = m / TI;
-  const int oy0 = (blockIdx.x / tilesx) * TI, ox0 = (blockIdx.x % tilesx) * TI;
-  const int CI = TI / 2 + kMaxTaps / 2 - 1;      // coefficient tile side (sized for db8)
-  float* s_ll = sm;
-  float* s_lh = s_ll + CI * CI;
-  float* s_hl = s_lh + CI * CI;
-  float* s_hh = s_hl + CI * CI;
-  float* s_lo = s_hh + CI * CI;                   // TI x CI
-  float* s_hi = s_lo + TI * CI;
-  constexpr int kOut = 8;                         // outputs per thread (TI^2 <= 8 * 256)
-  float accv[kOut];
-#pragma unroll
-  for (int t = 0; t < kOut; ++t) accv[t] = 0.f;
-  const int b_begin = finest ? 0 : blockIdx.y, b_end = finest ? kDb : blockIdx.y + 1;
-  for (int bi = b_begin; bi < b_end; ++bi) {
-    const int Lf = 2 * (bi + 1);
-    const int half = Lf / 2 - 1;
-    const int ky0 = oy0 / 2 - half, kx0 = ox0 / 2 - half;
-    const int CIb = TI / 2 + half;                 // rows/cols actually used by this basis
-    const size_t base = ((size_t)map * kBases + (bi + 1)) * (size_t)n * n;
-    const float* apx = coarsest ? nullptr : approx_in + ((size_t)map * kDb + bi) * (size_t)hm * hm;
-    for (int i = threadIdx.x; i < CIb * CIb; i += blockDim.x) {
-      const int r = i / CIb, c = i - r * CIb;
-      const int Yk = ((ky0 + r) % hm + hm) % hm, Xk = ((kx0 + c) % hm + hm) % hm;
-      s_ll[r * CI + c] = coarsest ? coef[base + (size_t)Yk * n + Xk] : apx[(size_t)Yk * hm + Xk];
-      s_hl[r * CI + c] = coef[base + (size_t)Yk * n + hm + Xk];
-      s_lh[r * CI + c] = coef[base + (size_t)(hm + Yk) * n + Xk];
-      s_hh[r * CI + c] = coef[base + (size_t)(hm + Yk) * n + hm + Xk];
-    }
-    __syncthreads();
-    const float* h = c_h[bi];
-    const float* g = c_g[bi];
-    // Along y: lo[r][c] = sum_j h[j] ll[kl][c] + g[j] lh[kl][c], kl = (r - j)/2 + half, j = r mod 2.
-    for (int i = threadIdx.x; i < TI * CIb; i += blockDim.x) {
-      const int r = i / CIb, c = i - r * CIb;
-      float lo = 0.f, hi = 0.f;
-      for (int j = (r & 1); j < Lf; j += 2) {
-        const int kl = ((r - j) >> 1) + half;
-        lo = fmaf(h[j], s_ll[kl * CI + c], fmaf(g[j], s_lh[kl * CI + c], lo));
-        hi = fmaf(h[j], s_hl[kl * CI + c], fmaf(g[j], s_hh[kl * CI + c], hi));
-      }
-      s_lo[r * CI + c] = lo;
-      s_hi[r * CI + c] = hi;
-    }
-    __syncthreads();
-    // Along x.
-#pragma unroll
-    for (int t = 0; t < kOut; ++t) {
-      const int i = threadIdx.x + t * blockDim.x;
-      if (i < TI * TI) {
-        const int r = i / TI, c = i - r * TI;
-        float v = 0.f;
-        for (int j = (c & 1); j < Lf; j += 2) {
-          const int kl = ((c - j) >> 1) + half;
-          v = fmaf(h[j], s_lo[r * CI + kl], fmaf(g[j], s_hi[r * CI + kl], v));
-        }
-        accv[t] += v;
-      }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int t = 0; t < kOut; ++t) {
-    const int i = threadIdx.x + t * blockDim.x;
-    if (i < TI * TI) {
-      const int r = i / TI, c = i - r * TI;
-      const int y = oy0 + r, x = ox0 + c;
-      if (finest) {
-        const size_t dirac = (size_t)map * kBases * (size_t)n * n + (size_t)y * n + x;
-        out[(size_t)map * n * n + (size_t)y * n + x] = (coef[dirac] + accv[t]) * (1.0f / 3.0f);
-      } else {
-        approx_out[((size_t)map * kDb + blockIdx.y) * (size_t)m * m + (size_t)y * m + x] = accv[t];
-      }
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Fast path for levels whose half size is >= 32: 32 x 32 output tiles, filter
 // length and tile shape known at compile time, each thread producing a strip of
@@ -186,19 +86,8 @@ constexpr int kA2Cols = 2 * kTO + 16;            // 80 staged input columns (cov
 constexpr int kA2Pitch = kA2Cols + 4;            // 84 = 20 mod 32 banks: row-parallel 16-byte reads conflict-free
 constexpr int kA2In = kRSmax * kA2Pitch;         // input tile
 constexpr int kPlo = kTO + 4;                    // row-filtered tiles (16-byte aligned rows)
-constexpr int kTI = 32;                          // synthesis output tile
-constexpr int kCImax = kTI / 2 + kMaxTaps / 2 - 1;   // 23
-constexpr int kPs = kCImax + 2;                  // 25
 
 __device__ __forceinline__ int wrap1(int v, int m) { return v < 0 ? v + m : (v >= m ? v - m : v); }
-
-// 4-byte asynchronous global->shared copies (cp.async), grouped and awaited per group.
-__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Rows: lo/hi[r][k] = sum_j h/g[j] in[r][2k + j], k in [0, TO). Each thread makes
 // four outputs of one row from 16-byte reads; the taps go in pairs,
@@ -597,7 +486,6 @@ __device__ __forceinline__ void ana_cols2(const float* __restrict__ lo_s, const 
 // second of two staging sets while basis i is filtered (2 CTAs/SM). NSET = 1: one staging
 // set, refilled for basis i + 1 once basis i's columns have read it, so the copy overlaps the
 // next basis' row pass; the smaller footprint fits 3 CTAs/SM (256 threads).
-constexpr int kAnaMFloats = kAnaPre + 4 * kStage;
 static size_t multi_analysis_smem(int nset = 2) {
   return (size_t)(kAnaPre + 2 * nset * kStage) * sizeof(float) + 32;
 }
@@ -764,145 +652,6 @@ __global__ void __launch_bounds__(256, 2) k_ana_pers(const float* __restrict__ i
     __syncthreads();   // lo/hi consumed before the next unit's rows
   }
 }
-
-// Synthesis of one basis on a TI x TI output tile, split in two steps so the
-// next basis' coefficients can be in flight (cp.async) while this one is filtered:
-//   syn_load     copies the four subband tiles (with the filter halo, periodic wrap);
-//   syn_compute  filters along y then x and adds to acc[4], this thread's outputs
-//                out[r][c0 .. c0+3] with r = tid % 32, c0 = 4 (tid / 32).
-// Each subband tile is loaded as rows of 32 floats starting 8 columns left of the
-// tile's coefficient origin (16-byte aligned), covering every halo width.
-constexpr int kSRow = 36;                         // floats per staged row (16-byte aligned pitch)
-constexpr int kSTile = kCImax * kSRow;            // one subband tile
-constexpr int kS4 = 4 * kSTile;                   // one set of four subband tiles
-__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-
-template <int LF>
-__device__ __forceinline__ void syn_load(const float* __restrict__ cb, const float* __restrict__ apx, int n, int m,
-                                         int oy0, int ox0, float* __restrict__ s4) {
-  constexpr int half = LF / 2 - 1;
-  constexpr int CI = kTI / 2 + half;
-  const int hm = m >> 1;
-  const int ky0 = oy0 / 2 - half, kxa = ox0 / 2 - 8;     // kxa: 16-byte aligned start column
-  // CI rows x 8 chunks of 4 floats, for each of the four subbands (chunks never straddle the wrap).
-  for (int i = threadIdx.x; i < 4 * CI * 8; i += blockDim.x) {
-    const int sb = i / (CI * 8), rc = i - sb * (CI * 8);
-    const int r = rc >> 3, k = rc & 7;
-    const int Yk = wrap1(ky0 + r, hm), Xk = wrap1(kxa + 4 * k, hm);
-    const float* src;
-    if (sb == 0) src = apx ? apx + (size_t)Yk * hm + Xk : cb + (size_t)Yk * n + Xk;   // LL
-    else if (sb == 1) src = cb + (size_t)(hm + Yk) * n + Xk;                         // LH (x-low, y-high)
-    else if (sb == 2) src = cb + (size_t)Yk * n + hm + Xk;                           // HL (x-high, y-low)
-    else src = cb + (size_t)(hm + Yk) * n + hm + Xk;                                 // HH
-    cp_async16(s4 + sb * kSTile + r * kSRow + 4 * k, src);
-  }
-}
-
-template <int LF>
-__device__ __forceinline__ void syn_compute(const float* __restrict__ s4, float* __restrict__ s_lo,
-                                            float* __restrict__ s_hi, float acc[4]) {
-  constexpr int half = LF / 2 - 1;
-  constexpr int CI = kTI / 2 + half;
-  constexpr int b = LF / 2 - 1;
-  const float* s_ll = s4 + (8 - half);             // column c of the halo tile = staged column c + 8 - half
-  const float* s_lh = s4 + kSTile + (8 - half);
-  const float* s_hl = s4 + 2 * kSTile + (8 - half);
-  const float* s_hh = s4 + 3 * kSTile + (8 - half);
-  // Along y: lo[r][c] = sum_{j = r mod 2} h[j] ll[(r - j)/2 + half][c] + g[j] lh[...]; coefficient
-  // row r0/2 + i feeds output row r0 + t through tap j = t - 2 (i - half).
-  for (int u = threadIdx.x; u < CI * (kTI / 4); u += blockDim.x) {
-    const int c = u % CI, r0 = (u / CI) * 4;
-    float lo[4] = {0.f, 0.f, 0.f, 0.f}, hi[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int i = 0; i < half + 2; ++i) {
-      const int o = (r0 / 2 + i) * kSRow + c;
-      const float vll = s_ll[o], vlh = s_lh[o], vhl = s_hl[o], vhh = s_hh[o];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int j = t - 2 * (i - half);
-        if (j >= 0 && j < LF) {
-          lo[t] = fmaf(c_h[b][j], vll, fmaf(c_g[b][j], vlh, lo[t]));
-          hi[t] = fmaf(c_h[b][j], vhl, fmaf(c_g[b][j], vhh, hi[t]));
-        }
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      s_lo[(r0 + t) * kPs + c] = lo[t];
-      s_hi[(r0 + t) * kPs + c] = hi[t];
-    }
-  }
-  __syncthreads();
-  // Along x: warp w owns output columns 4w .. 4w+3 of all 32 rows (row = lane), so the
-  // 32 lanes read 32 different rows at an odd pitch (no bank conflicts).
-  const int r = threadIdx.x & 31, c0 = (threadIdx.x >> 5) * 4;
-#pragma unroll
-  for (int i = 0; i < half + 2; ++i) {
-    const float vlo = s_lo[r * kPs + c0 / 2 + i], vhi = s_hi[r * kPs + c0 / 2 + i];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int j = t - 2 * (i - half);
-      if (j >= 0 && j < LF) acc[t] = fmaf(c_h[b][j], vlo, fmaf(c_g[b][j], vhi, acc[t]));
-    }
-  }
-}
-
-
-__device__ __forceinline__ void syn_load_dispatch(int bi, const float* cb, const float* apx, int n, int m, int oy0,
-                                                  int ox0, float* s4) {
-#define PS_L(LFv) syn_load<LFv>(cb, apx, n, m, oy0, ox0, s4)
-  PS_SWITCH_LF(bi, PS_L)
-#undef PS_L
-}
-__device__ __forceinline__ void syn_compute_dispatch(int bi, const float* s4, float* s_lo, float* s_hi, float acc[4]) {
-#define PS_C(LFv) syn_compute<LFv>(s4, s_lo, s_hi, acc)
-  PS_SWITCH_LF(bi, PS_C)
-#undef PS_C
-}
-
-constexpr int kSynSmemFloats = 2 * kS4 + 2 * kTI * kPs;
-
-// Finest level (m = n): all eight bases plus Dirac summed in registers -> Psi A.
-// Basis bi+1's tiles are copied asynchronously while basis bi is filtered.
-__global__ void __launch_bounds__(256, 3) k_syn_fine(const float* __restrict__ coef, const float* __restrict__ approx_in,
-                                                     int coarsest, int n, float* __restrict__ out) {
-  __shared__ __align__(16) float sm_s[kSynSmemFloats];
-  float* s4b[2] = {sm_s, sm_s + kS4};
-  float* s_lo = sm_s + 2 * kS4;
-  float* s_hi = s_lo + kTI * kPs;
-  const int map = blockIdx.z;
-  const int tilesx = n / kTI;
-  const int oy0 = (blockIdx.x / tilesx) * kTI, ox0 = (blockIdx.x % tilesx) * kTI;
-  const int hm = n >> 1;
-  auto cbp = [&](int bi) { return coef + ((size_t)map * kBases + bi + 1) * (size_t)n * n; };
-  auto apxp = [&](int bi) {
-    return coarsest ? (const float*)nullptr : approx_in + ((size_t)map * kDb + bi) * (size_t)hm * hm;
-  };
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  syn_load_dispatch(0, cbp(0), apxp(0), n, n, oy0, ox0, s4b[0]);
-  cp_async_commit();
-  for (int bi = 0; bi < kDb; ++bi) {
-    if (bi + 1 < kDb) {
-      syn_load_dispatch(bi + 1, cbp(bi + 1), apxp(bi + 1), n, n, oy0, ox0, s4b[(bi + 1) & 1]);
-      cp_async_commit();
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncthreads();
-    syn_compute_dispatch(bi, s4b[bi & 1], s_lo, s_hi, acc);
-    __syncthreads();
-  }
-  const int r = threadIdx.x & 31, c0 = (threadIdx.x >> 5) * 4;
-  const size_t o = (size_t)(oy0 + r) * n + ox0 + c0;
-  const float4 d = *reinterpret_cast<const float4*>(coef + (size_t)map * kBases * n * n + o);
-  const float k = 1.0f / 3.0f;
-  *reinterpret_cast<float4*>(out + (size_t)map * n * n + o) =
-      make_float4((d.x + acc[0]) * k, (d.y + acc[1]) * k, (d.z + acc[2]) * k, (d.w + acc[3]) * k);
-}
-
 
 // ---------------------------------------------------------------------------
 // Synthesis for levels with output side m >= 64: 64 x 64 output tiles.
@@ -1247,174 +996,416 @@ __global__ void __launch_bounds__(256, 3) k_syn2_lv(const float* __restrict__ co
 
 static size_t fast_analysis_smem() { return (size_t)kAnaFloats * sizeof(float) + 16; }
 
-static size_t synthesis_smem(int TI) {
-  const int CI = TI / 2 + kMaxTaps / 2 - 1;
-  return (size_t)(4 * CI * CI + 2 * TI * CI) * sizeof(float);
-}
 
 // ---------------------------------------------------------------------------
-// Coarse levels in one launch. The analysis levels whose input side is at most
-// kTail (all levels for images of at most kTail), and the synthesis levels whose
-// output side is at most kTailSyn (from the coarsest up to level 2), each take a few
-// microseconds of work but cost one dependent launch each when tiled. Here one CTA
-// per (basis, map) keeps a whole level in shared memory and runs the levels back to
-// back; periodic boundaries are indices modulo the level side (a power of two).
-constexpr int kTail = 64;      // analysis: fused levels have input side <= kTail
-constexpr int kTailSyn = 32;   // synthesis: fused levels have output side <= kTailSyn (tiled is faster above)
-constexpr int kTailThreads = 512;
+// Small levels in one launch: the analysis levels whose input side is at most kSmall, and
+// the synthesis levels whose output side is at most kSmallSyn (for an image of side n <=
+// kSmall: every level of both). One CTA per (basis, map) keeps the whole subtree on chip:
+// its coefficients are one m0 x m0 block of the Mallat layout. These levels are bound by
+// latency, not by bytes: the block (and, for the dual update, its thresholds) is read once,
+// before the first level, the levels then run from shared memory in register strips of four
+// outputs, and the block is written once at the end.
+// 64 x 64, 4 levels, 4 maps (back-to-back launches): analysis 12.4 -> 10.8 us against one
+// scalar pass per tap with the coefficients read level by level; synthesis 41.4 -> 10.4 us
+// against the coarse levels in one launch and the eight bases one after another in the next.
+constexpr int kSmall = 64;
+constexpr int kSmallSyn = 32;     // above it (images larger than kSmall) the tiled synthesis is faster
+constexpr int kSmallThreads = 256;
+__host__ __device__ constexpr int small_pitch(int m) { return m + 20; }   // row pitch of a level's input (16 wrapped columns)
 
-// One analysis level of side m held in img (m x m, row-major): rows then columns,
-// epilogue on the three detail subbands (and on LL at the last level, else LL
-// replaces img as the next level's input, side m/2).
+// One analysis level of side m. img: m rows of pitch small_pitch(m), columns m .. m + 15
+// repeating the row's start (periodic). lo, hi: m rows of pitch hm + 4. The coefficients a
+// (and thresholds t in the dual mode) are m0 x m0 blocks; the results replace a. The
+// approximation replaces img in the layout of the next level.
 template <int LF>
-__device__ __forceinline__ void tail_ana_level(float* img, float* lo, float* hi, int m, int bi, int map, int n,
-                                               int last, float* coef, float* thr, int mode, float scale, float gamma,
-                                               float delta) {
+__device__ __forceinline__ void small_ana_level(float* __restrict__ img, float* __restrict__ lo, float* __restrict__ hi,
+                                                float* __restrict__ a, const float* __restrict__ t, int m, int m0,
+                                                int last, int mode, float scale, float gamma, float delta) {
   constexpr int b = LF / 2 - 1;
-  const int hm = m >> 1, mask = m - 1;
-  for (int u = threadIdx.x; u < m * hm; u += blockDim.x) {      // lo/hi[r][k] = sum_j h/g[j] img[r][2k + j]
-    const int r = u / hm, k = u - r * hm;
-    const float* row = img + r * m;
-    float a = 0.f, c = 0.f;
+  const int hm = m >> 1, mask = m - 1, P = small_pitch(m), Q = hm + 4, PN = small_pitch(hm);
+  auto epi = [&](float v, int o) {
+    if (mode == SARA_DUAL) a[o] = fminf(fmaxf(fmaf(scale, v, a[o]), -t[o]), t[o]);
+    else a[o] = mode == SARA_APPLY ? scale * v : gamma * delta / (delta + fabsf(scale * v));
+  };
+  if (hm >= 4) {
+    constexpr int NV = (LF + 6 + 3) / 4;   // 16-byte reads of the samples of four outputs
+    for (int u = threadIdx.x; u < m * (hm >> 2); u += kSmallThreads) {
+      const int r = u & mask, k0 = (u / m) * 4;
+      const float4* row = reinterpret_cast<const float4*>(img + r * P + 2 * k0);
+      float x[4 * NV];
 #pragma unroll
-    for (int j = 0; j < LF; ++j) {
-      const float v = row[(2 * k + j) & mask];
-      a = fmaf(c_h[b][j], v, a);
-      c = fmaf(c_g[b][j], v, c);
-    }
-    lo[u] = a;
-    hi[u] = c;
-  }
-  __syncthreads();
-  const size_t base = ((size_t)map * kBases + (bi + 1)) * (size_t)n * n;
-  for (int u = threadIdx.x; u < hm * hm; u += blockDim.x) {     // columns: rows 2 ky + j of lo/hi
-    const int ky = u / hm, kx = u - ky * hm;
-    float ll = 0.f, lh = 0.f, hl = 0.f, hh = 0.f;
+      for (int v = 0; v < NV; ++v) {
+        const float4 q = row[v];
+        x[4 * v] = q.x, x[4 * v + 1] = q.y, x[4 * v + 2] = q.z, x[4 * v + 3] = q.w;
+      }
+      // One chain per output, in the order of the taps: a scalar FMA does as much per clock
+      // as a packed one, and the coarse coefficients are the ones whose rounding shows most.
+      float l[4] = {0.f, 0.f, 0.f, 0.f}, h[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int j = 0; j < LF; ++j) {
-      const int y = (2 * ky + j) & mask;
-      const float a = lo[y * hm + kx], c = hi[y * hm + kx];
-      ll = fmaf(c_h[b][j], a, ll);
-      lh = fmaf(c_g[b][j], a, lh);
-      hl = fmaf(c_h[b][j], c, hl);
-      hh = fmaf(c_g[b][j], c, hh);
+      for (int j = 0; j < LF; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          l[q] = fmaf(c_h[b][j], x[2 * q + j], l[q]);
+          h[q] = fmaf(c_g[b][j], x[2 * q + j], h[q]);
+        }
+      *reinterpret_cast<float4*>(lo + r * Q + k0) = make_float4(l[0], l[1], l[2], l[3]);
+      *reinterpret_cast<float4*>(hi + r * Q + k0) = make_float4(h[0], h[1], h[2], h[3]);
     }
-    sara_epilogue(mode, hl, base + (size_t)ky * n + (hm + kx), coef, thr, scale, gamma, delta);         // x-high, y-low
-    sara_epilogue(mode, lh, base + (size_t)(hm + ky) * n + kx, coef, thr, scale, gamma, delta);         // x-low, y-high
-    sara_epilogue(mode, hh, base + (size_t)(hm + ky) * n + (hm + kx), coef, thr, scale, gamma, delta);
-    if (last) sara_epilogue(mode, ll, base + (size_t)ky * n + kx, coef, thr, scale, gamma, delta);
-    else img[u] = ll;   // img was fully consumed by the row pass before the barrier above
+    __syncthreads();
+    const int qs = hm >> 2;   // column quads
+    for (int u = threadIdx.x; u < hm * qs; u += kSmallThreads) {
+      const int ky = u / qs, kx = (u - ky * qs) * 4;
+      u64 ll0 = 0ull, ll1 = 0ull, lh0 = 0ull, lh1 = 0ull, hl0 = 0ull, hl1 = 0ull, hh0 = 0ull, hh1 = 0ull;
+#pragma unroll
+      for (int j = 0; j < LF; ++j) {
+        const int o = ((2 * ky + j) & mask) * Q + kx;
+        const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(lo + o);
+        const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(hi + o);
+        const u64 ph = cdup(c_hd[b][j]), pg = cdup(c_gd[b][j]);
+        ll0 = ffma2(ph, x.x, ll0);
+        ll1 = ffma2(ph, x.y, ll1);
+        lh0 = ffma2(pg, x.x, lh0);
+        lh1 = ffma2(pg, x.y, lh1);
+        hl0 = ffma2(ph, y.x, hl0);
+        hl1 = ffma2(ph, y.y, hl1);
+        hh0 = ffma2(pg, y.x, hh0);
+        hh1 = ffma2(pg, y.y, hh1);
+      }
+      auto epi4 = [&](float4 v, int o) {
+        float4* dst = reinterpret_cast<float4*>(a + o);
+        if (mode == SARA_DUAL) {
+          *dst = f4clamp(f4fma(scale, v, *dst), *reinterpret_cast<const float4*>(t + o));
+        } else if (mode == SARA_APPLY) {
+          *dst = make_float4(scale * v.x, scale * v.y, scale * v.z, scale * v.w);
+        } else {
+          const float gd = gamma * delta;
+          *dst = make_float4(gd / (delta + fabsf(scale * v.x)), gd / (delta + fabsf(scale * v.y)),
+                             gd / (delta + fabsf(scale * v.z)), gd / (delta + fabsf(scale * v.w)));
+        }
+      };
+      epi4(f4of(hl0, hl1), ky * m0 + hm + kx);            // x-high, y-low
+      epi4(f4of(lh0, lh1), (hm + ky) * m0 + kx);          // x-low, y-high
+      epi4(f4of(hh0, hh1), (hm + ky) * m0 + hm + kx);
+      const float4 ll = f4of(ll0, ll1);
+      if (last) {
+        epi4(ll, ky * m0 + kx);
+      } else {   // img was consumed by the row pass, before the barrier above
+        for (int x = kx; x < hm + 16; x += hm) *reinterpret_cast<float4*>(img + ky * PN + x) = ll;
+      }
+    }
+  } else {       // sides 4 and 2: a handful of outputs
+    for (int u = threadIdx.x; u < m * hm; u += kSmallThreads) {
+      const int r = u / hm, k = u - r * hm;
+      float s = 0.f, d = 0.f;
+#pragma unroll
+      for (int j = 0; j < LF; ++j) {
+        const float v = img[r * P + ((2 * k + j) & mask)];
+        s = fmaf(c_h[b][j], v, s);
+        d = fmaf(c_g[b][j], v, d);
+      }
+      lo[r * Q + k] = s;
+      hi[r * Q + k] = d;
+    }
+    __syncthreads();
+    for (int u = threadIdx.x; u < hm * hm; u += kSmallThreads) {
+      const int ky = u / hm, kx = u - ky * hm;
+      float ll = 0.f, lh = 0.f, hl = 0.f, hh = 0.f;
+#pragma unroll
+      for (int j = 0; j < LF; ++j) {
+        const int o = ((2 * ky + j) & mask) * Q + kx;
+        ll = fmaf(c_h[b][j], lo[o], ll);
+        lh = fmaf(c_g[b][j], lo[o], lh);
+        hl = fmaf(c_h[b][j], hi[o], hl);
+        hh = fmaf(c_g[b][j], hi[o], hh);
+      }
+      epi(hl, ky * m0 + hm + kx);
+      epi(lh, (hm + ky) * m0 + kx);
+      epi(hh, (hm + ky) * m0 + hm + kx);
+      if (last) epi(ll, ky * m0 + kx);
+      else img[ky * PN + kx] = ll;
+    }
   }
   __syncthreads();
 }
 
-// Analysis levels l0..L in one CTA per (basis, map) = (blockIdx.x, blockIdx.y). The
-// input of level l0 (side m0 <= kTail) is X (l0 = 1) or that level's approximation
-// scratch (layout [map][basis][m0][m0]).
-__global__ void __launch_bounds__(kTailThreads) k_ana_tail(const float* __restrict__ in, int l0, int L, int n,
-                                                           float* __restrict__ coef, float* __restrict__ thr, int mode,
-                                                           float scale, float gamma, float delta) {
+// Analysis levels l0..L (sides m0 = n >> (l0 - 1) <= kSmall and below); one CTA per (basis,
+// map) = (blockIdx.x, blockIdx.y). The input of level l0 is X (l0 = 1) or that level's
+// approximation scratch (layout [map][basis][m0][m0]).
+__global__ void __launch_bounds__(kSmallThreads) k_ana_small(const float* __restrict__ in, int l0, int L, int n,
+                                                             float* __restrict__ coef, float* __restrict__ thr,
+                                                             int mode, float scale, float gamma, float delta) {
   extern __shared__ float4 smt[];
-  float* img = reinterpret_cast<float*>(smt);
   const int bi = blockIdx.x, map = blockIdx.y;
-  const int m0 = n >> (l0 - 1);
-  float* lo = img + m0 * m0;
-  float* hi = lo + m0 * (m0 >> 1);
+  const int m0 = n >> (l0 - 1), q0 = m0 >> 2, P = small_pitch(m0), Q = (m0 >> 1) + 4;
+  float* img = reinterpret_cast<float*>(smt);
+  float* lo = img + m0 * P;
+  float* hi = lo + m0 * Q;
+  float* a = hi + m0 * Q;
+  float* t = a + m0 * m0;
   const float* src = l0 == 1 ? in + (size_t)map * n * n : in + ((size_t)map * kDb + bi) * (size_t)m0 * m0;
-  for (int i = threadIdx.x; i < m0 * m0 / 4; i += blockDim.x)
-    reinterpret_cast<float4*>(img)[i] = reinterpret_cast<const float4*>(src)[i];
+  const size_t base = ((size_t)map * kBases + (bi + 1)) * (size_t)n * n;
+  for (int u = threadIdx.x; u < m0 * q0; u += kSmallThreads) {
+    const int y = u / q0, x = (u - y * q0) * 4;
+    const float4 v = *reinterpret_cast<const float4*>(src + (size_t)y * m0 + x);
+    float4 va, vt;
+    if (mode == SARA_DUAL) {
+      va = *reinterpret_cast<const float4*>(coef + base + (size_t)y * n + x);
+      vt = *reinterpret_cast<const float4*>(thr + base + (size_t)y * n + x);
+    }
+    for (int xx = x; xx < m0 + 16; xx += m0) *reinterpret_cast<float4*>(img + y * P + xx) = v;
+    if (mode == SARA_DUAL) {
+      *reinterpret_cast<float4*>(a + 4 * u) = va;
+      *reinterpret_cast<float4*>(t + 4 * u) = vt;
+    }
+  }
   __syncthreads();
   for (int l = l0, m = m0; l <= L; ++l, m >>= 1) {
-#define PS_TA(LFv) tail_ana_level<LFv>(img, lo, hi, m, bi, map, n, l == L, coef, thr, mode, scale, gamma, delta)
+#define PS_TA(LFv) small_ana_level<LFv>(img, lo, hi, a, t, m, m0, l == L, mode, scale, gamma, delta)
     PS_SWITCH_LF(bi, PS_TA)
 #undef PS_TA
   }
+  float* dst = (mode == SARA_REWEIGHT ? thr : coef) + base;
+  for (int u = threadIdx.x; u < m0 * q0; u += kSmallThreads) {
+    const int y = u / q0, x = (u - y * q0) * 4;
+    *reinterpret_cast<float4*>(dst + (size_t)y * n + x) = *reinterpret_cast<const float4*>(a + 4 * u);
+  }
 }
 
-// One synthesis level to output side m: LL (hm x hm) in shared memory; the level's
-// detail subbands are first copied from the coefficient plane cb into det
-// (LH, HL, HH, each hm x hm); output into out (m x m).
+// One synthesis level to output side m in place: the block's top-left m x m part (pitch B:
+// approximation, then the details) becomes the m x m approximation of the next level. Along
+// y into column-major intermediates (pitch m + 4), along x in 4 x 4 output blocks, as in
+// syn2_ypass / syn2_xpass, with periodic indices.
 template <int LF>
-__device__ __forceinline__ void tail_syn_level(const float* LLs, const float* __restrict__ cb, int n, int m,
-                                               float* det, float* lo, float* hi, float* out) {
-  constexpr int b = LF / 2 - 1;
-  const int hm = m >> 1, hmask = hm - 1, hh2 = hm * hm;
-  for (int i = threadIdx.x; i < 3 * hh2; i += blockDim.x) {
-    const int sb = i / hh2, k = i - sb * hh2, r = k / hm, c = k - r * hm;
-    det[i] = sb == 0 ? cb[(size_t)(hm + r) * n + c] : (sb == 1 ? cb[(size_t)r * n + hm + c]
-                                                             : cb[(size_t)(hm + r) * n + hm + c]);
+__device__ __forceinline__ void small_syn_level(float* __restrict__ blk, int B, int m, float* __restrict__ loT,
+                                                float* __restrict__ hiT) {
+  constexpr int b = LF / 2 - 1, half = LF / 2 - 1;
+  const int hm = m >> 1, hmask = hm - 1, P = m + 4;
+  if (hm == 1) {   // side 2: rows r and columns c of the four outputs
+    if (threadIdx.x < 2) {
+      const int r = threadIdx.x;
+      float l = 0.f, h = 0.f;
+#pragma unroll
+      for (int j = 0; j < LF; ++j)
+        if ((j & 1) == r) {
+          l = fmaf(c_h[b][j], blk[0], fmaf(c_g[b][j], blk[B], l));
+          h = fmaf(c_h[b][j], blk[1], fmaf(c_g[b][j], blk[B + 1], h));
+        }
+      loT[r] = l;
+      hiT[r] = h;
+    }
+    __syncthreads();
+    if (threadIdx.x < 4) {
+      const int r = threadIdx.x >> 1, c = threadIdx.x & 1;
+      float v = 0.f;
+#pragma unroll
+      for (int j = 0; j < LF; ++j)
+        if ((j & 1) == c) v = fmaf(c_h[b][j], loT[r], fmaf(c_g[b][j], hiT[r], v));
+      blk[r * B + c] = v;
+    }
+    __syncthreads();
+    return;
+  }
+  const int ncp = hm >> 1;
+  for (int u = threadIdx.x; u < ncp * (m >> 2); u += kSmallThreads) {
+    const int rg = u / ncp, c = 2 * (u - rg * ncp);
+    u64 lo[4], hi[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) lo[t] = hi[t] = 0ull;
+#pragma unroll
+    for (int i = 0; i < half + 2; ++i) {
+      const int kr = (2 * rg + i - half) & hmask;
+      const u64 vll = *reinterpret_cast<const u64*>(blk + kr * B + c);
+      const u64 vlh = *reinterpret_cast<const u64*>(blk + (hm + kr) * B + c);
+      const u64 vhl = *reinterpret_cast<const u64*>(blk + kr * B + hm + c);
+      const u64 vhh = *reinterpret_cast<const u64*>(blk + (hm + kr) * B + hm + c);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int j = t - 2 * (i - half);
+        if (j >= 0 && j < LF) {
+          const u64 ph = cdup(c_hd[b][j]), pg = cdup(c_gd[b][j]);
+          lo[t] = ffma2(ph, vll, ffma2(pg, vlh, lo[t]));
+          hi[t] = ffma2(ph, vhl, ffma2(pg, vhh, hi[t]));
+        }
+      }
+    }
+    float l0[4], l1[4], h0[4], h1[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      f2unpack(lo[t], l0[t], l1[t]);
+      f2unpack(hi[t], h0[t], h1[t]);
+    }
+    *reinterpret_cast<float4*>(loT + c * P + 4 * rg) = make_float4(l0[0], l0[1], l0[2], l0[3]);
+    *reinterpret_cast<float4*>(loT + (c + 1) * P + 4 * rg) = make_float4(l1[0], l1[1], l1[2], l1[3]);
+    *reinterpret_cast<float4*>(hiT + c * P + 4 * rg) = make_float4(h0[0], h0[1], h0[2], h0[3]);
+    *reinterpret_cast<float4*>(hiT + (c + 1) * P + 4 * rg) = make_float4(h1[0], h1[1], h1[2], h1[3]);
   }
   __syncthreads();
-  // Along y: output row R takes coefficient rows (R - j)/2 (mod hm) through taps j = R mod 2.
-  for (int u = threadIdx.x; u < m * hm; u += blockDim.x) {
-    const int R = u / hm, c = u - R * hm;
-    float a = 0.f, d = 0.f;
+  const int nq = m >> 2;
+  for (int u = threadIdx.x; u < nq * nq; u += kSmallThreads) {
+    const int cg = u / nq, rq = u - cg * nq;
+    u64 acc[8];
 #pragma unroll
-    for (int j = 0; j < LF; ++j) {
-      if ((j & 1) != (R & 1)) continue;
-      const int kr = ((R - j) >> 1) & hmask;
-      const float vll = LLs[kr * hm + c];
-      const float vlh = det[kr * hm + c];
-      const float vhl = det[hh2 + kr * hm + c];
-      const float vhh = det[2 * hh2 + kr * hm + c];
-      a = fmaf(c_h[b][j], vll, fmaf(c_g[b][j], vlh, a));
-      d = fmaf(c_h[b][j], vhl, fmaf(c_g[b][j], vhh, d));
-    }
-    lo[u] = a;
-    hi[u] = d;
-  }
-  __syncthreads();
-  // Along x.
-  for (int u = threadIdx.x; u < m * m; u += blockDim.x) {
-    const int R = u / m, X = u - R * m;
-    float v = 0.f;
+    for (int q = 0; q < 8; ++q) acc[q] = 0ull;
 #pragma unroll
-    for (int j = 0; j < LF; ++j) {
-      if ((j & 1) != (X & 1)) continue;
-      const int kc = ((X - j) >> 1) & hmask;
-      v = fmaf(c_h[b][j], lo[R * hm + kc], fmaf(c_g[b][j], hi[R * hm + kc], v));
+    for (int i = 0; i < half + 2; ++i) {
+      const int o = ((2 * cg + i - half) & hmask) * P + 4 * rq;
+      const ulonglong2 vlo = *reinterpret_cast<const ulonglong2*>(loT + o);
+      const ulonglong2 vhi = *reinterpret_cast<const ulonglong2*>(hiT + o);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int j = t - 2 * (i - half);
+        if (j >= 0 && j < LF) {
+          const u64 ph = cdup(c_hd[b][j]), pg = cdup(c_gd[b][j]);
+          acc[2 * t] = ffma2(ph, vlo.x, ffma2(pg, vhi.x, acc[2 * t]));
+          acc[2 * t + 1] = ffma2(ph, vlo.y, ffma2(pg, vhi.y, acc[2 * t + 1]));
+        }
+      }
     }
-    out[u] = v;
+#pragma unroll
+    for (int rr = 0; rr < 4; ++rr) *reinterpret_cast<float4*>(blk + (4 * rq + rr) * B + 4 * cg) = syn2_row(acc, rr);
   }
   __syncthreads();
 }
 
-// Synthesis levels L..l1 (l1 >= 2, output side of level l1 <= kTail) in one CTA per
-// (basis, map); the level-l1 output goes to approx_out ([map][basis][m][m]).
-__global__ void __launch_bounds__(kTailThreads) k_syn_tail(const float* __restrict__ coef, int L, int l1, int n,
-                                                           float* __restrict__ approx_out) {
+// out (this CTA's share of the rows of a tile) = (Dirac + sum over the cluster's partial
+// tiles) / 3: the CTAs of a cluster hold the partial sums of their bases in their shared
+// memory (`part`, ts rows of pitch B); the CTA of rank r writes rows [r, r + 1) ts / NS.
+template <int NS>
+__device__ __forceinline__ void cluster_sum(const float* part, int B, int ts, const float* __restrict__ dirac,
+                                            float* __restrict__ out, int n) {
+  const int rank = blockIdx.x % NS, q = ts >> 2;
+  for (int u = threadIdx.x; u < ts / NS * q; u += blockDim.x) {
+    const int y = rank * (ts / NS) + u / q, x = 4 * (u % q);
+    const float4 d = *reinterpret_cast<const float4*>(dirac + (size_t)y * n + x);
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int r = 0; r < NS; ++r) {
+      const float4 v = ld_cluster4(part + y * B + x, r);
+      s = make_float4(s.x + v.x, s.y + v.y, s.z + v.z, s.w + v.w);
+    }
+    const float k3 = 1.0f / 3.0f;
+    *reinterpret_cast<float4*>(out + (size_t)y * n + x) =
+        make_float4((d.x + s.x) * k3, (d.y + s.y) * k3, (d.z + s.z) * k3, (d.w + s.w) * k3);
+  }
+}
+
+// Synthesis levels L..l1 of one (basis, map) = (blockIdx.x, blockIdx.y); output side of level
+// l1 at most kSmall. FINEST (l1 = 1): the eight CTAs of a map are a cluster and sum their
+// bases and the Dirac part into Psi A; else the level-l1 output goes to approx_out
+// ([map][basis][m][m]).
+template <bool FINEST>
+__device__ __forceinline__ void syn_small(const float* __restrict__ coef, int L, int l1, int n,
+                                          float* __restrict__ dst) {
   extern __shared__ float4 smt[];
   const int bi = blockIdx.x, map = blockIdx.y;
-  const int mmax = n >> (l1 - 1);
-  float* bufA = reinterpret_cast<float*>(smt);          // mmax^2
-  float* bufB = bufA + mmax * mmax;                     // mmax^2 / 4
-  float* lo = bufB + mmax * mmax / 4;                   // mmax x mmax/2
-  float* hi = lo + mmax * (mmax >> 1);
-  float* det = hi + mmax * (mmax >> 1);                 // 3 x (mmax/2)^2
-  const float* cb = coef + ((size_t)map * kBases + bi + 1) * (size_t)n * n;
-  const int s0 = n >> L;                                // coarsest approximation side
-  // Level l writes bufA when l - l1 is even (the last level, the largest output, lands in
-  // bufA), so the coarsest approximation starts in the other buffer.
-  float* cur = (((L - l1) & 1) == 0) ? bufB : bufA;
-  for (int i = threadIdx.x; i < s0 * s0; i += blockDim.x) cur[i] = cb[(size_t)(i / s0) * n + (i % s0)];
+  const int m0 = n >> (l1 - 1), q0 = m0 >> 2, Bp = m0 + 4;
+  float* blk = reinterpret_cast<float*>(smt);
+  float* loT = blk + m0 * Bp;
+  float* hiT = loT + (m0 >> 1) * (m0 + 4);
+  const float* cmap = coef + (size_t)map * kBases * n * n;
+  const float* cb = cmap + (size_t)(bi + 1) * n * n;
+  for (int u = threadIdx.x; u < m0 * q0; u += kSmallThreads) {
+    const int y = u / q0, x = (u - y * q0) * 4;
+    *reinterpret_cast<float4*>(blk + y * Bp + x) = *reinterpret_cast<const float4*>(cb + (size_t)y * n + x);
+  }
   __syncthreads();
   for (int l = L; l >= l1; --l) {
     const int m = n >> (l - 1);
-    float* nxt = (cur == bufA) ? bufB : bufA;
-#define PS_TS(LFv) tail_syn_level<LFv>(cur, cb, n, m, det, lo, hi, nxt)
+#define PS_TS(LFv) small_syn_level<LFv>(blk, Bp, m, loT, hiT)
     PS_SWITCH_LF(bi, PS_TS)
 #undef PS_TS
-    cur = nxt;
   }
-  float* dst = approx_out + ((size_t)map * kDb + bi) * (size_t)mmax * mmax;
-  for (int i = threadIdx.x; i < mmax * mmax / 4; i += blockDim.x)
-    reinterpret_cast<float4*>(dst)[i] = reinterpret_cast<const float4*>(cur)[i];
+  if (FINEST) {
+    cluster_barrier();
+    cluster_sum<kDb>(blk, Bp, m0, cmap, dst + (size_t)map * n * n, n);
+    cluster_barrier();   // the partial images stay until every CTA has read them
+  } else {
+    float* o = dst + ((size_t)map * kDb + bi) * (size_t)m0 * m0;
+    for (int u = threadIdx.x; u < m0 * q0; u += kSmallThreads) {
+      const int y = u / q0, x = (u - y * q0) * 4;
+      *reinterpret_cast<float4*>(o + 4 * u) = *reinterpret_cast<const float4*>(blk + y * Bp + x);
+    }
+  }
+}
+__global__ void __cluster_dims__(kDb, 1, 1) __launch_bounds__(kSmallThreads)
+    k_syn_small(const float* __restrict__ coef, int L, int n, float* __restrict__ out) {
+  syn_small<true>(coef, L, 1, n, out);
+}
+__global__ void __launch_bounds__(kSmallThreads)
+    k_syn_tail(const float* __restrict__ coef, int L, int l1, int n, float* __restrict__ approx_out) {
+  syn_small<false>(coef, L, l1, n, approx_out);
 }
 
-static size_t ana_tail_smem(int m0) { return (size_t)2 * m0 * m0 * sizeof(float); }
-static size_t syn_tail_smem(int mmax) {
-  return (size_t)(mmax * mmax + mmax * mmax / 4 + mmax * mmax + 3 * (mmax / 2) * (mmax / 2)) * sizeof(float);
+static size_t ana_small_smem(int m0) {
+  return (size_t)(m0 * small_pitch(m0) + 2 * m0 * (m0 / 2 + 4) + 2 * m0 * m0) * sizeof(float);
 }
+static size_t syn_small_smem(int m0) { return (size_t)(m0 * (m0 + 4) + m0 * (m0 + 4)) * sizeof(float); }
+
+// The finest level with the bases of a tile spread over the NS CTAs of a cluster (NS = 8:
+// one basis each; NS = 4: db(r+1) and db(8-r), 18 taps in all for every rank), for images
+// with too few 64 x 64 tiles to fill the chip: the CTA runs its bases through one staging
+// set, leaves its partial tile in shared memory, and the cluster adds the partial tiles.
+template <int NS>
+__global__ void __cluster_dims__(NS, 1, 1) __launch_bounds__(256, 4)
+    k_syn2_split(const float* __restrict__ coef, const float* __restrict__ approx_in, int coarsest, int n,
+                 float* __restrict__ out, int* err, const __grid_constant__ SaraTma tm) {
+  extern __shared__ __align__(128) float4 sm2[];
+  __shared__ int failed;
+  float* const s4 = reinterpret_cast<float*>(sm2);
+  float* loT = s4 + kC2Set;
+  float* hiT = loT + kLoSize;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(hiT + kLoSize);
+  const int rank = blockIdx.x % NS, tile = blockIdx.x / NS, map = blockIdx.z, tilesx = n / kT2;
+  const int oy0 = (tile / tilesx) * kT2, ox0 = (tile % tilesx) * kT2, hm = n >> 1;
+  const float* cmap = coef + (size_t)map * kBases * n * n;
+  if (threadIdx.x == 0) {
+    failed = 0;
+    mbar_init(bar, 1);
+  }
+  __syncthreads();
+  auto issue = [&](int bi) {
+    syn2_issue_t(tm, (map * kBases + bi + 1) * n, (map * kDb + bi) * hm, bi, cmap + (size_t)(bi + 1) * n * n,
+                 coarsest ? nullptr : approx_in + ((size_t)map * kDb + bi) * (size_t)hm * hm, n, hm, oy0, ox0, s4, bar);
+  };
+  u64 acc[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) acc[q] = 0ull;
+  constexpr int NB = kDb / NS;
+  const int b_of[2] = {NS == kDb ? rank : kDb - 1 - rank, rank};
+  issue(b_of[0]);
+  for (int i = 0; i < NB; ++i) {
+    const bool ok = mbar_wait(bar, i & 1);
+    if (__syncthreads_or(!ok)) {   // the whole cluster's tile is left unwritten; its barriers are still met
+      if (threadIdx.x == 0) failed = 1;
+      syn2_abort(bar, i & 1, nullptr, 0u, err);
+      break;
+    }
+    const int bi = b_of[i];
+    syn2_ypass_dispatch(bi, s4, loT, hiT);
+    __syncthreads();
+    if (i + 1 < NB) issue(b_of[1]);
+    syn2_xpass_dispatch(bi, loT, hiT, acc);
+  }
+  // The staging set is free (the last y-pass has read it): it takes the partial tile.
+  const int rq = threadIdx.x & 15, cg = threadIdx.x >> 4;
+#pragma unroll
+  for (int rr = 0; rr < 4; ++rr)
+    *reinterpret_cast<float4*>(s4 + (4 * rq + rr) * kLoPitch + 4 * cg) = syn2_row(acc, rr);
+  cluster_barrier();
+  int bad = 0;
+#pragma unroll
+  for (int r = 0; r < NS; ++r) bad |= ld_cluster(&failed, r);
+  const size_t o = (size_t)oy0 * n + ox0;
+  if (!bad) cluster_sum<NS>(s4, kLoPitch, kT2, cmap + o, out + (size_t)map * n * n + o, n);
+  cluster_barrier();   // the partial tiles stay until every CTA has read them
+}
+static_assert(kT2 * kLoPitch <= kC2Set, "a partial tile fits the staging set");
+// (Tile, map) units up to which the bases are split. Eight ways while all 8 units' CTAs are
+// resident at once (4 CTAs on each of 152 SMs), four ways while the four-way grid is at most
+// two such waves; beyond that there are tiles enough, and the unsplit forms win. All of Psi,
+// 4 maps, 4 levels, us unsplit / 4 / 8: 128^2 (16 units) 43 / 27 / 25, 256^2 (64) 51 / 37 / 36,
+// 512^2 (256) 64 / 54 / 62, 1024^2 (1024, 6 levels) 133 / 147 / 182.
+constexpr int kSplit8Units = 76, kSplit4Units = 304;
 
 // ---- tensor maps (host side). cuTensorMapEncodeTiled comes from the driver through the
 // runtime's entry-point query, so the library links against the runtime alone; without it
@@ -1480,9 +1471,7 @@ static SaraTma synthesis_maps(const float* coef, const float* approx_in, int m, 
 cudaError_t configure_nufft_kernels();
 
 cudaError_t configure_kernels() {
-  cudaError_t e = cudaFuncSetAttribute((const void*)k_synthesis, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)synthesis_smem(32));
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   for (const void* f : {(const void*)k_ana_l1, (const void*)k_ana_lv}) {
     e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fast_analysis_smem());
     if (e != cudaSuccess) return e;
@@ -1518,12 +1507,15 @@ cudaError_t configure_kernels() {
   e = cudaFuncSetAttribute((const void*)k_ana_pers, cudaFuncAttributePreferredSharedMemoryCarveout,
                            cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute((const void*)k_ana_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)ana_tail_smem(kTail));
+  e = cudaFuncSetAttribute((const void*)k_ana_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)ana_small_smem(kSmall));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute((const void*)k_syn_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)syn_tail_smem(kTailSyn));
-  if (e != cudaSuccess) return e;
+  for (const void* f : {(const void*)k_syn2_split<8>, (const void*)k_syn2_split<4>}) {
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)syn2_smem(1));
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+  }
   return configure_nufft_kernels();
 }
 
@@ -1534,11 +1526,11 @@ cudaError_t sara_analysis(Handle* h, const float* X, float* coef, float* thr, in
   float* buf[2] = {h->approx, h->approx2};
   int lt = L + 1;                                   // first level of the fused tail
   for (int l = 1; l <= L; ++l)
-    if ((n >> (l - 1)) <= kTail) {
+    if ((n >> (l - 1)) <= kSmall) {
       lt = l;
       break;
     }
-  // Levels with input side > kTail: tiled, one launch per level (half side >= 128).
+  // Levels with input side > kSmall: tiled, one launch per level (half side >= 128).
   for (int l = 1; l < lt; ++l) {
     const int m = n >> (l - 1), hm = m / 2;
     const dim3 grid((hm / kTO) * (hm / kTO), kDb, nmaps);
@@ -1592,8 +1584,8 @@ cudaError_t sara_analysis(Handle* h, const float* X, float* coef, float* thr, in
   }
   if (lt <= L) {
     const float* in = lt == 1 ? X : buf[(lt - 2) & 1];
-    k_ana_tail<<<dim3(kDb, nmaps), kTailThreads, ana_tail_smem(n >> (lt - 1)), h->stream>>>(in, lt, L, n, coef, thr,
-                                                                                         mode, scale, gamma, delta);
+    k_ana_small<<<dim3(kDb, nmaps), kSmallThreads, ana_small_smem(n >> (lt - 1)), h->stream>>>(in, lt, L, n, coef, thr,
+                                                                                            mode, scale, gamma, delta);
     if (lt == 1 && fine_done) {
       const cudaError_t e = cudaEventRecord(fine_done, h->stream);
       if (e != cudaSuccess) return e;
@@ -1609,46 +1601,51 @@ static cudaError_t synthesis_levels(cudaStream_t stream, int n, int L, const flo
                                     float* approx1, int nmaps, int* err, int variant,
                                     cudaEvent_t fine_start = nullptr) {
   float* buf[2] = {approx0, approx1};
+  if (n <= kSmall) {
+    if (fine_start) {
+      const cudaError_t e = cudaEventRecord(fine_start, stream);
+      if (e != cudaSuccess) return e;
+    }
+    k_syn_small<<<dim3(kDb, nmaps), kSmallThreads, syn_small_smem(n), stream>>>(coef, L, n, out);
+    return cudaGetLastError();
+  }
   int lt = 0;                                       // lowest level of the fused tail (>= 2), 0: none
   for (int l = 2; l <= L; ++l)
-    if ((n >> (l - 1)) <= kTailSyn) {
+    if ((n >> (l - 1)) <= kSmallSyn) {
       lt = l;
       break;
     }
   if (lt)
-    k_syn_tail<<<dim3(kDb, nmaps), kTailThreads, syn_tail_smem(n >> (lt - 1)), stream>>>(coef, L, lt, n,
-                                                                                      buf[(lt - 1) & 1]);
-  for (int l = lt ? lt - 1 : L; l >= 1; --l) {
-    const int m = n >> (l - 1);
-    const int TI = m < 32 ? m : 32;
-    const int tiles = (m / TI) * (m / TI);
+    k_syn_tail<<<dim3(kDb, nmaps), kSmallThreads, syn_small_smem(n >> (lt - 1)), stream>>>(coef, L, lt, n,
+                                                                                         buf[(lt - 1) & 1]);
+  for (int l = lt ? lt - 1 : L; l >= 1; --l) {      // every side m >= 64 here
+    const int m = n >> (l - 1), tiles = (m / kT2) * (m / kT2);
     const float* ain = (l == L) ? nullptr : buf[l & 1];
-    float* aout = (l == 1) ? nullptr : buf[(l - 1) & 1];
-    if (l == 1 && fine_start) {
+    const SaraTma tm = synthesis_maps(coef, ain, m, n, nmaps);
+    if (l > 1) {
+      k_syn2_lv<<<dim3(tiles, nmaps, kDb), 256, syn2_smem(1), stream>>>(coef, ain, l == L, m, n, buf[(l - 1) & 1], err,
+                                                                        tm);
+      continue;
+    }
+    if (fine_start) {
       const cudaError_t e = cudaEventRecord(fine_start, stream);
       if (e != cudaSuccess) return e;
     }
-    const SaraTma tm = m >= kT2 ? synthesis_maps(coef, ain, m, n, nmaps) : SaraTma{};
-    if (m >= kT2 && l == 1) {
-      const dim3 grid((m / kT2) * (m / kT2), 1, nmaps);
-      if (variant == 2) {
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int units = (int)(grid.x * grid.z);
-        k_syn2_fine_pers<<<std::min(units, 4 * std::max(1, sms)), 256, syn2_smem(1), stream>>>(coef, ain, l == L, n,
-                                                                                              out, err, nmaps, tm);
-      } else if (variant == 1) k_syn2_fine<1><<<grid, 256, syn2_smem(1), stream>>>(coef, ain, l == L, n, out, err, tm);
-      else k_syn2_fine<2><<<grid, 256, syn2_smem(2), stream>>>(coef, ain, l == L, n, out, err, tm);
-    } else if (m >= kT2) {
-      k_syn2_lv<<<dim3((m / kT2) * (m / kT2), nmaps, kDb), 256, syn2_smem(1), stream>>>(coef, ain, l == L, m, n, aout,
-                                                                                     err, tm);
-    } else if (m >= kTI && l == 1) {
-      k_syn_fine<<<dim3(tiles, 1, nmaps), 256, 0, stream>>>(coef, ain, l == L, n, out);
-    } else {
-      dim3 grid(tiles, l == 1 ? 1 : kDb, nmaps);
-      k_synthesis<<<grid, 256, synthesis_smem(TI), stream>>>(coef, ain, l == L, m, TI, n, l == 1, aout, out);
-    }
+    const int units = tiles * nmaps;
+    if (units <= kSplit8Units)
+      k_syn2_split<8><<<dim3(8 * tiles, 1, nmaps), 256, syn2_smem(1), stream>>>(coef, ain, l == L, n, out, err, tm);
+    else if (units <= kSplit4Units)
+      k_syn2_split<4><<<dim3(4 * tiles, 1, nmaps), 256, syn2_smem(1), stream>>>(coef, ain, l == L, n, out, err, tm);
+    else if (variant == 2) {
+      int dev = 0, sms = 0;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      k_syn2_fine_pers<<<std::min(units, 4 * std::max(1, sms)), 256, syn2_smem(1), stream>>>(coef, ain, l == L, n, out,
+                                                                                            err, nmaps, tm);
+    } else if (variant == 1)
+      k_syn2_fine<1><<<dim3(tiles, 1, nmaps), 256, syn2_smem(1), stream>>>(coef, ain, l == L, n, out, err, tm);
+    else
+      k_syn2_fine<2><<<dim3(tiles, 1, nmaps), 256, syn2_smem(2), stream>>>(coef, ain, l == L, n, out, err, tm);
   }
   return cudaGetLastError();
 }
