@@ -123,7 +123,6 @@ static bool misaligned(const void* p, int device_ptrs) { return device_ptrs && p
     if (misaligned((p), (dp))) return fail((h), PS_EINVAL, std::string(what) + ": device pointer not 16-byte aligned"); \
   } while (0)
 
-static int sweep_blocks_host(int N) { return (N + 1023) / 1024; }
 
 static void free_vis(Handle* h) {
   const size_t M = h->M;
@@ -375,7 +374,7 @@ const char* ps_last_error(const ps_handle* h) { return h ? h->err.c_str() : g_cr
 int64_t ps_estimate_bytes(int32_t n, int32_t levels, int64_t M) {
   if (n < 16 || n > 2048 || !is_pow2(n) || levels < 1 || (n % (1 << levels)) != 0 || M < 0) return 0;
   const int64_t N = (int64_t)n * n, K = 2 * (int64_t)n;
-  const int64_t img = (28 + 72 + 16) * N * 4 + (8 * (int64_t)sweep_blocks_host((int)N) + 1024) * 8;
+  const int64_t img = (28 + 72 + 16) * N * 4 + (8 * (int64_t)ps::sweep_blocks((int)N) + 1024) * 8;
   const int64_t vis = M * (3 * 32 + 16 + 4 + 64) + (M / ps::kChunk + 64) * 24 + M / 2;   // + item and chunk lists
   const int64_t grid = 2 * (int64_t)n * K * 16 + 48 * K * K + K * 12 + (int64_t)n * 4;
   return img + vis + grid;
@@ -467,7 +466,7 @@ ps_status ps_create(const ps_config* cfg, void* cuda_stream, ps_handle** out) {
     return bail(PS_ECUDA);
   }
   const size_t N = h->N;
-  h->red_cap = 8 * sweep_blocks_host((int)N) + 1024;
+  h->red_cap = 8 * ps::sweep_blocks((int)N) + 1024;
   bool ok = dalloc(h, &h->S, 4 * N) == cudaSuccess && dalloc(h, &h->Z, 2 * N) == cudaSuccess &&
             dalloc(h, &h->C, 4 * N) == cudaSuccess && dalloc(h, &h->D, 2 * N) == cudaSuccess &&
             dalloc(h, &h->Xb, 4 * N) == cudaSuccess && dalloc(h, &h->PsiA, 4 * N) == cudaSuccess &&
@@ -1131,7 +1130,7 @@ ps_status ps_get_params(ps_handle* h, double* tau, double* rho1, double* rho2, d
 // relative-change partials (FP64) and writes the 8 sums and the device flags straight into the
 // mapped host buffer relc_host (no copy), and the event that marks them written.
 static ps_status relc_enqueue(Handle* h) {
-  CK(h, ps::relc_sums(h, sweep_blocks_host(h->N), h->relc_dev));
+  CK(h, ps::relc_sums(h, ps::sweep_blocks(h->N), h->relc_dev));
   CK(h, cudaEventRecord(h->relc_ev, h->stream));
   h->relc_pending = true;
   return PS_OK;

@@ -167,6 +167,7 @@ cudaError_t sara_analysis(Handle* h, const float* X, float* coef, float* thr, in
 cudaError_t sara_synthesis(Handle* h, const float* coef, float* out, cudaEvent_t fine_start = nullptr);
 
 // Elementwise / reductions (prox.cu).
+int sweep_blocks(int N);   // CTAs of the per-pixel sweep (8 FP64 partials each)
 cudaError_t primal_sweep(Handle* h);
 cudaError_t dirac_apply(Handle* h, const float* X, float* coef, float* thr, int mode,
                         float scale, float gamma, float delta);

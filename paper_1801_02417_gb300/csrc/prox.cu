@@ -16,7 +16,6 @@
 namespace ps {
 
 constexpr int kSweepThreads = 256;
-constexpr int kSweepPix = 4;   // pixels per thread
 
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
@@ -56,20 +55,35 @@ __device__ __forceinline__ void proj_e2(float r1, float r2, float r3, float d, f
   }
 }
 
-__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
-__device__ __forceinline__ float comp(const float4& v, int k) { return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w)); }
-__device__ __forceinline__ void setc(float4& v, int k, float x) {
-  if (k == 0) v.x = x;
-  else if (k == 1) v.y = x;
-  else if (k == 2) v.z = x;
-  else v.w = x;
+// P = 1 or 2 consecutive floats of a plane as one load or store.
+template <int P>
+struct Pix {
+  float v[P];
+};
+template <int P>
+__device__ __forceinline__ Pix<P> ldp(const float* p) {
+  Pix<P> r;
+  if constexpr (P == 1) {
+    r.v[0] = *p;
+  } else {
+    const float2 q = *reinterpret_cast<const float2*>(p);
+    r.v[0] = q.x, r.v[1] = q.y;
+  }
+  return r;
+}
+template <int P>
+__device__ __forceinline__ void stp(float* p, const Pix<P>& r) {
+  if constexpr (P == 1) *p = r.v[0];
+  else *reinterpret_cast<float2*>(p) = make_float2(r.v[0], r.v[1]);
 }
 
-// One thread = four consecutive pixels (float4 on every plane). grid.y indexes the problems
+// One thread = P consecutive pixels of every plane. grid.y indexes the problems
 // of a batch's size class, whose arrays follow one another (S, C, Xb, PsiA, Adj: 4 N floats
 // each; Z, D: 2 N; A, T: 4 cstride; partials: part_stride doubles); one problem: grid.y = 1.
-__global__ void __launch_bounds__(kSweepThreads, 3) k_primal(
+// Every load of the thread is issued before the first value is used: a small image is one
+// round trip to memory.
+template <int P>
+__global__ void __launch_bounds__(kSweepThreads) k_primal(
     int N, int mode, float tau, float rho1, float rho3, float* __restrict__ S, float* __restrict__ Z,
     float* __restrict__ C, float* __restrict__ D, const float* __restrict__ PsiA, const float* __restrict__ Adj,
     float* __restrict__ Xb, float* __restrict__ A, const float* __restrict__ T, size_t cstride,
@@ -89,109 +103,115 @@ __global__ void __launch_bounds__(kSweepThreads, 3) k_primal(
     part += p * part_stride;
   }
   float dss[4] = {0.f, 0.f, 0.f, 0.f}, ss[4] = {0.f, 0.f, 0.f, 0.f};
-  const int i = 4 * (blockIdx.x * kSweepThreads + threadIdx.x);
+  const int i = P * (blockIdx.x * kSweepThreads + threadIdx.x);
   const float inv_r3 = 1.0f / rho3;
   const float r1_3 = rho1 * (1.0f / 3.0f);
+  const bool tv = tv_mode(mode), con = constrained_mode(mode), sara = mode != PS_NNLS && !tv;
+  const bool split = mode == PS_POLARIZED || mode == PS_TV || mode == PS_L1TV;   // epigraph split (Alg. 1 / Alg. 3)
   if (i < N) {
-    float4 xb[4];
+    Pix<P> g[4], q[4], c[4], so[4], t[4], a[4], z[2], d[2];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const size_t o = (size_t)c * N + i;
-      float4 g = ld4(Adj + o);
-      // TV modes (Algorithm 3 step 3): Adj holds phi^dagger(Y - phi(S)), so the data
-      // gradient 1/2 phi^dagger(phi(S) - Y) is -Adj / 2.
-      if (tv_mode(mode)) g = make_float4(-0.5f * g.x, -0.5f * g.y, -0.5f * g.z, -0.5f * g.w);
-      if (mode != PS_NNLS) {
-        const float4 p = ld4(PsiA + o);
-        g = make_float4(g.x + p.x, g.y + p.y, g.z + p.z, g.w + p.w);
-      }
-      if (constrained_mode(mode)) {
-        const float4 q = ld4(C + o);
-        g = make_float4(g.x + q.x, g.y + q.y, g.z + q.z, g.w + q.w);
-      }
-      const float4 so = ld4(S + o);
-      float4 sn = make_float4(so.x - tau * g.x, so.y - tau * g.y, so.z - tau * g.z, so.w - tau * g.w);   // step 3
-      if (!constrained_mode(mode) && c == 0)                                                          // P_U'
-        sn = make_float4(fmaxf(sn.x, 0.f), fmaxf(sn.y, 0.f), fmaxf(sn.z, 0.f), fmaxf(sn.w, 0.f));
-      xb[c] = make_float4(2.f * sn.x - so.x, 2.f * sn.y - so.y, 2.f * sn.z - so.z, 2.f * sn.w - so.w);
-      dss[c] += (sn.x - so.x) * (sn.x - so.x) + (sn.y - so.y) * (sn.y - so.y) + (sn.z - so.z) * (sn.z - so.z) +
-                (sn.w - so.w) * (sn.w - so.w);
-      ss[c] += so.x * so.x + so.y * so.y + so.z * so.z + so.w * so.w;
-      st4(S + o, sn);
-      st4(Xb + o, xb[c]);
-      if (mode != PS_NNLS && !tv_mode(mode)) {                          // Dirac part of steps 5-6
-        const size_t ao = (size_t)c * cstride + i;
-        const float4 t = ld4(T + ao), a = ld4(A + ao);
-        st4(A + ao, make_float4(fminf(fmaxf(fmaf(r1_3, xb[c].x, a.x), -t.x), t.x),
-                                fminf(fmaxf(fmaf(r1_3, xb[c].y, a.y), -t.y), t.y),
-                                fminf(fmaxf(fmaf(r1_3, xb[c].z, a.z), -t.z), t.z),
-                                fminf(fmaxf(fmaf(r1_3, xb[c].w, a.w), -t.w), t.w)));
+    for (int k = 0; k < 4; ++k) {
+      const size_t o = (size_t)k * N + i;
+      g[k] = ldp<P>(Adj + o);
+      so[k] = ldp<P>(S + o);
+      if (mode != PS_NNLS) q[k] = ldp<P>(PsiA + o);
+      if (con) c[k] = ldp<P>(C + o);
+      if (sara) {
+        t[k] = ldp<P>(T + (size_t)k * cstride + i);
+        a[k] = ldp<P>(A + (size_t)k * cstride + i);
       }
     }
-    if (mode == PS_POLARIZED || mode == PS_TV || mode == PS_L1TV) {   // epigraph split (Alg. 1 / Alg. 3)
-      const float4 z1o = ld4(Z + i), z2o = ld4(Z + (size_t)N + i);
-      const float4 d1o = ld4(D + i), d2o = ld4(D + (size_t)N + i);
-      float4 c0 = ld4(C + i), c1 = ld4(C + (size_t)N + i), c2 = ld4(C + 2 * (size_t)N + i),
-             c3 = ld4(C + 3 * (size_t)N + i);
-      float4 z1n, z2n, d1n, d2n;
+    if (split) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        // Step 4: Z = P_V(Z - tau D).
-        const float za = comp(z1o, k), zb = comp(z2o, k);
-        float z1 = za - tau * comp(d1o, k), z2 = zb - tau * comp(d2o, k);
-        if (z1 + z2 > 0.f) {
-          const float a = 0.5f * (z1 - z2);
-          z2 = 0.5f * (z2 - z1);
-          z1 = a;
+      for (int k = 0; k < 2; ++k) {
+        z[k] = ldp<P>(Z + (size_t)k * N + i);
+        d[k] = ldp<P>(D + (size_t)k * N + i);
+      }
+    }
+    Pix<P> xb[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const size_t o = (size_t)k * N + i;
+      Pix<P> sn, an;
+#pragma unroll
+      for (int e = 0; e < P; ++e) {
+        // TV modes (Algorithm 3 step 3): Adj holds phi^dagger(Y - phi(S)), so the data
+        // gradient 1/2 phi^dagger(phi(S) - Y) is -Adj / 2.
+        float gr = tv ? -0.5f * g[k].v[e] : g[k].v[e];
+        if (mode != PS_NNLS) gr += q[k].v[e];
+        if (con) gr += c[k].v[e];
+        const float s0 = so[k].v[e];
+        float s1 = s0 - tau * gr;                                  // step 3
+        if (!con && k == 0) s1 = fmaxf(s1, 0.f);                   // P_U'
+        const float x = 2.f * s1 - s0, ds = s1 - s0;
+        sn.v[e] = s1;
+        xb[k].v[e] = x;
+        dss[k] += ds * ds;
+        ss[k] += s0 * s0;
+        if (sara) {                                                // Dirac part of steps 5-6
+          const float th = t[k].v[e];
+          an.v[e] = fminf(fmaxf(fmaf(r1_3, x, a[k].v[e]), -th), th);
         }
-        setc(z1n, k, z1);
-        setc(z2n, k, z2);
+      }
+      stp<P>(S + o, sn);
+      stp<P>(Xb + o, xb[k]);
+      if (sara) stp<P>(A + (size_t)k * cstride + i, an);
+    }
+    if (split) {
+#pragma unroll
+      for (int e = 0; e < P; ++e) {
+        // Step 4: Z = P_V(Z - tau D).
+        const float za = z[0].v[e], zb = z[1].v[e];
+        float z1 = za - tau * d[0].v[e], z2 = zb - tau * d[1].v[e];
+        if (z1 + z2 > 0.f) {
+          const float h = 0.5f * (z1 - z2);
+          z2 = 0.5f * (z2 - z1);
+          z1 = h;
+        }
+        z[0].v[e] = z1;
+        z[1].v[e] = z2;
         const float zb1 = 2.f * z1 - za, zb2 = 2.f * z2 - zb;
         // Steps 9-12.
-        const float ct0 = comp(c0, k) + rho3 * comp(xb[0], k), ct1 = comp(c1, k) + rho3 * comp(xb[1], k);
-        const float ct2 = comp(c2, k) + rho3 * comp(xb[2], k), ct3 = comp(c3, k) + rho3 * comp(xb[3], k);
-        const float dt1 = comp(d1o, k) + rho3 * zb1, dt2 = comp(d2o, k) + rho3 * zb2;
+        const float ct0 = c[0].v[e] + rho3 * xb[0].v[e], ct1 = c[1].v[e] + rho3 * xb[1].v[e];
+        const float ct2 = c[2].v[e] + rho3 * xb[2].v[e], ct3 = c[3].v[e] + rho3 * xb[3].v[e];
+        const float dt1 = d[0].v[e] + rho3 * zb1, dt2 = d[1].v[e] + rho3 * zb2;
         float pc, pd;
         proj_e1(ct0 * inv_r3, dt1 * inv_r3, pc, pd);
-        setc(c0, k, ct0 - rho3 * pc);
-        setc(d1n, k, dt1 - rho3 * pd);
+        c[0].v[e] = ct0 - rho3 * pc;
+        d[0].v[e] = dt1 - rho3 * pd;
         float p1, p2, p3, pd2;
         proj_e2(ct1 * inv_r3, ct2 * inv_r3, ct3 * inv_r3, dt2 * inv_r3, p1, p2, p3, pd2);
-        setc(c1, k, ct1 - rho3 * p1);
-        setc(c2, k, ct2 - rho3 * p2);
-        setc(c3, k, ct3 - rho3 * p3);
-        setc(d2n, k, dt2 - rho3 * pd2);
+        c[1].v[e] = ct1 - rho3 * p1;
+        c[2].v[e] = ct2 - rho3 * p2;
+        c[3].v[e] = ct3 - rho3 * p3;
+        d[1].v[e] = dt2 - rho3 * pd2;
       }
-      st4(Z + i, z1n);
-      st4(Z + (size_t)N + i, z2n);
-      st4(D + i, d1n);
-      st4(D + (size_t)N + i, d2n);
-      st4(C + i, c0);
-      st4(C + (size_t)N + i, c1);
-      st4(C + 2 * (size_t)N + i, c2);
-      st4(C + 3 * (size_t)N + i, c3);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        stp<P>(Z + (size_t)k * N + i, z[k]);
+        stp<P>(D + (size_t)k * N + i, d[k]);
+      }
     } else if (mode == PS_SOC) {
       // Direct cone dual: C = C~ - rho3 P_P(C~ / rho3), P_P = P_E2 with (r, d) = ((Q, U, V), I).
-      float4 c0 = ld4(C + i), c1 = ld4(C + (size_t)N + i), c2 = ld4(C + 2 * (size_t)N + i),
-             c3 = ld4(C + 3 * (size_t)N + i);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float ct0 = comp(c0, k) + rho3 * comp(xb[0], k), ct1 = comp(c1, k) + rho3 * comp(xb[1], k);
-        const float ct2 = comp(c2, k) + rho3 * comp(xb[2], k), ct3 = comp(c3, k) + rho3 * comp(xb[3], k);
+      for (int e = 0; e < P; ++e) {
+        const float ct0 = c[0].v[e] + rho3 * xb[0].v[e], ct1 = c[1].v[e] + rho3 * xb[1].v[e];
+        const float ct2 = c[2].v[e] + rho3 * xb[2].v[e], ct3 = c[3].v[e] + rho3 * xb[3].v[e];
         float p1, p2, p3, p0;
         proj_e2(ct1 * inv_r3, ct2 * inv_r3, ct3 * inv_r3, ct0 * inv_r3, p1, p2, p3, p0);
-        setc(c0, k, ct0 - rho3 * p0);
-        setc(c1, k, ct1 - rho3 * p1);
-        setc(c2, k, ct2 - rho3 * p2);
-        setc(c3, k, ct3 - rho3 * p3);
+        c[0].v[e] = ct0 - rho3 * p0;
+        c[1].v[e] = ct1 - rho3 * p1;
+        c[2].v[e] = ct2 - rho3 * p2;
+        c[3].v[e] = ct3 - rho3 * p3;
       }
-      st4(C + i, c0);
-      st4(C + (size_t)N + i, c1);
-      st4(C + 2 * (size_t)N + i, c2);
-      st4(C + 3 * (size_t)N + i, c3);
+    }
+    if (con) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) stp<P>(C + (size_t)k * N + i, c[k]);
     }
   }
-  // Partials for the relative-change statistic: FP32 within a warp (at most 128
+  // Partials for the relative-change statistic: FP32 within a warp (at most 64
   // terms), FP64 across warps and CTAs.
   double v[8];
 #pragma unroll
@@ -211,13 +231,21 @@ __global__ void __launch_bounds__(kSweepThreads, 3) k_primal(
   }
 }
 
-int sweep_blocks(int N) { return (N + kSweepThreads * kSweepPix - 1) / (kSweepThreads * kSweepPix); }
+// Pixels per thread: one while that is less than a wave of the chip's threads (a small image's
+// sweep is a latency: 64^2 10.1 -> 7.3 us, 256^2 10.5 -> 8.7 against four pixels in four CTAs,
+// resp. 64), two above, with all 28 loads of a pixel pair in flight (80 registers): 1024^2 39.7
+// us with four pixels and loads as the steps need them, 37.9 with all of four pixels' loads in
+// flight, 32.4 with two's (0.69 -> 0.84 of the copy bandwidth on 192 B per pixel); 2048^2 (cone
+// dual) 122 -> 104 us.
+static int sweep_pix(int N) { return N <= 65536 ? 1 : 2; }
+int sweep_blocks(int N) { return (N + kSweepThreads * sweep_pix(N) - 1) / (kSweepThreads * sweep_pix(N)); }
 
 cudaError_t primal_sweep(Handle* h) {
   const dim3 grid(sweep_blocks(h->N), h->problems);
-  k_primal<<<grid, kSweepThreads, 0, h->stream>>>(h->N, h->mode, (float)h->tau, (float)h->rho1, (float)h->rho3, h->S,
-                                                  h->Z, h->C, h->D, h->PsiA, h->Adj, h->Xb, h->A, h->T,
-                                                  (size_t)kBases * h->N, h->red, (size_t)h->red_cap);
+  auto kern = sweep_pix(h->N) == 1 ? k_primal<1> : k_primal<2>;
+  kern<<<grid, kSweepThreads, 0, h->stream>>>(h->N, h->mode, (float)h->tau, (float)h->rho1, (float)h->rho3, h->S, h->Z,
+                                              h->C, h->D, h->PsiA, h->Adj, h->Xb, h->A, h->T, (size_t)kBases * h->N,
+                                              h->red, (size_t)h->red_cap);
   return cudaGetLastError();
 }
 
