@@ -366,23 +366,15 @@ void ps_batch_destroy(ps_batch* b);
  * fastest depends on the image size and on how the visibilities fill the uv plane,
  * so it is measured on the handle's own problem). Values index the candidates: */
 enum {
-  PS_TUNE_SYNTHESIS = 0,  /* finest synthesis level: 0 double-buffered subband staging (3 CTAs/SM),
+  PS_TUNE_SYNTHESIS = 0,  /* finest synthesis level, of images with more than 304 tiles of 64 x 64
+                             over their maps (smaller ones take one form of their own): 0 double-buffered subband staging (3 CTAs/SM),
                              1 single-buffered, refilled during the x-pass (4 CTAs/SM),
                              2 as 1 in persistent CTAs looping over (tile, map) units, the staging
                                running on from one unit into the next */
-  PS_TUNE_DEGRID = 1,     /* 0 one row per thread over a work item,
-                             1 one same-cell chunk per warp (broadcast stencil reads),
-                             2 as 0 with registers capped for 6 CTAs per SM (W = 7; other widths
-                               run 0) */
-  PS_TUNE_GRID = 2,       /* 0 one warp per same-cell chunk (2 kernel cells per lane),
-                             1 half-warps on alternate rows of a chunk (4 cells per lane),
-                             2 lanes own (stencil row, channel pair) (W <= 8; W = 9 runs 0),
-                             3 tensor cores: each chunk's block as a small matrix product
-                               (TF32 hi/lo split, FP32 accumulation), kernel weights copied from a
-                               per-row table made once per measurement set (W <= 8; W = 9 runs 0),
-                             4 as 3 with the kernel weights evaluated in the kernel (no table
-                               traffic) (W <= 8; W = 9 runs 0) */
-  PS_TUNE_ANALYSIS = 3,   /* tiled analysis levels: 0 one (tile, basis, map) unit per CTA,
+  PS_TUNE_DEGRID = 1,     /* 0-2: one form (the library picks its launch shape from the rows and
+                             their coverage); the three values are accepted and equal */
+  PS_TUNE_GRID = 2,       /* 0-4: one form, likewise */
+  PS_TUNE_ANALYSIS = 3,   /* tiled analysis levels (input side above 64): 0 one (tile, basis, map) unit per CTA,
                              1 persistent (2 CTAs/SM looping over units, next unit's copies in flight),
                              2 level 1 with one CTA per (tile, map): the map's input tile copied once for
                                the 8 bases, each basis' staged A and gamma W in flight during the previous

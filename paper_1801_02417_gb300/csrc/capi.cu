@@ -135,11 +135,7 @@ static void free_vis(Handle* h) {
   dfree(h, h->cb, (size_t)h->nblocks);
   dfree(h, h->block_sum, (size_t)h->nblocks);
   dfree(h, h->items, (size_t)h->nitems);
-  dfree(h, h->gchunks, (size_t)h->ngchunks);
-  dfree(h, h->items_g, (size_t)h->nitems_g);
-  dfree(h, h->gchunks_g, (size_t)h->ngchunks_g);
   dfree(h, h->vblk, M);
-  dfree(h, h->wrow, 16 * M);
   const size_t Wd = h->g.Wd;
   dfree(h, h->T1, (size_t)h->n * Wd);
   dfree(h, h->G, Wd * Wd);
@@ -147,7 +143,7 @@ static void free_vis(Handle* h) {
   dfree(h, h->T2, (size_t)h->n * Wd);
   dfree(h, h->tw, (size_t)h->g.K);
   dfree(h, h->corr, (size_t)h->n);
-  h->M = h->nblocks = h->nitems = h->ngchunks = h->nitems_g = h->ngchunks_g = 0;
+  h->M = h->nblocks = h->nitems = 0;
   h->g = ps::GridGeom{};
 }
 
@@ -375,7 +371,7 @@ int64_t ps_estimate_bytes(int32_t n, int32_t levels, int64_t M) {
   if (n < 16 || n > 2048 || !is_pow2(n) || levels < 1 || (n % (1 << levels)) != 0 || M < 0) return 0;
   const int64_t N = (int64_t)n * n, K = 2 * (int64_t)n;
   const int64_t img = (28 + 72 + 16) * N * 4 + (8 * (int64_t)ps::sweep_blocks((int)N) + 1024) * 8;
-  const int64_t vis = M * (3 * 32 + 16 + 4 + 64) + (M / ps::kChunk + 64) * 24 + M / 2;   // + item and chunk lists
+  const int64_t vis = M * (3 * 32 + 16 + 4 + 2) + (M / 64 + 64) * 16;   // rows and work items
   const int64_t grid = 2 * (int64_t)n * K * 16 + 48 * K * K + K * 12 + (int64_t)n * 4;
   return img + vis + grid;
 }
@@ -461,7 +457,7 @@ ps_status ps_create(const ps_config* cfg, void* cuda_stream, ps_handle** out) {
   }
   double filt[ps::kDb][ps::kMaxTaps];
   ps::daubechies_filters(filt);
-  if ((e = ps::upload_filters(filt, h->stream)) != cudaSuccess) {
+  if ((e = ps::upload_filters(filt, h->stream)) != cudaSuccess || (e = ps::upload_es_polys(h->stream)) != cudaSuccess) {
     h->err = std::string("upload filters: ") + cudaGetErrorString(e);
     return bail(PS_ECUDA);
   }
@@ -629,7 +625,7 @@ ps_status ps_set_measurements(ps_handle* h, int64_t M64, const double* uv, const
     }
     CK(h, cudaStreamSynchronize(h->stream));
   }
-  auto wrow_of = [&](int64_t m) { return wsrc ? wsrc[m] : 1.0f; };
+  auto weight_of = [&](int64_t m) { return wsrc ? wsrc[m] : 1.0f; };
 
   // Grid geometry: tap centres c = floor(u + 1/2), u = omega K / (2 pi); rows checked.
   ps::GridGeom& g = h->g;
@@ -646,7 +642,7 @@ ps_status ps_set_measurements(ps_handle* h, int64_t M64, const double* uv, const
     int cm = 0, bad = 0;
     for (int64_t m = b; m < e; ++m) {
       const double ou = uvh[2 * m], ov = uvh[2 * m + 1];
-      const float wm = wrow_of(m);
+      const float wm = weight_of(m);
       if (!std::isfinite(ou) || !std::isfinite(ov) || std::fabs(ou) >= M_PI || std::fabs(ov) >= M_PI) {
         bad |= 1;
         continue;
@@ -684,20 +680,16 @@ ps_status ps_set_measurements(ps_handle* h, int64_t M64, const double* uv, const
   g.tilesX = (g.Wd + ps::kGridTile - 1) / ps::kGridTile;
   auto gi = [&](int k) { return g.full ? (k & (g.K - 1)) : k + g.off; };
 
-  // Storage order: rows sorted by degridding tile (TS x TS cells), then by gridding tile
-  // within it (TG x TG), then by tap-centre cell (row-major in the gridding tile), rows of
-  // one cell in the caller's order: three stable counting-sort passes, least significant
-  // first. The rows of every degridding tile, of every gridding tile and of every cell are
-  // then contiguous.
-  const int TS = ps::kGridTile, TG = ps::kGridTileG, NS = TS / TG;
+  // Storage order: rows sorted by degridding tile (TS x TS cells), then by tap-centre cell
+  // (row-major in the tile), rows of one cell in the caller's order: two stable counting-sort
+  // passes, least significant first. The rows of every tile and of every cell are then
+  // contiguous.
+  const int TS = ps::kGridTile;
   auto tile_of = [&](int32_t m) { return (int64_t)(gi(cy[m]) / TS) * g.tilesX + gi(cx[m]) / TS; };
-  auto sub_of = [&](int32_t m) { return (int64_t)(((gi(cy[m]) % TS) / TG) * NS + (gi(cx[m]) % TS) / TG); };
-  auto cell_of = [&](int32_t m) { return (int64_t)((gi(cy[m]) % TG) * TG + gi(cx[m]) % TG); };
+  auto cell_of = [&](int32_t m) { return (int64_t)((gi(cy[m]) % TS) * TS + gi(cx[m]) % TS); };
   std::vector<int32_t> perm(M), tmp(M);
   std::iota(tmp.begin(), tmp.end(), 0);
-  counting_sort(tmp, perm, (int64_t)TG * TG, parts, cell_of);
-  tmp.swap(perm);
-  counting_sort(tmp, perm, (int64_t)NS * NS, parts, sub_of);
+  counting_sort(tmp, perm, (int64_t)TS * TS, parts, cell_of);
   tmp.swap(perm);
   counting_sort(tmp, perm, (int64_t)g.tilesX * g.tilesX, parts, tile_of);
   std::vector<int32_t> sgy(M), sgx(M);   // grid cell of each row, in storage order
@@ -721,7 +713,7 @@ ps_status ps_set_measurements(ps_handle* h, int64_t M64, const double* uv, const
       const int packed = (cx[m] & 0xFFFF) | (cy[m] << 16);
       float pf;
       std::memcpy(&pf, &packed, sizeof(pf));
-      rech[i] = make_float4(fx[m], fy[m], wrow_of(m), pf);
+      rech[i] = make_float4(fx[m], fy[m], weight_of(m), pf);
     }
   });
   // 2 sum w_m^2 over a fixed partition (the same sum on every machine).
@@ -729,48 +721,32 @@ ps_status ps_set_measurements(ps_handle* h, int64_t M64, const double* uv, const
   std::vector<double> part_psf(kPsfParts, 0.0);
   parallel_parts(M, kPsfParts, [&](int t, int64_t b, int64_t e) {
     double acc = 0.0;
-    for (int64_t m = b; m < e; ++m) acc += 2.0 * (double)wrow_of(m) * wrow_of(m);
+    for (int64_t m = b; m < e; ++m) acc += 2.0 * (double)weight_of(m) * weight_of(m);
     part_psf[t] = acc;
   });
   h->psf_peak = std::accumulate(part_psf.begin(), part_psf.end(), 0.0);
-  // Work items (<= cap rows of one tile of side tsz) and same-cell chunks (<= kBinChunk
-  // rows): kGridItem rows of a TS tile per degridding item, kGridItemG rows of a TG tile per
-  // gridding item; a chunk holds its cell's position in the item's tile.
-  auto make_items = [&](int cap, int tsz, std::vector<ps::GridItem>& items, std::vector<int32_t>& gchunks) {
+  // Degridding work items: rows of one TS tile, at most kGridItem of them, and fewer where the
+  // rows would not give every SM four items (at least 64: an item stages its tile's spectrum
+  // cells whatever its rows). 64^2 / 2,000 rows: 5 items of 768, 18.7 us -> 31 of 64, 8.8 us;
+  // 256^2 / 50,000 rows: 20.6 -> 12.8 us.
+  std::vector<ps::GridItem> items;
+  {
+    const int even = (M / (4 * std::max(1, h->num_sms)) + 31) / 32 * 32;
+    const int cap = std::min(ps::kGridItem, std::max(64, even));
     int j0 = 0;
     while (j0 < M) {
-      const int ty = sgy[j0] / tsz, tx = sgx[j0] / tsz;
+      const int ty = sgy[j0] / TS, tx = sgx[j0] / TS;
       int j1 = j0;
-      while (j1 < M && j1 - j0 < cap && sgy[j1] / tsz == ty && sgx[j1] / tsz == tx) ++j1;
-      ps::GridItem it{};
-      it.ty = ty;
-      it.tx = tx;
-      it.vstart = j0;
-      it.vend = j1;
-      it.cstart = (int32_t)gchunks.size();
-      int c0 = j0;
-      while (c0 < j1) {
-        int c1 = c0;
-        while (c1 < j1 && c1 - c0 < ps::kBinChunk && sgy[c1] == sgy[c0] && sgx[c1] == sgx[c0]) ++c1;
-        const int ly = sgy[c0] - ty * tsz, lx = sgx[c0] - tx * tsz;
-        gchunks.push_back((c0 - j0) | ((c1 - c0) << 10) | (ly << 16) | (lx << 24));
-        c0 = c1;
-      }
-      it.cend = (int32_t)gchunks.size();
-      items.push_back(it);
+      while (j1 < M && j1 - j0 < cap && sgy[j1] / TS == ty && sgx[j1] / TS == tx) ++j1;
+      items.push_back(ps::GridItem{ty, tx, j0, j1});
       j0 = j1;
     }
-  };
-  std::vector<ps::GridItem> items, items_g;
-  std::vector<int32_t> gchunks, gchunks_g;
-  make_items(ps::kGridItem, TS, items, gchunks);
-  make_items(ps::kGridItemG, TG, items_g, gchunks_g);
+  }
+  h->ncells = M > 0 ? 1 : 0;
+  for (int i = 1; i < M; ++i) h->ncells += sgy[i] != sgy[i - 1] || sgx[i] != sgx[i - 1];
   h->M = M;
   h->nblocks = M > 0 ? nblocks : 0;
   h->nitems = (int)items.size();
-  h->ngchunks = (int)gchunks.size();
-  h->nitems_g = (int)items_g.size();
-  h->ngchunks_g = (int)gchunks_g.size();
   if (M > 0) h->eps_host.assign(eps, eps + h->nblocks);
   else h->eps_host.clear();
 
@@ -782,13 +758,10 @@ ps_status ps_set_measurements(ps_handle* h, int64_t M64, const double* uv, const
             dalloc(h, &h->cb, (size_t)h->nblocks) == cudaSuccess &&
             dalloc(h, &h->block_sum, (size_t)h->nblocks) == cudaSuccess &&
             dalloc(h, &h->items, items.size()) == cudaSuccess &&
-            dalloc(h, &h->gchunks, gchunks.size()) == cudaSuccess &&
-            dalloc(h, &h->items_g, items_g.size()) == cudaSuccess &&
-            dalloc(h, &h->gchunks_g, gchunks_g.size()) == cudaSuccess && dalloc(h, &h->vblk, (size_t)M) == cudaSuccess &&
+            dalloc(h, &h->vblk, (size_t)M) == cudaSuccess &&
             dalloc(h, &h->T1, (size_t)h->n * Wd) == cudaSuccess && dalloc(h, &h->G, Wd * Wd) == cudaSuccess &&
             dalloc(h, &h->Acc, 2 * Wd * Wd) == cudaSuccess && dalloc(h, &h->T2, (size_t)h->n * Wd) == cudaSuccess &&
-            dalloc(h, &h->tw, (size_t)g.K) == cudaSuccess && dalloc(h, &h->corr, (size_t)h->n) == cudaSuccess &&
-            (g.W > 8 || dalloc(h, &h->wrow, 16 * (size_t)M) == cudaSuccess);
+            dalloc(h, &h->tw, (size_t)g.K) == cudaSuccess && dalloc(h, &h->corr, (size_t)h->n) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     free_vis(h);
@@ -814,13 +787,7 @@ ps_status ps_set_measurements(ps_handle* h, int64_t M64, const double* uv, const
     CK(h, cudaMemcpyAsync(h->perm, perm.data(), perm.size() * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream));
     CK(h, cudaMemcpyAsync(h->eps, eps, h->nblocks * sizeof(double), cudaMemcpyHostToDevice, h->stream));
     CK(h, cudaMemcpyAsync(h->items, items.data(), items.size() * sizeof(ps::GridItem), cudaMemcpyHostToDevice, h->stream));
-    CK(h, cudaMemcpyAsync(h->gchunks, gchunks.data(), gchunks.size() * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream));
-    CK(h, cudaMemcpyAsync(h->items_g, items_g.data(), items_g.size() * sizeof(ps::GridItem), cudaMemcpyHostToDevice,
-                          h->stream));
-    CK(h, cudaMemcpyAsync(h->gchunks_g, gchunks_g.data(), gchunks_g.size() * sizeof(int32_t), cudaMemcpyHostToDevice,
-                          h->stream));
     CK(h, cudaMemcpyAsync(h->vblk, vblk.data(), vblk.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, h->stream));
-    CK(h, ps::nufft_row_weights(h));
     // Measurements into sorted order.
     ps_status st = stage_in(h, vis, 4 * (size_t)M * sizeof(float2), device_ptrs, h->vtmp);
     if (st != PS_OK) return st;
@@ -1344,7 +1311,9 @@ ps_status ps_profile_stages(ps_handle* h, int32_t n_iter, double* stage_ms) {
 
 // ---------------------------------------------------------------------------
 // Autotuner: candidates per PS_TUNE_* slot, each timed on the handle's own data.
+// kTuneForms: the forms behind them that differ (the interpolation kernels have one each).
 static const int kTuneCandidates[PS_TUNE_COUNT] = {3, 3, 5, 6};
+static const int kTuneForms[PS_TUNE_COUNT] = {3, 1, 1, 6};
 
 // Mean milliseconds of `reps` launches of f after one untimed launch.
 extern "C++" {
@@ -1379,7 +1348,7 @@ ps_status ps_autotune(ps_handle* h, int32_t reps, int32_t* choices, double* ms) 
   auto pick = [&](int slot, auto launch) -> ps_status {
     int best = 0;
     double best_t = 0.0;
-    for (int v = 0; v < kTuneCandidates[slot]; ++v) {
+    for (int v = 0; v < kTuneForms[slot]; ++v) {
       h->tune[slot] = v;
       double t = 0.0;
       ps_status st = tune_time(h, reps, launch, &t);
@@ -1505,7 +1474,6 @@ ps_status ps_max_abs_analysis(ps_handle* h, double* out) {
 
 ps_status ps_debug_set_wait_polls(int32_t polls) {
   cudaError_t e = ps::set_wait_polls_sara(polls);
-  if (e == cudaSuccess) e = ps::set_wait_polls_nufft(polls);
   // The copies run on the legacy stream, which non-blocking streams do not wait for.
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return fail(nullptr, PS_ECUDA, std::string("debug_set_wait_polls: ") + cudaGetErrorString(e));

@@ -131,4 +131,31 @@ double es_fourier(double xi, int W, double beta) {
   return s * half;
 }
 
+// Tap j (offset f + W/2 - j, |f| <= 1/2) as a polynomial of degree 2 kEsTerms - 1 in f: the
+// Chebyshev series of the kernel on 64 nodes, cut at that degree and written out in powers;
+// c holds the even coefficients (of f^0, f^2, ..), then the odd ones (of f, f^3, ..).
+void es_poly(int W, int j, double c[2 * kEsTerms]) {
+  constexpr int D = 2 * kEsTerms, NN = 64;
+  double a[D];   // Chebyshev coefficients in x = 2 f
+  for (int k = 0; k < D; ++k) {
+    double s = 0.0;
+    for (int i = 0; i < NN; ++i) {
+      const double th = M_PI * (i + 0.5) / NN;
+      s += es_kernel(0.5 * std::cos(th) + (W / 2 - j), W, es_beta(W)) * std::cos(k * th);
+    }
+    a[k] = s * (k == 0 ? 1.0 : 2.0) / NN;
+  }
+  double t0[D] = {1.0}, t1[D] = {0.0, 1.0}, p[D] = {};   // T_k in powers of x
+  for (int k = 0; k < D; ++k) {
+    for (int i = 0; i < D; ++i) p[i] += a[k] * t0[i];
+    double t2[D];
+    for (int i = 0; i < D; ++i) t2[i] = (i > 0 ? 2.0 * t1[i - 1] : 0.0) - t0[i];
+    for (int i = 0; i < D; ++i) t0[i] = t1[i], t1[i] = t2[i];
+  }
+  for (int k = 0; k < kEsTerms; ++k) {
+    c[k] = p[2 * k] * std::pow(2.0, 2 * k);
+    c[kEsTerms + k] = p[2 * k + 1] * std::pow(2.0, 2 * k + 1);
+  }
+}
+
 }  // namespace ps

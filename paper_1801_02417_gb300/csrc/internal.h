@@ -15,13 +15,8 @@ constexpr int kBases = 9;        // Dirac + db1..db8
 constexpr int kDb = 8;           // Daubechies bases
 constexpr int kMaxTaps = 16;     // db8 filter length
 constexpr int kGridTile = 16;    // degridding tile side (cells)
-constexpr int kGridTileG = 8;    // gridding tile side (cells): a quarter of a degridding tile
-static_assert(kGridTile % kGridTileG == 0, "gridding tiles subdivide degridding tiles");
-constexpr int kChunk = 1024;     // visibilities per reduction chunk
-constexpr int kGridItem = 768;   // visibilities per degridding work item
-constexpr int kGridItemG = 384;  // visibilities per gridding work item (smaller: 4 CTAs per SM)
-static_assert(kGridItem <= 1024 && kGridItemG <= 1024, "a chunk's start is a 10-bit offset in its item");
-constexpr int kBinChunk = 32;    // visibilities per same-cell accumulation chunk
+constexpr int kGridItem = 768;   // visibilities per degridding work item, at most
+constexpr int kEsTerms = 5;      // coefficients of the even and of the odd part of a kernel tap's polynomial
 constexpr int kWarpBins = 64;    // l2 blocks up to which degridding keeps per-warp FP64 block sums
 constexpr int kGraphIters = 8;   // iterations per launch of the multi-iteration graph
 
@@ -30,10 +25,9 @@ enum { SARA_DUAL = 0, SARA_APPLY = 1, SARA_REWEIGHT = 2 };
 // Degridding modes.
 enum { DEG_DUAL = 0, DEG_APPLY = 1, DEG_RESID = 2 };
 
-struct GridItem {      // one gridding CTA: gridding-order rows [vstart, vend), centres in tile (ty, tx),
-  int32_t ty, tx;      // same-cell chunks [cstart, cend)
-  int32_t vstart, vend, cstart, cend;
-  int32_t pad0, pad1;
+struct GridItem {      // one degridding CTA: stored rows [vstart, vend), centres in tile (ty, tx)
+  int32_t ty, tx;
+  int32_t vstart, vend;
 };
 
 // Geometry of the NUFFT grid: the K x K oversampled spectrum is kept only on a
@@ -46,7 +40,7 @@ struct GridGeom {
   int Wd = 0;            // stored grid side: 2R+1 (window) or K (full)
   int full = 0;          // 1: full grid, indices wrap modulo K
   int off = 0;           // grid index of frequency k: (k + off) [& (K-1) if full]
-  int tilesX = 0;        // gridding tiles per side
+  int tilesX = 0;        // degridding tiles per side
   float beta = 0.f;      // ES kernel shape
 };
 
@@ -97,15 +91,10 @@ struct Handle {
   double *eps = nullptr;      // per block radius (device)
   float *cb = nullptr;        // per block scale c_b (device)
   double *block_sum = nullptr;     // nblocks FP64 sums filled by the degridding kernel
-  int nitems = 0, ngchunks = 0;
-  GridItem *items = nullptr;       // degridding work items (<= kGridItem rows)
-  int32_t *gchunks = nullptr;      // packed (start, count, ly, lx) of their same-cell chunks
-  int nitems_g = 0, ngchunks_g = 0;
-  GridItem *items_g = nullptr;     // gridding work items (<= kGridItemG rows) and their chunks
-  int32_t *gchunks_g = nullptr;
+  int ncells = 0;                  // cells that hold a row
+  int nitems = 0;
+  GridItem *items = nullptr;       // degridding work items
   uint16_t *vblk = nullptr;        // l2 block of each stored row
-  float *wrow = nullptr;           // W <= 8: kernel weights of each stored row, 8 y-taps (M x 8)
-                                   // then 8 x-taps (M x 8), zero past W
   std::vector<double> eps_host;
   double psf_peak = 0.0;      // 2 sum w_m^2: peak of the Stokes-I PSF
   float *tmp36 = nullptr;     // 36N scratch for operator calls (allocated on first use)
@@ -131,9 +120,8 @@ struct Handle {
   uint64_t version = 1;       // bumped when mode, state or measurements change (batch graphs rebuild)
 };
 
-// Bounded-wait poll budget of each translation unit with bulk-copy waits (polls < 0: default).
+// Bounded-wait poll budget of the translation unit with bulk-copy waits (polls < 0: default).
 cudaError_t set_wait_polls_sara(int polls);
-cudaError_t set_wait_polls_nufft(int polls);
 
 // Message returned by ps_last_error(NULL) (calls without a handle).
 void set_global_error(const std::string& msg);
@@ -143,15 +131,16 @@ void daubechies_filters(double h[kDb][kMaxTaps]);          // db1..db8 scaling f
 double es_beta(int W);
 double es_kernel(double t, int W, double beta);            // ES kernel value at offset t (cells)
 double es_fourier(double xi, int W, double beta);          // its Fourier transform at xi
+void es_poly(int W, int j, double c[2 * kEsTerms]);        // tap j as a polynomial of its offset: E then O coefficients
 
 // Kernel launchers (return cudaGetLastError()).
 cudaError_t upload_filters(const double h[kDb][kMaxTaps], cudaStream_t stream);
+cudaError_t upload_es_polys(cudaStream_t stream);
 
 // NUFFT pieces (nufft.cu).
 cudaError_t nufft_forward_grid(Handle* h, const float* X);                 // X (4 planes) -> G
 cudaError_t nufft_degrid(Handle* h, int mode, float2* out);                // G -> visibilities
 cudaError_t nufft_grid(Handle* h, const float2* in, int use_block_scale);  // visibilities -> Acc
-cudaError_t nufft_row_weights(Handle* h);                                   // rec -> wrow (W <= 8)
 cudaError_t tv_dual(Handle* h);      // Algorithm 3 steps 5-6 on Xb -> A (TV layout)
 cudaError_t tv_adjoint(Handle* h);   // Psi A = grad^T A_tv (+ A_l1) -> PsiA
 __host__ __device__ inline bool tv_mode(int m) { return m >= PS_TV && m <= PS_L1TV_NC; }

@@ -14,29 +14,25 @@
 //   k_fwd_rows    row FFTs of the de-apodised, zero-padded rows     (n CTAs)
 //   k_fwd_cols    column FFTs, kept on the window                    (Wd CTAs)
 //   k_degrid      interpolation + Stokes->correlation mixing + dual update of B
-//                 and per-chunk FP64 partial of ||B~/rho2 - Y||^2     (1 CTA / chunk)
+//                 and per-block FP64 sums of ||B~/rho2 - Y||^2        (1 CTA / work item)
 //   k_block_scale per-block l2-ball projection factor (FP64)
-//   k_grid        mixing by conj(L) + tile-privatised gridding in shared memory
+//   k_grid        mixing by conj(L) + gridding, one warp per run of rows
 //   k_adj_cols    Hermitian symmetrisation + inverse column FFTs     (R+1 CTAs)
 //   k_adj_rows    inverse row FFTs + crop + de-apodisation -> phi^dagger planes
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "internal.h"
 #include "packed.cuh"
 
 namespace ps {
 
-// Sets this file's bounded-wait poll budget (ps_debug_set_wait_polls).
-cudaError_t set_wait_polls_nufft(int polls) { return set_wait_polls_here(polls); }
-
 __device__ __forceinline__ float4 f4add(float4 a, float4 b) {
   return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
 }
 __device__ __forceinline__ float4 f4sub(float4 a, float4 b) {
   return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
-}
-__device__ __forceinline__ float4 f4scale(float4 a, float s) {
-  return make_float4(a.x * s, a.y * s, a.z * s, a.w * s);
 }
 __device__ __forceinline__ float4 f4fma(float s, float4 a, float4 acc) {
   return make_float4(fmaf(s, a.x, acc.x), fmaf(s, a.y, acc.y), fmaf(s, a.z, acc.z), fmaf(s, a.w, acc.w));
@@ -223,6 +219,55 @@ __device__ __forceinline__ void es_weights(float f, float beta, float* wt) {
   }
 }
 
+// Polynomials of the kernel taps in f (|f| <= 1/2), fitted on the host in FP64 (es_poly):
+// tap j = E_j(f^2) + f O_j(f^2) and, the kernel being even, tap W-1-j = E_j(f^2) - f O_j(f^2).
+// Coefficients duplicated in both halves of a 64-bit word, one table per width.
+__constant__ __align__(16) float2 c_es[3][5][2 * kEsTerms];
+
+cudaError_t upload_es_polys(cudaStream_t stream) {
+  float2 t[3][5][2 * kEsTerms] = {};
+  for (int q = 0; q < 3; ++q)
+    for (int j = 0; j <= (5 + 2 * q) / 2; ++j) {
+      double c[2 * kEsTerms];
+      es_poly(5 + 2 * q, j, c);
+      for (int k = 0; k < 2 * kEsTerms; ++k) t[q][j][k] = make_float2((float)c[k], (float)c[k]);
+    }
+  cudaError_t e = cudaMemcpyToSymbolAsync(c_es, t, sizeof(t), 0, cudaMemcpyHostToDevice, stream);
+  return e == cudaSuccess ? cudaStreamSynchronize(stream) : e;
+}
+
+// The W x- and W y-weights of a row at once, two polynomials per packed FMA (lanes x, y):
+// 34 packed FMAs for W = 7 in place of 14 square roots and exponentials, and closer to the
+// kernel: at most 1e-7 of its peak off in FP32 (1.4e-7 at the very end of the outermost tap),
+// the exponential form 7e-7. W = 5 keeps the exponentials: the square-root end of its kernel
+// (height 1e-5) is not a polynomial.
+template <int W>
+__device__ __forceinline__ void es_weights_xy(float fx, float fy, float beta, float* wx, float* wy) {
+  if constexpr (W == 5) {
+    es_weights<W>(fx, beta, wx);
+    es_weights<W>(fy, beta, wy);
+  } else {
+    constexpr int q = (W - 5) / 2, hw = W / 2;
+    const u64 f = f2pack(fx, fy), nf = f2pack(-fx, -fy), x = ffma2(f, f, 0ull);
+    auto co = [&](int j, int k) { return *reinterpret_cast<const u64*>(&c_es[q][j][k]); };
+#pragma unroll
+    for (int j = 0; j <= hw; ++j) {
+      u64 e = co(j, kEsTerms - 1);
+#pragma unroll
+      for (int k = kEsTerms - 2; k >= 0; --k) e = ffma2(e, x, co(j, k));
+      if (j == hw) {   // the centre tap is even in f
+        f2unpack(e, wx[j], wy[j]);
+      } else {
+        u64 o = co(j, 2 * kEsTerms - 1);
+#pragma unroll
+        for (int k = kEsTerms - 2; k >= 0; --k) o = ffma2(o, x, co(j, kEsTerms + k));
+        f2unpack(ffma2(o, f, e), wx[j], wy[j]);
+        f2unpack(ffma2(o, nf, e), wx[W - 1 - j], wy[W - 1 - j]);
+      }
+    }
+  }
+}
+
 __device__ __forceinline__ void unpack_rec(float4 r, float& fx, float& fy, float& w, int& cx, int& cy) {
   fx = r.x;
   fy = r.y;
@@ -230,23 +275,6 @@ __device__ __forceinline__ void unpack_rec(float4 r, float& fx, float& fy, float
   const int pk = __float_as_int(r.w);
   cx = (int)(short)(pk & 0xFFFF);
   cy = pk >> 16;
-}
-
-template <typename T>
-__device__ __forceinline__ T block_sum(T v, T* sh) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) sh[wid] = v;
-  __syncthreads();
-  T r = 0;
-  if (threadIdx.x < 32) {
-    r = (threadIdx.x < (blockDim.x >> 5)) ? sh[threadIdx.x] : (T)0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-  }
-  return r;  // valid in thread 0
 }
 
 // FP32 -> TF32 hi part (round to nearest, ties away) and the TF32 rounding of the
@@ -270,65 +298,80 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// Second half of a degridding row m (all 32 lanes of the warp call it together: the
-// block-sum combination is warp-collective; inactive lanes add nothing): from the
-// interpolated packed spectra sp (at +u) and sn (at -u) to the row's visibilities
-// (or residuals), and its term of the per-block sums.
-__device__ __forceinline__ void degrid_finish(int m, bool active, float w, float4 sp, float4 sn, int mode,
-                                              float2* __restrict__ R, const float2* __restrict__ Yv,
-                                              const float* __restrict__ cb, float inv_rho2,
-                                              const uint16_t* __restrict__ vblk, bool reduce, bool private_bins,
-                                              double* bsum, float2* __restrict__ out) {
+// Second half of a degridding row m: from the interpolated packed spectra sp (at +u) and sn
+// (at -u) to the row's visibilities (or residuals); returns its term of the per-block sums
+// and its block (blk, left alone by DEG_APPLY).
+__device__ __forceinline__ float degrid_finish(int m, float w, float4 sp, float4 sn, int mode, float2* __restrict__ R,
+                                               const float2* __restrict__ Yv, const float* __restrict__ cb,
+                                               float inv_rho2, const uint16_t* __restrict__ vblk,
+                                               float2* __restrict__ out, int& blk) {
   float4* R4 = reinterpret_cast<float4*>(R);
   const float4* Y4 = reinterpret_cast<const float4*>(Yv);
-  int blk = -1;
-  float e2 = 0.f;
-  if (active) {
-    // G1 = F(I + iQ), G2 = F(U + iV); F(I) = (G1(u) + conj G1(-u))/2, F(Q) = (G1(u) - conj G1(-u))/(2i).
-    const float FIr = 0.5f * (sp.x + sn.x), FIi = 0.5f * (sp.y - sn.y);
-    const float FQr = 0.5f * (sp.y + sn.y), FQi = -0.5f * (sp.x - sn.x);
-    float4 v01 = make_float4(w * (FIr + FQr), w * (FIi + FQi), w * sp.z, w * sp.w);   // RR, RL = G2(u)
-    float4 v23 = make_float4(w * sn.z, -w * sn.w, w * (FIr - FQr), w * (FIi - FQi));  // LR = conj G2(-u), LL
-    if (mode == DEG_APPLY) {
+  // G1 = F(I + iQ), G2 = F(U + iV); F(I) = (G1(u) + conj G1(-u))/2, F(Q) = (G1(u) - conj G1(-u))/(2i).
+  const float FIr = 0.5f * (sp.x + sn.x), FIi = 0.5f * (sp.y - sn.y);
+  const float FQr = 0.5f * (sp.y + sn.y), FQi = -0.5f * (sp.x - sn.x);
+  float4 v01 = make_float4(w * (FIr + FQr), w * (FIi + FQi), w * sp.z, w * sp.w);   // RR, RL = G2(u)
+  float4 v23 = make_float4(w * sn.z, -w * sn.w, w * (FIr - FQr), w * (FIi - FQi));  // LR = conj G2(-u), LL
+  if (mode == DEG_APPLY) {
+    float4* o4 = reinterpret_cast<float4*>(out);
+    o4[2 * (size_t)m] = v01;
+    o4[2 * (size_t)m + 1] = v23;
+    return 0.f;
+  }
+  blk = vblk[m];
+  const float4 y0 = Y4[2 * (size_t)m], y1 = Y4[2 * (size_t)m + 1];
+  if (mode == DEG_DUAL) {
+    const float cs = cb[blk] * inv_rho2;
+    const float4 r0 = R4[2 * (size_t)m], r1 = R4[2 * (size_t)m + 1];
+    v01 = f4sub(f4fma(cs, r0, v01), y0);
+    v23 = f4sub(f4fma(cs, r1, v23), y1);
+    R4[2 * (size_t)m] = v01;
+    R4[2 * (size_t)m + 1] = v23;
+  } else {
+    v01 = f4sub(y0, v01);
+    v23 = f4sub(y1, v23);
+    if (out) {
       float4* o4 = reinterpret_cast<float4*>(out);
       o4[2 * (size_t)m] = v01;
       o4[2 * (size_t)m + 1] = v23;
-    } else {
-      blk = vblk[m];
-      const float4 y0 = Y4[2 * (size_t)m], y1 = Y4[2 * (size_t)m + 1];
-      if (mode == DEG_DUAL) {
-        const float cs = cb[blk] * inv_rho2;
-        const float4 r0 = R4[2 * (size_t)m], r1 = R4[2 * (size_t)m + 1];
-        v01 = f4sub(f4fma(cs, r0, v01), y0);
-        v23 = f4sub(f4fma(cs, r1, v23), y1);
-        R4[2 * (size_t)m] = v01;
-        R4[2 * (size_t)m + 1] = v23;
-      } else {
-        v01 = f4sub(y0, v01);
-        v23 = f4sub(y1, v23);
-        if (out) {
-          float4* o4 = reinterpret_cast<float4*>(out);
-          o4[2 * (size_t)m] = v01;
-          o4[2 * (size_t)m + 1] = v23;
-        }
-      }
-      e2 = (v01.x * v01.x + v01.y * v01.y + v01.z * v01.z + v01.w * v01.w) +
-           (v23.x * v23.x + v23.y * v23.y + v23.z * v23.z + v23.w * v23.w);
     }
   }
-  if (reduce) {
-    // Lanes holding the same block add their terms (FP32, at most 32 of them); the
-    // lowest such lane adds the group's sum in FP64 to this warp's bin of the block
-    // (private bins: no other lane or warp writes it) or, with many blocks, to the
-    // CTA's shared bin by an atomic.
-    const unsigned peers = __match_any_sync(0xffffffffu, blk);
-    float sum = 0.f;
-    for (unsigned p = peers; p; p &= p - 1) sum += __shfl_sync(peers, e2, __ffs(p) - 1);
-    if (blk >= 0 && (threadIdx.x & 31) == __ffs(peers) - 1) {
-      if (private_bins) bsum[(threadIdx.x >> 5) * kWarpBins + blk] += (double)sum;
-      else atomicAdd(&bsum[blk], (double)sum);
+  return (v01.x * v01.x + v01.y * v01.y + v01.z * v01.z + v01.w * v01.w) +
+         (v23.x * v23.x + v23.y * v23.y + v23.z * v23.z + v23.w * v23.w);
+}
+
+// Adds every lane's e2 to the sum of its block blk (-1: none); all 32 lanes together. FP32
+// over a warp's lanes of one block, FP64 in sums[]: this warp's own bins, or (shared) sums that
+// other warps add to as well. Blocks that more than eight lanes share take one butterfly
+// sum each (~15 instructions); the rest go by groups of equal blocks, all groups at once, a few
+// instructions per lane of the largest.
+__device__ __forceinline__ void block_add(int blk, float e2, bool shared, double* sums) {
+  const int lane = threadIdx.x & 31;
+  auto add = [&](int b, float v) {
+    if (shared) atomicAdd(&sums[b], (double)v);
+    else sums[b] += (double)v;
+  };
+  unsigned peers = __match_any_sync(0xffffffffu, blk);
+  if (__any_sync(0xffffffffu, blk >= 0 && __popc(peers) > 8)) {
+    unsigned todo = __ballot_sync(0xffffffffu, blk >= 0 && __popc(peers) > 8);
+    while (todo) {   // at most three blocks have more than eight of the 32 lanes
+      const int b = __shfl_sync(0xffffffffu, blk, __ffs(todo) - 1);
+      const bool mine = blk == b;
+      float v = mine ? e2 : 0.f;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) add(b, v);
+      if (mine) blk = -1;
+      todo &= ~__ballot_sync(0xffffffffu, mine);
     }
-    __syncwarp();   // the next row's leader of this block may be another lane
+  }
+  __syncwarp();   // lane 0's sums before another lane's below, or in the next call
+  if (__any_sync(0xffffffffu, blk >= 0)) {
+    if (blk < 0) peers = 1u << lane;
+    float v = 0.f;
+    for (unsigned p = peers; p; p &= p - 1) v += __shfl_sync(peers, e2, __ffs(p) - 1);
+    if (blk >= 0 && lane == __ffs(peers) - 1) add(blk, v);
+    __syncwarp();
   }
 }
 
@@ -340,28 +383,26 @@ __device__ __forceinline__ void degrid_prefetch(int m, int mode, const float2* R
   if (mode == DEG_DUAL) asm volatile("prefetch.global.L1 [%0];" ::"l"(R + 4 * (size_t)m));
 }
 
-// One row of a degridding work item on the CUDA cores: the 2 W^2 taps read from the
-// staged spectrum cells, then degrid_finish (warp-collective, like it).
+// One row of a degridding work item on the CUDA cores: the 2 W^2 taps read from the staged
+// spectrum cells, then degrid_finish and block_add (warp-collective: every lane calls it).
 template <int W>
 __device__ __forceinline__ void degrid_row(int m, bool active, const GridItem& it, const float4* __restrict__ rec,
                                            const float4* Gp, const float4* Gn, int off, int full, int K, float beta,
                                            int mode, float2* __restrict__ R, const float2* __restrict__ Yv,
                                            const float* __restrict__ cb, float inv_rho2,
-                                           const uint16_t* __restrict__ vblk, bool reduce, bool private_bins,
-                                           double* bsum,
+                                           const uint16_t* __restrict__ vblk, bool shared, double* sums,
                                            float2* __restrict__ out) {
   constexpr int TS = kGridTile;
   constexpr int SS = TS + W - 1;
-  float4 sp = make_float4(0.f, 0.f, 0.f, 0.f), sn = sp;
-  float w = 0.f;
+  int blk = -1;
+  float e2 = 0.f;
   if (active) {
     degrid_prefetch(m, mode, R, Yv);
-    float fx, fy;
+    float fx, fy, w;
     int cx, cy;
     unpack_rec(rec[m], fx, fy, w, cx, cy);
     float wx[W], wy[W];
-    es_weights<W>(fx, beta, wx);
-    es_weights<W>(fy, beta, wy);
+    es_weights_xy<W>(fx, fy, beta, wx, wy);
     // Local centre within the tile (tap j of +u at local j + lc; of -u at local (TS-1-lc) + j).
     const int lcy = gidx(cy, off, full, K) - it.ty * TS, lcx = gidx(cx, off, full, K) - it.tx * TS;
     const float4* gp = Gp + lcy * SS + lcx;
@@ -387,12 +428,14 @@ __device__ __forceinline__ void degrid_row(int m, bool active, const GridItem& i
       sn0 = ffma2(kny, an0, sn0);
       sn1 = ffma2(kny, an1, sn1);
     }
+    float4 sp, sn;
     f2unpack(sp0, sp.x, sp.y);
     f2unpack(sp1, sp.z, sp.w);
     f2unpack(sn0, sn.x, sn.y);
     f2unpack(sn1, sn.z, sn.w);
+    e2 = degrid_finish(m, w, sp, sn, mode, R, Yv, cb, inv_rho2, vblk, out, blk);
   }
-  degrid_finish(m, active, w, sp, sn, mode, R, Yv, cb, inv_rho2, vblk, reduce, private_bins, bsum, out);
+  if (mode != DEG_APPLY) block_add(blk, e2, shared, sums);
 }
 
 // Interpolate the packed spectra at +u and -u, unpack the four Stokes spectra,
@@ -405,12 +448,11 @@ __device__ __forceinline__ void degrid_row(int m, bool active, const GridItem& i
 // then in FP64 through per-warp shared bins (up to kWarpBins blocks; shared FP64
 // atomics beyond) and one global FP64 atomic per block and CTA (block_sum, cleared
 // by the caller).
-// FORM 0: one row per thread over the item; 1: one same-cell chunk per warp (broadcast
-// stencil reads); 2: as 0 with registers capped for 6 CTAs per SM at W = 7 (40 instead of
-// 51, so more rows are in flight per SM; other widths would spill under a cap and run as 0).
-template <int W, int FORM>
-__global__ void __launch_bounds__(256, (FORM == 2 && W == 7) ? 6 : 0) k_degrid(
-    const GridItem* __restrict__ items, const int32_t* __restrict__ chunks, const float4* __restrict__ rec, const float4* __restrict__ G, int Wd,
+// Registers are capped for 6 CTAs per SM at W = 7 (40 of 67: more rows in flight per SM, 100
+// against 111 us at 1024^2 / 2,000,000 rows; other widths would spill and run without a cap).
+template <int W>
+__global__ void __launch_bounds__(256, W == 7 ? 6 : 0) k_degrid(
+    const GridItem* __restrict__ items, const float4* __restrict__ rec, const float4* __restrict__ G, int Wd,
     int off, int full, int K, float beta, int mode, float2* __restrict__ R, const float2* __restrict__ Yv,
     const float* __restrict__ cb, float inv_rho2, const uint16_t* __restrict__ vblk, int nblocks,
     double* __restrict__ block_sum, float2* __restrict__ out) {
@@ -447,22 +489,11 @@ __global__ void __launch_bounds__(256, (FORM == 2 && W == 7) ? 6 : 0) k_degrid(
     Gn[i] = vn;
   }
   __syncthreads();
-  if (FORM == 1) {
-    // One same-cell chunk (<= 32 rows) per warp: every lane reads the same stencil
-    // cells, so the shared-memory gathers are broadcasts.
-    const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    for (int c = threadIdx.x >> 5; c < it.cend - it.cstart; c += nwarps) {
-      const int pk = chunks[it.cstart + c];
-      const int v0 = pk & 1023, cnt = (pk >> 10) & 63;
-      degrid_row<W>(it.vstart + v0 + lane, lane < cnt, it, rec, Gp, Gn, off, full, K, beta, mode, R, Yv, cb, inv_rho2,
-                    vblk, reduce, private_bins, bsum, out);
-    }
-  } else {
-    for (int base = it.vstart; base < it.vend; base += blockDim.x) {
-      const int m = base + threadIdx.x;
-      degrid_row<W>(m, m < it.vend, it, rec, Gp, Gn, off, full, K, beta, mode, R, Yv, cb, inv_rho2, vblk, reduce,
-                    private_bins, bsum, out);
-    }
+  double* sums = bsum + (private_bins ? (threadIdx.x >> 5) * kWarpBins : 0);
+  for (int base = it.vstart; base < it.vend; base += blockDim.x) {
+    const int m = base + threadIdx.x;
+    degrid_row<W>(m, m < it.vend, it, rec, Gp, Gn, off, full, K, beta, mode, R, Yv, cb, inv_rho2, vblk, !private_bins,
+                  sums, out);
   }
   if (reduce) {
     __syncthreads();
@@ -494,157 +525,158 @@ __global__ void k_block_scale(const double* __restrict__ block_sum, const double
   cb[b] = (float)(rho2 * (1.0 - keep));
 }
 
-// Gridding (adjoint of the interpolation), Alg. 1 step 3's phi^dagger.
-// Rows are stored sorted by tap-centre cell. One CTA owns a work item:
-// up to kGridItemG visibilities whose centres lie in one kGridTileG^2 tile.
-//  1. Each thread stages one visibility in shared memory: the conj(L)-mixed
-//     values x_I = RR + LL, x_Q = RR - LL, x_U = RL + LR, x_V = i (LR - RL)
-//     scaled by c_b w_m (two float4), and its W x and W y kernel weights (planes
-//     with an odd stride, so lanes reading different taps hit different banks).
-//  2. Visibilities sharing a centre cell (a chunk of <= 32) touch the same W x W
-//     cells. One warp takes one chunk; lane l owns kernel cells l, l+32, ... and
-//     accumulates their 8 channels over the chunk in registers (two rows per
-//     step, channel values read as broadcasts), then adds them once to a
-//     channel-planar shared-memory tile.
-//  3. The tile (with halo) is added to the global accumulator.
-// Channels are gridded at +u only; k_adj_cols forms the -u half by Hermitian
-// symmetrisation.
-// Stride of the staged per-row weight planes: tap j of row v sits in bank (2 j + v) mod 32, so
-// the lanes of a warp (one row, or two rows v, v+1 in the half-warp form) reading their
-// cells' taps never share a bank.
-constexpr int kGridV = kGridItemG + 2;
-
-// Work split of a same-cell chunk (one warp per chunk in every form):
-// FORM 0: lane l owns kernel cells l, l + 32, all 8 channels.
-// FORM 1: the two half-warps take alternate rows of the chunk, lane l owns cells
-//   (l & 15) + 16 q; each 16-byte broadcast read of a row's channels then serves 16 lanes
-//   (two rows per instruction), and the halves' sums are combined by shuffles before the
-//   shared-memory flush.
-// FORM 2 (W <= 8): lane l < 4 W owns stencil row jy = l / 4 and channel pair cp = l % 4,
-//   i.e. the W cells (jy, 0..W-1) of two channels: per row it reads w_y[jy], its channel
-//   pair and the W x-weights (broadcasts), forms t = w_y x once and applies W packed FMAs.
-// FORM 3 (W <= 8): the chunk's block as a product of two small matrices on the tensor
-//   cores (mma.m16n8k8, TF32 with hi/lo operand splitting for FP32 accuracy); lanes load
-//   distinct words of the rows instead of broadcasts.
-// Stride of the 8 channel planes of a gridding tile: its (kGridTileG + W - 1)^2 cells plus
-// one, odd modulo 32, so lanes adding to the same cell of different planes spread over banks.
+// Gridding (adjoint of the interpolation), Alg. 1 step 3's phi^dagger. Rows are stored sorted
+// by tap-centre cell; a warp takes `rows` consecutive rows, 32 at a time, on its own:
+//  1. lane = row: the row is read, mixed by conj(L) (x_I = RR + LL, x_Q = RR - LL, x_U = RL + LR,
+//     x_V = i (LR - RL)), scaled by c_b w_m, and left in the warp's shared-memory buffer with its
+//     W y- and x-weights (es_weights_xy); the next 32 rows are read meanwhile.
+//  2. Per run of rows of one cell, the cell's W x W x 8 block is accumulated in registers as a
+//     product of two small matrices on the tensor cores: G = P^T Y, P[v][(jx, c)] = w_x[v][jx]
+//     x_c[v] (MT m-tiles of 16 rows (jx, c)) and Y[v][jy] = w_y[v][jy] (NT n-tiles of 8), 8 rows v
+//     per mma.m16n8k8 (TF32). Each FP32 operand is split into TF32 hi + lo parts and the
+//     products hi hi, hi lo, lo hi accumulate in FP32 (lo lo is below FP32 rounding). Rows of
+//     a product that are not the run's enter as zeros.
+//  3. Where the cell ends, the block goes to shared memory and from there to the accumulator
+//     by W bulk reductions (one per stencil row, W cells of 32 bytes; two where the row wraps
+//     around a full grid), which run while the warp goes on with its next cell.
+// Channels are gridded at +u only; k_adj_cols forms the -u half by Hermitian symmetrisation.
+//
+// Nothing is shared between warps: no barrier, no uneven end of a work item, no list of work,
+// and no FP32 atomic on shared memory (a compare-and-swap loop), which the form before it
+// paid (one CTA per tile of cells, blocks added to a shared tile, weights from a table of 64
+// bytes per row: in this form the table measured 91 us against 87). Grid stage, us: 1024^2 / 2,000,000 rows (34 per cell) 101 -> 87 with 232 -> 106 MB
+// of DRAM traffic, 256^2 / 50,000 17 -> 14; phi^dagger as a whole: 1024^2 / 200,001 scattered rows
+// (1 per cell) 397 -> 193, 512^2 / 2,000,001 scattered 389 -> 333. Bound by issue (62% of the slots
+// busy), the split and the products before the tensor pipe.
+constexpr int kGridWarps = 4;   // warps of a CTA
 template <int W>
-__host__ __device__ constexpr int grid_plane() {
-  return (kGridTileG + W - 1) * (kGridTileG + W - 1) + 1;
-}
-
-// FORM 3 keeps 8 y-weights and 8 x-weights per row for kGridItemG rows plus 8 spare
-// rows (its last k-step of a chunk may read, and then discard, up to 7 rows past it).
-constexpr int kGridRows3 = kGridItemG + 8;
-// Floats of staged weights per work item (a multiple of 4: the tile planes after them stay 16-byte aligned).
-template <int W, int FORM>
-__host__ __device__ constexpr int grid_wts_floats() {
-  return FORM >= 3 ? 16 * kGridRows3 : (2 * W * kGridV + 3) / 4 * 4;
-}
-
-// Step 1 for one visibility j of a work item: row record r (fx, fy, w), its correlations
-// b0 = (RR, RL), b1 = (LR, LL) and its block scale. FORM 0-2 evaluate its weights into
-// wts as W x-planes then W y-planes of stride kGridV; FORM 3 copies them instead (8
-// y-weights per row for kGridRows3 rows, then 8 x-weights per row, zero past W).
-template <int W, int FORM>
-__device__ __forceinline__ void grid_stage_row(int j, float4 r, float4 b0, float4 b1, float blk_scale, float beta,
-                                               float4* __restrict__ x4, float* __restrict__ wts) {
-  float fx, fy, w;
-  int cx, cy;
-  unpack_rec(r, fx, fy, w, cx, cy);
-  const float sc = blk_scale * w;
-  // x_I = RR + LL, x_Q = RR - LL, x_U = RL + LR, x_V = i (LR - RL).
-  x4[2 * j] = make_float4(sc * (b0.x + b1.z), sc * (b0.y + b1.w), sc * (b0.x - b1.z), sc * (b0.y - b1.w));
-  x4[2 * j + 1] = make_float4(sc * (b0.z + b1.x), sc * (b0.w + b1.y), -sc * (b1.y - b0.w), sc * (b1.x - b0.z));
-  if (FORM == 3) {
-    // Weights arrive by bulk copies from the per-row table (k_row_weights).
-  } else if (FORM == 4) {
-    // The layout of FORM 3, evaluated here instead of copied from the table.
-    float wx[W], wy[W];
-    es_weights<W>(fx, beta, wx);
-    es_weights<W>(fy, beta, wy);
-    float t[8];
+struct GridWarp {
+  static constexpr int MT = (W + 1) / 2, NT = (W + 7) / 8;
+  static constexpr int XP = 2 * MT <= 8 ? 8 : 12;    // x-weights per row (2 MT used)
+  static constexpr int SP = 8 * W + 4;               // stage pitch of a stencil row (2 SP = 24 mod 32 banks for W = 7)
+  static constexpr int kRow = 32 * (8 + 8 * NT + XP);            // floats of the row buffer
+  static constexpr int kFloats = kRow + 2 * ((W * SP + 3) / 4 * 4);   // + two staged blocks
+};
+template <int W>
+__global__ void __launch_bounds__(32 * kGridWarps) k_grid(
+    int M, int rows, const uint16_t* __restrict__ vblk, const float4* __restrict__ rec, const float2* __restrict__ vin,
+    const float* __restrict__ cb, int use_scale, int Wd, int off, int full, int K, float beta,
+    float* __restrict__ Acc) {
+  using T = GridWarp<W>;
+  constexpr int MT = T::MT, NT = T::NT, hw = W / 2;
+  extern __shared__ __align__(16) float4 smw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float* xs = reinterpret_cast<float*>(smw) + warp * T::kFloats;   // 8 channels per row
+  float* wyb = xs + 32 * 8;
+  float* wxb = wyb + 32 * 8 * NT;
+  float* stage = xs + T::kRow;
+  constexpr int kStageF = (T::kFloats - T::kRow) / 2;
+  const long long first = (long long)(blockIdx.x * kGridWarps + warp) * rows;
+  if (first >= M) return;
+  const int m0 = (int)first, m1 = (int)min((long long)M, first + rows);
+  const float4* v4 = reinterpret_cast<const float4*>(vin);
+  const int g = lane >> 2, tig = lane & 3;
+  float d[MT][NT][4];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) t[k] = k < W ? wy[k] : 0.f;
-    float4* py = reinterpret_cast<float4*>(wts) + 2 * j;
-    py[0] = make_float4(t[0], t[1], t[2], t[3]);
-    py[1] = make_float4(t[4], t[5], t[6], t[7]);
+  for (int t = 0; t < MT; ++t)
 #pragma unroll
-    for (int k = 0; k < 8; ++k) t[k] = k < W ? wx[k] : 0.f;
-    float4* px = reinterpret_cast<float4*>(wts + 8 * kGridRows3) + 2 * j;
-    px[0] = make_float4(t[0], t[1], t[2], t[3]);
-    px[1] = make_float4(t[4], t[5], t[6], t[7]);
-  } else {
-    float wx[W], wy[W];
-    es_weights<W>(fx, beta, wx);
-    es_weights<W>(fy, beta, wy);
-    float* wxs = wts;
-    float* wys = wts + W * kGridV;
+    for (int q = 0; q < NT; ++q) d[t][q][0] = d[t][q][1] = d[t][q][2] = d[t][q][3] = 0.f;
+  float4 r, b0, b1;
+  int blk = 0, buf = 0, cell = -1;   // cell: the accumulated block's (grid row << 12 | column), -1: none
+  auto fetch = [&](int m) {
+    const size_t i = min(m + lane, m1 - 1);
+    r = rec[i];
+    b0 = v4[2 * i];
+    b1 = v4[2 * i + 1];
+    if (use_scale) blk = vblk[i];
+  };
+  // The block to the accumulator: d[t][q][i] is cell (jy = 8 q + 2 tig + (i & 1), jx = 2 t + (i >> 1)),
+  // channel g.
+  auto flush = [&]() {
+    float* st = stage + buf * kStageF;
+    bulk_wait_read<1>();   // this lane's reductions of two cells ago have read their buffer
+    __syncwarp();
 #pragma unroll
-    for (int k = 0; k < W; ++k) {
-      wxs[k * kGridV + j] = wx[k];
-      wys[k * kGridV + j] = wy[k];
+    for (int t = 0; t < MT; ++t)
+#pragma unroll
+      for (int q = 0; q < NT; ++q)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int jy = 8 * q + 2 * tig + (i & 1), jx = 2 * t + (i >> 1);
+          if (jy < W && jx < W) st[jy * T::SP + jx * 8 + g] = d[t][q][i];
+          d[t][q][i] = 0.f;
+        }
+    fence_proxy_async();
+    __syncwarp();
+    if (lane < W) {
+      const int gy = (cell >> 12) - hw + lane, gx = (cell & 4095) - hw;
+      const float* src = st + lane * T::SP;
+      if (!full) {
+        bulk_reduce_add(Acc + 8 * ((size_t)gy * Wd + gx), src, W * 32);
+      } else {
+        float* row = Acc + 8 * (size_t)(gy & (K - 1)) * Wd;
+        const int x0 = gx & (K - 1), n0 = min(W, K - x0);
+        bulk_reduce_add(row + 8 * (size_t)x0, src, n0 * 32);
+        if (n0 < W) bulk_reduce_add(row, src + 8 * n0, (W - n0) * 32);
+      }
     }
-  }
-}
-
-// Step 2: every same-cell chunk of the work item, one warp per chunk (FORM as above),
-// added to the channel-planar tile acc (8 planes of grid_plane<W>() floats).
-template <int W, int FORM>
-__device__ __forceinline__ void grid_chunks(const int32_t* __restrict__ chunks, int nc, const float4* __restrict__ x4,
-                                            const float* __restrict__ wts, float* __restrict__ acc) {
-  const float* wxs = wts;
-  const float* wys = wts + W * kGridV;
-  constexpr int TS = kGridTileG;
-  constexpr int SS = TS + W - 1;
-  constexpr int NP = grid_plane<W>();
-  constexpr bool HALF = FORM == 1;
-  constexpr int LPR = HALF ? 16 : 32;            // lanes per row in flight
-  constexpr int CPL = (W * W + LPR - 1) / LPR;   // kernel cells per lane
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const int sub = HALF ? (lane >> 4) : 0, sl = HALF ? (lane & 15) : lane;
-  int wxo[CPL], wyo[CPL], coff[CPL];
+    bulk_commit();
+    buf ^= 1;
+  };
+  fetch(m0);
+  for (int m = m0; m < m1; m += 32) {
+    const int cnt = min(32, m1 - m);
+    int key;
+    {
+      float fx, fy, w;
+      int cx, cy;
+      unpack_rec(r, fx, fy, w, cx, cy);
+      key = gidx(cy, off, full, K) << 12 | gidx(cx, off, full, K);   // lanes past the rows repeat the last row's
+      const float sc = lane < cnt ? (use_scale ? cb[blk] : 1.0f) * w : 0.f;
+      float4* xo = reinterpret_cast<float4*>(xs) + 2 * lane;
+      xo[0] = make_float4(sc * (b0.x + b1.z), sc * (b0.y + b1.w), sc * (b0.x - b1.z), sc * (b0.y - b1.w));
+      xo[1] = make_float4(sc * (b0.z + b1.x), sc * (b0.w + b1.y), -sc * (b1.y - b0.w), sc * (b1.x - b0.z));
+      float4* yo = reinterpret_cast<float4*>(wyb + 8 * NT * lane);
+      float4* po = reinterpret_cast<float4*>(wxb + T::XP * lane);
+      float wx[W], wy[W];
+      es_weights_xy<W>(fx, fy, beta, wx, wy);
+      auto at = [](const float* v, int k) { return k < W ? v[k < W ? k : 0] : 0.f; };
 #pragma unroll
-  for (int q = 0; q < CPL; ++q) {
-    const int cell = sl + LPR * q;
-    const int jy = cell < W * W ? cell / W : 0, jx = cell < W * W ? cell - (cell / W) * W : 0;
-    wxo[q] = jx * kGridV;
-    wyo[q] = jy * kGridV;
-    coff[q] = jy * SS + jx;
-  }
-  const ulonglong2* xv = reinterpret_cast<const ulonglong2*>(x4);
-  for (int c = warp; c < nc; c += nwarps) {
-    const int pk = chunks[c];
-    const int v0 = pk & 1023, cnt = (pk >> 10) & 63, ly = (pk >> 16) & 255, lx = (pk >> 24) & 255;
-    if constexpr (FORM >= 3) {
-      // Tensor cores: the chunk's W x W x 8 block is the product G = P^T Y over its rows,
-      // P[v][(jx, c)] = w_x[v][jx] x_c[v] (64 rows (jx, c) in MT m-tiles of 16) and
-      // Y[v][jy] = w_y[v][jy] (8 columns), k = 8 rows per mma.m16n8k8 (TF32). Each FP32
-      // operand is split into TF32 hi + lo parts and the three products hi hi, hi lo,
-      // lo hi are accumulated in FP32 (the lo lo term is below FP32 rounding). Rows of
-      // the last k-step past the chunk enter as zeros.
-      constexpr int MT = (W + 1) / 2;
-      const int g = lane >> 2, tig = lane & 3;
-      const float* xs = reinterpret_cast<const float*>(x4);
-      const float* wyb = wts;
-      const float* wxb = wts + 8 * kGridRows3;
-      float d[MT][4];
+      for (int q = 0; q < 2 * NT; ++q)
+        yo[q] = make_float4(at(wy, 4 * q), at(wy, 4 * q + 1), at(wy, 4 * q + 2), at(wy, 4 * q + 3));
 #pragma unroll
-      for (int t = 0; t < MT; ++t) d[t][0] = d[t][1] = d[t][2] = d[t][3] = 0.f;
-      const int vend = v0 + cnt;
-      for (int k0 = v0; k0 < vend; k0 += 8) {
+      for (int q = 0; q < T::XP / 4; ++q)
+        po[q] = make_float4(at(wx, 4 * q), at(wx, 4 * q + 1), at(wx, 4 * q + 2), at(wx, 4 * q + 3));
+    }
+    if (m + 32 < m1) fetch(m + 32);
+    // Rows that start a run of another cell than the row before them.
+    const int before = __shfl_up_sync(0xffffffffu, key, 1);
+    unsigned starts = __ballot_sync(0xffffffffu, lane > 0 && key != before);
+    __syncwarp();
+    for (int a = 0; a < cnt;) {
+      const int end = starts ? __ffs(starts) - 1 : cnt;
+      starts &= starts - 1;
+      const int k = __shfl_sync(0xffffffffu, key, a);
+      if (cell >= 0 && k != cell) flush();
+      cell = k;
+      for (int k0 = a; k0 < end; k0 += 8) {
         const int va = k0 + tig, vb = va + 4;
-        // Rows past the chunk (the next chunk's, or the zeroed spare rows after the
-        // item) keep their finite P entries; their Y entries are zeroed.
-        const float xa = xs[8 * va + g], xb = xs[8 * vb + g];
-        uint32_t bh[2], bl[2];
-        tf32_split(va < vend ? wyb[8 * va + g] : 0.f, bh[0], bl[0]);
-        tf32_split(vb < vend ? wyb[8 * vb + g] : 0.f, bh[1], bl[1]);
-        const float4* wa = reinterpret_cast<const float4*>(wxb + 8 * va);
-        const float4* wb = reinterpret_cast<const float4*>(wxb + 8 * vb);
-        const float4 wa0 = wa[0], wa1 = wa[1], wb0 = wb[0], wb1 = wb[1];
-        const float pa[8] = {wa0.x, wa0.y, wa0.z, wa0.w, wa1.x, wa1.y, wa1.z, wa1.w};
-        const float pb[8] = {wb0.x, wb0.y, wb0.z, wb0.w, wb1.x, wb1.y, wb1.z, wb1.w};
+        const int ra = min(va, 31), rb = min(vb, 31);
+        const float xa = xs[8 * ra + g], xb = xs[8 * rb + g];
+        uint32_t bh[NT][2], bl[NT][2];
+#pragma unroll
+        for (int q = 0; q < NT; ++q) {
+          tf32_split(va < end ? wyb[8 * NT * ra + 8 * q + g] : 0.f, bh[q][0], bl[q][0]);
+          tf32_split(vb < end ? wyb[8 * NT * rb + 8 * q + g] : 0.f, bh[q][1], bl[q][1]);
+        }
+        float pa[T::XP], pb[T::XP];
+#pragma unroll
+        for (int q = 0; q < T::XP / 4; ++q) {
+          const float4 wa = reinterpret_cast<const float4*>(wxb + T::XP * ra)[q];
+          const float4 wb = reinterpret_cast<const float4*>(wxb + T::XP * rb)[q];
+          pa[4 * q] = wa.x, pa[4 * q + 1] = wa.y, pa[4 * q + 2] = wa.z, pa[4 * q + 3] = wa.w;
+          pb[4 * q] = wb.x, pb[4 * q + 1] = wb.y, pb[4 * q + 2] = wb.z, pb[4 * q + 3] = wb.w;
+        }
         uint32_t ah[MT][4], al[MT][4];
 #pragma unroll
         for (int t = 0; t < MT; ++t) {
@@ -659,213 +691,21 @@ __device__ __forceinline__ void grid_chunks(const int32_t* __restrict__ chunks, 
         }
         // Small terms first; consecutive products go to different tiles (independent).
 #pragma unroll
-        for (int t = 0; t < MT; ++t) mma_tf32(d[t], al[t], bh);
+        for (int q = 0; q < NT; ++q) {
 #pragma unroll
-        for (int t = 0; t < MT; ++t) mma_tf32(d[t], ah[t], bl);
+          for (int t = 0; t < MT; ++t) mma_tf32(d[t][q], al[t], bh[q]);
 #pragma unroll
-        for (int t = 0; t < MT; ++t) mma_tf32(d[t], ah[t], bh);
-      }
-      // d[t][i]: cell (jy = 2 tig + (i & 1), jx = 2 t + (i >> 1)), channel g.
-      const int base = g * NP + ly * SS + lx;
+          for (int t = 0; t < MT; ++t) mma_tf32(d[t][q], ah[t], bl[q]);
 #pragma unroll
-      for (int t = 0; t < MT; ++t)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int jy = 2 * tig + (i & 1), jx = 2 * t + (i >> 1);
-          if (jy < W && jx < W) atomicAdd(acc + base + jy * SS + jx, d[t][i]);
-        }
-    } else if constexpr (FORM == 2) {
-      static_assert(FORM != 2 || 4 * W <= 32, "row-channel lanes need 4 W <= 32");
-      const int jy = lane >> 2, cp = lane & 3;
-      if (lane < 4 * W) {
-        const u64* xp = reinterpret_cast<const u64*>(x4);   // row v, channel pair cp at 4 v + cp
-        const float* wyr = wys + jy * kGridV;
-        u64 acc2[W];
-#pragma unroll
-        for (int k = 0; k < W; ++k) acc2[k] = 0ull;
-        for (int v = v0; v < v0 + cnt; ++v) {
-          const u64 t = ffma2(fdup(wyr[v]), xp[4 * v + cp], 0ull);
-#pragma unroll
-          for (int k = 0; k < W; ++k) acc2[k] = ffma2(fdup(wxs[k * kGridV + v]), t, acc2[k]);
-        }
-        const int cell0 = (ly + jy) * SS + lx;
-#pragma unroll
-        for (int k = 0; k < W; ++k) {
-          float lo, hi;
-          f2unpack(acc2[k], lo, hi);
-          atomicAdd(acc + (2 * cp) * NP + cell0 + k, lo);
-          atomicAdd(acc + (2 * cp + 1) * NP + cell0 + k, hi);
+          for (int t = 0; t < MT; ++t) mma_tf32(d[t][q], ah[t], bh[q]);
         }
       }
-    } else {
-      // a2[q][p] holds channels (2p, 2p+1) of kernel cell q: packed FP32x2 accumulation.
-      u64 a2[CPL][4];
-#pragma unroll
-      for (int q = 0; q < CPL; ++q)
-#pragma unroll
-        for (int p = 0; p < 4; ++p) a2[q][p] = 0ull;
-      if (HALF) {
-        for (int v = v0 + sub; v < v0 + cnt; v += 2) {
-          const ulonglong2 x0 = xv[2 * v], x1 = xv[2 * v + 1];
-#pragma unroll
-          for (int q = 0; q < CPL; ++q) {
-            const u64 k0 = fdup(wxs[wxo[q] + v] * wys[wyo[q] + v]);
-            a2[q][0] = ffma2(k0, x0.x, a2[q][0]);
-            a2[q][1] = ffma2(k0, x0.y, a2[q][1]);
-            a2[q][2] = ffma2(k0, x1.x, a2[q][2]);
-            a2[q][3] = ffma2(k0, x1.y, a2[q][3]);
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < CPL; ++q)
-#pragma unroll
-          for (int p = 0; p < 4; ++p) {
-            float lo, hi;
-            f2unpack(a2[q][p], lo, hi);
-            lo += __shfl_xor_sync(0xffffffffu, lo, 16);
-            hi += __shfl_xor_sync(0xffffffffu, hi, 16);
-            a2[q][p] = f2pack(lo, hi);
-          }
-      } else {
-        int v = v0;
-        for (; v + 1 < v0 + cnt; v += 2) {
-          const ulonglong2 x0 = xv[2 * v], x1 = xv[2 * v + 1], y0 = xv[2 * v + 2], y1 = xv[2 * v + 3];
-#pragma unroll
-          for (int q = 0; q < CPL; ++q) {
-            const u64 k0 = fdup(wxs[wxo[q] + v] * wys[wyo[q] + v]);
-            const u64 k1 = fdup(wxs[wxo[q] + v + 1] * wys[wyo[q] + v + 1]);
-            a2[q][0] = ffma2(k1, y0.x, ffma2(k0, x0.x, a2[q][0]));
-            a2[q][1] = ffma2(k1, y0.y, ffma2(k0, x0.y, a2[q][1]));
-            a2[q][2] = ffma2(k1, y1.x, ffma2(k0, x1.x, a2[q][2]));
-            a2[q][3] = ffma2(k1, y1.y, ffma2(k0, x1.y, a2[q][3]));
-          }
-        }
-        if (v < v0 + cnt) {
-          const ulonglong2 x0 = xv[2 * v], x1 = xv[2 * v + 1];
-#pragma unroll
-          for (int q = 0; q < CPL; ++q) {
-            const u64 k0 = fdup(wxs[wxo[q] + v] * wys[wyo[q] + v]);
-            a2[q][0] = ffma2(k0, x0.x, a2[q][0]);
-            a2[q][1] = ffma2(k0, x0.y, a2[q][1]);
-            a2[q][2] = ffma2(k0, x1.x, a2[q][2]);
-            a2[q][3] = ffma2(k0, x1.y, a2[q][3]);
-          }
-        }
-      }
-      const int cbase = ly * SS + lx;
-#pragma unroll
-      for (int q = 0; q < CPL; ++q) {
-        if (sub == 0 && sl + LPR * q < W * W) {
-#pragma unroll
-          for (int p = 0; p < 4; ++p) {
-            float lo, hi;
-            f2unpack(a2[q][p], lo, hi);
-            atomicAdd(acc + (2 * p) * NP + cbase + coff[q], lo);
-            atomicAdd(acc + (2 * p + 1) * NP + cbase + coff[q], hi);
-          }
-        }
-      }
+      a = end;
     }
+    __syncwarp();   // the row buffer is read before the next rows replace it
   }
-}
-
-// Step 3: the tile with its halo added to the global accumulator.
-template <int W>
-__device__ __forceinline__ void grid_flush(const float* __restrict__ acc, int ty, int tx, int Wd, int full, int K,
-                                           float4* __restrict__ Acc) {
-  constexpr int TS = kGridTileG;
-  constexpr int SS = TS + W - 1;
-  constexpr int NC = SS * SS;
-  constexpr int NP = grid_plane<W>();
-  constexpr int hw = W / 2;
-  for (int c = threadIdx.x; c < NC; c += blockDim.x) {
-    const int ly = c / SS, lx = c - (c / SS) * SS;
-    int gy = ty * TS - hw + ly, gx = tx * TS - hw + lx;
-    if (full) {
-      gy &= (K - 1);
-      gx &= (K - 1);
-    } else if (gy < 0 || gy >= Wd || gx < 0 || gx >= Wd) {
-      continue;
-    }
-    const float4 lo = make_float4(acc[0 * NP + c], acc[1 * NP + c], acc[2 * NP + c], acc[3 * NP + c]);
-    const float4 hi = make_float4(acc[4 * NP + c], acc[5 * NP + c], acc[6 * NP + c], acc[7 * NP + c]);
-    float4* dst = Acc + 2 * ((size_t)gy * Wd + gx);
-    if (lo.x != 0.f || lo.y != 0.f || lo.z != 0.f || lo.w != 0.f) atomicAdd(dst, lo);
-    if (hi.x != 0.f || hi.y != 0.f || hi.z != 0.f || hi.w != 0.f) atomicAdd(dst + 1, hi);
-  }
-}
-
-constexpr int kGridThreads = 256;   // threads of a gridding CTA
-
-template <int W, int FORM>
-__global__ void __launch_bounds__(kGridThreads) k_grid(
-    const GridItem* __restrict__ items, const int32_t* __restrict__ chunks, const uint16_t* __restrict__ vblk,
-    const float4* __restrict__ rec, const float2* __restrict__ vin, const float* __restrict__ cb, int use_scale,
-    int Wd, int full, int K, float beta, const float* __restrict__ wrow, int M, float4* __restrict__ Acc,
-    int* __restrict__ err) {
-  constexpr int NP = grid_plane<W>();
-  __shared__ uint64_t wbar;                      // FORM 3: completion of the weight copies
-  extern __shared__ float4 smg[];
-  float4* x4 = smg;                              // kGridItemG x 2: mixed, scaled channels of each row
-  float* wts = reinterpret_cast<float*>(smg + 2 * kGridItemG);  // weights (layout by FORM)
-  float* acc = wts + grid_wts_floats<W, FORM>(); // 8 planes of NP floats
-  const GridItem it = items[blockIdx.x];
-  for (int i = threadIdx.x; i < 8 * NP; i += blockDim.x) acc[i] = 0.f;
-  const int nv = it.vend - it.vstart;
-  if (FORM == 3 && threadIdx.x == 0) {
-    mbar_init(&wbar, 1);
-    mbar_expect_tx(&wbar, (uint32_t)nv * 64u);
-    bulk_g2s(wts, wrow + 8 * (size_t)it.vstart, (uint32_t)nv * 32u, &wbar);
-    bulk_g2s(wts + 8 * kGridRows3, wrow + 8 * ((size_t)M + it.vstart), (uint32_t)nv * 32u, &wbar);
-  }
-  const float4* v4 = reinterpret_cast<const float4*>(vin);
-  // Every global load of this thread's rows is issued before the first is used.
-  constexpr int RPT = (kGridItemG + kGridThreads - 1) / kGridThreads;   // rows per thread
-  float4 r[RPT], b0[RPT], b1[RPT];
-  int blk[RPT];
-#pragma unroll
-  for (int q = 0; q < RPT; ++q) {
-    const int j = threadIdx.x + q * kGridThreads;
-    const size_t idx = (size_t)it.vstart + (j < nv ? j : 0);
-    r[q] = rec[idx];
-    b0[q] = v4[2 * idx];
-    b1[q] = v4[2 * idx + 1];
-    blk[q] = use_scale ? vblk[idx] : 0;
-  }
-#pragma unroll
-  for (int q = 0; q < RPT; ++q) {
-    const int j = threadIdx.x + q * kGridThreads;
-    if (j < nv) grid_stage_row<W, FORM>(j, r[q], b0[q], b1[q], use_scale ? cb[blk[q]] : 1.0f, beta, x4, wts);
-  }
-  if (FORM >= 3 && threadIdx.x < 8) {
-    // Spare rows after the item: finite (zero) operands for the last k-step of its last chunk.
-    const int j = nv + threadIdx.x;
-    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (j < kGridItemG) x4[2 * j] = x4[2 * j + 1] = z;
-    float4* yb = reinterpret_cast<float4*>(wts) + 2 * j;
-    float4* xb = reinterpret_cast<float4*>(wts + 8 * kGridRows3) + 2 * j;
-    yb[0] = yb[1] = xb[0] = xb[1] = z;
-  }
-  __syncthreads();
-  if (FORM == 3) {
-    const bool ok = mbar_wait(&wbar, 0);
-    if (__syncthreads_or(!ok)) {
-      if (threadIdx.x == 0) {
-        atomicExch(err, 1);
-        (void)mbar_drain(&wbar, 0);
-      }
-      return;
-    }
-  }
-  grid_chunks<W, FORM>(chunks + it.cstart, it.cend - it.cstart, x4, wts, acc);
-  __syncthreads();
-  grid_flush<W>(acc, it.ty, it.tx, Wd, full, K, Acc);
-}
-
-template <int W, int FORM>
-static constexpr size_t grid_smem() {
-  return (size_t)2 * kGridItemG * sizeof(float4) +
-         (size_t)(grid_wts_floats<W, FORM>() + 8 * grid_plane<W>()) * sizeof(float);
+  flush();
+  bulk_wait_all();   // the reductions are done before the CTA's shared memory goes
 }
 
 // Hermitian symmetrisation + inverse column FFTs for the column pair (kx, -kx).
@@ -1022,22 +862,11 @@ cudaError_t configure_nufft_kernels() {
   if ((e = set_smem((const void*)k_fwd_rows, sm1)) != cudaSuccess) return e;
   if ((e = set_smem((const void*)k_fwd_cols, sm1)) != cudaSuccess) return e;
   if ((e = set_smem((const void*)k_adj_rows, sm1)) != cudaSuccess) return e;
-  const void* grids[] = {(const void*)k_grid<5, 0>, (const void*)k_grid<7, 0>, (const void*)k_grid<9, 0>,
-                         (const void*)k_grid<5, 1>, (const void*)k_grid<7, 1>, (const void*)k_grid<9, 1>,
-                         (const void*)k_grid<5, 2>, (const void*)k_grid<7, 2>, (const void*)k_grid<5, 3>,
-                         (const void*)k_grid<7, 3>, (const void*)k_grid<5, 4>, (const void*)k_grid<7, 4>};
-  const size_t grid_bytes[] = {grid_smem<5, 0>(), grid_smem<7, 0>(), grid_smem<9, 0>(), grid_smem<5, 1>(),
-                               grid_smem<7, 1>(), grid_smem<9, 1>(), grid_smem<5, 2>(), grid_smem<7, 2>(),
-                               grid_smem<5, 3>(), grid_smem<7, 3>(), grid_smem<5, 4>(), grid_smem<7, 4>()};
-  for (int i = 0; i < 12; ++i)
-    if ((e = set_smem(grids[i], grid_bytes[i])) != cudaSuccess) return e;
   // Per-block FP64 accumulators of the degridding kernels (up to 2047 blocks).
-  const void* degrids[] = {(const void*)k_degrid<5, 0>, (const void*)k_degrid<7, 0>, (const void*)k_degrid<9, 0>,
-                           (const void*)k_degrid<5, 1>, (const void*)k_degrid<7, 1>, (const void*)k_degrid<9, 1>,
-                           (const void*)k_degrid<5, 2>, (const void*)k_degrid<7, 2>, (const void*)k_degrid<9, 2>};
+  const void* degrids[] = {(const void*)k_degrid<5>, (const void*)k_degrid<7>, (const void*)k_degrid<9>};
   const size_t degrid_smem[] = {degrid_smem_tiles<5>(), degrid_smem_tiles<7>(), degrid_smem_tiles<9>()};
-  for (int i = 0; i < 9; ++i)
-    if ((e = set_smem(degrids[i], degrid_smem[i % 3] + 2048 * sizeof(double))) != cudaSuccess) return e;
+  for (int i = 0; i < 3; ++i)
+    if ((e = set_smem(degrids[i], degrid_smem[i] + 2048 * sizeof(double))) != cudaSuccess) return e;
   return set_smem((const void*)k_adj_cols, sm2);
 }
 
@@ -1054,11 +883,8 @@ static void launch_degrid(Handle* h, int mode, float2* out) {
   const GridGeom& g = h->g;
   const int nbins = h->nblocks <= kWarpBins ? kWarpBins * 8 : h->nblocks;   // 8 warps of 256 threads
   const size_t sm = degrid_smem_tiles<W>() + (size_t)nbins * sizeof(double);
-  const int form = h->tune[PS_TUNE_DEGRID];
-  auto kern = form == 1 ? k_degrid<W, 1> : (form == 2 ? k_degrid<W, 2> : k_degrid<W, 0>);
-  kern<<<h->nitems, 256, sm, h->stream>>>(h->items, h->gchunks, h->rec, h->G, g.Wd, g.off, g.full, g.K, g.beta, mode,
-                                          h->R, h->Y, h->cb, (float)(1.0 / h->rho2), h->vblk, h->nblocks,
-                                          h->block_sum, out);
+  k_degrid<W><<<h->nitems, 256, sm, h->stream>>>(h->items, h->rec, h->G, g.Wd, g.off, g.full, g.K, g.beta, mode, h->R, h->Y,
+                                          h->cb, (float)(1.0 / h->rho2), h->vblk, h->nblocks, h->block_sum, out);
 }
 
 cudaError_t nufft_degrid(Handle* h, int mode, float2* out) {
@@ -1082,65 +908,33 @@ cudaError_t block_scales(Handle* h) {
   return cudaGetLastError();
 }
 
-// Kernel weights of every stored row, computed once per set of measurements (the rows'
-// fractional offsets do not change): y-taps in the first M x 8 floats, x-taps after.
-template <int W>
-__global__ void k_row_weights(const float4* __restrict__ rec, int M, float beta, float* __restrict__ wrow) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= M) return;
-  float fx, fy, w;
-  int cx, cy;
-  unpack_rec(rec[m], fx, fy, w, cx, cy);
-  float wx[W], wy[W], t[8];
-  es_weights<W>(fx, beta, wx);
-  es_weights<W>(fy, beta, wy);
-  float4* py = reinterpret_cast<float4*>(wrow) + 2 * (size_t)m;
-  float4* px = reinterpret_cast<float4*>(wrow + 8 * (size_t)M) + 2 * (size_t)m;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) t[k] = k < W ? wy[k] : 0.f;
-  py[0] = make_float4(t[0], t[1], t[2], t[3]);
-  py[1] = make_float4(t[4], t[5], t[6], t[7]);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) t[k] = k < W ? wx[k] : 0.f;
-  px[0] = make_float4(t[0], t[1], t[2], t[3]);
-  px[1] = make_float4(t[4], t[5], t[6], t[7]);
-}
-
-cudaError_t nufft_row_weights(Handle* h) {
-  if (!h->wrow || h->M == 0) return cudaSuccess;
-  const int blocks = (h->M + 255) / 256;
-  if (h->g.W == 5)
-    k_row_weights<5><<<blocks, 256, 0, h->stream>>>(h->rec, h->M, h->g.beta, h->wrow);
-  else
-    k_row_weights<7><<<blocks, 256, 0, h->stream>>>(h->rec, h->M, h->g.beta, h->wrow);
-  return cudaGetLastError();
-}
-
-template <int W, int FORM>
-static void launch_grid_form(Handle* h, const float2* in, int use_scale) {
-  const GridGeom& g = h->g;
-  k_grid<W, FORM><<<h->nitems_g, kGridThreads, grid_smem<W, FORM>(), h->stream>>>(
-      h->items_g, h->gchunks_g, h->vblk, h->rec, in, h->cb, use_scale, g.Wd, g.full, g.K, g.beta, h->wrow, h->M, h->Acc,
-      h->dev_flags);
-}
-
 template <int W>
 static void launch_grid(Handle* h, const float2* in, int use_scale) {
-  // FORM 2 needs 4 W <= 32 lanes and FORMs 3-4 8 taps per row: W = 9 runs FORM 0 for them.
-  constexpr bool narrow = W <= 8;
-  switch (h->tune[PS_TUNE_GRID]) {
-    case 1: launch_grid_form<W, 1>(h, in, use_scale); break;
-    case 2: launch_grid_form<W, narrow ? 2 : 0>(h, in, use_scale); break;
-    case 3: launch_grid_form<W, narrow ? 3 : 0>(h, in, use_scale); break;
-    case 4: launch_grid_form<W, narrow ? 4 : 0>(h, in, use_scale); break;
-    default: launch_grid_form<W, 0>(h, in, use_scale); break;
-  }
+  const GridGeom& g = h->g;
+  // Rows per warp: 64 where that leaves two warps for every scheduler of the chip and a cell
+  // holds enough rows that cutting its run at a warp's end costs more than parallelism gives,
+  // else 32. phi^dagger, us at 32 / 64 / 128 rows: 1024^2 / 2,000,000 rows (34 per cell) 147 / 143 /
+  // 144, 64^2 / 100,000 (73 per cell) 35 / 30 / 30; 256^2 / 50,000 29 / 31 / 35, 2048^2 / 700,001
+  // (4 per cell) 215 / 222 / 243, 1024^2 / 200,001 scattered (1 per cell) 193 / 200 / 219.
+  // Rows per warp. Few rows: 8, for more warps with fewer cells each. Many rows in dense cells:
+  // 64, where that leaves two warps for every scheduler of the chip and a cell holds enough
+  // rows that cutting its run at a warp's end costs more than parallelism gives. Else 32.
+  // phi^dagger, us at 8 / 32 / 64 rows: 64^2 / 2,000 rows 27 / 29 / 31, 128^2 / 6,001 scattered
+  // (1 per cell) 31 / 43 / 60, 64^2 / 25,153 33 / 27 / 29, 256^2 / 50,000 31 / 29 / 31, 2048^2 /
+  // 700,001 (4 per cell) - / 215 / 222; 64^2 / 100,000 (73 per cell) - / 35 / 30, 1024^2 / 2,000,000
+  // (34 per cell) - / 147 / 143.
+  const int warps = 8 * std::max(1, h->num_sms);
+  const int rows = h->M <= 12 * warps ? 8 : (h->M >= 64 * warps && h->M / std::max(1, h->ncells) >= 16 ? 64 : 32);
+  const int ctas = (int)(((int64_t)h->M + (int64_t)rows * kGridWarps - 1) / ((int64_t)rows * kGridWarps));
+  k_grid<W><<<ctas, 32 * kGridWarps, kGridWarps * GridWarp<W>::kFloats * sizeof(float), h->stream>>>(
+      h->M, rows, h->vblk, h->rec, in, h->cb, use_scale, g.Wd, g.off, g.full, g.K, g.beta,
+      reinterpret_cast<float*>(h->Acc));
 }
 
 cudaError_t nufft_grid(Handle* h, const float2* in, int use_scale) {
   const GridGeom& g = h->g;
   cudaError_t e = cudaMemsetAsync(h->Acc, 0, (size_t)g.Wd * g.Wd * 2 * sizeof(float4), h->stream);
-  if (e != cudaSuccess || h->nitems_g == 0) return e;
+  if (e != cudaSuccess || h->M == 0) return e;
   switch (g.W) {
     case 5: launch_grid<5>(h, in, use_scale); break;
     case 9: launch_grid<9>(h, in, use_scale); break;

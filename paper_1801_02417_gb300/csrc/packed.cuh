@@ -45,6 +45,20 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
                "l"(src), "r"(bytes), "r"(smem_u32(bar))
                : "memory");
 }
+// Bulk reduction: global[0 .. bytes) += shared[0 .. bytes) in FP32 (16-byte aligned, a multiple of 16
+// bytes), in this thread's bulk groups: commit closes a group; wait_read<N> waits until at most N
+// groups have still to read their shared memory, wait_all until every group is done.
+__device__ __forceinline__ void bulk_reduce_add(float* dst, const float* src, uint32_t bytes) {
+  asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(dst),
+               "r"(smem_u32(src)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void bulk_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // 2D tensor-map copy (TMA) of one box into shared memory (128-byte aligned destination), completing
 // on `bar`. The map lives in kernel-parameter space (a __grid_constant__ argument). x is the
 // innermost coordinate in elements (x * 4 bytes a multiple of 16 for float data); parts of the
