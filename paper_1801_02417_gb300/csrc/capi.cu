@@ -6,8 +6,7 @@
 //   k_analysis x levels         steps 5-6 (Psi^dagger of 2S'-S, soft-threshold dual)
 //   k_synthesis x levels        Psi A^(k+1) for the next step 3
 //   k_fwd_rows, k_fwd_cols      F Z of phi(2S'-S)                  (step 7)
-//   k_degrid                    G, mixing by L, B~ and ||B~/rho2 - Y||^2 partials
-//   k_block_scale               step 8 (l2-ball factor per block)
+//   k_degrid                    G, mixing by L, B~ and ||B~/rho2 - Y||^2; step 8 (l2-ball factor per block)
 //   k_grid, k_adj_cols, k_adj_rows   phi^dagger B^(k+1) for the next step 3
 // B is kept as R = B~/rho2 - Y with a per-block factor: B = c_b R, c_b =
 // rho2 (1 - min(1, eps_b / ||R_b||)), which is the step-8 result written out.
@@ -134,6 +133,8 @@ static void free_vis(Handle* h) {
   dfree(h, h->eps, (size_t)h->nblocks);
   dfree(h, h->cb, (size_t)h->nblocks);
   dfree(h, h->block_sum, (size_t)h->nblocks);
+  dfree(h, h->block_norm_sq, (size_t)h->nblocks);
+  dfree(h, h->block_done, 1);
   dfree(h, h->items, (size_t)h->nitems);
   dfree(h, h->vblk, M);
   const size_t Wd = h->g.Wd;
@@ -213,7 +214,7 @@ static ps_status compute_derived(Handle* h) {
   }
   CK(h, ps::sara_synthesis(h, h->A, h->PsiA));
   if (h->M > 0) {
-    CK(h, ps::nufft_grid(h, h->R, 1));
+    CK(h, ps::nufft_grid(h, h->R, 1, false));
     CK(h, ps::nufft_adjoint_image(h, h->Adj));
   } else {
     CK(h, cudaMemsetAsync(h->Adj, 0, 4 * (size_t)h->N * sizeof(float), h->stream));
@@ -238,16 +239,26 @@ static cudaError_t nufft_chain(Handle* h, cudaEvent_t* ev) {
   auto mark = [&](int i) { return ev ? cudaEventRecord(ev[i], h->stream) : cudaSuccess; };
   cudaError_t e;
   if ((e = mark(PS_STAGE_FWD_FFT)) != cudaSuccess) return e;
-  if (h->M > 0 && (e = ps::nufft_forward_grid(h, h->Xb)) != cudaSuccess) return e;
+  if (h->M > 0 && (e = ps::nufft_forward_grid(h, h->Xb, true)) != cudaSuccess) return e;
   if ((e = mark(PS_STAGE_DEGRID)) != cudaSuccess) return e;
   if (h->M > 0 && (e = ps::nufft_degrid(h, ps::DEG_DUAL, nullptr)) != cudaSuccess) return e;
   if ((e = mark(PS_STAGE_BALL)) != cudaSuccess) return e;
-  if (h->M > 0 && (e = ps::block_scales(h)) != cudaSuccess) return e;
   if ((e = mark(PS_STAGE_GRID)) != cudaSuccess) return e;
-  if (h->M > 0 && (e = ps::nufft_grid(h, h->R, 1)) != cudaSuccess) return e;
+  if (h->M > 0 && (e = ps::nufft_grid(h, h->R, 1, true)) != cudaSuccess) return e;
   if ((e = mark(PS_STAGE_ADJ_FFT)) != cudaSuccess) return e;
   if (h->M > 0 && (e = ps::nufft_adjoint_image(h, h->Adj)) != cudaSuccess) return e;
   return mark(PS_NSTAGES);
+}
+
+// The NUFFT chain beside a SARA chain. Where the SARA chain is the longer one (above 64^2), the
+// early start of NUFFT kernels takes room that it would use: us per iteration with early NUFFT
+// launches / ordinary ones (SARA launches early in both): 64^2 26.4 / 30.5, 128^2 41.7 / 39.2, 256^2
+// 65.1 / 58.6, 512^2 125 / 120, 1024^2 454.7 / 455.9, 2048^2 1185 / 1177.
+static cudaError_t nufft_chain_beside(Handle* h) {
+  h->early = h->n <= 64;
+  const cudaError_t e = nufft_chain(h, nullptr);
+  h->early = true;
+  return e;
 }
 
 // Algorithm 3: the data-term gradient of the next primal step, at the new S:
@@ -257,12 +268,12 @@ static cudaError_t nufft_gradient_chain(Handle* h, cudaEvent_t* ev) {
   auto mark = [&](int i) { return ev ? cudaEventRecord(ev[i], h->stream) : cudaSuccess; };
   cudaError_t e;
   if ((e = mark(PS_STAGE_FWD_FFT)) != cudaSuccess) return e;
-  if (h->M > 0 && (e = ps::nufft_forward_grid(h, h->S)) != cudaSuccess) return e;
+  if (h->M > 0 && (e = ps::nufft_forward_grid(h, h->S, true)) != cudaSuccess) return e;
   if ((e = mark(PS_STAGE_DEGRID)) != cudaSuccess) return e;
   if (h->M > 0 && (e = ps::nufft_degrid(h, ps::DEG_RESID, h->vtmp)) != cudaSuccess) return e;
   if ((e = mark(PS_STAGE_BALL)) != cudaSuccess) return e;
   if ((e = mark(PS_STAGE_GRID)) != cudaSuccess) return e;
-  if (h->M > 0 && (e = ps::nufft_grid(h, h->vtmp, 0)) != cudaSuccess) return e;
+  if (h->M > 0 && (e = ps::nufft_grid(h, h->vtmp, 0, true)) != cudaSuccess) return e;
   if ((e = mark(PS_STAGE_ADJ_FFT)) != cudaSuccess) return e;
   if (h->M > 0 && (e = ps::nufft_adjoint_image(h, h->Adj)) != cudaSuccess) return e;
   return mark(PS_NSTAGES);
@@ -326,7 +337,7 @@ static cudaError_t one_iteration(Handle* h, cudaEvent_t* ev = nullptr) {
   h->stream = main;
   if (e != cudaSuccess) return e;
   if (e2 != cudaSuccess) return e2;
-  if ((e = nufft_chain(h, nullptr)) != cudaSuccess) return e;
+  if ((e = nufft_chain_beside(h)) != cudaSuccess) return e;
   return cudaStreamWaitEvent(h->stream, h->ev_join, 0);
 }
 
@@ -757,6 +768,7 @@ ps_status ps_set_measurements(ps_handle* h, int64_t M64, const double* uv, const
             dalloc(h, &h->perm, (size_t)M) == cudaSuccess && dalloc(h, &h->eps, (size_t)h->nblocks) == cudaSuccess &&
             dalloc(h, &h->cb, (size_t)h->nblocks) == cudaSuccess &&
             dalloc(h, &h->block_sum, (size_t)h->nblocks) == cudaSuccess &&
+            dalloc(h, &h->block_norm_sq, (size_t)h->nblocks) == cudaSuccess && dalloc(h, &h->block_done, 1) == cudaSuccess &&
             dalloc(h, &h->items, items.size()) == cudaSuccess &&
             dalloc(h, &h->vblk, (size_t)M) == cudaSuccess &&
             dalloc(h, &h->T1, (size_t)h->n * Wd) == cudaSuccess && dalloc(h, &h->G, Wd * Wd) == cudaSuccess &&
@@ -780,6 +792,8 @@ ps_status ps_set_measurements(ps_handle* h, int64_t M64, const double* uv, const
     corrh[q] = (float)(1.0 / ps::es_fourier(2.0 * M_PI * (q - h->n / 2) / g.K, g.W, g.beta));
     if (q > 0 && q < h->n / 2) corrh[h->n - q] = corrh[q];
   }
+  CK(h, cudaMemsetAsync(h->block_done, 0, sizeof(int), h->stream));
+  if (h->nblocks > 0) CK(h, cudaMemsetAsync(h->block_sum, 0, h->nblocks * sizeof(double), h->stream));
   CK(h, cudaMemcpyAsync(h->tw, twh.data(), twh.size() * sizeof(float2), cudaMemcpyHostToDevice, h->stream));
   CK(h, cudaMemcpyAsync(h->corr, corrh.data(), corrh.size() * sizeof(float), cudaMemcpyHostToDevice, h->stream));
   if (M > 0) {
@@ -858,9 +872,9 @@ static ps_status opnorm_lanczos(Handle* h) {
   std::vector<double> al, be;
   double theta = 0.0, beta = 0.0;
   for (int j = 0; j < 300; ++j) {
-    CK(h, ps::nufft_forward_grid(h, v));
+    CK(h, ps::nufft_forward_grid(h, v, true));
     CK(h, ps::nufft_degrid(h, ps::DEG_APPLY, h->vtmp));
-    CK(h, ps::nufft_grid(h, h->vtmp, 0));
+    CK(h, ps::nufft_grid(h, h->vtmp, 0, true));
     CK(h, ps::nufft_adjoint_image(h, w));
     CK(h, ps::reduce_dot(h, w, v, N4, dres));
     CK(h, cudaMemcpyAsync(h->red_host, dres, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
@@ -896,7 +910,7 @@ static ps_status default_gamma(Handle* h) {
     h->gamma_default = h->cfg.gamma;
   } else if (h->M > 0 && h->opnorm_sq > 0) {
     double* dres = h->red + (size_t)h->red_cap - 600;
-    CK(h, ps::nufft_grid(h, h->Y, 0));
+    CK(h, ps::nufft_grid(h, h->Y, 0, false));
     CK(h, ps::nufft_adjoint_image(h, h->Adj));
     CK(h, ps::dirac_apply(h, h->Adj, h->A, nullptr, ps::SARA_APPLY, 1.0f / 3.0f, 0.f, 0.f));
     CK(h, ps::sara_analysis(h, h->Adj, h->A, nullptr, ps::SARA_APPLY, 1.0f / 3.0f, 0.f, 0.f));
@@ -1146,12 +1160,12 @@ ps_status ps_compute_stats(ps_handle* h, double zeta_sigma, ps_stats* out) {
   std::vector<double> bsum(h->nblocks);
   double rms = 0.0;
   if (h->M > 0) {
-    CK(h, ps::nufft_forward_grid(h, h->S));
+    CK(h, ps::nufft_forward_grid(h, h->S, true));
     CK(h, ps::nufft_degrid(h, ps::DEG_RESID, h->vtmp));
-    CK(h, cudaMemcpyAsync(bsum.data(), h->block_sum, bsum.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, ps::nufft_grid(h, h->vtmp, 0));
+    CK(h, ps::nufft_grid(h, h->vtmp, 0, true));
     CK(h, ps::nufft_adjoint_image(h, h->tmp4));
     CK(h, ps::reduce_dot(h, h->tmp4, h->tmp4, N, dres));
+    CK(h, cudaMemcpyAsync(bsum.data(), h->block_norm_sq, bsum.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaMemcpyAsync(h->red_host, dres, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     rms = std::sqrt(h->red_host[0] / (double)N);
@@ -1200,7 +1214,7 @@ ps_status ps_apply_phi(ps_handle* h, const float* S, float* Y, int32_t device_pt
     CK(h, cudaMemcpyAsync(h->tmp4, S, N4 * sizeof(float), cudaMemcpyHostToDevice, h->stream));
     X = h->tmp4;
   }
-  CK(h, ps::nufft_forward_grid(h, X));
+  CK(h, ps::nufft_forward_grid(h, X, false));
   CK(h, ps::nufft_degrid(h, ps::DEG_APPLY, h->vtmp));
   if (device_ptrs) {
     CK(h, ps::scatter_vis(h, h->vtmp, (float2*)Y));
@@ -1237,7 +1251,7 @@ ps_status ps_apply_phi_adjoint(ps_handle* h, const float* Yin, float* S, int32_t
     CK(h, e);
   }
   if (h->M > 0) {
-    CK(h, ps::nufft_grid(h, h->vtmp, 0));
+    CK(h, ps::nufft_grid(h, h->vtmp, 0, false));
     CK(h, ps::nufft_adjoint_image(h, out));
   }
   if (!device_ptrs) return copy_out(h, h->tmp4, S, N4 * sizeof(float), 0);
@@ -1380,15 +1394,15 @@ ps_status ps_autotune(ps_handle* h, int32_t reps, int32_t* choices, double* ms) 
   // from the spectrum of the current S, on a scratch copy of the dual: the candidates read and
   // write the visibility rows as in the iteration, and the state's dual is untouched.
   if (h->M > 0) {
-    CK(h, ps::nufft_forward_grid(h, h->S));
+    CK(h, ps::nufft_forward_grid(h, h->S, false));
     CK(h, cudaMemcpyAsync(h->vtmp, h->R, 4 * (size_t)h->M * sizeof(float2), cudaMemcpyDeviceToDevice, h->stream));
     float2* const R_state = h->R;
     h->R = h->vtmp;
-    st = pick(PS_TUNE_DEGRID, [&] { return ps::nufft_degrid(h, ps::DEG_DUAL, nullptr); });
+    st = pick(PS_TUNE_DEGRID, [&] { return ps::nufft_degrid(h, ps::DEG_DUAL, nullptr, true); });
     h->R = R_state;
     if (st != PS_OK) return st;
     // Gridding: the current dual into the accumulator (an intermediate; phi^dagger B is kept).
-    st = pick(PS_TUNE_GRID, [&] { return ps::nufft_grid(h, h->R, 1); });
+    st = pick(PS_TUNE_GRID, [&] { return ps::nufft_grid(h, h->R, 1, false); });
     if (st != PS_OK) return st;
   }
   if (ps::tv_mode(h->mode)) h->derived_valid = false;   // the SARA synthesis timing wrote PsiA
@@ -1421,8 +1435,8 @@ int32_t ps_kernels_per_iteration(const ps_handle* h) {
   if (!h) return 0;
   int k = 1;                                   // k_primal
   if (ps::tv_mode(h->mode)) return k + 2 + (h->M > 0 ? 2 + 1 + 1 + 2 : 0);   // TV dual + adjoint, gradient chain
-  if (h->mode != PS_NNLS) k += 2 * h->L;       // analysis + synthesis levels
-  if (h->M > 0) k += 2 + 1 + 1 + 1 + 2;        // fwd rows/cols, degrid, block scale, grid, adj cols/rows
+  if (h->mode != PS_NNLS) k += ps::sara_launches(h->n, h->L);
+  if (h->M > 0) k += 2 + 1 + 1 + 2;            // fwd rows/cols, degrid, grid, adj cols/rows
   return k;
 }
 
@@ -1825,7 +1839,7 @@ static ps_status batch_build(ps_batch* b) {
     for (Handle* h : c.hs) {
       const size_t i = index_of(h);
       if (err == cudaSuccess) err = cudaStreamWaitEvent(h->stream, c.ev_primal, 0);
-      if (err == cudaSuccess) err = nufft_chain(h, nullptr);
+      if (err == cudaSuccess) err = nufft_chain_beside(h);
       if (err == cudaSuccess) err = cudaEventRecord(b->join[i], h->stream);
       if (err == cudaSuccess) err = cudaStreamWaitEvent(b->stream, b->join[i], 0);
     }

@@ -90,7 +90,9 @@ struct Handle {
   float2 *vtmp = nullptr;     // M x 4 scratch
   double *eps = nullptr;      // per block radius (device)
   float *cb = nullptr;        // per block scale c_b (device)
-  double *block_sum = nullptr;     // nblocks FP64 sums filled by the degridding kernel
+  double *block_sum = nullptr;     // nblocks FP64 sums of a running degridding launch (zero between launches)
+  double *block_norm_sq = nullptr; // those of the last one that formed them
+  int *block_done = nullptr;       // its finished CTAs (zero between launches)
   int ncells = 0;                  // cells that hold a row
   int nitems = 0;
   GridItem *items = nullptr;       // degridding work items
@@ -112,6 +114,9 @@ struct Handle {
   // Launch choices (PS_TUNE_* slots) and the device's SM count (persistent grids).
   int32_t tune[PS_TUNE_COUNT] = {};
   int num_sms = 0;
+
+  // Whether NUFFT launches may start before the kernel before them has ended (launch_after).
+  bool early = true;
 
   // CUDA graph of one iteration.
   cudaGraphExec_t graph = nullptr;
@@ -138,15 +143,16 @@ cudaError_t upload_filters(const double h[kDb][kMaxTaps], cudaStream_t stream);
 cudaError_t upload_es_polys(cudaStream_t stream);
 
 // NUFFT pieces (nufft.cu).
-cudaError_t nufft_forward_grid(Handle* h, const float* X);                 // X (4 planes) -> G
-cudaError_t nufft_degrid(Handle* h, int mode, float2* out);                // G -> visibilities
-cudaError_t nufft_grid(Handle* h, const float2* in, int use_block_scale);  // visibilities -> Acc
+// X (4 planes) -> G; clear_acc: the gridding accumulator too, for the nufft_grid(.., cleared) that follows.
+cudaError_t nufft_forward_grid(Handle* h, const float* X, bool clear_acc);
+// G -> visibilities; DEG_DUAL also steps the l2-ball factors c_b, unless keep_cb.
+cudaError_t nufft_degrid(Handle* h, int mode, float2* out, bool keep_cb = false);
+cudaError_t nufft_grid(Handle* h, const float2* in, int use_block_scale, bool cleared);  // visibilities -> Acc
 cudaError_t tv_dual(Handle* h);      // Algorithm 3 steps 5-6 on Xb -> A (TV layout)
 cudaError_t tv_adjoint(Handle* h);   // Psi A = grad^T A_tv (+ A_l1) -> PsiA
 __host__ __device__ inline bool tv_mode(int m) { return m >= PS_TV && m <= PS_L1TV_NC; }
 __host__ __device__ inline bool constrained_mode(int m) { return m == PS_POLARIZED || m == PS_SOC || m == PS_TV || m == PS_L1TV; }
 cudaError_t nufft_adjoint_image(Handle* h, float* out);                    // Acc -> 4 planes
-cudaError_t block_scales(Handle* h);                                        // chunk partials -> c_b
 
 // SARA pieces (sara.cu).
 // `fine_done` (may be null) is recorded on h->stream after the level-1 analysis launch;
@@ -154,6 +160,8 @@ cudaError_t block_scales(Handle* h);                                        // c
 cudaError_t sara_analysis(Handle* h, const float* X, float* coef, float* thr, int mode,
                           float scale, float gamma, float delta, cudaEvent_t fine_done = nullptr);
 cudaError_t sara_synthesis(Handle* h, const float* coef, float* out, cudaEvent_t fine_start = nullptr);
+
+int sara_launches(int n, int L);   // kernels of one analysis and one synthesis
 
 // Elementwise / reductions (prox.cu).
 int sweep_blocks(int N);   // CTAs of the per-pixel sweep (8 FP64 partials each)

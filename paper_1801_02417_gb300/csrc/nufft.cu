@@ -14,8 +14,8 @@
 //   k_fwd_rows    row FFTs of the de-apodised, zero-padded rows     (n CTAs)
 //   k_fwd_cols    column FFTs, kept on the window                    (Wd CTAs)
 //   k_degrid      interpolation + Stokes->correlation mixing + dual update of B
-//                 and per-block FP64 sums of ||B~/rho2 - Y||^2        (1 CTA / work item)
-//   k_block_scale per-block l2-ball projection factor (FP64)
+//                 + per-block FP64 sums of ||B~/rho2 - Y||^2 and the l2-ball factors
+//                                                                   (1 CTA / work item)
 //   k_grid        mixing by conj(L) + gridding, one warp per run of rows
 //   k_adj_cols    Hermitian symmetrisation + inverse column FFTs     (R+1 CTAs)
 //   k_adj_rows    inverse row FFTs + crop + de-apodisation -> phi^dagger planes
@@ -165,8 +165,12 @@ __device__ __forceinline__ int gidx(int k, int off, int full, int K) {
 // ---------------------------------------------------------------- forward
 __global__ void k_fwd_rows(const float* __restrict__ X, int n, int N, const float* __restrict__ corr,
                            const float2* __restrict__ tw, int K, int logK, float4* __restrict__ T1,
-                           int Wd, int off, int full) {
+                           int Wd, int off, int full, float4* __restrict__ clear, int nclear) {
   extern __shared__ float4 sm[];
+  pdl_wait();
+  // The accumulator of the gridding that follows in the chain (none: nclear = 0).
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nclear; i += gridDim.x * blockDim.x)
+    clear[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   float4* buf = sm;
   const int p = blockIdx.x;
   const float cy = corr[p];
@@ -191,6 +195,7 @@ __global__ void k_fwd_rows(const float* __restrict__ X, int n, int N, const floa
 __global__ void k_fwd_cols(const float4* __restrict__ T1, int n, const float2* __restrict__ tw, int K,
                            int logK, float4* __restrict__ G, int Wd, int off, int full) {
   extern __shared__ float4 sm[];
+  pdl_wait();
   float4* buf = sm;
   const int gx = blockIdx.x;
   for (int p = threadIdx.x; p < n; p += blockDim.x) {
@@ -302,7 +307,7 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
 // (at -u) to the row's visibilities (or residuals); returns its term of the per-block sums
 // and its block (blk, left alone by DEG_APPLY).
 __device__ __forceinline__ float degrid_finish(int m, float w, float4 sp, float4 sn, int mode, float2* __restrict__ R,
-                                               const float2* __restrict__ Yv, const float* __restrict__ cb,
+                                               const float2* __restrict__ Yv, const float* cb,
                                                float inv_rho2, const uint16_t* __restrict__ vblk,
                                                float2* __restrict__ out, int& blk) {
   float4* R4 = reinterpret_cast<float4*>(R);
@@ -389,7 +394,7 @@ template <int W>
 __device__ __forceinline__ void degrid_row(int m, bool active, const GridItem& it, const float4* __restrict__ rec,
                                            const float4* Gp, const float4* Gn, int off, int full, int K, float beta,
                                            int mode, float2* __restrict__ R, const float2* __restrict__ Yv,
-                                           const float* __restrict__ cb, float inv_rho2,
+                                           const float* cb, float inv_rho2,
                                            const uint16_t* __restrict__ vblk, bool shared, double* sums,
                                            float2* __restrict__ out) {
   constexpr int TS = kGridTile;
@@ -446,16 +451,28 @@ __device__ __forceinline__ void degrid_row(int m, bool active, const GridItem& i
 // fixed offsets from its centre. Per-block sums of ||B~/rho2 - Y||^2 (DUAL) or
 // ||Y - phi X||^2 (RESID): per row and per warp group of same-block lanes in FP32,
 // then in FP64 through per-warp shared bins (up to kWarpBins blocks; shared FP64
-// atomics beyond) and one global FP64 atomic per block and CTA (block_sum, cleared
-// by the caller).
+// atomics beyond) and one global FP64 atomic per block and CTA; the last CTA to end takes
+// the l2-ball step.
+// The per-block sums and what becomes of them at the end of a launch: sum (cleared before and after),
+// done (CTAs that have added theirs; 0 between launches), norm_sq, and the factors cb (null: kept).
+struct BallStep {
+  double* sum;
+  int* done;
+  double* norm_sq;
+  float* cb;
+  const double* eps;
+  double rho2;
+  int literal;
+};
+
 // Registers are capped for 6 CTAs per SM at W = 7 (40 of 67: more rows in flight per SM, 100
 // against 111 us at 1024^2 / 2,000,000 rows; other widths would spill and run without a cap).
 template <int W>
 __global__ void __launch_bounds__(256, W == 7 ? 6 : 0) k_degrid(
     const GridItem* __restrict__ items, const float4* __restrict__ rec, const float4* __restrict__ G, int Wd,
     int off, int full, int K, float beta, int mode, float2* __restrict__ R, const float2* __restrict__ Yv,
-    const float* __restrict__ cb, float inv_rho2, const uint16_t* __restrict__ vblk, int nblocks,
-    double* __restrict__ block_sum, float2* __restrict__ out) {
+    const float* cb, float inv_rho2, const uint16_t* __restrict__ vblk, int nblocks, BallStep ball,
+    float2* __restrict__ out) {
   constexpr int TS = kGridTile;
   constexpr int SS = TS + W - 1;
   constexpr int hw = W / 2;
@@ -463,6 +480,8 @@ __global__ void __launch_bounds__(256, W == 7 ? 6 : 0) k_degrid(
   float4* Gp = smd;                 // +u cells: grid rows/cols ty*TS - hw + [0, SS)
   float4* Gn = smd + SS * SS;       // -u cells: mirrored rows/cols -(ty*TS + TS-1) - hw + [0, SS)
   double* bsum = reinterpret_cast<double*>(smd + 2 * SS * SS);
+  __shared__ int s_last;
+  pdl_wait();
   const GridItem it = items[blockIdx.x];
   const bool reduce = (mode != DEG_APPLY);
   const bool private_bins = nblocks <= kWarpBins;   // per-warp bins: kWarpBins x 8 warps doubles
@@ -503,7 +522,28 @@ __global__ void __launch_bounds__(256, W == 7 ? 6 : 0) k_degrid(
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += bsum[w * kWarpBins + b];
       else
         t = bsum[b];
-      if (t != 0.0) atomicAdd(&block_sum[b], t);
+      if (t != 0.0) atomicAdd(&ball.sum[b], t);
+    }
+    // The CTA that finds every other one done turns the sums into the l2-ball factors
+    // (Algorithm 1 step 8: with r = ||B~/rho2 - Y||_b, c_b = rho2 (1 - min(1, radius / r))) and
+    // leaves the sums cleared for the next launch.
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(ball.done, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (s_last) {
+      __threadfence();
+      for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
+        const double q = __ldcg(&ball.sum[b]);
+        ball.sum[b] = 0.0;
+        ball.norm_sq[b] = q;
+        if (ball.cb) {
+          const double r = sqrt(q);
+          const double radius = ball.literal ? ball.eps[b] / ball.rho2 : ball.eps[b];
+          ball.cb[b] = (float)(ball.rho2 * (1.0 - (r > radius ? radius / r : 1.0)));
+        }
+      }
+      if (threadIdx.x == 0) *ball.done = 0;
     }
   }
 }
@@ -511,18 +551,6 @@ __global__ void __launch_bounds__(256, W == 7 ? 6 : 0) k_degrid(
 template <int W>
 static constexpr size_t degrid_smem_tiles() {
   return (size_t)2 * (kGridTile + W - 1) * (kGridTile + W - 1) * sizeof(float4);
-}
-
-// Per-block factor c_b of B = c_b R after the l2-ball step (Algorithm 1 step 8):
-// with r = ||B~/rho2 - Y||_b, c_b = rho2 (1 - min(1, radius / r)).
-__global__ void k_block_scale(const double* __restrict__ block_sum, const double* __restrict__ eps, int nblocks,
-                              double rho2, int literal, float* __restrict__ cb) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nblocks) return;
-  const double r = sqrt(block_sum[b]);
-  const double radius = literal ? eps[b] / rho2 : eps[b];
-  const double keep = (r > radius) ? radius / r : 1.0;
-  cb[b] = (float)(rho2 * (1.0 - keep));
 }
 
 // Gridding (adjoint of the interpolation), Alg. 1 step 3's phi^dagger. Rows are stored sorted
@@ -572,6 +600,7 @@ __global__ void __launch_bounds__(32 * kGridWarps) k_grid(
   float* stage = xs + T::kRow;
   constexpr int kStageF = (T::kFloats - T::kRow) / 2;
   const long long first = (long long)(blockIdx.x * kGridWarps + warp) * rows;
+  pdl_wait();
   if (first >= M) return;
   const int m0 = (int)first, m1 = (int)min((long long)M, first + rows);
   const float4* v4 = reinterpret_cast<const float4*>(vin);
@@ -714,6 +743,7 @@ __global__ void __launch_bounds__(32 * kGridWarps) k_grid(
 __global__ void k_adj_cols(const float4* __restrict__ Acc, int n, const float2* __restrict__ tw, int K,
                            int logK, float4* __restrict__ T2, int Wd, int off, int full) {
   extern __shared__ float4 sm[];
+  pdl_wait();
   float4* bp = sm;
   float4* bm = sm + K;
   const int kx = blockIdx.x;
@@ -796,6 +826,7 @@ __global__ void k_adj_rows(const float4* __restrict__ T2, int n, int N, const fl
                            const float2* __restrict__ tw, int K, int logK, int Wd, int off, int full,
                            float* __restrict__ out) {
   extern __shared__ float4 sm[];
+  pdl_wait();
   float4* buf = sm;
   const int p = blockIdx.x;
   int st;
@@ -870,46 +901,37 @@ cudaError_t configure_nufft_kernels() {
   return set_smem((const void*)k_adj_cols, sm2);
 }
 
-cudaError_t nufft_forward_grid(Handle* h, const float* X) {
+cudaError_t nufft_forward_grid(Handle* h, const float* X, bool clear_acc) {
   const GridGeom& g = h->g;
   const size_t sm1 = fft_smem_bytes(g.K, 1);
-  k_fwd_rows<<<h->n, 256, sm1, h->stream>>>(X, h->n, h->N, h->corr, h->tw, g.K, g.logK, h->T1, g.Wd, g.off, g.full);
-  k_fwd_cols<<<g.Wd, 512, sm1, h->stream>>>(h->T1, h->n, h->tw, g.K, g.logK, h->G, g.Wd, g.off, g.full);
-  return cudaGetLastError();
+  cudaError_t e = launch_after(h->early, k_fwd_rows, h->n, 256, sm1, h->stream, X, h->n, h->N, h->corr, h->tw, g.K, g.logK, h->T1,
+                               g.Wd, g.off, g.full, h->Acc, clear_acc ? 2 * g.Wd * g.Wd : 0);
+  if (e != cudaSuccess) return e;
+  return launch_after(h->early, k_fwd_cols, g.Wd, 512, sm1, h->stream, h->T1, h->n, h->tw, g.K, g.logK, h->G, g.Wd, g.off, g.full);
 }
 
 template <int W>
-static void launch_degrid(Handle* h, int mode, float2* out) {
+static cudaError_t launch_degrid(Handle* h, int mode, float2* out, bool keep_cb) {
   const GridGeom& g = h->g;
   const int nbins = h->nblocks <= kWarpBins ? kWarpBins * 8 : h->nblocks;   // 8 warps of 256 threads
   const size_t sm = degrid_smem_tiles<W>() + (size_t)nbins * sizeof(double);
-  k_degrid<W><<<h->nitems, 256, sm, h->stream>>>(h->items, h->rec, h->G, g.Wd, g.off, g.full, g.K, g.beta, mode, h->R, h->Y,
-                                          h->cb, (float)(1.0 / h->rho2), h->vblk, h->nblocks, h->block_sum, out);
+  const BallStep ball{h->block_sum, h->block_done, h->block_norm_sq, mode == DEG_DUAL && !keep_cb ? h->cb : nullptr,
+                      h->eps,       h->rho2,       h->cfg.literal_ball};
+  return launch_after(h->early, k_degrid<W>, h->nitems, 256, sm, h->stream, h->items, h->rec, h->G, g.Wd, g.off, g.full, g.K,
+                      g.beta, mode, h->R, h->Y, h->cb, (float)(1.0 / h->rho2), h->vblk, h->nblocks, ball, out);
 }
 
-cudaError_t nufft_degrid(Handle* h, int mode, float2* out) {
+cudaError_t nufft_degrid(Handle* h, int mode, float2* out, bool keep_cb) {
   if (h->M == 0) return cudaSuccess;
-  if (mode != DEG_APPLY) {
-    cudaError_t e = cudaMemsetAsync(h->block_sum, 0, (size_t)h->nblocks * sizeof(double), h->stream);
-    if (e != cudaSuccess) return e;
-  }
   switch (h->g.W) {
-    case 5: launch_degrid<5>(h, mode, out); break;
-    case 9: launch_degrid<9>(h, mode, out); break;
-    default: launch_degrid<7>(h, mode, out); break;
+    case 5: return launch_degrid<5>(h, mode, out, keep_cb);
+    case 9: return launch_degrid<9>(h, mode, out, keep_cb);
+    default: return launch_degrid<7>(h, mode, out, keep_cb);
   }
-  return cudaGetLastError();
-}
-
-cudaError_t block_scales(Handle* h) {
-  if (h->nblocks == 0) return cudaSuccess;
-  k_block_scale<<<(h->nblocks + 127) / 128, 128, 0, h->stream>>>(h->block_sum, h->eps, h->nblocks, h->rho2,
-                                                                 h->cfg.literal_ball, h->cb);
-  return cudaGetLastError();
 }
 
 template <int W>
-static void launch_grid(Handle* h, const float2* in, int use_scale) {
+static cudaError_t launch_grid(Handle* h, const float2* in, int use_scale) {
   const GridGeom& g = h->g;
   // Rows per warp: 64 where that leaves two warps for every scheduler of the chip and a cell
   // holds enough rows that cutting its run at a warp's end costs more than parallelism gives,
@@ -926,30 +948,34 @@ static void launch_grid(Handle* h, const float2* in, int use_scale) {
   const int warps = 8 * std::max(1, h->num_sms);
   const int rows = h->M <= 12 * warps ? 8 : (h->M >= 64 * warps && h->M / std::max(1, h->ncells) >= 16 ? 64 : 32);
   const int ctas = (int)(((int64_t)h->M + (int64_t)rows * kGridWarps - 1) / ((int64_t)rows * kGridWarps));
-  k_grid<W><<<ctas, 32 * kGridWarps, kGridWarps * GridWarp<W>::kFloats * sizeof(float), h->stream>>>(
-      h->M, rows, h->vblk, h->rec, in, h->cb, use_scale, g.Wd, g.off, g.full, g.K, g.beta,
-      reinterpret_cast<float*>(h->Acc));
+  return launch_after(h->early, k_grid<W>, ctas, 32 * kGridWarps, kGridWarps * GridWarp<W>::kFloats * sizeof(float), h->stream, h->M,
+                      rows, h->vblk, h->rec, in, h->cb, use_scale, g.Wd, g.off, g.full, g.K, g.beta,
+                      reinterpret_cast<float*>(h->Acc));
 }
 
-cudaError_t nufft_grid(Handle* h, const float2* in, int use_scale) {
+cudaError_t nufft_grid(Handle* h, const float2* in, int use_scale, bool cleared) {
   const GridGeom& g = h->g;
-  cudaError_t e = cudaMemsetAsync(h->Acc, 0, (size_t)g.Wd * g.Wd * 2 * sizeof(float4), h->stream);
-  if (e != cudaSuccess || h->M == 0) return e;
-  switch (g.W) {
-    case 5: launch_grid<5>(h, in, use_scale); break;
-    case 9: launch_grid<9>(h, in, use_scale); break;
-    default: launch_grid<7>(h, in, use_scale); break;
+  if (!cleared) {
+    const cudaError_t e = cudaMemsetAsync(h->Acc, 0, (size_t)g.Wd * g.Wd * 2 * sizeof(float4), h->stream);
+    if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  if (h->M == 0) return cudaSuccess;
+  switch (g.W) {
+    case 5: return launch_grid<5>(h, in, use_scale);
+    case 9: return launch_grid<9>(h, in, use_scale);
+    default: return launch_grid<7>(h, in, use_scale);
+  }
 }
 
 cudaError_t nufft_adjoint_image(Handle* h, float* out) {
   const GridGeom& g = h->g;
   const size_t sm2 = fft_smem_bytes(g.K, 2), sm1 = fft_smem_bytes(g.K, 1);
   const int ncols = g.full ? (g.K / 2 + 1) : (g.R + 1);
-  k_adj_cols<<<ncols, 512, sm2, h->stream>>>(h->Acc, h->n, h->tw, g.K, g.logK, h->T2, g.Wd, g.off, g.full);
-  k_adj_rows<<<h->n, 256, sm1, h->stream>>>(h->T2, h->n, h->N, h->corr, h->tw, g.K, g.logK, g.Wd, g.off, g.full, out);
-  return cudaGetLastError();
+  cudaError_t e = launch_after(h->early, k_adj_cols, ncols, 512, sm2, h->stream, h->Acc, h->n, h->tw, g.K, g.logK, h->T2, g.Wd, g.off,
+                               g.full);
+  if (e != cudaSuccess) return e;
+  return launch_after(h->early, k_adj_rows, h->n, 256, sm1, h->stream, h->T2, h->n, h->N, h->corr, h->tw, g.K, g.logK, g.Wd, g.off,
+                      g.full, out);
 }
 
 }  // namespace ps

@@ -406,6 +406,7 @@ __global__ void __launch_bounds__(256, 3) k_ana_lv(const float* __restrict__ app
                                                    float* __restrict__ approx_out, int mode, float scale, float gamma,
                                                    float delta, int* err, const __grid_constant__ SaraTma tm) {
   extern __shared__ __align__(128) float4 sma[];
+  pdl_wait();
   const AnaSmem S = ana_smem(sma);
   const int bi = blockIdx.y, map = blockIdx.z;
   const int hm = m >> 1, tilesx = hm / kTO;
@@ -579,6 +580,7 @@ __global__ void __launch_bounds__(256, 2) k_ana_pers(const float* __restrict__ i
                                                      int mode, float scale, float gamma, float delta, int* err,
                                                      int nmaps, const __grid_constant__ SaraTma tm) {
   extern __shared__ __align__(128) float4 smp[];
+  pdl_wait();
   float* in_s = reinterpret_cast<float*>(smp);
   float* lo_s = in_s + kA2In;
   float* hi_s = lo_s + kRSmax * kPlo;
@@ -843,6 +845,7 @@ __global__ void __launch_bounds__(256, NBUF == 1 ? 4 : 3)
     k_syn2_fine(const float* __restrict__ coef, const float* __restrict__ approx_in, int coarsest, int n,
                 float* __restrict__ out, int* err, const __grid_constant__ SaraTma tm) {
   extern __shared__ __align__(128) float4 sm2[];
+  pdl_wait();
   float* const s4 = reinterpret_cast<float*>(sm2);   // staging set(s): basis b in set b % NBUF
   float* loT = s4 + NBUF * kC2Set;
   float* hiT = loT + kLoSize;
@@ -906,6 +909,7 @@ __global__ void __launch_bounds__(256, 4)
     k_syn2_fine_pers(const float* __restrict__ coef, const float* __restrict__ approx_in, int coarsest, int n,
                      float* __restrict__ out, int* err, int nmaps, const __grid_constant__ SaraTma tm) {
   extern __shared__ __align__(128) float4 sm2[];
+  pdl_wait();
   float* const s4 = reinterpret_cast<float*>(sm2);
   float* loT = s4 + kC2Set;
   float* hiT = loT + kLoSize;
@@ -964,6 +968,7 @@ __global__ void __launch_bounds__(256, 3) k_syn2_lv(const float* __restrict__ co
                                                     int coarsest, int m, int n, float* __restrict__ approx_out,
                                                     int* err, const __grid_constant__ SaraTma tm) {
   extern __shared__ __align__(128) float4 sm2[];
+  pdl_wait();
   float* s4 = reinterpret_cast<float*>(sm2);
   float* loT = s4 + kC2Set;
   float* hiT = loT + kLoSize;
@@ -1135,6 +1140,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_ana_small(const float* __rest
                                                              float* __restrict__ coef, float* __restrict__ thr,
                                                              int mode, float scale, float gamma, float delta) {
   extern __shared__ float4 smt[];
+  pdl_wait();
   const int bi = blockIdx.x, map = blockIdx.y;
   const int m0 = n >> (l0 - 1), q0 = m0 >> 2, P = small_pitch(m0), Q = (m0 >> 1) + 4;
   float* img = reinterpret_cast<float*>(smt);
@@ -1297,6 +1303,7 @@ template <bool FINEST>
 __device__ __forceinline__ void syn_small(const float* __restrict__ coef, int L, int l1, int n,
                                           float* __restrict__ dst) {
   extern __shared__ float4 smt[];
+  pdl_wait();
   const int bi = blockIdx.x, map = blockIdx.y;
   const int m0 = n >> (l1 - 1), q0 = m0 >> 2, Bp = m0 + 4;
   float* blk = reinterpret_cast<float*>(smt);
@@ -1351,6 +1358,7 @@ __global__ void __cluster_dims__(NS, 1, 1) __launch_bounds__(256, 4)
                  float* __restrict__ out, int* err, const __grid_constant__ SaraTma tm) {
   extern __shared__ __align__(128) float4 sm2[];
   __shared__ int failed;
+  pdl_wait();
   float* const s4 = reinterpret_cast<float*>(sm2);
   float* loT = s4 + kC2Set;
   float* hiT = loT + kLoSize;
@@ -1560,9 +1568,13 @@ cudaError_t sara_analysis(Handle* h, const float* X, float* coef, float* thr, in
       const float* in = l == 1 ? X : buf[(l - 2) & 1];
       const size_t in_map = l == 1 ? (size_t)n * n : (size_t)kDb * m * m, in_basis = l == 1 ? 0 : (size_t)m * m;
       const SaraTma tm = analysis_maps(in, m, l == 1 ? nmaps : kDb * nmaps, coef, thr, n, nmaps, mode);
-      k_ana_pers<<<ctas, 256, pers_analysis_smem(), h->stream>>>(in, in_map, in_basis, m, n, l == L, coef, thr,
-                                                                 buf[(l - 1) & 1], mode, scale, gamma, delta,
-                                                                 h->dev_flags, nmaps, tm);
+      if (l == 1)
+        k_ana_pers<<<ctas, 256, pers_analysis_smem(), h->stream>>>(in, in_map, in_basis, m, n, l == L, coef, thr,
+                                                                   buf[(l - 1) & 1], mode, scale, gamma, delta,
+                                                                   h->dev_flags, nmaps, tm);
+      else
+        launch_after(true, k_ana_pers, ctas, 256, pers_analysis_smem(), h->stream, in, in_map, in_basis, m, n, l == L, coef, thr,
+                     buf[(l - 1) & 1], mode, scale, gamma, delta, h->dev_flags, nmaps, tm);
       if (l == 1 && fine_done) {
         const cudaError_t e = cudaEventRecord(fine_done, h->stream);
         if (e != cudaSuccess) return e;
@@ -1577,15 +1589,18 @@ cudaError_t sara_analysis(Handle* h, const float* X, float* coef, float* thr, in
       }
     } else {
       const SaraTma tm = analysis_maps(buf[(l - 2) & 1], m, kDb * nmaps, coef, thr, n, nmaps, mode);
-      k_ana_lv<<<grid, 256, fast_analysis_smem(), h->stream>>>(buf[(l - 2) & 1], m, n, l == L, coef, thr,
-                                                              buf[(l - 1) & 1], mode, scale, gamma, delta,
-                                                              h->dev_flags, tm);
+      launch_after(true, k_ana_lv, grid, 256, fast_analysis_smem(), h->stream, buf[(l - 2) & 1], m, n, l == L, coef, thr,
+                   buf[(l - 1) & 1], mode, scale, gamma, delta, h->dev_flags, tm);
     }
   }
   if (lt <= L) {
     const float* in = lt == 1 ? X : buf[(lt - 2) & 1];
-    k_ana_small<<<dim3(kDb, nmaps), kSmallThreads, ana_small_smem(n >> (lt - 1)), h->stream>>>(in, lt, L, n, coef, thr,
-                                                                                            mode, scale, gamma, delta);
+    if (lt == 1)
+      k_ana_small<<<dim3(kDb, nmaps), kSmallThreads, ana_small_smem(n), h->stream>>>(in, lt, L, n, coef, thr, mode, scale,
+                                                                                  gamma, delta);
+    else
+      launch_after(true, k_ana_small, dim3(kDb, nmaps), kSmallThreads, ana_small_smem(n >> (lt - 1)), h->stream, in, lt, L, n, coef,
+                   thr, mode, scale, gamma, delta);
     if (lt == 1 && fine_done) {
       const cudaError_t e = cudaEventRecord(fine_done, h->stream);
       if (e != cudaSuccess) return e;
@@ -1606,8 +1621,7 @@ static cudaError_t synthesis_levels(cudaStream_t stream, int n, int L, const flo
       const cudaError_t e = cudaEventRecord(fine_start, stream);
       if (e != cudaSuccess) return e;
     }
-    k_syn_small<<<dim3(kDb, nmaps), kSmallThreads, syn_small_smem(n), stream>>>(coef, L, n, out);
-    return cudaGetLastError();
+    return launch_after(true, k_syn_small, dim3(kDb, nmaps), kSmallThreads, syn_small_smem(n), stream, coef, L, n, out);
   }
   int lt = 0;                                       // lowest level of the fused tail (>= 2), 0: none
   for (int l = 2; l <= L; ++l)
@@ -1616,15 +1630,15 @@ static cudaError_t synthesis_levels(cudaStream_t stream, int n, int L, const flo
       break;
     }
   if (lt)
-    k_syn_tail<<<dim3(kDb, nmaps), kSmallThreads, syn_small_smem(n >> (lt - 1)), stream>>>(coef, L, lt, n,
-                                                                                         buf[(lt - 1) & 1]);
+    launch_after(true, k_syn_tail, dim3(kDb, nmaps), kSmallThreads, syn_small_smem(n >> (lt - 1)), stream, coef, L, lt, n,
+                 buf[(lt - 1) & 1]);
   for (int l = lt ? lt - 1 : L; l >= 1; --l) {      // every side m >= 64 here
     const int m = n >> (l - 1), tiles = (m / kT2) * (m / kT2);
     const float* ain = (l == L) ? nullptr : buf[l & 1];
     const SaraTma tm = synthesis_maps(coef, ain, m, n, nmaps);
     if (l > 1) {
-      k_syn2_lv<<<dim3(tiles, nmaps, kDb), 256, syn2_smem(1), stream>>>(coef, ain, l == L, m, n, buf[(l - 1) & 1], err,
-                                                                        tm);
+      launch_after(true, k_syn2_lv, dim3(tiles, nmaps, kDb), 256, syn2_smem(1), stream, coef, ain, l == L, m, n,
+                   buf[(l - 1) & 1], err, tm);
       continue;
     }
     if (fine_start) {
@@ -1633,21 +1647,32 @@ static cudaError_t synthesis_levels(cudaStream_t stream, int n, int L, const flo
     }
     const int units = tiles * nmaps;
     if (units <= kSplit8Units)
-      k_syn2_split<8><<<dim3(8 * tiles, 1, nmaps), 256, syn2_smem(1), stream>>>(coef, ain, l == L, n, out, err, tm);
+      launch_after(true, k_syn2_split<8>, dim3(8 * tiles, 1, nmaps), 256, syn2_smem(1), stream, coef, ain, l == L, n, out, err, tm);
     else if (units <= kSplit4Units)
-      k_syn2_split<4><<<dim3(4 * tiles, 1, nmaps), 256, syn2_smem(1), stream>>>(coef, ain, l == L, n, out, err, tm);
+      launch_after(true, k_syn2_split<4>, dim3(4 * tiles, 1, nmaps), 256, syn2_smem(1), stream, coef, ain, l == L, n, out, err, tm);
     else if (variant == 2) {
       int dev = 0, sms = 0;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      k_syn2_fine_pers<<<std::min(units, 4 * std::max(1, sms)), 256, syn2_smem(1), stream>>>(coef, ain, l == L, n, out,
-                                                                                            err, nmaps, tm);
+      launch_after(true, k_syn2_fine_pers, std::min(units, 4 * std::max(1, sms)), 256, syn2_smem(1), stream, coef, ain, l == L, n,
+                   out, err, nmaps, tm);
     } else if (variant == 1)
-      k_syn2_fine<1><<<dim3(tiles, 1, nmaps), 256, syn2_smem(1), stream>>>(coef, ain, l == L, n, out, err, tm);
+      launch_after(true, k_syn2_fine<1>, dim3(tiles, 1, nmaps), 256, syn2_smem(1), stream, coef, ain, l == L, n, out, err, tm);
     else
-      k_syn2_fine<2><<<dim3(tiles, 1, nmaps), 256, syn2_smem(2), stream>>>(coef, ain, l == L, n, out, err, tm);
+      launch_after(true, k_syn2_fine<2>, dim3(tiles, 1, nmaps), 256, syn2_smem(2), stream, coef, ain, l == L, n, out, err, tm);
   }
   return cudaGetLastError();
+}
+
+// First level of side at most `side` from level l on (L + 1: none).
+static int first_level(int n, int L, int l, int side) {
+  while (l <= L && (n >> (l - 1)) > side) ++l;
+  return l;
+}
+
+int sara_launches(int n, int L) {
+  const int la = first_level(n, L, 1, kSmall), ls = n <= kSmall ? 1 : first_level(n, L, 2, kSmallSyn);
+  return (la - 1) + (la <= L) + (ls - 1) + (ls <= L);   // tiled levels and the fused small ones, each way
 }
 
 cudaError_t sara_synthesis(Handle* h, const float* coef, float* out, cudaEvent_t fine_start) {
