@@ -481,7 +481,7 @@ ps_status ps_create(const ps_config* cfg, void* cuda_stream, ps_handle** out) {
             dalloc(h, &h->A, 36 * N) == cudaSuccess && dalloc(h, &h->T, 36 * N) == cudaSuccess &&
             dalloc(h, &h->approx, 16 * N) == cudaSuccess && dalloc(h, &h->red, (size_t)h->red_cap) == cudaSuccess &&
             dalloc(h, &h->dev_flags, 4) == cudaSuccess &&
-            cudaMallocHost((void**)&h->red_host, 1024 * sizeof(double)) == cudaSuccess &&
+            cudaMallocHost((void**)&h->red_host, 2048 * sizeof(double)) == cudaSuccess &&
             cudaHostAlloc((void**)&h->relc_host, 16 * sizeof(double), cudaHostAllocMapped) == cudaSuccess &&
             cudaHostGetDevicePointer((void**)&h->relc_dev, h->relc_host, 0) == cudaSuccess;
   if (!ok) {
@@ -540,15 +540,16 @@ void ps_destroy(ps_handle* h) {
 
 // Reads the device error flags after a synchronisation: a bounded in-kernel wait
 // that gave up is reported as PS_ETIMEOUT (the flag is then cleared).
+static ps_status report_flag(Handle* h, int flag) {
+  if (!flag) return PS_OK;
+  CK(h, cudaMemsetAsync(h->dev_flags, 0, 4 * sizeof(int), h->stream));
+  return fail(h, PS_ETIMEOUT, "a bounded device wait (bulk-copy barrier) gave up; results of that launch are invalid");
+}
 static ps_status check_flags(Handle* h) {
   int f[4] = {0, 0, 0, 0};
   CK(h, cudaMemcpyAsync(f, h->dev_flags, sizeof(f), cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
-  if (f[0]) {
-    CK(h, cudaMemsetAsync(h->dev_flags, 0, sizeof(f), h->stream));
-    return fail(h, PS_ETIMEOUT, "a bounded device wait (bulk-copy barrier) gave up; results of that launch are invalid");
-  }
-  return PS_OK;
+  return report_flag(h, f[0]);
 }
 
 ps_status ps_synchronize(ps_handle* h) {
@@ -868,7 +869,7 @@ static ps_status opnorm_lanczos(Handle* h) {
   // On the handle's (non-blocking) stream, so the iterations below are ordered after the copy.
   CK(h, cudaMemcpyAsync(v, x.data(), N4 * sizeof(float), cudaMemcpyHostToDevice, h->stream));
   CK(h, cudaMemsetAsync(u, 0, N4 * sizeof(float), h->stream));
-  double* dres = h->red + (size_t)h->red_cap - 600;
+  double* dres = h->red + (size_t)h->red_cap - 1020;
   std::vector<double> al, be;
   double theta = 0.0, beta = 0.0;
   for (int j = 0; j < 300; ++j) {
@@ -909,7 +910,7 @@ static ps_status default_gamma(Handle* h) {
   if (h->cfg.gamma > 0) {
     h->gamma_default = h->cfg.gamma;
   } else if (h->M > 0 && h->opnorm_sq > 0) {
-    double* dres = h->red + (size_t)h->red_cap - 600;
+    double* dres = h->red + (size_t)h->red_cap - 1020;
     CK(h, ps::nufft_grid(h, h->Y, 0, false));
     CK(h, ps::nufft_adjoint_image(h, h->Adj));
     CK(h, ps::dirac_apply(h, h->Adj, h->A, nullptr, ps::SARA_APPLY, 1.0f / 3.0f, 0.f, 0.f));
@@ -1120,11 +1121,8 @@ static ps_status relc_enqueue(Handle* h) {
 // The relative change from the landed sums (and the flags copied with them).
 static ps_status relc_finish(Handle* h, double* out4) {
   h->relc_pending = false;
-  const int* f = reinterpret_cast<const int*>(h->relc_host + 8);
-  if (f[0]) {
-    CK(h, cudaMemsetAsync(h->dev_flags, 0, 4 * sizeof(int), h->stream));
-    return fail(h, PS_ETIMEOUT, "a bounded device wait (bulk-copy barrier) gave up; results of that launch are invalid");
-  }
+  const ps_status st = report_flag(h, reinterpret_cast<const int*>(h->relc_host + 8)[0]);
+  if (st != PS_OK) return st;
   bool finite = true;
   for (int c = 0; c < 4; ++c) {
     const double num = h->relc_host[c], den = h->relc_host[4 + c];
@@ -1145,46 +1143,46 @@ ps_status ps_compute_stats(ps_handle* h, double zeta_sigma, ps_stats* out) {
   if (!h->have_meas) return fail(h, PS_ESTATE, "compute_stats: call ps_set_measurements first");
   if (!(zeta_sigma > 0)) zeta_sigma = h->cfg.zeta_sigma;
   const size_t N = h->N;
-  double* dres = h->red + (size_t)h->red_cap - 600;
-  // Relative change of the last iteration (from the partials written by k_primal).
+  double* dres = h->red + (size_t)h->red_cap - 1020;
   out->stop_flags = 0;
   out->converged = 0;
-  {
-    ps_status st = relc_enqueue(h);
-    if (st != PS_OK) return st;
-    CK(h, cudaStreamSynchronize(h->stream));
-    st = relc_finish(h, out->rel_change);
-    if (st != PS_OK) return st;
-  }
-  // Residual Y - phi(S) per block, and the residual image.
-  std::vector<double> bsum(h->nblocks);
-  double rms = 0.0;
+  ps_status st = ensure_tmp36(h);
+  if (st != PS_OK) return st;
+  // Everything is queued before the first wait: the relative change of the last iteration (from
+  // the partials written by k_primal); beside each other the weighted norm (analysis of S) and the
+  // residual Y - phi(S) per block with the residual image; then the violations, whose zeta comes
+  // from the image's sum of squares on the device. The results land in mapped host memory.
+  if ((st = relc_enqueue(h)) != PS_OK) return st;
+  CK(h, cudaEventRecord(h->ev_fork, h->stream));
+  CK(h, cudaStreamWaitEvent(h->aux, h->ev_fork, 0));
+  cudaStream_t main = h->stream;
+  h->stream = h->aux;                     // the launchers use h->stream
+  cudaError_t e = ps::dirac_apply(h, h->S, h->tmp36, nullptr, ps::SARA_APPLY, 1.0f / 3.0f, 0.f, 0.f);
+  if (e == cudaSuccess) e = ps::sara_analysis(h, h->S, h->tmp36, nullptr, ps::SARA_APPLY, 1.0f / 3.0f, 0.f, 0.f);
+  if (e == cudaSuccess) e = ps::weighted_l1(h, h->tmp36, h->T, h->relc_dev + 13);
+  h->stream = main;
+  CK(h, e);
+  CK(h, cudaEventRecord(h->ev_join, h->aux));
   if (h->M > 0) {
     CK(h, ps::nufft_forward_grid(h, h->S, true));
     CK(h, ps::nufft_degrid(h, ps::DEG_RESID, h->vtmp));
     CK(h, ps::nufft_grid(h, h->vtmp, 0, true));
     CK(h, ps::nufft_adjoint_image(h, h->tmp4));
     CK(h, ps::reduce_dot(h, h->tmp4, h->tmp4, N, dres));
-    CK(h, cudaMemcpyAsync(bsum.data(), h->block_norm_sq, bsum.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaMemcpyAsync(h->red_host, dres, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
-    rms = std::sqrt(h->red_host[0] / (double)N);
+    CK(h, cudaMemcpyAsync(h->red_host, h->block_norm_sq, h->nblocks * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   }
+  CK(h, cudaStreamWaitEvent(h->stream, h->ev_join, 0));
+  CK(h, ps::violation_count(h, h->S, h->M > 0 ? dres : nullptr, zeta_sigma, h->relc_dev + 10));
   CK(h, cudaStreamSynchronize(h->stream));
+  if ((st = relc_finish(h, out->rel_change)) != PS_OK) return st;
+  const double rms = std::sqrt(h->relc_host[10] / (double)N);
+  const double* bsum = h->red_host;
   if (out->block_residual)
     for (int b = 0; b < std::min(out->nblocks, h->nblocks); ++b) out->block_residual[b] = std::sqrt(bsum[b]);
   out->zeta = h->psf_peak > 0 ? zeta_sigma * rms / h->psf_peak : 0.0;
-  CK(h, ps::violation_count(h, h->S, out->zeta, dres + 2));
-  ps_status st = ensure_tmp36(h);
-  if (st != PS_OK) return st;
-  CK(h, ps::dirac_apply(h, h->S, h->tmp36, nullptr, ps::SARA_APPLY, 1.0f / 3.0f, 0.f, 0.f));
-  CK(h, ps::sara_analysis(h, h->S, h->tmp36, nullptr, ps::SARA_APPLY, 1.0f / 3.0f, 0.f, 0.f));
-  CK(h, ps::weighted_l1(h, h->tmp36, h->T, dres + 4));
-  CK(h, cudaMemcpyAsync(h->red_host, dres, 6 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  CK(h, cudaStreamSynchronize(h->stream));
-  out->violations = (int64_t)h->red_host[2];
-  out->violations_raw = (int64_t)h->red_host[3];
-  out->weighted_l1 = h->red_host[4];
+  out->violations = (int64_t)h->relc_host[11];
+  out->violations_raw = (int64_t)h->relc_host[12];
+  out->weighted_l1 = h->relc_host[13];
   out->iterations = h->iterations;
   // Stopping rule of Section 5.5: every criterion that applies in the mode.
   int flags = 0;
@@ -1199,7 +1197,7 @@ ps_status ps_compute_stats(ps_handle* h, double zeta_sigma, ps_stats* out) {
     flags |= PS_STOP_NP;
   out->stop_flags = flags;
   out->converged = flags == (PS_STOP_REL | PS_STOP_RESID | PS_STOP_NP);
-  return check_flags(h);
+  return report_flag(h, reinterpret_cast<const int*>(h->relc_host + 14)[0]);
 }
 
 ps_status ps_apply_phi(ps_handle* h, const float* S, float* Y, int32_t device_ptrs) {
@@ -1476,7 +1474,7 @@ ps_status ps_max_abs_analysis(ps_handle* h, double* out) {
   if (!h || !out) return h ? fail(h, PS_EINVAL, "max_abs_analysis: null output") : PS_EINVAL;
   ps_status st = ensure_tmp36(h);
   if (st != PS_OK) return st;
-  double* dres = h->red + (size_t)h->red_cap - 600;
+  double* dres = h->red + (size_t)h->red_cap - 1020;
   CK(h, ps::dirac_apply(h, h->S, h->tmp36, nullptr, ps::SARA_APPLY, 1.0f / 3.0f, 0.f, 0.f));
   CK(h, ps::sara_analysis(h, h->S, h->tmp36, nullptr, ps::SARA_APPLY, 1.0f / 3.0f, 0.f, 0.f));
   CK(h, ps::max_abs(h, h->tmp36, 36 * (size_t)h->N, dres + 8));

@@ -75,11 +75,12 @@ struct Handle {
   double *red = nullptr;      // reduction partials
   int red_cap = 0;
   double *red_host = nullptr; // pinned
-  double *relc_host = nullptr; // pinned, mapped: relative-change sums (8) and the device flags of the last request
+  double *relc_host = nullptr; // pinned, mapped: relative-change sums (8) and the device flags (2) of the last request;
+                               // ps_compute_stats: sum, counts (10-12), weighted norm (13), flags (14-15)
   double *relc_dev = nullptr;  // the device's address of relc_host
   cudaEvent_t relc_ev = nullptr;
   bool relc_pending = false;
-  int *dev_flags = nullptr;   // device error flags: [0] a bounded wait gave up
+  int *dev_flags = nullptr;   // [0] error flag: a bounded wait gave up; [1], [2] counters of the reductions
 
   // Visibility-domain state, rows stored in tap-centre-cell order (tile-major).
   int M = 0, nblocks = 0;
@@ -170,8 +171,8 @@ cudaError_t dirac_apply(Handle* h, const float* X, float* coef, float* thr, int 
                         float scale, float gamma, float delta);
 cudaError_t reduce_dot(Handle* h, const float* a, const float* b, size_t len, double* dev_out);
 cudaError_t relc_sums(Handle* h, int nb, double* out);   // 8 column sums of k_primal's partials + the flags
-cudaError_t violation_count(Handle* h, const float* S, double zeta, double* dev_out);
-cudaError_t weighted_l1(Handle* h, const float* coef, const float* thr, double* dev_out);
+cudaError_t violation_count(Handle* h, const float* S, const double* rms_sum, double zeta_sigma, double* out);
+cudaError_t weighted_l1(Handle* h, const float* coef, const float* thr, double* out);
 cudaError_t max_abs(Handle* h, const float* c, size_t len, double* dev_out);
 cudaError_t scale_copy(Handle* h, const float* x, float* y, size_t len, double s);
 cudaError_t lanczos_update(Handle* h, float* w, const float* v, const float* u, size_t len, double alpha,

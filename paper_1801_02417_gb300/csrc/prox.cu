@@ -268,35 +268,43 @@ cudaError_t dirac_apply(Handle* h, const float* X, float* coef, float* thr, int 
   return cudaGetLastError();
 }
 
-// Deterministic two-stage FP64 reductions: per-CTA partials then one CTA.
-__global__ void k_dot_partial(const float* __restrict__ a, const float* __restrict__ b, size_t len,
-                              double* __restrict__ part) {
+// Deterministic FP64 reductions in one launch: per-CTA partials, which the last CTA to end sums in
+// a fixed order. `done` counts the CTAs that have written theirs (0 between launches).
+template <typename T>
+__device__ __forceinline__ T cta_sum(T v, T* sh) {   // valid in thread 0; sh: 32 values
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  T t = 0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
+  __syncthreads();
+  return t;
+}
+__device__ __forceinline__ bool last_cta(int* done) {   // after the partials are written by thread 0
+  __shared__ int last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(done, 1) == (int)gridDim.x - 1;
+    if (last) *done = 0;
+    __threadfence();
+  }
+  __syncthreads();
+  return last;
+}
+
+__global__ void k_dot(const float* __restrict__ a, const float* __restrict__ b, size_t len, double* part, int* done,
+                      double* out) {
   __shared__ double sh[32];
   double s = 0.0;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (size_t)gridDim.x * blockDim.x)
     s += (double)a[i] * (double)b[i];
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
-    part[blockIdx.x] = t;
-  }
-}
-
-__global__ void k_sum_partials(const double* __restrict__ part, int np, double* __restrict__ out) {
-  __shared__ double sh[32];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < np; i += blockDim.x) s += part[i];
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
-    *out = t;
-  }
+  s = cta_sum(s, sh);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  if (!last_cta(done)) return;
+  s = threadIdx.x < gridDim.x ? __ldcg(&part[threadIdx.x]) : 0.0;   // at most blockDim CTAs
+  s = cta_sum(s, sh);
+  if (threadIdx.x == 0) *out = s;
 }
 
 // Column sums of the per-CTA relative-change partials that k_primal writes (8 per CTA: the
@@ -328,17 +336,26 @@ cudaError_t relc_sums(Handle* h, int nb, double* out) {
   return cudaGetLastError();
 }
 
+// CTAs (and threads of each) of the one-launch reductions; their partials are the last
+// 2 kRedBlocks doubles of `red`, the weighted norm's the kRedBlocks before them (it runs beside
+// the others), their counters dev_flags[1] and [2].
 static constexpr int kRedBlocks = 256;
+static double* red_partials(Handle* h, int back) { return h->red + (size_t)h->red_cap - back * kRedBlocks; }
 
 cudaError_t reduce_dot(Handle* h, const float* a, const float* b, size_t len, double* dev_out) {
-  double* part = h->red + (size_t)h->red_cap - 2 * kRedBlocks;
-  k_dot_partial<<<kRedBlocks, 256, 0, h->stream>>>(a, b, len, part);
-  k_sum_partials<<<1, 256, 0, h->stream>>>(part, kRedBlocks, dev_out);
+  k_dot<<<kRedBlocks, kRedBlocks, 0, h->stream>>>(a, b, len, red_partials(h, 2), h->dev_flags + 1, dev_out);
   return cudaGetLastError();
 }
 
-__global__ void k_violations(int N, const float* __restrict__ S, double zeta, double* __restrict__ part) {
-  __shared__ double sh[2][32];
+// Pixels with -I + ||(Q, U, V)|| above zeta and above zero, zeta = zeta_sigma rms / psf_peak from the sum
+// of squares *rms_sum of the residual image (null: zeta = 0). The last CTA writes out[0] = that
+// sum, out[1 .. 2] = the counts and out[4 .. 5] = the device flags (as ints); `out` may be mapped
+// host memory.
+__global__ void k_violations(int N, const float* __restrict__ S, const double* rms_sum, double zeta_sigma,
+                             double psf_peak, double* part, int* flags, double* out) {
+  __shared__ double sh[32];
+  const double q = rms_sum ? *rms_sum : 0.0;
+  const double zeta = psf_peak > 0.0 ? zeta_sigma * sqrt(q / (double)N) / psf_peak : 0.0;
   double c0 = 0.0, c1 = 0.0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
     const double I = S[i], Q = S[(size_t)N + i], U = S[2 * (size_t)N + i], V = S[3 * (size_t)N + i];
@@ -346,86 +363,79 @@ __global__ void k_violations(int N, const float* __restrict__ S, double zeta, do
     c0 += (p > zeta) ? 1.0 : 0.0;
     c1 += (p > 0.0) ? 1.0 : 0.0;
   }
-  c0 = warp_sum(c0);
-  c1 = warp_sum(c1);
-  if ((threadIdx.x & 31) == 0) {
-    sh[0][threadIdx.x >> 5] = c0;
-    sh[1][threadIdx.x >> 5] = c1;
+  c0 = cta_sum(c0, sh);
+  c1 = cta_sum(c1, sh);
+  if (threadIdx.x == 0) {
+    part[2 * blockIdx.x] = c0;
+    part[2 * blockIdx.x + 1] = c1;
   }
-  __syncthreads();
-  if (threadIdx.x < 2) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[threadIdx.x][w];
-    part[2 * blockIdx.x + threadIdx.x] = t;
-  }
-}
-
-__global__ void k_sum_pairs(const double* __restrict__ part, int np, double* __restrict__ out) {
-  if (threadIdx.x < 2) {
-    double s = 0.0;
-    for (int i = 0; i < np; ++i) s += part[2 * i + threadIdx.x];
-    out[threadIdx.x] = s;
+  if (!last_cta(flags + 1)) return;
+  c0 = threadIdx.x < gridDim.x ? __ldcg(&part[2 * threadIdx.x]) : 0.0;
+  c1 = threadIdx.x < gridDim.x ? __ldcg(&part[2 * threadIdx.x + 1]) : 0.0;
+  c0 = cta_sum(c0, sh);
+  c1 = cta_sum(c1, sh);
+  if (threadIdx.x == 0) {
+    out[0] = q;
+    out[1] = c0;
+    out[2] = c1;
+    for (int k = 0; k < 4; ++k) reinterpret_cast<int*>(out + 4)[k] = k ? 0 : flags[k];
+    __threadfence_system();
   }
 }
 
-cudaError_t violation_count(Handle* h, const float* S, double zeta, double* dev_out) {
-  double* part = h->red + (size_t)h->red_cap - 2 * kRedBlocks;
-  k_violations<<<kRedBlocks / 2, 256, 0, h->stream>>>(h->N, S, zeta, part);
-  k_sum_pairs<<<1, 32, 0, h->stream>>>(part, kRedBlocks / 2, dev_out);
+cudaError_t violation_count(Handle* h, const float* S, const double* rms_sum, double zeta_sigma, double* out) {
+  k_violations<<<kRedBlocks, kRedBlocks, 0, h->stream>>>(h->N, S, rms_sum, zeta_sigma, h->psf_peak, red_partials(h, 2),
+                                                         h->dev_flags, out);
   return cudaGetLastError();
 }
 
-__global__ void k_wl1_partial(const float* __restrict__ c, const float* __restrict__ t, size_t len,
-                              double* __restrict__ part) {
+__global__ void k_wl1(const float* __restrict__ c, const float* __restrict__ t, size_t len, double* part, int* done,
+                      double* out) {
   __shared__ double sh[32];
   double s = 0.0;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (size_t)gridDim.x * blockDim.x)
     s += (double)t[i] * fabs((double)c[i]);
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-  __syncthreads();
+  s = cta_sum(s, sh);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  if (!last_cta(done)) return;
+  s = threadIdx.x < gridDim.x ? __ldcg(&part[threadIdx.x]) : 0.0;
+  s = cta_sum(s, sh);
   if (threadIdx.x == 0) {
-    double r = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += sh[w];
-    part[blockIdx.x] = r;
+    *out = s;
+    __threadfence_system();
   }
 }
 
-cudaError_t weighted_l1(Handle* h, const float* coef, const float* thr, double* dev_out) {
-  double* part = h->red + (size_t)h->red_cap - 2 * kRedBlocks;
-  k_wl1_partial<<<kRedBlocks, 256, 0, h->stream>>>(coef, thr, (size_t)36 * h->N, part);
-  k_sum_partials<<<1, 256, 0, h->stream>>>(part, kRedBlocks, dev_out);
+cudaError_t weighted_l1(Handle* h, const float* coef, const float* thr, double* out) {
+  k_wl1<<<kRedBlocks, kRedBlocks, 0, h->stream>>>(coef, thr, (size_t)36 * h->N, red_partials(h, 3), h->dev_flags + 2, out);
   return cudaGetLastError();
 }
 
-__global__ void k_maxabs_partial(const float* __restrict__ c, size_t len, float* __restrict__ part) {
+__global__ void k_maxabs(const float* __restrict__ c, size_t len, float* part, int* done, double* out) {
   __shared__ float sh[32];
+  auto cta_max = [&](float m) {   // valid in thread 0
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, sh[w]);
+    __syncthreads();
+    return m;
+  };
   float m = 0.f;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (size_t)gridDim.x * blockDim.x)
     m = fmaxf(m, fabsf(c[i]));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float r = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r = fmaxf(r, sh[w]);
-    part[blockIdx.x] = r;
-  }
-}
-
-__global__ void k_max_partials(const float* __restrict__ part, int np, double* __restrict__ out) {
-  if (threadIdx.x == 0) {
-    float r = 0.f;
-    for (int i = 0; i < np; ++i) r = fmaxf(r, part[i]);
-    *out = (double)r;
-  }
+  m = cta_max(m);
+  if (threadIdx.x == 0) part[blockIdx.x] = m;
+  if (!last_cta(done)) return;
+  m = cta_max(threadIdx.x < gridDim.x ? __ldcg(&part[threadIdx.x]) : 0.f);
+  if (threadIdx.x == 0) *out = (double)m;
 }
 
 cudaError_t max_abs(Handle* h, const float* c, size_t len, double* dev_out) {
-  float* part = reinterpret_cast<float*>(h->red + (size_t)h->red_cap - 2 * kRedBlocks);
-  k_maxabs_partial<<<kRedBlocks, 256, 0, h->stream>>>(c, len, part);
-  k_max_partials<<<1, 32, 0, h->stream>>>(part, kRedBlocks, dev_out);
+  k_maxabs<<<kRedBlocks, kRedBlocks, 0, h->stream>>>(c, len, reinterpret_cast<float*>(red_partials(h, 2)),
+                                                     h->dev_flags + 1, dev_out);
   return cudaGetLastError();
 }
 
