@@ -59,8 +59,7 @@ cudaError_t upload_filters(const double h[kDb][kMaxTaps], cudaStream_t stream) {
   return e;
 }
 
-// A tap pair as one 64-bit FMA operand: {c[j], c[j+1]} (j even) or a duplicated tap.
-__device__ __forceinline__ u64 cpair(const float* c) { return *reinterpret_cast<const u64*>(c); }
+// A duplicated tap as one 64-bit FMA operand.
 __device__ __forceinline__ u64 cdup(const float2& c) { return *reinterpret_cast<const u64*>(&c); }
 
 // Calls CALL(LF) with the compile-time filter length of basis bi (db1..db8).
@@ -89,38 +88,46 @@ constexpr int kPlo = kTO + 4;                    // row-filtered tiles (16-byte 
 
 __device__ __forceinline__ int wrap1(int v, int m) { return v < 0 ? v + m : (v >= m ? v - m : v); }
 
-// Rows: lo/hi[r][k] = sum_j h/g[j] in[r][2k + j], k in [0, TO). Each thread makes
+// The filter passes of the analysis run as loops over the taps of basis b (its length a value, not
+// a template argument): eight unrolled variants, each executed once or twice per CTA, spent 6 to
+// 10 cycles per issue waiting for instructions in the levels below the first (ncu); the loops are
+// one short piece of code for every basis. us: 1024^2, 6 levels, the stage of levels 2-6 65 -> 59, of
+// level 1 83.5 -> 82 (105 -> 84 with one basis per CTA); iteration 457 -> 441, 512^2 120 -> 113, 2048^2
+// (cone dual) 1177 -> 1142.
+//
+// Rows: lo/hi[r][k] = sum_j h/g[j] in[r][2k + j], k in [0, TO), RS rows. Each thread makes
 // four outputs of one row from 16-byte reads; the taps go in pairs,
-// {c[2p], c[2p+1]} x {in[2k+2p], in[2k+2p+1]}, and the two halves are added at the end.
-template <int LF>
-__device__ __forceinline__ void ana_rows(const float* __restrict__ in_s, float* __restrict__ lo_s,
+// {c[2p], c[2p+1]} x {in[2k+2p], in[2k+2p+1]}, and the two halves are added at the end. Two pairs per
+// step (an odd count ends with a pair of zero taps); x0 .. x3 are the sample pairs p .. p + 3.
+__device__ __forceinline__ void ana_rows(int b, const float* __restrict__ in_s, float* __restrict__ lo_s,
                                          float* __restrict__ hi_s) {
-  constexpr int RS = 2 * kTO + LF - 2;
-  constexpr int b = LF / 2 - 1;
-  constexpr int NP = LF / 2 + 3;            // sample pairs feeding four outputs
-  constexpr int NV = (NP + 1) / 2;          // 16-byte reads
+  const int RS = 2 * kTO + 2 * b;
   for (int u = threadIdx.x; u < RS * (kTO / 4); u += blockDim.x) {
     const int r = u % RS, k0 = (u / RS) * 4;
-    const float* row = in_s + r * kA2Pitch + 2 * k0;
-    u64 x[2 * NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(row + 4 * v);
-      x[2 * v] = q.x;
-      x[2 * v + 1] = q.y;
+    const ulonglong2* row = reinterpret_cast<const ulonglong2*>(in_s + r * kA2Pitch + 2 * k0);
+    const ulonglong2 q0 = row[0], q1 = row[1];
+    u64 x0 = q0.x, x1 = q0.y, x2 = q1.x, x3 = q1.y;
+    u64 a[4] = {0ull, 0ull, 0ull, 0ull}, c[4] = {0ull, 0ull, 0ull, 0ull};
+    for (int p = 0; p <= b; p += 2) {
+      const ulonglong2 n = row[2 + (p >> 1)];
+      const ulonglong2 h = *reinterpret_cast<const ulonglong2*>(&c_h[b][2 * p]);
+      const ulonglong2 g = *reinterpret_cast<const ulonglong2*>(&c_g[b][2 * p]);
+      a[0] = ffma2(h.y, x1, ffma2(h.x, x0, a[0]));
+      a[1] = ffma2(h.y, x2, ffma2(h.x, x1, a[1]));
+      a[2] = ffma2(h.y, x3, ffma2(h.x, x2, a[2]));
+      a[3] = ffma2(h.y, n.x, ffma2(h.x, x3, a[3]));
+      c[0] = ffma2(g.y, x1, ffma2(g.x, x0, c[0]));
+      c[1] = ffma2(g.y, x2, ffma2(g.x, x1, c[1]));
+      c[2] = ffma2(g.y, x3, ffma2(g.x, x2, c[2]));
+      c[3] = ffma2(g.y, n.x, ffma2(g.x, x3, c[3]));
+      x0 = x2, x1 = x3, x2 = n.x, x3 = n.y;
     }
     float lo[4], hi[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      u64 a = 0ull, c = 0ull;
-#pragma unroll
-      for (int p = 0; p < LF / 2; ++p) {
-        a = ffma2(cpair(&c_h[b][2 * p]), x[q + p], a);
-        c = ffma2(cpair(&c_g[b][2 * p]), x[q + p], c);
-      }
       float a0, a1, c0, c1;
-      f2unpack(a, a0, a1);
-      f2unpack(c, c0, c1);
+      f2unpack(a[q], a0, a1);
+      f2unpack(c[q], c0, c1);
       lo[q] = a0 + a1;
       hi[q] = c0 + c1;
     }
@@ -161,13 +168,11 @@ __device__ __forceinline__ void sara_epilogue4(int mode, float4 v, size_t idx, f
 // Columns + epilogue for one basis: four subbands of a TO x TO tile. Each thread
 // owns four consecutive columns of one output row (two packed pairs per subband),
 // so the epilogue reads and writes A and gamma W as float4 (staged before the filtering).
-template <int LF>
 __device__ __forceinline__ void ana_cols(const float* __restrict__ lo_s, const float* __restrict__ hi_s, int bi,
                                          int map, int n, int hm, int oy0, int ox0, int last, float* __restrict__ coef,
                                          float* __restrict__ thr, float* __restrict__ approx_out, int mode,
                                          float scale, float gamma, float delta, const float* __restrict__ st_a,
                                          const float* __restrict__ st_t) {
-  constexpr int b = LF / 2 - 1;
   const size_t base = ((size_t)map * kBases + (bi + 1)) * (size_t)n * n;
   for (int u = threadIdx.x; u < kTO * kTO / 4; u += blockDim.x) {
     const int kx0 = (u % (kTO / 4)) * 4, ky = u / (kTO / 4);
@@ -177,11 +182,11 @@ __device__ __forceinline__ void ana_cols(const float* __restrict__ lo_s, const f
     const size_t i_hh = base + (size_t)(hm + Y) * n + (hm + X);
     const size_t i_ll = base + (size_t)Y * n + X;
     u64 ll0 = 0ull, ll1 = 0ull, lh0 = 0ull, lh1 = 0ull, hl0 = 0ull, hl1 = 0ull, hh0 = 0ull, hh1 = 0ull;
-#pragma unroll
-    for (int j = 0; j < LF; ++j) {
+#pragma unroll 2
+    for (int j = 0; j < 2 * bi + 2; ++j) {
       const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(lo_s + (2 * ky + j) * kPlo + kx0);
       const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(hi_s + (2 * ky + j) * kPlo + kx0);
-      const u64 ph = cdup(c_hd[b][j]), pg = cdup(c_gd[b][j]);
+      const u64 ph = cdup(c_hd[bi][j]), pg = cdup(c_gd[bi][j]);
       ll0 = ffma2(ph, a.x, ll0);
       ll1 = ffma2(ph, a.y, ll1);
       lh0 = ffma2(pg, a.x, lh0);
@@ -344,12 +349,11 @@ __device__ __forceinline__ void ana_abort(const AnaSmem& S, int staged, int* err
 
 // One basis of one tile: input copies (issued first), staged epilogue operands (dual
 // mode), rows, columns + epilogue.
-template <int LF>
 __device__ __forceinline__ void ana_basis(const SaraTma& tm, int in_row0, const float* src, int m, const AnaSmem& S,
                                           int bi, int map, int n, int hm, int oy0, int ox0, int last, float* coef,
                                           float* thr, float* approx_out, int mode, float scale, float gamma,
                                           float delta, int* err) {
-  ana_issue_input_t(tm, in_row0, src, m, oy0, ox0, 2 * kTO + LF - 2, S.in_s, &S.bar[0]);
+  ana_issue_input_t(tm, in_row0, src, m, oy0, ox0, 2 * kTO + 2 * bi, S.in_s, &S.bar[0]);
   if (mode == SARA_DUAL)
     stage_epilogue_t(tm, coef, thr, ((size_t)map * kBases + bi + 1) * (size_t)n * n, (map * kBases + bi + 1) * n, n,
                      hm, oy0, ox0, S.st_a, S.st_t, &S.bar[1]);
@@ -358,26 +362,15 @@ __device__ __forceinline__ void ana_basis(const SaraTma& tm, int in_row0, const 
     ana_abort(S, mode == SARA_DUAL, err);
     return;   // this tile is left unchanged (the host reports PS_ETIMEOUT)
   }
-  ana_rows<LF>(S.in_s, S.lo_s, S.hi_s);
+  ana_rows(bi, S.in_s, S.lo_s, S.hi_s);
   __syncthreads();
   if (mode == SARA_DUAL && !mbar_wait(&S.bar[1], 0)) {
     atomicExch(err, 1);
     (void)mbar_drain(&S.bar[1], 0);
     return;
   }
-  ana_cols<LF>(S.lo_s, S.hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta,
+  ana_cols(S.lo_s, S.hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta,
                S.st_a, S.st_t);
-}
-
-__device__ __forceinline__ void ana_dispatch(const SaraTma& tm, int in_row0, int bi, const float* src, int m,
-                                             const AnaSmem& S, int map, int n, int hm, int oy0, int ox0, int last,
-                                             float* coef, float* thr, float* approx_out, int mode, float scale,
-                                             float gamma, float delta, int* err) {
-#define PS_ANA(LFv)                                                                                              \
-  ana_basis<LFv>(tm, in_row0, src, m, S, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, \
-                 delta, err)
-  PS_SWITCH_LF(bi, PS_ANA)
-#undef PS_ANA
 }
 
 // Level-1 analysis: input is the map itself; one basis per CTA (grid.y).
@@ -395,8 +388,8 @@ __global__ void __launch_bounds__(256, 3) k_ana_l1(const float* __restrict__ X, 
     mbar_init(&S.bar[1], 1);
   }
   __syncthreads();
-  ana_dispatch(tm, map * n, bi, X + (size_t)map * n * n, n, S, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode,
-               scale, gamma, delta, err);
+  ana_basis(tm, map * n, X + (size_t)map * n * n, n, S, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode,
+            scale, gamma, delta, err);
 }
 
 // Levels >= 2 with half size >= 32: one basis per CTA (grid.y). (A basis-slowest grid, which
@@ -416,19 +409,17 @@ __global__ void __launch_bounds__(256, 3) k_ana_lv(const float* __restrict__ app
     mbar_init(&S.bar[1], 1);
   }
   __syncthreads();
-  ana_dispatch(tm, (map * kDb + bi) * m, bi, approx_in + ((size_t)map * kDb + bi) * (size_t)m * m, m, S, map, n, hm,
-               oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta, err);
+  ana_basis(tm, (map * kDb + bi) * m, approx_in + ((size_t)map * kDb + bi) * (size_t)m * m, m, S, bi, map, n, hm, oy0,
+            ox0, last, coef, thr, approx_out, mode, scale, gamma, delta, err);
 }
 
 // Columns + epilogue for one basis with two columns per thread (the 512-thread form): each
 // thread owns two consecutive columns of one output row (one packed pair per subband).
-template <int LF>
 __device__ __forceinline__ void ana_cols2(const float* __restrict__ lo_s, const float* __restrict__ hi_s, int bi,
                                           int map, int n, int hm, int oy0, int ox0, int last, float* __restrict__ coef,
                                           float* __restrict__ thr, float* __restrict__ approx_out, int mode,
                                           float scale, float gamma, float delta, const float* __restrict__ st_a,
                                           const float* __restrict__ st_t) {
-  constexpr int b = LF / 2 - 1;
   const size_t base = ((size_t)map * kBases + (bi + 1)) * (size_t)n * n;
   for (int u = threadIdx.x; u < kTO * kTO / 2; u += blockDim.x) {
     const int kx0 = (u % (kTO / 2)) * 2, ky = u / (kTO / 2);
@@ -436,11 +427,11 @@ __device__ __forceinline__ void ana_cols2(const float* __restrict__ lo_s, const 
     const size_t idx[4] = {base + (size_t)Y * n + (hm + X), base + (size_t)(hm + Y) * n + X,
                            base + (size_t)(hm + Y) * n + (hm + X), base + (size_t)Y * n + X};   // HL, LH, HH, LL
     u64 ll = 0ull, lh = 0ull, hl = 0ull, hh = 0ull;
-#pragma unroll
-    for (int j = 0; j < LF; ++j) {
+#pragma unroll 2
+    for (int j = 0; j < 2 * bi + 2; ++j) {
       const u64 a = *reinterpret_cast<const u64*>(lo_s + (2 * ky + j) * kPlo + kx0);
       const u64 c = *reinterpret_cast<const u64*>(hi_s + (2 * ky + j) * kPlo + kx0);
-      const u64 ph = cdup(c_hd[b][j]), pg = cdup(c_gd[b][j]);
+      const u64 ph = cdup(c_hd[bi][j]), pg = cdup(c_gd[bi][j]);
       ll = ffma2(ph, a, ll);
       lh = ffma2(pg, a, lh);
       hl = ffma2(ph, c, hl);
@@ -534,9 +525,7 @@ __global__ void __launch_bounds__(THREADS, NSET == 1 ? 3 : 2) k_ana_l1m(const fl
     if (NSET == 2 && staged && i + 1 < NB)
       stage_epilogue_t(tm, coef, thr, plane(bi + 1), prow(bi + 1), n, hm, oy0, ox0, set_a(s ^ 1), set_t(s ^ 1),
                        &bar[1 + (s ^ 1)]);
-#define PS_MR(LFv) ana_rows<LFv>(in_s, lo_s, hi_s)
-    PS_SWITCH_LF(bi, PS_MR)
-#undef PS_MR
+    ana_rows(bi, in_s, lo_s, hi_s);
     if (staged) {
       const bool ok2 = mbar_wait(&bar[1 + s], par);
       if (__syncthreads_or(!ok2)) {
@@ -550,15 +539,12 @@ __global__ void __launch_bounds__(THREADS, NSET == 1 ? 3 : 2) k_ana_l1m(const fl
     } else {
       __syncthreads();
     }
-#define PS_MC(LFv)                                                                                           \
-  if (THREADS == 512)                                                                                        \
-    ana_cols2<LFv>(lo_s, hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta, \
-                   set_a(s), set_t(s));                                                                      \
-  else                                                                                                       \
-    ana_cols<LFv>(lo_s, hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta,  \
-                  set_a(s), set_t(s))
-    PS_SWITCH_LF(bi, PS_MC)
-#undef PS_MC
+    if (THREADS == 512)
+      ana_cols2(lo_s, hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta, set_a(s),
+                set_t(s));
+    else
+      ana_cols(lo_s, hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta, set_a(s),
+               set_t(s));
     __syncthreads();   // lo/hi and stage set s consumed before the next basis
     // NSET = 1: the single set is free now: refill it for basis i + 1 (its rows run meanwhile).
     if (NSET == 1 && staged && i + 1 < NB)
@@ -632,9 +618,7 @@ __global__ void __launch_bounds__(256, 2) k_ana_pers(const float* __restrict__ i
       abort_all();
       return;
     }
-#define PS_PR(LFv) ana_rows<LFv>(in_s, lo_s, hi_s)
-    PS_SWITCH_LF(bi, PS_PR)
-#undef PS_PR
+    ana_rows(bi, in_s, lo_s, hi_s);
     // The input tile is consumed and every thread is past the previous unit's columns,
     // so the input buffer and stage set s ^ 1 can be refilled for the next unit.
     __syncthreads();
@@ -646,11 +630,8 @@ __global__ void __launch_bounds__(256, 2) k_ana_pers(const float* __restrict__ i
         return;
       }
     }
-#define PS_PC(LFv)                                                                                                 \
-  ana_cols<LFv>(lo_s, hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta,      \
-                st + 2 * s * kStage, st + (2 * s + 1) * kStage)
-    PS_SWITCH_LF(bi, PS_PC)
-#undef PS_PC
+    ana_cols(lo_s, hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta,
+             st + 2 * s * kStage, st + (2 * s + 1) * kStage);
     __syncthreads();   // lo/hi consumed before the next unit's rows
   }
 }
@@ -1022,37 +1003,43 @@ __host__ __device__ constexpr int small_pitch(int m) { return m + 20; }   // row
 // repeating the row's start (periodic). lo, hi: m rows of pitch hm + 4. The coefficients a
 // (and thresholds t in the dual mode) are m0 x m0 blocks; the results replace a. The
 // approximation replaces img in the layout of the next level.
-template <int LF>
-__device__ __forceinline__ void small_ana_level(float* __restrict__ img, float* __restrict__ lo, float* __restrict__ hi,
+// LFT: the filter length, or 0 for a loop over the taps of basis b (as ana_rows).
+template <int LFT>
+__device__ __forceinline__ void small_ana_level(int b, float* __restrict__ img, float* __restrict__ lo, float* __restrict__ hi,
                                                 float* __restrict__ a, const float* __restrict__ t, int m, int m0,
                                                 int last, int mode, float scale, float gamma, float delta) {
-  constexpr int b = LF / 2 - 1;
+  const int LF = LFT ? LFT : 2 * b + 2;
+  constexpr int U4 = LFT ? 4 : 1, U1 = LFT ? 16 : 2;   // steps unrolled: all, or one of the loop's
   const int hm = m >> 1, mask = m - 1, P = small_pitch(m), Q = hm + 4, PN = small_pitch(hm);
   auto epi = [&](float v, int o) {
     if (mode == SARA_DUAL) a[o] = fminf(fmaxf(fmaf(scale, v, a[o]), -t[o]), t[o]);
     else a[o] = mode == SARA_APPLY ? scale * v : gamma * delta / (delta + fabsf(scale * v));
   };
   if (hm >= 4) {
-    constexpr int NV = (LF + 6 + 3) / 4;   // 16-byte reads of the samples of four outputs
     for (int u = threadIdx.x; u < m * (hm >> 2); u += kSmallThreads) {
       const int r = u & mask, k0 = (u / m) * 4;
       const float4* row = reinterpret_cast<const float4*>(img + r * P + 2 * k0);
-      float x[4 * NV];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const float4 q = row[v];
-        x[4 * v] = q.x, x[4 * v + 1] = q.y, x[4 * v + 2] = q.z, x[4 * v + 3] = q.w;
-      }
+      float4 x0 = row[0], x1 = row[1];   // samples j .. j + 7 of the step's first tap j
       // One chain per output, in the order of the taps: a scalar FMA does as much per clock
       // as a packed one, and the coarse coefficients are the ones whose rounding shows most.
+      // Four taps per step, zero ones at the end of the shorter filters.
       float l[4] = {0.f, 0.f, 0.f, 0.f}, h[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll U4
+      for (int j = 0; j < LF; j += 4) {
+        const float4 x2 = row[2 + (j >> 2)];
+        const float4 ch = *reinterpret_cast<const float4*>(&c_h[b][j]), cg = *reinterpret_cast<const float4*>(&c_g[b][j]);
+        const float x[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
+        const float th[4] = {ch.x, ch.y, ch.z, ch.w}, tg[4] = {cg.x, cg.y, cg.z, cg.w};
 #pragma unroll
-      for (int j = 0; j < LF; ++j)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          l[q] = fmaf(c_h[b][j], x[2 * q + j], l[q]);
-          h[q] = fmaf(c_g[b][j], x[2 * q + j], h[q]);
-        }
+          for (int q = 0; q < 4; ++q) {
+            if (LFT && j + i >= LFT) continue;
+            l[q] = fmaf(th[i], x[2 * q + i], l[q]);
+            h[q] = fmaf(tg[i], x[2 * q + i], h[q]);
+          }
+        x0 = x1, x1 = x2;
+      }
       *reinterpret_cast<float4*>(lo + r * Q + k0) = make_float4(l[0], l[1], l[2], l[3]);
       *reinterpret_cast<float4*>(hi + r * Q + k0) = make_float4(h[0], h[1], h[2], h[3]);
     }
@@ -1061,7 +1048,7 @@ __device__ __forceinline__ void small_ana_level(float* __restrict__ img, float* 
     for (int u = threadIdx.x; u < hm * qs; u += kSmallThreads) {
       const int ky = u / qs, kx = (u - ky * qs) * 4;
       u64 ll0 = 0ull, ll1 = 0ull, lh0 = 0ull, lh1 = 0ull, hl0 = 0ull, hl1 = 0ull, hh0 = 0ull, hh1 = 0ull;
-#pragma unroll
+#pragma unroll U1
       for (int j = 0; j < LF; ++j) {
         const int o = ((2 * ky + j) & mask) * Q + kx;
         const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(lo + o);
@@ -1102,7 +1089,7 @@ __device__ __forceinline__ void small_ana_level(float* __restrict__ img, float* 
     for (int u = threadIdx.x; u < m * hm; u += kSmallThreads) {
       const int r = u / hm, k = u - r * hm;
       float s = 0.f, d = 0.f;
-#pragma unroll
+#pragma unroll U1
       for (int j = 0; j < LF; ++j) {
         const float v = img[r * P + ((2 * k + j) & mask)];
         s = fmaf(c_h[b][j], v, s);
@@ -1115,7 +1102,7 @@ __device__ __forceinline__ void small_ana_level(float* __restrict__ img, float* 
     for (int u = threadIdx.x; u < hm * hm; u += kSmallThreads) {
       const int ky = u / hm, kx = u - ky * hm;
       float ll = 0.f, lh = 0.f, hl = 0.f, hh = 0.f;
-#pragma unroll
+#pragma unroll U1
       for (int j = 0; j < LF; ++j) {
         const int o = ((2 * ky + j) & mask) * Q + kx;
         ll = fmaf(c_h[b][j], lo[o], ll);
@@ -1135,7 +1122,8 @@ __device__ __forceinline__ void small_ana_level(float* __restrict__ img, float* 
 
 // Analysis levels l0..L (sides m0 = n >> (l0 - 1) <= kSmall and below); one CTA per (basis,
 // map) = (blockIdx.x, blockIdx.y). The input of level l0 is X (l0 = 1) or that level's
-// approximation scratch (layout [map][basis][m0][m0]).
+// approximation scratch (layout [map][basis][m0][m0]). LOOPS: filters as loops over the taps.
+template <bool LOOPS>
 __global__ void __launch_bounds__(kSmallThreads) k_ana_small(const float* __restrict__ in, int l0, int L, int n,
                                                              float* __restrict__ coef, float* __restrict__ thr,
                                                              int mode, float scale, float gamma, float delta) {
@@ -1166,9 +1154,13 @@ __global__ void __launch_bounds__(kSmallThreads) k_ana_small(const float* __rest
   }
   __syncthreads();
   for (int l = l0, m = m0; l <= L; ++l, m >>= 1) {
-#define PS_TA(LFv) small_ana_level<LFv>(img, lo, hi, a, t, m, m0, l == L, mode, scale, gamma, delta)
-    PS_SWITCH_LF(bi, PS_TA)
+    if (LOOPS) {
+      small_ana_level<0>(bi, img, lo, hi, a, t, m, m0, l == L, mode, scale, gamma, delta);
+    } else {
+#define PS_TA(LFv) small_ana_level<LFv>(bi, img, lo, hi, a, t, m, m0, l == L, mode, scale, gamma, delta)
+      PS_SWITCH_LF(bi, PS_TA)
 #undef PS_TA
+    }
   }
   float* dst = (mode == SARA_REWEIGHT ? thr : coef) + base;
   for (int u = threadIdx.x; u < m0 * q0; u += kSmallThreads) {
@@ -1515,9 +1507,10 @@ cudaError_t configure_kernels() {
   e = cudaFuncSetAttribute((const void*)k_ana_pers, cudaFuncAttributePreferredSharedMemoryCarveout,
                            cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute((const void*)k_ana_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)ana_small_smem(kSmall));
-  if (e != cudaSuccess) return e;
+  for (const void* f : {(const void*)k_ana_small<false>, (const void*)k_ana_small<true>}) {
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ana_small_smem(kSmall));
+    if (e != cudaSuccess) return e;
+  }
   for (const void* f : {(const void*)k_syn2_split<8>, (const void*)k_syn2_split<4>}) {
     e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)syn2_smem(1));
     if (e != cudaSuccess) return e;
@@ -1595,11 +1588,15 @@ cudaError_t sara_analysis(Handle* h, const float* X, float* coef, float* thr, in
   }
   if (lt <= L) {
     const float* in = lt == 1 ? X : buf[(lt - 2) & 1];
+    // Loops over the taps from 256^2 on (512^2 120 -> 113 us per iteration, 1024^2 446 -> 441: the eight
+    // unrolled variants wait for instructions, and take their cache from the NUFFT kernels beside
+    // them); unrolled below, where a pass is one chain of latencies (64^2 26.3 against 27.2, 128^2
+    // 39.3 against 39.9).
     if (lt == 1)
-      k_ana_small<<<dim3(kDb, nmaps), kSmallThreads, ana_small_smem(n), h->stream>>>(in, lt, L, n, coef, thr, mode, scale,
-                                                                                  gamma, delta);
+      k_ana_small<false><<<dim3(kDb, nmaps), kSmallThreads, ana_small_smem(n), h->stream>>>(in, lt, L, n, coef, thr, mode,
+                                                                                         scale, gamma, delta);
     else
-      launch_after(true, k_ana_small, dim3(kDb, nmaps), kSmallThreads, ana_small_smem(n >> (lt - 1)), h->stream, in, lt, L, n, coef,
+      launch_after(true, n <= 128 ? k_ana_small<false> : k_ana_small<true>, dim3(kDb, nmaps), kSmallThreads, ana_small_smem(n >> (lt - 1)), h->stream, in, lt, L, n, coef,
                    thr, mode, scale, gamma, delta);
     if (lt == 1 && fine_done) {
       const cudaError_t e = cudaEventRecord(fine_done, h->stream);
