@@ -165,60 +165,73 @@ __device__ __forceinline__ void sara_epilogue4(int mode, float4 v, size_t idx, f
   }
 }
 
-// Columns + epilogue for one basis: four subbands of a TO x TO tile. Each thread
-// owns four consecutive columns of one output row (two packed pairs per subband),
-// so the epilogue reads and writes A and gamma W as float4 (staged before the filtering).
+// Columns + epilogue for one basis: four subbands of a TO x TO tile, 256 threads. Half of them
+// filter the low rows (LL and LH), half the high rows (HL and HH); a thread owns four consecutive
+// columns (two packed pairs) of two output rows, whose 2 LF taps reach over LF + 2 input rows, so
+// it reads 18 rows of 16 bytes for db8 where one output row of all four subbands took 32. The
+// epilogue reads and writes A and gamma W as float4 (staged before the filtering).
 __device__ __forceinline__ void ana_cols(const float* __restrict__ lo_s, const float* __restrict__ hi_s, int bi,
                                          int map, int n, int hm, int oy0, int ox0, int last, float* __restrict__ coef,
                                          float* __restrict__ thr, float* __restrict__ approx_out, int mode,
                                          float scale, float gamma, float delta, const float* __restrict__ st_a,
                                          const float* __restrict__ st_t) {
   const size_t base = ((size_t)map * kBases + (bi + 1)) * (size_t)n * n;
-  for (int u = threadIdx.x; u < kTO * kTO / 4; u += blockDim.x) {
-    const int kx0 = (u % (kTO / 4)) * 4, ky = u / (kTO / 4);
-    const int Y = oy0 + ky, X = ox0 + kx0;
-    const size_t i_hl = base + (size_t)Y * n + (hm + X);
-    const size_t i_lh = base + (size_t)(hm + Y) * n + X;
-    const size_t i_hh = base + (size_t)(hm + Y) * n + (hm + X);
-    const size_t i_ll = base + (size_t)Y * n + X;
-    u64 ll0 = 0ull, ll1 = 0ull, lh0 = 0ull, lh1 = 0ull, hl0 = 0ull, hl1 = 0ull, hh0 = 0ull, hh1 = 0ull;
-#pragma unroll 2
-    for (int j = 0; j < 2 * bi + 2; ++j) {
-      const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(lo_s + (2 * ky + j) * kPlo + kx0);
-      const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(hi_s + (2 * ky + j) * kPlo + kx0);
-      const u64 ph = cdup(c_hd[bi][j]), pg = cdup(c_gd[bi][j]);
-      ll0 = ffma2(ph, a.x, ll0);
-      ll1 = ffma2(ph, a.y, ll1);
-      lh0 = ffma2(pg, a.x, lh0);
-      lh1 = ffma2(pg, a.y, lh1);
-      hl0 = ffma2(ph, c.x, hl0);
-      hl1 = ffma2(ph, c.y, hl1);
-      hh0 = ffma2(pg, c.x, hh0);
-      hh1 = ffma2(pg, c.y, hh1);
-    }
+  const bool high = threadIdx.x >= 128;   // warp-uniform
+  const int kx0 = (threadIdx.x & 7) * 4, ky0 = 2 * ((threadIdx.x >> 3) & 15);
+  const float* col = (high ? hi_s : lo_s) + 2 * ky0 * kPlo + kx0;
+  u64 h[2][2], g[2][2];   // [output row][column pair] through the low and the high filter
+#pragma unroll
+  for (int r = 0; r < 2; ++r) h[r][0] = h[r][1] = g[r][0] = g[r][1] = 0ull;
+  // Input rows 2 q and 2 q + 1 meet taps 2 q, 2 q + 1 of the first output row and 2 q - 2, 2 q - 1 of the second.
+  auto step = [&](int r, ulonglong2 x0, ulonglong2 x1, ulonglong2 th, ulonglong2 tg) {
+    h[r][0] = ffma2(th.y, x1.x, ffma2(th.x, x0.x, h[r][0]));
+    h[r][1] = ffma2(th.y, x1.y, ffma2(th.x, x0.y, h[r][1]));
+    g[r][0] = ffma2(tg.y, x1.x, ffma2(tg.x, x0.x, g[r][0]));
+    g[r][1] = ffma2(tg.y, x1.y, ffma2(tg.x, x0.y, g[r][1]));
+  };
+  const ulonglong2* ch = reinterpret_cast<const ulonglong2*>(&c_hd[bi][0]);
+  const ulonglong2* cg = reinterpret_cast<const ulonglong2*>(&c_gd[bi][0]);
+  auto row = [&](int i) { return *reinterpret_cast<const ulonglong2*>(col + i * kPlo); };
+  ulonglong2 th = ch[0], tg = cg[0], x0 = row(0), x1 = row(1);
+  step(0, x0, x1, th, tg);
+  for (int q = 1; q <= bi; ++q) {
+    x0 = row(2 * q), x1 = row(2 * q + 1);
+    step(1, x0, x1, th, tg);
+    th = ch[q], tg = cg[q];
+    step(0, x0, x1, th, tg);
+  }
+  x0 = row(2 * bi + 2), x1 = row(2 * bi + 3);
+  step(1, x0, x1, th, tg);
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int ky = ky0 + r, Y = oy0 + ky, X = ox0 + kx0, so = ky * kTO + kx0;
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 a_hl = z, a_lh = z, a_hh = z, a_ll = z, t_hl = z, t_lh = z, t_hh = z, t_ll = z;
-    if (mode == SARA_DUAL) {
-      // Staged by the bulk-copy engine: [subband][row][32].
-      const int so = ky * kTO + kx0;
-      a_hl = *reinterpret_cast<const float4*>(st_a + so);
-      a_lh = *reinterpret_cast<const float4*>(st_a + kTO * kTO + so);
-      a_hh = *reinterpret_cast<const float4*>(st_a + 2 * kTO * kTO + so);
-      t_hl = *reinterpret_cast<const float4*>(st_t + so);
-      t_lh = *reinterpret_cast<const float4*>(st_t + kTO * kTO + so);
-      t_hh = *reinterpret_cast<const float4*>(st_t + 2 * kTO * kTO + so);
+    auto out = [&](u64 v0, u64 v1, int sb, size_t o) {   // staged by the bulk-copy engine: [subband][row][32]
+      float4 a = z, t = z;
+      if (mode == SARA_DUAL) {
+        a = *reinterpret_cast<const float4*>(st_a + sb * kTO * kTO + so);
+        t = *reinterpret_cast<const float4*>(st_t + sb * kTO * kTO + so);
+      }
+      sara_epilogue4(mode, f4of(v0, v1), base + o, a, t, coef, thr, scale, gamma, delta);
+    };
+    if (high) {
+      out(h[r][0], h[r][1], 0, (size_t)Y * n + (hm + X));          // x-high, y-low
+      out(g[r][0], g[r][1], 2, (size_t)(hm + Y) * n + (hm + X));
+    } else {
+      out(g[r][0], g[r][1], 1, (size_t)(hm + Y) * n + X);          // x-low, y-high
+      const size_t o = base + (size_t)Y * n + X;
       if (last) {
-        a_ll = *reinterpret_cast<const float4*>(coef + i_ll);
-        t_ll = *reinterpret_cast<const float4*>(thr + i_ll);
+        float4 a = z, t = z;
+        if (mode == SARA_DUAL) {
+          a = *reinterpret_cast<const float4*>(coef + o);
+          t = *reinterpret_cast<const float4*>(thr + o);
+        }
+        sara_epilogue4(mode, f4of(h[r][0], h[r][1]), o, a, t, coef, thr, scale, gamma, delta);
+      } else {
+        *reinterpret_cast<float4*>(approx_out + ((size_t)map * kDb + bi) * (size_t)hm * hm + (size_t)Y * hm + X) =
+            f4of(h[r][0], h[r][1]);
       }
     }
-    sara_epilogue4(mode, f4of(hl0, hl1), i_hl, a_hl, t_hl, coef, thr, scale, gamma, delta);   // x-high, y-low
-    sara_epilogue4(mode, f4of(lh0, lh1), i_lh, a_lh, t_lh, coef, thr, scale, gamma, delta);   // x-low, y-high
-    sara_epilogue4(mode, f4of(hh0, hh1), i_hh, a_hh, t_hh, coef, thr, scale, gamma, delta);
-    if (last) sara_epilogue4(mode, f4of(ll0, ll1), i_ll, a_ll, t_ll, coef, thr, scale, gamma, delta);
-    else
-      *reinterpret_cast<float4*>(approx_out + ((size_t)map * kDb + bi) * (size_t)hm * hm + (size_t)Y * hm + X) =
-          f4of(ll0, ll1);
   }
 }
 
@@ -713,16 +726,26 @@ __device__ __forceinline__ void syn2_issue_t(const SaraTma& tm, int prow, int ap
 
 // Along y for basis LF: lo/hi at output rows 4 rg + t (t = 0..3) and staged columns
 // c, c + 1, from coefficient rows 2 rg + i (i = 0 .. half + 1) through tap
-// j = t - 2 (i - half). Columns start at the even column at or left of 8 - half.
+// j = t - 2 (i - half). Columns start at the even column at or left of 8 - half. The 256 threads take
+// the tile's own 16 column pairs x 16 row groups, a half-warp 8 pairs of two row groups and a
+// quarter-warp 4 of them, so that neither the 8-byte reads (row groups 16 banks apart) nor the
+// 16-byte column-major writes share a bank; the first 64 then take the halo's pairs. (One running
+// index over all pairs: 3.9 M conflicts in 11.5 M wavefronts at 1024^2.)
 template <int LF>
 __device__ __forceinline__ void syn2_ypass(const float* __restrict__ s4, float* __restrict__ loT,
                                            float* __restrict__ hiT) {
   constexpr int half = LF / 2 - 1;
   constexpr int cs = (8 - half) & ~1;
-  constexpr int NCP = (kC2Cols - cs) / 2;
-  for (int u = threadIdx.x; u < NCP * (kT2 / 4); u += blockDim.x) {
-    const int cp = u % NCP, rg = u / NCP;
-    const int c = cs + 2 * cp;
+  constexpr int NCR = (8 - cs) / 2;       // column pairs left of the tile's own 16
+  const int l = threadIdx.x & 31;
+#pragma unroll 1
+  for (int k = 0; k < 2; ++k) {
+    int c = 8 + 2 * ((l & 3) | ((l >> 1) & 12)), rg = 2 * (threadIdx.x >> 5) + ((l >> 2) & 1);
+    if (k) {
+      if (threadIdx.x >= 64 || (l & 3) >= NCR) break;
+      c = cs + 2 * (l & 3);
+      rg = threadIdx.x >> 2;
+    }
     u64 lo[4], hi[4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) lo[t] = hi[t] = 0ull;
