@@ -362,39 +362,27 @@ ps_status ps_batch_synchronize(ps_batch* b);
 void ps_batch_destroy(ps_batch* b);
 
 /* Launch choices of the kernels (the paper runs the same operators in every
- * iteration of Algorithm 1 and prescribes no implementation; which launch shape is
- * fastest depends on the image size and on how the visibilities fill the uv plane,
- * so it is measured on the handle's own problem). Values index the candidates: */
+ * iteration of Algorithm 1 and prescribes no implementation). The library picks each
+ * kernel's launch shape by rules on the image size, the number of maps and how the
+ * visibilities fill the uv plane, so every slot has one form; the values that selected
+ * forms of their own before are accepted and equal. */
 enum {
-  PS_TUNE_SYNTHESIS = 0,  /* finest synthesis level, of images with more than 304 tiles of 64 x 64
-                             over their maps (smaller ones take one form of their own): 0 double-buffered subband staging (3 CTAs/SM),
-                             1 single-buffered, refilled during the x-pass (4 CTAs/SM),
-                             2 as 1 in persistent CTAs looping over (tile, map) units, the staging
-                               running on from one unit into the next */
-  PS_TUNE_DEGRID = 1,     /* 0-2: one form (the library picks its launch shape from the rows and
-                             their coverage); the three values are accepted and equal */
-  PS_TUNE_GRID = 2,       /* 0-4: one form, likewise */
-  PS_TUNE_ANALYSIS = 3,   /* tiled analysis levels (input side above 64): 0 one (tile, basis, map) unit per CTA,
-                             1 persistent (2 CTAs/SM looping over units, next unit's copies in flight),
-                             2 level 1 with one CTA per (tile, map): the map's input tile copied once for
-                               the 8 bases, each basis' staged A and gamma W in flight during the previous
-                               basis (levels >= 2 as 0),
-                             3 as 2 with one CTA per (tile, 4 bases, map),
-                             4 as 3 with 512 threads per CTA (two columns per thread),
-                             5 as 3 with one staging set, refilled for the next basis during its
-                               row pass (3 CTAs/SM) */
+  PS_TUNE_SYNTHESIS = 0,  /* finest synthesis level: 0-2 */
+  PS_TUNE_DEGRID = 1,     /* 0-2 */
+  PS_TUNE_GRID = 2,       /* 0-4 */
+  PS_TUNE_ANALYSIS = 3,   /* tiled analysis levels: 0-5 */
   PS_TUNE_COUNT = 4
 };
 
-/* Autotuner: after ps_set_measurements, time every candidate of every PS_TUNE_*
- * slot on the handle's data (reps launches each, CUDA events on the handle's
- * stream, after one untimed launch) and keep the fastest. The state of the
+/* Autotuner: after ps_set_measurements, time the form of every PS_TUNE_* slot on the
+ * handle's data (reps launches each, CUDA events on the handle's
+ * stream, after one untimed launch) and set the slots to it. The state of the
  * iteration is unchanged (the timed launches run the analysis dual update on scratch
  * coefficients, recompute Psi A of the current A in place, run the degridding dual update
  * on a scratch copy of the data dual and grid the current dual into the gridding
  * accumulator, an intermediate; phi^dagger B is kept). Uses (and on first use allocates) the handle's
  * 36N operator scratch. choices (nullable) receives the
- * PS_TUNE_COUNT picks; ms (nullable) receives, per slot, the time of the pick in
+ * PS_TUNE_COUNT picks (0); ms (nullable) receives, per slot, its time in
  * milliseconds. Synchronises the stream. PS_ESTATE before measurements. */
 ps_status ps_autotune(ps_handle* h, int32_t reps, int32_t* choices, double* ms);
 

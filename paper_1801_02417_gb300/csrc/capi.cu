@@ -1322,10 +1322,8 @@ ps_status ps_profile_stages(ps_handle* h, int32_t n_iter, double* stage_ms) {
 }
 
 // ---------------------------------------------------------------------------
-// Autotuner: candidates per PS_TUNE_* slot, each timed on the handle's own data.
-// kTuneForms: the forms behind them that differ (the interpolation kernels have one each).
-static const int kTuneCandidates[PS_TUNE_COUNT] = {3, 3, 5, 6};
-static const int kTuneForms[PS_TUNE_COUNT] = {3, 1, 1, 6};
+// Autotuner: the PS_TUNE_* slots, timed on the handle's own data.
+static const int kTuneCandidates[PS_TUNE_COUNT] = {3, 3, 5, 6};   // values that are accepted
 
 // Mean milliseconds of `reps` launches of f after one untimed launch.
 extern "C++" {
@@ -1357,22 +1355,11 @@ ps_status ps_autotune(ps_handle* h, int32_t reps, int32_t* choices, double* ms) 
     if (st != PS_OK) return st;
   }
   double best_ms[PS_TUNE_COUNT] = {0.0, 0.0, 0.0, 0.0};
+  // Every slot has one form (the launch shapes follow rules on the sizes): the pick is 0, and its
+  // time is measured.
   auto pick = [&](int slot, auto launch) -> ps_status {
-    int best = 0;
-    double best_t = 0.0;
-    for (int v = 0; v < kTuneForms[slot]; ++v) {
-      h->tune[slot] = v;
-      double t = 0.0;
-      ps_status st = tune_time(h, reps, launch, &t);
-      if (st != PS_OK) return st;
-      if (v == 0 || t < best_t) {
-        best = v;
-        best_t = t;
-      }
-    }
-    h->tune[slot] = best;
-    best_ms[slot] = best_t;
-    return PS_OK;
+    h->tune[slot] = 0;
+    return tune_time(h, reps, launch, &best_ms[slot]);
   };
   // Analysis: the dual update of steps 5-6 as the iteration runs it (staged A and gamma W
   // reads), on scratch coefficients so the state's A is untouched.

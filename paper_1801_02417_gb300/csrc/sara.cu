@@ -309,7 +309,7 @@ __device__ __forceinline__ void stage_epilogue(const float* coef, const float* t
     const size_t off = sb == 0 ? base + (size_t)Y * n + hm + ox0
                                : (sb == 1 ? base + (size_t)(hm + Y) * n + ox0 : base + (size_t)(hm + Y) * n + hm + ox0);
     float* dst = (arr ? st_t : st_a) + sb * kTO * kTO + r * kTO;
-    fence_proxy_async();   // the persistent form refills buffers its threads have read
+    fence_proxy_async();   // k_ana_l1m refills buffers its threads have read
     bulk_g2s(dst, (arr ? thr : coef) + off, kTO * sizeof(float), bar);
   }
 }
@@ -325,7 +325,7 @@ __device__ __forceinline__ void stage_epilogue_t(const SaraTma& tm, const float*
   }
   if (threadIdx.x == 0) {
     mbar_expect_tx(bar, 2u * kStage * sizeof(float));
-    fence_proxy_async();   // the persistent and multi-basis forms refill buffers their threads have read
+    fence_proxy_async();   // k_ana_l1m refills buffers its threads have read
     const int xs[3] = {hm + ox0, ox0, hm + ox0}, ys[3] = {prow + oy0, prow + hm + oy0, prow + hm + oy0};
 #pragma unroll
     for (int sb = 0; sb < 3; ++sb) {
@@ -426,226 +426,62 @@ __global__ void __launch_bounds__(256, 3) k_ana_lv(const float* __restrict__ app
             ox0, last, coef, thr, approx_out, mode, scale, gamma, delta, err);
 }
 
-// Columns + epilogue for one basis with two columns per thread (the 512-thread form): each
-// thread owns two consecutive columns of one output row (one packed pair per subband).
-__device__ __forceinline__ void ana_cols2(const float* __restrict__ lo_s, const float* __restrict__ hi_s, int bi,
-                                          int map, int n, int hm, int oy0, int ox0, int last, float* __restrict__ coef,
-                                          float* __restrict__ thr, float* __restrict__ approx_out, int mode,
-                                          float scale, float gamma, float delta, const float* __restrict__ st_a,
-                                          const float* __restrict__ st_t) {
-  const size_t base = ((size_t)map * kBases + (bi + 1)) * (size_t)n * n;
-  for (int u = threadIdx.x; u < kTO * kTO / 2; u += blockDim.x) {
-    const int kx0 = (u % (kTO / 2)) * 2, ky = u / (kTO / 2);
-    const int Y = oy0 + ky, X = ox0 + kx0;
-    const size_t idx[4] = {base + (size_t)Y * n + (hm + X), base + (size_t)(hm + Y) * n + X,
-                           base + (size_t)(hm + Y) * n + (hm + X), base + (size_t)Y * n + X};   // HL, LH, HH, LL
-    u64 ll = 0ull, lh = 0ull, hl = 0ull, hh = 0ull;
-#pragma unroll 2
-    for (int j = 0; j < 2 * bi + 2; ++j) {
-      const u64 a = *reinterpret_cast<const u64*>(lo_s + (2 * ky + j) * kPlo + kx0);
-      const u64 c = *reinterpret_cast<const u64*>(hi_s + (2 * ky + j) * kPlo + kx0);
-      const u64 ph = cdup(c_hd[bi][j]), pg = cdup(c_gd[bi][j]);
-      ll = ffma2(ph, a, ll);
-      lh = ffma2(pg, a, lh);
-      hl = ffma2(ph, c, hl);
-      hh = ffma2(pg, c, hh);
-    }
-    const u64 v[4] = {hl, lh, hh, ll};
-    const int nsb = last ? 4 : 3;
-    for (int sb = 0; sb < nsb; ++sb) {
-      float v0, v1;
-      f2unpack(v[sb], v0, v1);
-      float2* dst = reinterpret_cast<float2*>(coef + idx[sb]);
-      if (mode == SARA_DUAL) {
-        float2 a2, t2;
-        if (sb < 3) {
-          a2 = *reinterpret_cast<const float2*>(st_a + sb * kTO * kTO + ky * kTO + kx0);
-          t2 = *reinterpret_cast<const float2*>(st_t + sb * kTO * kTO + ky * kTO + kx0);
-        } else {
-          a2 = *reinterpret_cast<const float2*>(coef + idx[sb]);
-          t2 = *reinterpret_cast<const float2*>(thr + idx[sb]);
-        }
-        *dst = make_float2(fminf(fmaxf(fmaf(scale, v0, a2.x), -t2.x), t2.x),
-                           fminf(fmaxf(fmaf(scale, v1, a2.y), -t2.y), t2.y));
-      } else if (mode == SARA_APPLY) {
-        *dst = make_float2(scale * v0, scale * v1);
-      } else {
-        const float gd = gamma * delta;
-        *reinterpret_cast<float2*>(thr + idx[sb]) =
-            make_float2(gd / (delta + fabsf(scale * v0)), gd / (delta + fabsf(scale * v1)));
-      }
-    }
-    if (!last) {
-      float a0, a1;
-      f2unpack(ll, a0, a1);
-      *reinterpret_cast<float2*>(approx_out + ((size_t)map * kDb + bi) * (size_t)hm * hm + (size_t)Y * hm + X) =
-          make_float2(a0, a1);
-    }
-  }
-}
-
-// Level-1 analysis with the input tile shared by NB bases: one CTA per (tile, group of NB
-// bases, map). The 2 TO + 14 rows the db8 filter needs cover every shorter filter (same
+// Level-1 analysis with the input tile shared by four bases: one CTA per (tile, half of the bases,
+// map). The 2 TO + 14 rows the db8 filter needs cover every shorter filter (same
 // origin), so the map's tile is copied once and each basis filters it from shared memory.
-// NSET = 2: the staged A and gamma W rows of basis i + 1 (dual mode) are copied into the
-// second of two staging sets while basis i is filtered (2 CTAs/SM). NSET = 1: one staging
-// set, refilled for basis i + 1 once basis i's columns have read it, so the copy overlaps the
-// next basis' row pass; the smaller footprint fits 3 CTAs/SM (256 threads).
-static size_t multi_analysis_smem(int nset = 2) {
-  return (size_t)(kAnaPre + 2 * nset * kStage) * sizeof(float) + 32;
-}
+// One staging set holds A and gamma W (dual mode), refilled for basis i + 1 once basis i's
+// columns have read it, so the copy overlaps the next basis' row pass; 73 KB, 3 CTAs/SM.
+// (Two sets at 2 CTAs/SM, eight bases per CTA, 512 threads and a persistent form over all
+// units were slower: 85-88, 94 and 139 us at 1024^2 against 82.)
+constexpr int kL1Bases = 4;
+static size_t multi_analysis_smem() { return (size_t)(kAnaPre + 2 * kStage) * sizeof(float) + 32; }
 
-template <int NB, int THREADS, int NSET = 2>
-__global__ void __launch_bounds__(THREADS, NSET == 1 ? 3 : 2) k_ana_l1m(const float* __restrict__ X, int n, int last,
+__global__ void __launch_bounds__(256, 3) k_ana_l1m(const float* __restrict__ X, int n, int last,
                                                     float* __restrict__ coef, float* __restrict__ thr,
                                                     float* __restrict__ approx_out, int mode, float scale,
                                                     float gamma, float delta, int* err,
                                                     const __grid_constant__ SaraTma tm) {
   extern __shared__ __align__(128) float4 smm[];
-  float* in_s = reinterpret_cast<float*>(smm);
-  float* lo_s = in_s + kA2In;
-  float* hi_s = lo_s + kRSmax * kPlo;
-  float* st = in_s + kAnaPre;                                          // set s: A at st + 2 s kStage, gamma W after it
-  uint64_t* bar = reinterpret_cast<uint64_t*>(st + 2 * NSET * kStage);    // [0] input tile, [1 + s] stage set s
-  const int map = blockIdx.z, b0 = blockIdx.y * NB;
+  const AnaSmem S = ana_smem(smm);
+  const int map = blockIdx.z, b0 = blockIdx.y * kL1Bases;
   const int hm = n >> 1, tilesx = hm / kTO;
   const int oy0 = (blockIdx.x / tilesx) * kTO, ox0 = (blockIdx.x % tilesx) * kTO;
   const bool staged = mode == SARA_DUAL;
-  auto plane = [&](int bi) { return ((size_t)map * kBases + bi + 1) * (size_t)n * n; };
-  auto prow = [&](int bi) { return (map * kBases + bi + 1) * n; };
-  auto set_a = [&](int s) { return st + 2 * s * kStage; };
-  auto set_t = [&](int s) { return st + (2 * s + 1) * kStage; };
-  if (threadIdx.x == 0)
-    for (int q = 0; q < 1 + NSET; ++q) mbar_init(&bar[q], 1);
+  auto stage = [&](int bi) {
+    stage_epilogue_t(tm, coef, thr, ((size_t)map * kBases + bi + 1) * (size_t)n * n, (map * kBases + bi + 1) * n, n, hm,
+                     oy0, ox0, S.st_a, S.st_t, &S.bar[1]);
+  };
+  if (threadIdx.x == 0) {
+    mbar_init(&S.bar[0], 1);
+    mbar_init(&S.bar[1], 1);
+  }
   __syncthreads();
-  ana_issue_input_t(tm, map * n, X + (size_t)map * n * n, n, oy0, ox0, kRSmax, in_s, &bar[0]);
-  if (staged) stage_epilogue_t(tm, coef, thr, plane(b0), prow(b0), n, hm, oy0, ox0, set_a(0), set_t(0), &bar[1]);
-  const bool ok = mbar_wait(&bar[0], 0);
+  ana_issue_input_t(tm, map * n, X + (size_t)map * n * n, n, oy0, ox0, kRSmax, S.in_s, &S.bar[0]);
+  if (staged) stage(b0);
+  const bool ok = mbar_wait(&S.bar[0], 0);
   if (__syncthreads_or(!ok)) {
-    if (threadIdx.x == 0) {
-      atomicExch(err, 1);
-      (void)mbar_drain(&bar[0], 0);
-      if (staged) (void)mbar_drain(&bar[1], 0);
-    }
+    ana_abort(S, staged, err);
     return;   // the CTA's tiles are left unchanged (the host reports PS_ETIMEOUT)
   }
-  for (int i = 0; i < NB; ++i) {
-    const int bi = b0 + i, s = NSET == 2 ? (i & 1) : 0;
-    // Phase of set s's barrier for basis i (each use completes one phase).
-    const uint32_t par = NSET == 2 ? (uint32_t)((i >> 1) & 1) : (uint32_t)(i & 1);
-    // NSET = 2: set s ^ 1 was last read by basis i - 1, which ended at a barrier: refill it
-    // for basis i + 1.
-    if (NSET == 2 && staged && i + 1 < NB)
-      stage_epilogue_t(tm, coef, thr, plane(bi + 1), prow(bi + 1), n, hm, oy0, ox0, set_a(s ^ 1), set_t(s ^ 1),
-                       &bar[1 + (s ^ 1)]);
-    ana_rows(bi, in_s, lo_s, hi_s);
+  for (int i = 0; i < kL1Bases; ++i) {
+    const int bi = b0 + i;
+    ana_rows(bi, S.in_s, S.lo_s, S.hi_s);
     if (staged) {
-      const bool ok2 = mbar_wait(&bar[1 + s], par);
+      const bool ok2 = mbar_wait(&S.bar[1], i & 1);   // each refill completes one phase
       if (__syncthreads_or(!ok2)) {
         if (threadIdx.x == 0) {
           atomicExch(err, 1);
-          (void)mbar_drain(&bar[1 + s], par);
-          if (NSET == 2 && i + 1 < NB) (void)mbar_drain(&bar[1 + (s ^ 1)], (uint32_t)(((i + 1) >> 1) & 1));
+          (void)mbar_drain(&S.bar[1], i & 1);
         }
         return;
       }
     } else {
       __syncthreads();
     }
-    if (THREADS == 512)
-      ana_cols2(lo_s, hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta, set_a(s),
-                set_t(s));
-    else
-      ana_cols(lo_s, hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta, set_a(s),
-               set_t(s));
-    __syncthreads();   // lo/hi and stage set s consumed before the next basis
-    // NSET = 1: the single set is free now: refill it for basis i + 1 (its rows run meanwhile).
-    if (NSET == 1 && staged && i + 1 < NB)
-      stage_epilogue_t(tm, coef, thr, plane(bi + 1), prow(bi + 1), n, hm, oy0, ox0, set_a(0), set_t(0), &bar[1]);
-  }
-}
-
-// Persistent form of the tiled analysis levels: 2 CTAs per SM loop over the units
-// (tile, basis, map) of a level, tile fastest. A unit's input rows are copied while
-// the previous unit's columns are filtered, and its staged A and gamma W rows
-// (double-buffered) while the whole previous unit runs, so the copy latency that the
-// one-unit-per-CTA form exposes once per CTA is hidden behind compute.
-constexpr int kAnaPFloats = kAnaPre + 4 * kStage;
-static size_t pers_analysis_smem() { return (size_t)kAnaPFloats * sizeof(float) + 32; }
-
-__global__ void __launch_bounds__(256, 2) k_ana_pers(const float* __restrict__ in, size_t in_map, size_t in_basis, int m,
-                                                     int n, int last, float* __restrict__ coef,
-                                                     float* __restrict__ thr, float* __restrict__ approx_out,
-                                                     int mode, float scale, float gamma, float delta, int* err,
-                                                     int nmaps, const __grid_constant__ SaraTma tm) {
-  extern __shared__ __align__(128) float4 smp[];
-  pdl_wait();
-  float* in_s = reinterpret_cast<float*>(smp);
-  float* lo_s = in_s + kA2In;
-  float* hi_s = lo_s + kRSmax * kPlo;
-  float* st = in_s + kAnaPre;                                        // set s: A at st + 2 s kStage, gamma W after it
-  uint64_t* bar = reinterpret_cast<uint64_t*>(st + 4 * kStage);     // [0] input rows, [1 + s] stage set s
-  const int hm = m >> 1, tilesx = hm / kTO, tiles = tilesx * tilesx;
-  const int units = tiles * kDb * nmaps;
-  const bool staged = mode == SARA_DUAL;
-  if (threadIdx.x == 0)
-    for (int q = 0; q < 3; ++q) mbar_init(&bar[q], 1);
-  __syncthreads();
-  int issued_in = 0, issued_st[2] = {0, 0};
-  auto decode = [&](int u, int& bi, int& map, int& oy0, int& ox0) {
-    const int t = u % tiles, r = u / tiles;
-    bi = r % kDb;
-    map = r / kDb;
-    oy0 = (t / tilesx) * kTO;
-    ox0 = (t % tilesx) * kTO;
-  };
-  auto issue = [&](int u, int s) {
-    int bi, map, oy0, ox0;
-    decode(u, bi, map, oy0, ox0);
-    const size_t in_off = (size_t)map * in_map + (size_t)bi * in_basis;
-    ana_issue_input_t(tm, (int)(in_off / (size_t)m), in + in_off, m, oy0, ox0, 2 * kTO + 2 * (bi + 1) - 2, in_s,
-                      &bar[0]);
-    ++issued_in;
-    if (staged) {
-      stage_epilogue_t(tm, coef, thr, ((size_t)map * kBases + bi + 1) * (size_t)n * n, (map * kBases + bi + 1) * n, n,
-                       hm, oy0, ox0, st + 2 * s * kStage, st + (2 * s + 1) * kStage, &bar[1 + s]);
-      ++issued_st[s];
-    }
-  };
-  auto abort_all = [&]() {
-    if (threadIdx.x == 0) {
-      atomicExch(err, 1);
-      if (issued_in) (void)mbar_drain(&bar[0], (issued_in - 1) & 1);
-      for (int q = 0; q < 2; ++q)
-        if (issued_st[q]) (void)mbar_drain(&bar[1 + q], (issued_st[q] - 1) & 1);
-    }
-  };
-  int u = blockIdx.x;
-  if (u < units) issue(u, 0);
-  for (int i = 0; u < units; ++i, u += gridDim.x) {
-    const int s = i & 1;
-    int bi, map, oy0, ox0;
-    decode(u, bi, map, oy0, ox0);
-    const bool ok = mbar_wait(&bar[0], i & 1);
-    if (__syncthreads_or(!ok)) {
-      abort_all();
-      return;
-    }
-    ana_rows(bi, in_s, lo_s, hi_s);
-    // The input tile is consumed and every thread is past the previous unit's columns,
-    // so the input buffer and stage set s ^ 1 can be refilled for the next unit.
-    __syncthreads();
-    if (u + (int)gridDim.x < units) issue(u + gridDim.x, s ^ 1);
-    if (staged) {
-      const bool ok2 = mbar_wait(&bar[1 + s], (i >> 1) & 1);
-      if (__syncthreads_or(!ok2)) {
-        abort_all();
-        return;
-      }
-    }
-    ana_cols(lo_s, hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta,
-             st + 2 * s * kStage, st + (2 * s + 1) * kStage);
-    __syncthreads();   // lo/hi consumed before the next unit's rows
+    ana_cols(S.lo_s, S.hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta, S.st_a,
+             S.st_t);
+    __syncthreads();   // lo/hi and the stage set consumed before the next basis
+    if (staged && i + 1 < kL1Bases) stage(bi + 1);
   }
 }
 
@@ -827,70 +663,56 @@ __device__ __forceinline__ float4 syn2_row(const u64 acc[8], int rr) {
   return make_float4(v[0], v[1], v[2], v[3]);
 }
 
-static size_t syn2_smem(int sets) { return (size_t)(sets * kC2Set + 2 * kLoSize) * sizeof(float) + 16; }
+static size_t syn2_smem() { return (size_t)(kC2Set + 2 * kLoSize) * sizeof(float) + 16; }
 
 // After a bounded wait gave up somewhere in the CTA: raise the flag (when given),
 // give the copies still in flight a bounded chance to land, and let the caller return.
-__device__ __forceinline__ void syn2_abort(uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1, int* err) {
+__device__ __forceinline__ void syn2_abort(uint64_t* bar, uint32_t parity, int* err) {
   if (threadIdx.x == 0) {
     if (err) atomicExch(err, 1);
-    (void)mbar_drain(b0, p0);
-    if (b1) (void)mbar_drain(b1, p1);
+    (void)mbar_drain(bar, parity);
   }
   __syncthreads();
 }
 
-// Finest level (m = n >= 64): the eight bases plus the Dirac part summed in registers -> Psi A.
-// NBUF = 2: two staging sets, basis b+1 copied while basis b is filtered (3 CTAs per SM).
-// NBUF = 1: one staging set, refilled with basis b+1 as soon as the y-pass of basis b
-// has read it, so the copy overlaps the x-pass (4 CTAs per SM hide the rest).
-template <int NBUF>
-__global__ void __launch_bounds__(256, NBUF == 1 ? 4 : 3)
+// Finest level: the eight bases plus the Dirac part summed in registers -> Psi A. One staging set,
+// refilled with basis b+1 as soon as the y-pass of basis b has read it, so the copy overlaps the
+// x-pass (4 CTAs per SM hide the rest; two sets at 3 CTAs per SM and a persistent form whose
+// staging runs on across tiles were slower: 78 and 80 us at 1024^2 against 72).
+__global__ void __launch_bounds__(256, 4)
     k_syn2_fine(const float* __restrict__ coef, const float* __restrict__ approx_in, int coarsest, int n,
                 float* __restrict__ out, int* err, const __grid_constant__ SaraTma tm) {
   extern __shared__ __align__(128) float4 sm2[];
   pdl_wait();
-  float* const s4 = reinterpret_cast<float*>(sm2);   // staging set(s): basis b in set b % NBUF
-  float* loT = s4 + NBUF * kC2Set;
+  float* const s4 = reinterpret_cast<float*>(sm2);
+  float* loT = s4 + kC2Set;
   float* hiT = loT + kLoSize;
   uint64_t* bar = reinterpret_cast<uint64_t*>(hiT + kLoSize);
   const int map = blockIdx.z, tilesx = n / kT2;
   const int oy0 = (blockIdx.x / tilesx) * kT2, ox0 = (blockIdx.x % tilesx) * kT2;
   const int hm = n >> 1;
   const float* cmap = coef + (size_t)map * kBases * n * n;
-  auto cbp = [&](int bi) { return cmap + (size_t)(bi + 1) * n * n; };
-  auto apxp = [&](int bi) {
-    return coarsest ? (const float*)nullptr : approx_in + ((size_t)map * kDb + bi) * (size_t)hm * hm;
-  };
-  auto set = [&](int bi) { return s4 + (bi % NBUF) * kC2Set; };
   auto issue = [&](int bi) {
-    syn2_issue_t(tm, (map * kBases + bi + 1) * n, (map * kDb + bi) * hm, bi, cbp(bi), apxp(bi), n, hm, oy0, ox0, set(bi),
-                 &bar[bi % NBUF]);
+    syn2_issue_t(tm, (map * kBases + bi + 1) * n, (map * kDb + bi) * hm, bi, cmap + (size_t)(bi + 1) * n * n,
+                 coarsest ? nullptr : approx_in + ((size_t)map * kDb + bi) * (size_t)hm * hm, n, hm, oy0, ox0, s4, bar);
   };
-  // Barrier of basis bi and the parity of its phase (each barrier completes once per use).
-  auto bar_of = [&](int bi) { return &bar[bi % NBUF]; };
-  auto par_of = [&](int bi) { return (uint32_t)((bi / NBUF) & 1); };
-  if (threadIdx.x == 0)
-    for (int q = 0; q < NBUF; ++q) mbar_init(&bar[q], 1);
+  if (threadIdx.x == 0) mbar_init(bar, 1);
   __syncthreads();
   issue(0);
   u64 acc[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) acc[q] = 0ull;
   for (int bi = 0; bi < kDb; ++bi) {
-    // NBUF = 2: set (bi+1)&1 last fed the y-pass of basis bi-1, which ended at a barrier.
-    if (NBUF == 2 && bi + 1 < kDb) issue(bi + 1);
-    const bool ok = mbar_wait(bar_of(bi), par_of(bi));
+    const bool ok = mbar_wait(bar, bi & 1);
     // Also orders the previous x-pass' reads of loT/hiT before this y-pass writes them.
     if (__syncthreads_or(!ok)) {
-      const bool next = NBUF == 2 && bi + 1 < kDb;
-      syn2_abort(bar_of(bi), par_of(bi), next ? bar_of(bi + 1) : nullptr, next ? par_of(bi + 1) : 0u, err);
+      syn2_abort(bar, bi & 1, err);
       return;
     }
-    syn2_ypass_dispatch(bi, set(bi), loT, hiT);
+    syn2_ypass_dispatch(bi, s4, loT, hiT);
     __syncthreads();
-    // NBUF = 1: the set is free once every y-pass read of it has passed the barrier above.
-    if (NBUF == 1 && bi + 1 < kDb) issue(bi + 1);
+    // The set is free once every y-pass read of it has passed the barrier above.
+    if (bi + 1 < kDb) issue(bi + 1);
     syn2_xpass_dispatch(bi, loT, hiT, acc);
   }
   const int rq = threadIdx.x & 15, cg = threadIdx.x >> 4;
@@ -902,67 +724,6 @@ __global__ void __launch_bounds__(256, NBUF == 1 ? 4 : 3)
     const float4 s = syn2_row(acc, rr);
     *reinterpret_cast<float4*>(out + (size_t)map * n * n + o) =
         make_float4((d.x + s.x) * k3, (d.y + s.y) * k3, (d.z + s.z) * k3, (d.w + s.w) * k3);
-  }
-}
-
-// Persistent form of the finest level: the CTAs (4 per SM) loop over the (tile, map) units,
-// and the single staging set runs on across units: the copies of the next unit's first
-// basis go out right after the y-pass of the current unit's last basis, so neither a
-// CTA's start nor the end of a unit exposes a copy's latency, and no wave runs part-full.
-__global__ void __launch_bounds__(256, 4)
-    k_syn2_fine_pers(const float* __restrict__ coef, const float* __restrict__ approx_in, int coarsest, int n,
-                     float* __restrict__ out, int* err, int nmaps, const __grid_constant__ SaraTma tm) {
-  extern __shared__ __align__(128) float4 sm2[];
-  pdl_wait();
-  float* const s4 = reinterpret_cast<float*>(sm2);
-  float* loT = s4 + kC2Set;
-  float* hiT = loT + kLoSize;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(hiT + kLoSize);
-  const int tilesx = n / kT2, units = tilesx * tilesx * nmaps;
-  const int hm = n >> 1;
-  auto issue = [&](int unit, int bi) {
-    const int map = unit / (tilesx * tilesx), t = unit % (tilesx * tilesx);
-    const int oy0 = (t / tilesx) * kT2, ox0 = (t % tilesx) * kT2;
-    const float* cb = coef + ((size_t)map * kBases + bi + 1) * (size_t)n * n;
-    const float* apx = coarsest ? nullptr : approx_in + ((size_t)map * kDb + bi) * (size_t)hm * hm;
-    syn2_issue_t(tm, (map * kBases + bi + 1) * n, (map * kDb + bi) * hm, bi, cb, apx, n, hm, oy0, ox0, s4, bar);
-  };
-  if (threadIdx.x == 0) mbar_init(bar, 1);
-  __syncthreads();
-  uint32_t phase = 0;            // uses of the barrier so far (each copy set completes one phase)
-  int unit = blockIdx.x;
-  if (unit < units) issue(unit, 0);
-  for (; unit < units; unit += gridDim.x) {
-    const int map = unit / (tilesx * tilesx), t = unit % (tilesx * tilesx);
-    const int oy0 = (t / tilesx) * kT2, ox0 = (t % tilesx) * kT2;
-    u64 acc[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = 0ull;
-    for (int bi = 0; bi < kDb; ++bi, ++phase) {
-      const bool ok = mbar_wait(bar, phase & 1);
-      // Also orders the previous x-pass' reads of loT/hiT before this y-pass writes them.
-      if (__syncthreads_or(!ok)) {
-        syn2_abort(bar, phase & 1, nullptr, 0u, err);
-        return;
-      }
-      syn2_ypass_dispatch(bi, s4, loT, hiT);
-      __syncthreads();
-      // The staging set is free once every y-pass read of it has passed the barrier above.
-      if (bi + 1 < kDb) issue(unit, bi + 1);
-      else if (unit + (int)gridDim.x < units) issue(unit + gridDim.x, 0);
-      syn2_xpass_dispatch(bi, loT, hiT, acc);
-    }
-    const int rq = threadIdx.x & 15, cg = threadIdx.x >> 4;
-    const float k3 = 1.0f / 3.0f;
-    const float* cmap = coef + (size_t)map * kBases * n * n;
-#pragma unroll
-    for (int rr = 0; rr < 4; ++rr) {
-      const size_t o = (size_t)(oy0 + 4 * rq + rr) * n + ox0 + 4 * cg;
-      const float4 d = *reinterpret_cast<const float4*>(cmap + o);
-      const float4 sv = syn2_row(acc, rr);
-      *reinterpret_cast<float4*>(out + (size_t)map * n * n + o) =
-          make_float4((d.x + sv.x) * k3, (d.y + sv.y) * k3, (d.z + sv.z) * k3, (d.w + sv.w) * k3);
-    }
   }
 }
 
@@ -987,7 +748,7 @@ __global__ void __launch_bounds__(256, 3) k_syn2_lv(const float* __restrict__ co
   syn2_issue_t(tm, (map * kBases + bi + 1) * n, (map * kDb + bi) * hm, bi, cb, apx, n, hm, oy0, ox0, s4, bar);
   const bool ok = mbar_wait(bar, 0);
   if (__syncthreads_or(!ok)) {
-    syn2_abort(bar, 0, nullptr, 0, err);
+    syn2_abort(bar, 0, err);
     return;
   }
   syn2_ypass_dispatch(bi, s4, loT, hiT);
@@ -1400,7 +1161,7 @@ __global__ void __cluster_dims__(NS, 1, 1) __launch_bounds__(256, 4)
     const bool ok = mbar_wait(bar, i & 1);
     if (__syncthreads_or(!ok)) {   // the whole cluster's tile is left unwritten; its barriers are still met
       if (threadIdx.x == 0) failed = 1;
-      syn2_abort(bar, i & 1, nullptr, 0u, err);
+      syn2_abort(bar, i & 1, err);
       break;
     }
     const int bi = b_of[i];
@@ -1501,33 +1262,15 @@ cudaError_t configure_kernels() {
     e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
   }
-  e = cudaFuncSetAttribute((const void*)k_syn2_fine<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)syn2_smem(2));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute((const void*)k_syn2_fine<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)syn2_smem(1));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute((const void*)k_syn2_lv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)syn2_smem(1));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute((const void*)k_syn2_fine_pers, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)syn2_smem(1));
-  if (e != cudaSuccess) return e;
-  for (const void* f : {(const void*)k_syn2_fine<2>, (const void*)k_syn2_fine<1>, (const void*)k_syn2_lv,
-                        (const void*)k_syn2_fine_pers}) {
-    e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-  }
-  for (const void* f : {(const void*)k_ana_l1m<8, 256>, (const void*)k_ana_l1m<4, 256>,
-                        (const void*)k_ana_l1m<4, 512>, (const void*)k_ana_l1m<4, 256, 1>}) {
-    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)multi_analysis_smem());
+  for (const void* f : {(const void*)k_syn2_fine, (const void*)k_syn2_lv}) {
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)syn2_smem());
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
   }
-  e = cudaFuncSetAttribute((const void*)k_ana_pers, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)pers_analysis_smem());
+  e = cudaFuncSetAttribute((const void*)k_ana_l1m, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)multi_analysis_smem());
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute((const void*)k_ana_pers, cudaFuncAttributePreferredSharedMemoryCarveout,
+  e = cudaFuncSetAttribute((const void*)k_ana_l1m, cudaFuncAttributePreferredSharedMemoryCarveout,
                            cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
   for (const void* f : {(const void*)k_ana_small<false>, (const void*)k_ana_small<true>}) {
@@ -1535,13 +1278,19 @@ cudaError_t configure_kernels() {
     if (e != cudaSuccess) return e;
   }
   for (const void* f : {(const void*)k_syn2_split<8>, (const void*)k_syn2_split<4>}) {
-    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)syn2_smem(1));
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)syn2_smem());
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
   }
   return configure_nufft_kernels();
 }
+
+// (Tile, map) units of the first analysis level from which its tiles serve four bases per CTA; with
+// fewer, one basis per CTA keeps more of the chip busy. us, one basis / four: 256^2 (64 units) 14.8 /
+// 21, 512^2 (256) 28 / 34, 1024^2 (1024) 87 / 80, 2048^2 (4096) 317 / 283;
+// a batch whose 512^2 class has 512 units 415 / 411 per iteration.
+constexpr int kSharedTiles = 512;
 
 cudaError_t sara_analysis(Handle* h, const float* X, float* coef, float* thr, int mode, float scale, float gamma,
                           float delta, cudaEvent_t fine_done) {
@@ -1558,55 +1307,22 @@ cudaError_t sara_analysis(Handle* h, const float* X, float* coef, float* thr, in
   for (int l = 1; l < lt; ++l) {
     const int m = n >> (l - 1), hm = m / 2;
     const dim3 grid((hm / kTO) * (hm / kTO), kDb, nmaps);
-    if (l == 1 && h->tune[PS_TUNE_ANALYSIS] >= 2) {
-      const int choice = h->tune[PS_TUNE_ANALYSIS], nb = choice == 2 ? 8 : 4;
-      const dim3 gm((hm / kTO) * (hm / kTO), kDb / nb, nmaps);
-      const SaraTma tm = analysis_maps(X, n, nmaps, coef, thr, n, nmaps, mode);
-      if (choice == 2)
-        k_ana_l1m<8, 256><<<gm, 256, multi_analysis_smem(), h->stream>>>(X, n, l == L, coef, thr, buf[0], mode,
-                                                                         scale, gamma, delta, h->dev_flags, tm);
-      else if (choice == 3)
-        k_ana_l1m<4, 256><<<gm, 256, multi_analysis_smem(), h->stream>>>(X, n, l == L, coef, thr, buf[0], mode,
-                                                                         scale, gamma, delta, h->dev_flags, tm);
-      else if (choice == 4)
-        k_ana_l1m<4, 512><<<gm, 512, multi_analysis_smem(), h->stream>>>(X, n, l == L, coef, thr, buf[0], mode,
-                                                                         scale, gamma, delta, h->dev_flags, tm);
-      else
-        k_ana_l1m<4, 256, 1><<<gm, 256, multi_analysis_smem(1), h->stream>>>(X, n, l == L, coef, thr, buf[0], mode,
-                                                                            scale, gamma, delta, h->dev_flags, tm);
-      if (fine_done) {
-        const cudaError_t e = cudaEventRecord(fine_done, h->stream);
-        if (e != cudaSuccess) return e;
-      }
-    } else if (h->tune[PS_TUNE_ANALYSIS] == 1) {
-      const int units = (int)(grid.x * grid.y * grid.z);
-      const int ctas = std::min(units, 2 * std::max(1, h->num_sms));
-      const float* in = l == 1 ? X : buf[(l - 2) & 1];
-      const size_t in_map = l == 1 ? (size_t)n * n : (size_t)kDb * m * m, in_basis = l == 1 ? 0 : (size_t)m * m;
-      const SaraTma tm = analysis_maps(in, m, l == 1 ? nmaps : kDb * nmaps, coef, thr, n, nmaps, mode);
-      if (l == 1)
-        k_ana_pers<<<ctas, 256, pers_analysis_smem(), h->stream>>>(in, in_map, in_basis, m, n, l == L, coef, thr,
-                                                                   buf[(l - 1) & 1], mode, scale, gamma, delta,
-                                                                   h->dev_flags, nmaps, tm);
-      else
-        launch_after(true, k_ana_pers, ctas, 256, pers_analysis_smem(), h->stream, in, in_map, in_basis, m, n, l == L, coef, thr,
-                     buf[(l - 1) & 1], mode, scale, gamma, delta, h->dev_flags, nmaps, tm);
-      if (l == 1 && fine_done) {
-        const cudaError_t e = cudaEventRecord(fine_done, h->stream);
-        if (e != cudaSuccess) return e;
-      }
-    } else if (l == 1) {
-      const SaraTma tm = analysis_maps(X, n, nmaps, coef, thr, n, nmaps, mode);
-      k_ana_l1<<<grid, 256, fast_analysis_smem(), h->stream>>>(X, n, l == L, coef, thr, buf[(l - 1) & 1], mode, scale,
-                                                              gamma, delta, h->dev_flags, tm);
-      if (fine_done) {
-        const cudaError_t e = cudaEventRecord(fine_done, h->stream);
-        if (e != cudaSuccess) return e;
-      }
-    } else {
-      const SaraTma tm = analysis_maps(buf[(l - 2) & 1], m, kDb * nmaps, coef, thr, n, nmaps, mode);
+    const SaraTma tm = analysis_maps(l == 1 ? X : buf[(l - 2) & 1], m, l == 1 ? nmaps : kDb * nmaps, coef, thr, n, nmaps,
+                                     mode);
+    if (l > 1) {
       launch_after(true, k_ana_lv, grid, 256, fast_analysis_smem(), h->stream, buf[(l - 2) & 1], m, n, l == L, coef, thr,
                    buf[(l - 1) & 1], mode, scale, gamma, delta, h->dev_flags, tm);
+      continue;
+    }
+    if ((int)(grid.x * grid.z) >= kSharedTiles)
+      k_ana_l1m<<<dim3(grid.x, kDb / kL1Bases, nmaps), 256, multi_analysis_smem(), h->stream>>>(
+          X, n, l == L, coef, thr, buf[0], mode, scale, gamma, delta, h->dev_flags, tm);
+    else
+      k_ana_l1<<<grid, 256, fast_analysis_smem(), h->stream>>>(X, n, l == L, coef, thr, buf[0], mode, scale, gamma, delta,
+                                                              h->dev_flags, tm);
+    if (fine_done) {
+      const cudaError_t e = cudaEventRecord(fine_done, h->stream);
+      if (e != cudaSuccess) return e;
     }
   }
   if (lt <= L) {
@@ -1630,11 +1346,9 @@ cudaError_t sara_analysis(Handle* h, const float* X, float* coef, float* thr, in
 }
 
 // Psi A on `stream` with `approx` as the per-level approximation scratch
-// (2 x 32 x (n/2)^2 floats); `err` (may be null) receives the bounded-wait flag;
-// `variant` is the PS_TUNE_SYNTHESIS choice of the finest level.
+// (2 x 32 x (n/2)^2 floats); `err` (may be null) receives the bounded-wait flag.
 static cudaError_t synthesis_levels(cudaStream_t stream, int n, int L, const float* coef, float* out, float* approx0,
-                                    float* approx1, int nmaps, int* err, int variant,
-                                    cudaEvent_t fine_start = nullptr) {
+                                    float* approx1, int nmaps, int* err, cudaEvent_t fine_start = nullptr) {
   float* buf[2] = {approx0, approx1};
   if (n <= kSmall) {
     if (fine_start) {
@@ -1657,7 +1371,7 @@ static cudaError_t synthesis_levels(cudaStream_t stream, int n, int L, const flo
     const float* ain = (l == L) ? nullptr : buf[l & 1];
     const SaraTma tm = synthesis_maps(coef, ain, m, n, nmaps);
     if (l > 1) {
-      launch_after(true, k_syn2_lv, dim3(tiles, nmaps, kDb), 256, syn2_smem(1), stream, coef, ain, l == L, m, n,
+      launch_after(true, k_syn2_lv, dim3(tiles, nmaps, kDb), 256, syn2_smem(), stream, coef, ain, l == L, m, n,
                    buf[(l - 1) & 1], err, tm);
       continue;
     }
@@ -1667,19 +1381,11 @@ static cudaError_t synthesis_levels(cudaStream_t stream, int n, int L, const flo
     }
     const int units = tiles * nmaps;
     if (units <= kSplit8Units)
-      launch_after(true, k_syn2_split<8>, dim3(8 * tiles, 1, nmaps), 256, syn2_smem(1), stream, coef, ain, l == L, n, out, err, tm);
+      launch_after(true, k_syn2_split<8>, dim3(8 * tiles, 1, nmaps), 256, syn2_smem(), stream, coef, ain, l == L, n, out, err, tm);
     else if (units <= kSplit4Units)
-      launch_after(true, k_syn2_split<4>, dim3(4 * tiles, 1, nmaps), 256, syn2_smem(1), stream, coef, ain, l == L, n, out, err, tm);
-    else if (variant == 2) {
-      int dev = 0, sms = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      launch_after(true, k_syn2_fine_pers, std::min(units, 4 * std::max(1, sms)), 256, syn2_smem(1), stream, coef, ain, l == L, n,
-                   out, err, nmaps, tm);
-    } else if (variant == 1)
-      launch_after(true, k_syn2_fine<1>, dim3(tiles, 1, nmaps), 256, syn2_smem(1), stream, coef, ain, l == L, n, out, err, tm);
+      launch_after(true, k_syn2_split<4>, dim3(4 * tiles, 1, nmaps), 256, syn2_smem(), stream, coef, ain, l == L, n, out, err, tm);
     else
-      launch_after(true, k_syn2_fine<2>, dim3(tiles, 1, nmaps), 256, syn2_smem(2), stream, coef, ain, l == L, n, out, err, tm);
+      launch_after(true, k_syn2_fine, dim3(tiles, 1, nmaps), 256, syn2_smem(), stream, coef, ain, l == L, n, out, err, tm);
   }
   return cudaGetLastError();
 }
@@ -1696,9 +1402,7 @@ int sara_launches(int n, int L) {
 }
 
 cudaError_t sara_synthesis(Handle* h, const float* coef, float* out, cudaEvent_t fine_start) {
-  return synthesis_levels(h->stream, h->n, h->L, coef, out, h->approx, h->approx2, h->nmaps, h->dev_flags,
-                          h->tune[PS_TUNE_SYNTHESIS],
-                          fine_start);
+  return synthesis_levels(h->stream, h->n, h->L, coef, out, h->approx, h->approx2, h->nmaps, h->dev_flags, fine_start);
 }
 
 // ---------------------------------------------------------------------------
@@ -1787,8 +1491,7 @@ extern "C" ps_status ps_apply_psi_static(const float* A, float* S, int32_t n, in
   }
   e = cudaMemsetAsync(flag, 0, sizeof(int), (cudaStream_t)cuda_stream);
   if (e == cudaSuccess)
-    e = synthesis_levels((cudaStream_t)cuda_stream, n, levels, A, S, scratch, scratch + kStaticScratchFloats / 2, 4, flag,
-                         0);
+    e = synthesis_levels((cudaStream_t)cuda_stream, n, levels, A, S, scratch, scratch + kStaticScratchFloats / 2, 4, flag);
   if (e != cudaSuccess) {
     set_global_error(std::string("apply_psi_static: launch: ") + cudaGetErrorString(e));
     return PS_ECUDA;

@@ -63,3 +63,35 @@ def test_dual_update_and_reweight_match_oracle(n, levels):
     # The weights of the state that was read: gamma delta / (delta + |coefficient|).
     coef = wav.psi_adjoint(got["S"].astype(np.float64), levels)
     assert rel_err(T, 0.02 * 0.01 / (0.01 + np.abs(coef))) <= 1e-5
+
+
+def test_dual_update_of_shared_tiles_and_its_bounded_wait():
+    """1024^2: the first analysis level with its input tiles shared by four bases. One iteration without
+    data from a random state, A of one map against clamp(A + rho1 Psi^dagger (2 S' - S), +-gamma W); then
+    a launch whose waits give up at once is reported and the handle goes on."""
+    n, levels = 1024, 2
+    rng = np.random.default_rng(41)
+    st = {k: (0.05 * rng.normal(size=s)).astype(np.float32)
+          for k, s in (("S", (4, n, n)), ("Z", (2, n, n)), ("A", (4, 9, n, n)), ("C", (4, n, n)), ("D", (2, n, n)))}
+    with PolarizedSARA(n, levels, tau=0.3, rho1=0.8, rho2=1.0, rho3=0.9) as s:
+        s.set_measurements(np.zeros((0, 2)), np.zeros((0, 4), np.complex64), None, np.zeros(1, np.int64), np.zeros(0))
+        s.set_sara_weights(None, 0.06)
+        s.set_state(st)
+        s.pd_iterate(1)
+        got = s.get_state()
+        try:
+            B.ps_debug_set_wait_polls(0)
+            s.pd_iterate(1)
+            with pytest.raises(B.PolsaraError) as e:
+                s.synchronize()
+            assert e.value.status == B.PS_ETIMEOUT
+        finally:
+            B.ps_debug_set_wait_polls(-1)
+        s.set_state(st)
+        s.pd_iterate(1)
+        again = s.get_state()
+    X = 2 * got["S"][2:3].astype(np.float64) - st["S"][2:3]
+    want = np.clip(st["A"][2:3] + 0.8 * wav.psi_adjoint(X, levels), -0.06, 0.06)
+    assert rel_err(got["A"][2:3], want) <= 2e-5
+    for k in ("S", "A", "C"):
+        assert np.array_equal(got[k], again[k]), k
