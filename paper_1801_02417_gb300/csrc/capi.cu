@@ -1047,17 +1047,11 @@ ps_status ps_get_state(ps_handle* h, const ps_state_view* v) {
   if (v->C && (st = copy_out(h, h->C, v->C, 4 * N * sizeof(float), dp)) != PS_OK) return st;
   if (v->D && (st = copy_out(h, h->D, v->D, 2 * N * sizeof(float), dp)) != PS_OK) return st;
   if (v->B && h->M > 0) {
-    float2* tmp = nullptr;
-    CK(h, dalloc(h, &tmp, 4 * (size_t)h->M));
-    cudaError_t e = cudaMemcpyAsync(h->vtmp, h->R, 4 * (size_t)h->M * sizeof(float2), cudaMemcpyDeviceToDevice, h->stream);
-    if (e == cudaSuccess) e = ps::scale_vis(h, h->vtmp);
-    if (e == cudaSuccess) e = ps::scatter_vis(h, h->vtmp, tmp);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(v->B, tmp, 4 * (size_t)h->M * sizeof(float2),
-                          dp ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    dfree(h, tmp, 4 * (size_t)h->M);
-    CK(h, e);
+    float2* dst = dp ? reinterpret_cast<float2*>(v->B) : h->vtmp;
+    CK(h, ps::read_dual(h, dst));
+    if (!dp)
+      CK(h, cudaMemcpyAsync(v->B, dst, 4 * (size_t)h->M * sizeof(float2), cudaMemcpyDeviceToHost, h->stream));
+    CK(h, cudaStreamSynchronize(h->stream));
   }
   return PS_OK;
 }
@@ -1213,18 +1207,9 @@ ps_status ps_apply_phi(ps_handle* h, const float* S, float* Y, int32_t device_pt
     X = h->tmp4;
   }
   CK(h, ps::nufft_forward_grid(h, X, false));
-  CK(h, ps::nufft_degrid(h, ps::DEG_APPLY, h->vtmp));
-  if (device_ptrs) {
-    CK(h, ps::scatter_vis(h, h->vtmp, (float2*)Y));
-    return PS_OK;
-  }
-  float2* tmp = nullptr;
-  CK(h, dalloc(h, &tmp, V));
-  cudaError_t e = ps::scatter_vis(h, h->vtmp, tmp);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(Y, tmp, V * sizeof(float2), cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  dfree(h, tmp, V);
-  CK(h, e);
+  float2* out = device_ptrs ? reinterpret_cast<float2*>(Y) : h->vtmp;
+  CK(h, ps::nufft_degrid(h, ps::DEG_APPLY, out, false, h->perm));
+  if (!device_ptrs) return copy_out(h, out, Y, V * sizeof(float2), 0);
   return PS_OK;
 }
 
@@ -1237,19 +1222,13 @@ ps_status ps_apply_phi_adjoint(ps_handle* h, const float* Yin, float* S, int32_t
   float* out = device_ptrs ? S : h->tmp4;
   if (h->M == 0) {
     CK(h, cudaMemsetAsync(out, 0, N4 * sizeof(float), h->stream));
-  } else if (device_ptrs) {
-    CK(h, ps::gather_vis(h, (const float2*)Yin, h->vtmp));
   } else {
-    float2* tmp = nullptr;
-    CK(h, dalloc(h, &tmp, V));
-    cudaError_t e = cudaMemcpyAsync(tmp, Yin, V * sizeof(float2), cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess) e = ps::gather_vis(h, tmp, h->vtmp);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    dfree(h, tmp, V);
-    CK(h, e);
-  }
-  if (h->M > 0) {
-    CK(h, ps::nufft_grid(h, h->vtmp, 0, false));
+    const float2* in = reinterpret_cast<const float2*>(Yin);
+    if (!device_ptrs) {
+      CK(h, cudaMemcpyAsync(h->vtmp, Yin, V * sizeof(float2), cudaMemcpyHostToDevice, h->stream));
+      in = h->vtmp;
+    }
+    CK(h, ps::nufft_grid(h, in, 0, false, h->perm));
     CK(h, ps::nufft_adjoint_image(h, out));
   }
   if (!device_ptrs) return copy_out(h, h->tmp4, S, N4 * sizeof(float), 0);

@@ -146,9 +146,11 @@ cudaError_t upload_es_polys(cudaStream_t stream);
 // NUFFT pieces (nufft.cu).
 // X (4 planes) -> G; clear_acc: the gridding accumulator too, for the nufft_grid(.., cleared) that follows.
 cudaError_t nufft_forward_grid(Handle* h, const float* X, bool clear_acc);
-// G -> visibilities; DEG_DUAL also steps the l2-ball factors c_b, unless keep_cb.
-cudaError_t nufft_degrid(Handle* h, int mode, float2* out, bool keep_cb = false);
-cudaError_t nufft_grid(Handle* h, const float2* in, int use_block_scale, bool cleared);  // visibilities -> Acc
+// G -> visibilities; DEG_DUAL also steps the l2-ball factors c_b, unless keep_cb. perm: DEG_APPLY writes
+// the caller's row order (stored order without).
+cudaError_t nufft_degrid(Handle* h, int mode, float2* out, bool keep_cb = false, const int32_t* perm = nullptr);
+// Visibilities -> Acc; `in` in stored order, or in the caller's (perm).
+cudaError_t nufft_grid(Handle* h, const float2* in, int use_block_scale, bool cleared, const int32_t* perm = nullptr);
 cudaError_t tv_dual(Handle* h);      // Algorithm 3 steps 5-6 on Xb -> A (TV layout)
 cudaError_t tv_adjoint(Handle* h);   // Psi A = grad^T A_tv (+ A_l1) -> PsiA
 __host__ __device__ inline bool tv_mode(int m) { return m >= PS_TV && m <= PS_L1TV_NC; }
@@ -178,7 +180,6 @@ cudaError_t scale_copy(Handle* h, const float* x, float* y, size_t len, double s
 cudaError_t lanczos_update(Handle* h, float* w, const float* v, const float* u, size_t len, double alpha,
                            double beta);                                    // w -= alpha v + beta u
 cudaError_t gather_vis(Handle* h, const float2* user, float2* sorted);
-cudaError_t scatter_vis(Handle* h, const float2* sorted, float2* user);
-cudaError_t scale_vis(Handle* h, float2* v);   // v = c_b v per block (state readout)
+cudaError_t read_dual(Handle* h, float2* user);   // c_b R in the caller's row order (state readout)
 
 }  // namespace ps

@@ -304,9 +304,9 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
 }
 
 // Second half of a degridding row m: from the interpolated packed spectra sp (at +u) and sn
-// (at -u) to the row's visibilities (or residuals); returns its term of the per-block sums
-// and its block (blk, left alone by DEG_APPLY).
-__device__ __forceinline__ float degrid_finish(int m, float w, float4 sp, float4 sn, int mode, float2* __restrict__ R,
+// (at -u) to the row's visibilities (row mo of out) or residuals; returns its term of the
+// per-block sums and its block (blk, left alone by DEG_APPLY).
+__device__ __forceinline__ float degrid_finish(int m, int mo, float w, float4 sp, float4 sn, int mode, float2* __restrict__ R,
                                                const float2* __restrict__ Yv, const float* cb,
                                                float inv_rho2, const uint16_t* __restrict__ vblk,
                                                float2* __restrict__ out, int& blk) {
@@ -319,8 +319,8 @@ __device__ __forceinline__ float degrid_finish(int m, float w, float4 sp, float4
   float4 v23 = make_float4(w * sn.z, -w * sn.w, w * (FIr - FQr), w * (FIi - FQi));  // LR = conj G2(-u), LL
   if (mode == DEG_APPLY) {
     float4* o4 = reinterpret_cast<float4*>(out);
-    o4[2 * (size_t)m] = v01;
-    o4[2 * (size_t)m + 1] = v23;
+    o4[2 * (size_t)mo] = v01;
+    o4[2 * (size_t)mo + 1] = v23;
     return 0.f;
   }
   blk = vblk[m];
@@ -396,13 +396,14 @@ __device__ __forceinline__ void degrid_row(int m, bool active, const GridItem& i
                                            int mode, float2* __restrict__ R, const float2* __restrict__ Yv,
                                            const float* cb, float inv_rho2,
                                            const uint16_t* __restrict__ vblk, bool shared, double* sums,
-                                           float2* __restrict__ out) {
+                                           const int32_t* __restrict__ perm, float2* __restrict__ out) {
   constexpr int TS = kGridTile;
   constexpr int SS = TS + W - 1;
   int blk = -1;
   float e2 = 0.f;
   if (active) {
     degrid_prefetch(m, mode, R, Yv);
+    const int mo = mode == DEG_APPLY && perm ? perm[m] : m;
     float fx, fy, w;
     int cx, cy;
     unpack_rec(rec[m], fx, fy, w, cx, cy);
@@ -438,7 +439,7 @@ __device__ __forceinline__ void degrid_row(int m, bool active, const GridItem& i
     f2unpack(sp1, sp.z, sp.w);
     f2unpack(sn0, sn.x, sn.y);
     f2unpack(sn1, sn.z, sn.w);
-    e2 = degrid_finish(m, w, sp, sn, mode, R, Yv, cb, inv_rho2, vblk, out, blk);
+    e2 = degrid_finish(m, mo, w, sp, sn, mode, R, Yv, cb, inv_rho2, vblk, out, blk);
   }
   if (mode != DEG_APPLY) block_add(blk, e2, shared, sums);
 }
@@ -467,12 +468,12 @@ struct BallStep {
 
 // Registers are capped for 6 CTAs per SM at W = 7 (40 of 67: more rows in flight per SM, 100
 // against 111 us at 1024^2 / 2,000,000 rows; other widths would spill and run without a cap).
-template <int W>
+template <int W, bool APPLY>
 __global__ void __launch_bounds__(256, W == 7 ? 6 : 0) k_degrid(
     const GridItem* __restrict__ items, const float4* __restrict__ rec, const float4* __restrict__ G, int Wd,
-    int off, int full, int K, float beta, int mode, float2* __restrict__ R, const float2* __restrict__ Yv,
+    int off, int full, int K, float beta, int step_mode, float2* __restrict__ R, const float2* __restrict__ Yv,
     const float* cb, float inv_rho2, const uint16_t* __restrict__ vblk, int nblocks, BallStep ball,
-    float2* __restrict__ out) {
+    const int32_t* __restrict__ perm, float2* __restrict__ out) {
   constexpr int TS = kGridTile;
   constexpr int SS = TS + W - 1;
   constexpr int hw = W / 2;
@@ -481,6 +482,7 @@ __global__ void __launch_bounds__(256, W == 7 ? 6 : 0) k_degrid(
   float4* Gn = smd + SS * SS;       // -u cells: mirrored rows/cols -(ty*TS + TS-1) - hw + [0, SS)
   double* bsum = reinterpret_cast<double*>(smd + 2 * SS * SS);
   __shared__ int s_last;
+  const int mode = APPLY ? (int)DEG_APPLY : step_mode;
   pdl_wait();
   const GridItem it = items[blockIdx.x];
   const bool reduce = (mode != DEG_APPLY);
@@ -512,7 +514,7 @@ __global__ void __launch_bounds__(256, W == 7 ? 6 : 0) k_degrid(
   for (int base = it.vstart; base < it.vend; base += blockDim.x) {
     const int m = base + threadIdx.x;
     degrid_row<W>(m, m < it.vend, it, rec, Gp, Gn, off, full, K, beta, mode, R, Yv, cb, inv_rho2, vblk, !private_bins,
-                  sums, out);
+                  sums, perm, out);
   }
   if (reduce) {
     __syncthreads();
@@ -585,9 +587,10 @@ struct GridWarp {
   static constexpr int kRow = 32 * (8 + 8 * NT + XP);            // floats of the row buffer
   static constexpr int kFloats = kRow + 2 * ((W * SP + 3) / 4 * 4);   // + two staged blocks
 };
-template <int W>
+template <int W, bool PERM>
 __global__ void __launch_bounds__(32 * kGridWarps) k_grid(
     int M, int rows, const uint16_t* __restrict__ vblk, const float4* __restrict__ rec, const float2* __restrict__ vin,
+    const int32_t* __restrict__ perm,
     const float* __restrict__ cb, int use_scale, int Wd, int off, int full, int K, float beta,
     float* __restrict__ Acc) {
   using T = GridWarp<W>;
@@ -612,11 +615,14 @@ __global__ void __launch_bounds__(32 * kGridWarps) k_grid(
     for (int q = 0; q < NT; ++q) d[t][q][0] = d[t][q][1] = d[t][q][2] = d[t][q][3] = 0.f;
   float4 r, b0, b1;
   int blk = 0, buf = 0, cell = -1;   // cell: the accumulated block's (grid row << 12 | column), -1: none
+  // vin in stored order, or (PERM) in the caller's; the index of a row is read one step ahead of it.
+  int next = PERM ? perm[min(m0 + lane, m1 - 1)] : 0;
   auto fetch = [&](int m) {
-    const size_t i = min(m + lane, m1 - 1);
+    const size_t i = min(m + lane, m1 - 1), v = PERM ? next : i;
     r = rec[i];
-    b0 = v4[2 * i];
-    b1 = v4[2 * i + 1];
+    b0 = v4[2 * v];
+    b1 = v4[2 * v + 1];
+    if (PERM) next = perm[min(m + 32 + lane, m1 - 1)];
     if (use_scale) blk = vblk[i];
   };
   // The block to the accumulator: d[t][q][i] is cell (jy = 8 q + 2 tig + (i & 1), jx = 2 t + (i >> 1)),
@@ -894,10 +900,11 @@ cudaError_t configure_nufft_kernels() {
   if ((e = set_smem((const void*)k_fwd_cols, sm1)) != cudaSuccess) return e;
   if ((e = set_smem((const void*)k_adj_rows, sm1)) != cudaSuccess) return e;
   // Per-block FP64 accumulators of the degridding kernels (up to 2047 blocks).
-  const void* degrids[] = {(const void*)k_degrid<5>, (const void*)k_degrid<7>, (const void*)k_degrid<9>};
+  const void* degrids[] = {(const void*)k_degrid<5, false>, (const void*)k_degrid<7, false>, (const void*)k_degrid<9, false>,
+                           (const void*)k_degrid<5, true>,  (const void*)k_degrid<7, true>,  (const void*)k_degrid<9, true>};
   const size_t degrid_smem[] = {degrid_smem_tiles<5>(), degrid_smem_tiles<7>(), degrid_smem_tiles<9>()};
-  for (int i = 0; i < 3; ++i)
-    if ((e = set_smem(degrids[i], degrid_smem[i] + 2048 * sizeof(double))) != cudaSuccess) return e;
+  for (int i = 0; i < 6; ++i)
+    if ((e = set_smem(degrids[i], degrid_smem[i % 3] + 2048 * sizeof(double))) != cudaSuccess) return e;
   return set_smem((const void*)k_adj_cols, sm2);
 }
 
@@ -911,27 +918,27 @@ cudaError_t nufft_forward_grid(Handle* h, const float* X, bool clear_acc) {
 }
 
 template <int W>
-static cudaError_t launch_degrid(Handle* h, int mode, float2* out, bool keep_cb) {
+static cudaError_t launch_degrid(Handle* h, int mode, float2* out, bool keep_cb, const int32_t* perm) {
   const GridGeom& g = h->g;
   const int nbins = h->nblocks <= kWarpBins ? kWarpBins * 8 : h->nblocks;   // 8 warps of 256 threads
   const size_t sm = degrid_smem_tiles<W>() + (size_t)nbins * sizeof(double);
   const BallStep ball{h->block_sum, h->block_done, h->block_norm_sq, mode == DEG_DUAL && !keep_cb ? h->cb : nullptr,
                       h->eps,       h->rho2,       h->cfg.literal_ball};
-  return launch_after(h->early, k_degrid<W>, h->nitems, 256, sm, h->stream, h->items, h->rec, h->G, g.Wd, g.off, g.full, g.K,
-                      g.beta, mode, h->R, h->Y, h->cb, (float)(1.0 / h->rho2), h->vblk, h->nblocks, ball, out);
+  return launch_after(h->early, mode == DEG_APPLY ? k_degrid<W, true> : k_degrid<W, false>, h->nitems, 256, sm, h->stream, h->items, h->rec, h->G, g.Wd, g.off, g.full, g.K,
+                      g.beta, mode, h->R, h->Y, h->cb, (float)(1.0 / h->rho2), h->vblk, h->nblocks, ball, perm, out);
 }
 
-cudaError_t nufft_degrid(Handle* h, int mode, float2* out, bool keep_cb) {
+cudaError_t nufft_degrid(Handle* h, int mode, float2* out, bool keep_cb, const int32_t* perm) {
   if (h->M == 0) return cudaSuccess;
   switch (h->g.W) {
-    case 5: return launch_degrid<5>(h, mode, out, keep_cb);
-    case 9: return launch_degrid<9>(h, mode, out, keep_cb);
-    default: return launch_degrid<7>(h, mode, out, keep_cb);
+    case 5: return launch_degrid<5>(h, mode, out, keep_cb, perm);
+    case 9: return launch_degrid<9>(h, mode, out, keep_cb, perm);
+    default: return launch_degrid<7>(h, mode, out, keep_cb, perm);
   }
 }
 
 template <int W>
-static cudaError_t launch_grid(Handle* h, const float2* in, int use_scale) {
+static cudaError_t launch_grid(Handle* h, const float2* in, int use_scale, const int32_t* perm) {
   const GridGeom& g = h->g;
   // Rows per warp: 64 where that leaves two warps for every scheduler of the chip and a cell
   // holds enough rows that cutting its run at a warp's end costs more than parallelism gives,
@@ -948,12 +955,12 @@ static cudaError_t launch_grid(Handle* h, const float2* in, int use_scale) {
   const int warps = 8 * std::max(1, h->num_sms);
   const int rows = h->M <= 12 * warps ? 8 : (h->M >= 64 * warps && h->M / std::max(1, h->ncells) >= 16 ? 64 : 32);
   const int ctas = (int)(((int64_t)h->M + (int64_t)rows * kGridWarps - 1) / ((int64_t)rows * kGridWarps));
-  return launch_after(h->early, k_grid<W>, ctas, 32 * kGridWarps, kGridWarps * GridWarp<W>::kFloats * sizeof(float), h->stream, h->M,
-                      rows, h->vblk, h->rec, in, h->cb, use_scale, g.Wd, g.off, g.full, g.K, g.beta,
+  return launch_after(h->early, perm ? k_grid<W, true> : k_grid<W, false>, ctas, 32 * kGridWarps, kGridWarps * GridWarp<W>::kFloats * sizeof(float),
+                      h->stream, h->M, rows, h->vblk, h->rec, in, perm, h->cb, use_scale, g.Wd, g.off, g.full, g.K, g.beta,
                       reinterpret_cast<float*>(h->Acc));
 }
 
-cudaError_t nufft_grid(Handle* h, const float2* in, int use_scale, bool cleared) {
+cudaError_t nufft_grid(Handle* h, const float2* in, int use_scale, bool cleared, const int32_t* perm) {
   const GridGeom& g = h->g;
   if (!cleared) {
     const cudaError_t e = cudaMemsetAsync(h->Acc, 0, (size_t)g.Wd * g.Wd * 2 * sizeof(float4), h->stream);
@@ -961,9 +968,9 @@ cudaError_t nufft_grid(Handle* h, const float2* in, int use_scale, bool cleared)
   }
   if (h->M == 0) return cudaSuccess;
   switch (g.W) {
-    case 5: return launch_grid<5>(h, in, use_scale);
-    case 9: return launch_grid<9>(h, in, use_scale);
-    default: return launch_grid<7>(h, in, use_scale);
+    case 5: return launch_grid<5>(h, in, use_scale, perm);
+    case 9: return launch_grid<9>(h, in, use_scale, perm);
+    default: return launch_grid<7>(h, in, use_scale, perm);
   }
 }
 

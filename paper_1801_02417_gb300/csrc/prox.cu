@@ -474,15 +474,6 @@ __global__ void k_gather_vis(int M, const int32_t* __restrict__ perm, const floa
   sorted[2 * (size_t)m + 1] = user[2 * u + 1];
 }
 
-__global__ void k_scatter_vis(int M, const int32_t* __restrict__ perm, const float4* __restrict__ sorted,
-                              float4* __restrict__ user) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= M) return;
-  const size_t u = (size_t)perm[m];
-  user[2 * u] = sorted[2 * (size_t)m];
-  user[2 * u + 1] = sorted[2 * (size_t)m + 1];
-}
-
 cudaError_t gather_vis(Handle* h, const float2* user, float2* sorted) {
   if (h->M == 0) return cudaSuccess;
   k_gather_vis<<<(h->M + 255) / 256, 256, 0, h->stream>>>(h->M, h->perm, reinterpret_cast<const float4*>(user),
@@ -490,26 +481,22 @@ cudaError_t gather_vis(Handle* h, const float2* user, float2* sorted) {
   return cudaGetLastError();
 }
 
-cudaError_t scatter_vis(Handle* h, const float2* sorted, float2* user) {
-  if (h->M == 0) return cudaSuccess;
-  k_scatter_vis<<<(h->M + 255) / 256, 256, 0, h->stream>>>(h->M, h->perm, reinterpret_cast<const float4*>(sorted),
-                                                           reinterpret_cast<float4*>(user));
-  return cudaGetLastError();
-}
-
-__global__ void k_scale_vis(int M, const uint16_t* __restrict__ vblk, const float* __restrict__ cb,
-                            float4* __restrict__ v) {
+__global__ void k_read_dual(int M, const int32_t* __restrict__ perm, const uint16_t* __restrict__ vblk,
+                            const float* __restrict__ cb, const float4* __restrict__ R, float4* __restrict__ user) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= M) return;
   const float s = cb[vblk[m]];
-  const float4 a = v[2 * (size_t)m], b = v[2 * (size_t)m + 1];
-  v[2 * (size_t)m] = make_float4(a.x * s, a.y * s, a.z * s, a.w * s);
-  v[2 * (size_t)m + 1] = make_float4(b.x * s, b.y * s, b.z * s, b.w * s);
+  const size_t u = (size_t)perm[m];
+  const float4 a = R[2 * (size_t)m], b = R[2 * (size_t)m + 1];
+  user[2 * u] = make_float4(a.x * s, a.y * s, a.z * s, a.w * s);
+  user[2 * u + 1] = make_float4(b.x * s, b.y * s, b.z * s, b.w * s);
 }
 
-cudaError_t scale_vis(Handle* h, float2* v) {
+cudaError_t read_dual(Handle* h, float2* user) {
   if (h->M == 0) return cudaSuccess;
-  k_scale_vis<<<(h->M + 255) / 256, 256, 0, h->stream>>>(h->M, h->vblk, h->cb, reinterpret_cast<float4*>(v));
+  k_read_dual<<<(h->M + 255) / 256, 256, 0, h->stream>>>(h->M, h->perm, h->vblk, h->cb,
+                                                         reinterpret_cast<const float4*>(h->R),
+                                                         reinterpret_cast<float4*>(user));
   return cudaGetLastError();
 }
 
