@@ -492,10 +492,7 @@ ps_status ps_create(const ps_config* cfg, void* cuda_stream, ps_handle** out) {
   h->approx2 = h->approx + 8 * N;
   if (reset_state(h) != PS_OK) return bail(PS_ECUDA);
   // Thresholds default to 1 (gamma = 1, W = 1).
-  std::vector<float> ones(36 * N, 1.0f);
-  if (cudaMemcpyAsync(h->T, ones.data(), ones.size() * sizeof(float), cudaMemcpyHostToDevice, h->stream) !=
-          cudaSuccess ||
-      cudaStreamSynchronize(h->stream) != cudaSuccess) {
+  if (ps::fill(h, h->T, 36 * N, 1.0f) != cudaSuccess || cudaStreamSynchronize(h->stream) != cudaSuccess) {
     h->err = "ps_create: initialisation failed";
     return bail(PS_ECUDA);
   }
@@ -572,13 +569,6 @@ static ps_status default_gamma(Handle* h);
 static __global__ void k_fill(float* p, int n, float v) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) p[i] = v;
-}
-
-// p[0 .. len) = v, grid-stride, float4 stores (p 16-byte aligned, len a multiple of 4).
-static __global__ void k_fill4(float4* p, size_t len4, float v) {
-  const float4 q = make_float4(v, v, v, v);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < len4; i += (size_t)gridDim.x * blockDim.x)
-    p[i] = q;
 }
 
 extern "C" {
@@ -789,8 +779,9 @@ ps_status ps_set_measurements(ps_handle* h, int64_t M64, const double* uv, const
     }
   std::vector<float> corrh(h->n);
   // phihat is even: q and n - q (offsets -d and +d from the centre) share a value.
+  const std::vector<double> ft = ps::es_fourier(2.0 * M_PI / g.K, h->n / 2 + 1, g.W);
   for (int q = 0; q <= h->n / 2; ++q) {
-    corrh[q] = (float)(1.0 / ps::es_fourier(2.0 * M_PI * (q - h->n / 2) / g.K, g.W, g.beta));
+    corrh[q] = (float)(1.0 / ft[h->n / 2 - q]);
     if (q > 0 && q < h->n / 2) corrh[h->n - q] = corrh[q];
   }
   CK(h, cudaMemsetAsync(h->block_done, 0, sizeof(int), h->stream));
@@ -849,55 +840,49 @@ static double tridiag_max_eig(const std::vector<double>& a, const std::vector<do
 // ||phi||_sp^2, the step-size bound of Section 4.3.3, as the largest eigenvalue of
 // phi^dagger phi by Lanczos iterations (three-term recurrence, FP32 vectors, FP64
 // coefficients; the largest Ritz value rises monotonically to it). Stops when that
-// value changes by <= 1e-9 relative, or the Krylov space is invariant. Scratch: tmp4,
-// Xb and Adj (all cleared by the caller's reset of the state).
+// value changes by <= 1e-9 relative, or the Krylov space is invariant. The coefficients stay on
+// the device, where the next step takes them; the host reads them every kLanczosAhead
+// steps and ignores the ones past the stop. Scratch: tmp4,
+// Xb and Adj (all cleared by the caller's reset of the state) and the partials of `red`.
 static ps_status opnorm_lanczos(Handle* h) {
+  constexpr int kLanczosAhead = 4, kMost = 300;
   h->opnorm_sq = 0.0;
   if (h->M == 0) return PS_OK;
   const size_t N4 = 4 * (size_t)h->N;
-  std::vector<float> x(N4);
-  uint64_t s = 0x9E3779B97F4A7C15ull;
-  double nrm = 0.0;
-  for (size_t i = 0; i < N4; ++i) {
-    s = s * 6364136223846793005ull + 1442695040888963407ull;
-    x[i] = (float)((double)(s >> 11) / 9007199254740992.0 - 0.5);
-    nrm += (double)x[i] * x[i];
-  }
-  const float inv = (float)(1.0 / std::sqrt(nrm));
-  for (auto& v : x) v *= inv;
   float *v = h->tmp4, *u = h->Xb, *w = h->Adj;   // current, previous and new Lanczos vectors
-  // On the handle's (non-blocking) stream, so the iterations below are ordered after the copy.
-  CK(h, cudaMemcpyAsync(v, x.data(), N4 * sizeof(float), cudaMemcpyHostToDevice, h->stream));
+  // alpha_j at coef[2 j], beta_j^2 (|w|^2 after the step) at coef[2 j + 1].
+  double* coef = h->red + (size_t)h->red_cap - 1020;
+  CK(h, ps::lanczos_start(h, v, N4, coef));
   CK(h, cudaMemsetAsync(u, 0, N4 * sizeof(float), h->stream));
-  double* dres = h->red + (size_t)h->red_cap - 1020;
   std::vector<double> al, be;
-  double theta = 0.0, beta = 0.0;
-  for (int j = 0; j < 300; ++j) {
-    CK(h, ps::nufft_forward_grid(h, v, true));
-    CK(h, ps::nufft_degrid(h, ps::DEG_APPLY, h->vtmp));
-    CK(h, ps::nufft_grid(h, h->vtmp, 0, true));
-    CK(h, ps::nufft_adjoint_image(h, w));
-    CK(h, ps::reduce_dot(h, w, v, N4, dres));
-    CK(h, cudaMemcpyAsync(h->red_host, dres, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  double theta = 0.0;
+  bool done = false;
+  for (int j0 = 0; j0 < kMost && !done; j0 += kLanczosAhead) {
+    for (int j = j0; j < j0 + kLanczosAhead; ++j) {
+      double* c = coef + 2 * (j % kLanczosAhead);
+      const double* last = j > 0 ? coef + 2 * ((j - 1) % kLanczosAhead) + 1 : nullptr;
+      CK(h, ps::nufft_forward_grid(h, v, true));
+      CK(h, ps::nufft_degrid(h, ps::DEG_APPLY, h->vtmp));
+      CK(h, ps::nufft_grid(h, h->vtmp, 0, true));
+      CK(h, ps::nufft_adjoint_image(h, w));
+      CK(h, ps::reduce_dot(h, w, v, N4, c));
+      CK(h, ps::lanczos_update(h, w, v, u, N4, c, last));
+      CK(h, ps::lanczos_scale(h, w, u, N4, c + 1));   // the new vector over the previous one
+      std::swap(u, v);
+    }
+    CK(h, cudaMemcpyAsync(h->red_host, coef, 2 * kLanczosAhead * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
-    const double alpha = h->red_host[0];
-    if (!std::isfinite(alpha)) return fail(h, PS_ENONFINITE, "Lanczos: non-finite phi^dagger phi x");
-    CK(h, ps::lanczos_update(h, w, v, u, N4, alpha, beta));
-    CK(h, ps::reduce_dot(h, w, w, N4, dres + 1));
-    CK(h, cudaMemcpyAsync(h->red_host + 1, dres + 1, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
-    const double beta_new = std::sqrt(h->red_host[1]);
-    if (!std::isfinite(beta_new)) return fail(h, PS_ENONFINITE, "Lanczos: non-finite phi^dagger phi x");
-    al.push_back(alpha);
-    const double theta_new = tridiag_max_eig(al, be);
-    if (!(theta_new > 0)) return fail(h, PS_ENONFINITE, "Lanczos: zero phi^dagger phi x");
-    const bool done = (j >= 4 && std::fabs(theta_new - theta) <= 1e-9 * theta_new) || beta_new <= 1e-12 * theta_new;
-    theta = theta_new;
-    if (done) break;
-    be.push_back(beta_new);
-    CK(h, ps::scale_copy(h, w, u, N4, 1.0 / beta_new));   // the new vector over the previous one
-    std::swap(u, v);
-    beta = beta_new;
+    for (int j = j0; j < j0 + kLanczosAhead && !done; ++j) {
+      const double alpha = h->red_host[2 * (j - j0)], beta = std::sqrt(h->red_host[2 * (j - j0) + 1]);
+      if (!std::isfinite(alpha) || !std::isfinite(beta))
+        return fail(h, PS_ENONFINITE, "Lanczos: non-finite phi^dagger phi x");
+      al.push_back(alpha);
+      const double theta_new = tridiag_max_eig(al, be);
+      if (!(theta_new > 0)) return fail(h, PS_ENONFINITE, "Lanczos: zero phi^dagger phi x");
+      done = (j >= 4 && std::fabs(theta_new - theta) <= 1e-9 * theta_new) || beta <= 1e-12 * theta_new;
+      theta = theta_new;
+      be.push_back(beta);
+    }
   }
   h->opnorm_sq = theta;
   return PS_OK;
@@ -926,8 +911,7 @@ static ps_status default_gamma(Handle* h) {
   }
   h->gamma = h->gamma_default;
   const size_t len = 36 * (size_t)h->N;
-  k_fill4<<<1024, 256, 0, h->stream>>>(reinterpret_cast<float4*>(h->T), len / 4, (float)h->gamma);
-  CK(h, cudaGetLastError());
+  CK(h, ps::fill(h, h->T, len, (float)h->gamma));
   return PS_OK;
 }
 
@@ -943,8 +927,7 @@ ps_status ps_set_sara_weights(ps_handle* h, const float* W, double gamma, int32_
     if (st != PS_OK) return st;
     CK(h, ps::scale_copy(h, h->T, h->T, len, gamma));
   } else {   // W = 1: gamma W filled on the device
-    k_fill4<<<1024, 256, 0, h->stream>>>(reinterpret_cast<float4*>(h->T), len / 4, (float)gamma);
-    CK(h, cudaGetLastError());
+    CK(h, ps::fill(h, h->T, len, (float)gamma));
   }
   h->gamma = gamma;
   if (!device_ptrs) CK(h, cudaStreamSynchronize(h->stream));

@@ -114,21 +114,29 @@ static void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w
   }
 }
 
-double es_fourier(double xi, int W, double beta) {
+std::vector<double> es_fourier(double step, int count, int W) {
   // phihat(xi) = int_{-W/2}^{W/2} phi(t) cos(xi t) dt; phi is even. The quadrature rule is
-  // built once (thread-safe static initialisation: handles may be prepared concurrently).
+  // built once (thread-safe static initialisation: handles may be prepared concurrently). The
+  // frequencies are equally spaced, so each node's cosines come by rotation.
   struct Rule {
     std::vector<double> x, w;
     Rule() { gauss_legendre(400, x, w); }
   };
   static const Rule rule;
   const double half = 0.5 * W;
-  double s = 0.0;
-  for (size_t i = 0; i < rule.x.size(); ++i) {
-    const double t = half * rule.x[i];
-    s += rule.w[i] * es_kernel(t, W, beta) * std::cos(xi * t);
+  std::vector<double> out(count, 0.0);
+  for (size_t i = 0; i < rule.x.size() / 2; ++i) {   // the nodes come in pairs +-x
+    const double t = half * rule.x[i], a = 2.0 * half * rule.w[i] * es_kernel(t, W, es_beta(W));
+    const double dc = std::cos(step * t), ds = std::sin(step * t);
+    double c = 1.0, s = 0.0;
+    for (int k = 0; k < count; ++k) {
+      out[k] += a * c;
+      const double n = c * dc - s * ds;
+      s = s * dc + c * ds;
+      c = n;
+    }
   }
-  return s * half;
+  return out;
 }
 
 // Tap j (offset f + W/2 - j, |f| <= 1/2) as a polynomial of degree 2 kEsTerms - 1 in f: the

@@ -136,7 +136,7 @@ void set_global_error(const std::string& msg);
 void daubechies_filters(double h[kDb][kMaxTaps]);          // db1..db8 scaling filters
 double es_beta(int W);
 double es_kernel(double t, int W, double beta);            // ES kernel value at offset t (cells)
-double es_fourier(double xi, int W, double beta);          // its Fourier transform at xi
+std::vector<double> es_fourier(double step, int count, int W);   // its Fourier transform at k step, k < count (beta = es_beta)
 void es_poly(int W, int j, double c[2 * kEsTerms]);        // tap j as a polynomial of its offset: E then O coefficients
 
 // Kernel launchers (return cudaGetLastError()).
@@ -177,8 +177,11 @@ cudaError_t violation_count(Handle* h, const float* S, const double* rms_sum, do
 cudaError_t weighted_l1(Handle* h, const float* coef, const float* thr, double* out);
 cudaError_t max_abs(Handle* h, const float* c, size_t len, double* dev_out);
 cudaError_t scale_copy(Handle* h, const float* x, float* y, size_t len, double s);
-cudaError_t lanczos_update(Handle* h, float* w, const float* v, const float* u, size_t len, double alpha,
-                           double beta);                                    // w -= alpha v + beta u
+cudaError_t fill(Handle* h, float* p, size_t len, float v);      // len a multiple of 4
+cudaError_t lanczos_start(Handle* h, float* v, size_t len, double* scratch);   // the normalised start vector
+cudaError_t lanczos_update(Handle* h, float* w, const float* v, const float* u, size_t len, double* coef,
+                           const double* last);                             // w -= alpha v + beta u; |w|^2
+cudaError_t lanczos_scale(Handle* h, const float* w, float* u, size_t len, const double* norm_sq);   // u = w / |w|
 cudaError_t gather_vis(Handle* h, const float2* user, float2* sorted);
 cudaError_t read_dual(Handle* h, float2* user);   // c_b R in the caller's row order (state readout)
 

@@ -450,17 +450,81 @@ cudaError_t scale_copy(Handle* h, const float* x, float* y, size_t len, double s
   return cudaGetLastError();
 }
 
-// Lanczos three-term recurrence: w = w - alpha v - beta u (FP32 vectors, FP64 coefficients).
-__global__ void k_lanczos_update(float* __restrict__ w, const float* __restrict__ v, const float* __restrict__ u,
-                                 size_t len, double alpha, double beta) {
-  const float a = (float)alpha, b = (float)beta;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (size_t)gridDim.x * blockDim.x)
-    w[i] = fmaf(-b, u[i], fmaf(-a, v[i], w[i]));
+__global__ void k_fill4(float4* p, size_t len4, float v) {
+  const float4 q = make_float4(v, v, v, v);
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < len4; i += (size_t)gridDim.x * blockDim.x)
+    p[i] = q;
 }
 
-cudaError_t lanczos_update(Handle* h, float* w, const float* v, const float* u, size_t len, double alpha,
-                           double beta) {
-  k_lanczos_update<<<1024, 256, 0, h->stream>>>(w, v, u, len, alpha, beta);
+cudaError_t fill(Handle* h, float* p, size_t len, float v) {
+  k_fill4<<<1024, 256, 0, h->stream>>>(reinterpret_cast<float4*>(p), len / 4, v);
+  return cudaGetLastError();
+}
+
+// The Lanczos start vector: sample i is the (i + 1)-th state of a 64-bit linear congruential
+// generator, its top 53 bits as a number in [-1/2, 1/2). A thread jumps to its first sample by
+// powers of the generator's affine map (square and multiply) and steps on from there.
+constexpr int kLcgRun = 16;
+__global__ void k_lanczos_start(float* __restrict__ x, size_t len) {
+  const size_t i0 = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * kLcgRun;
+  if (i0 >= len) return;
+  unsigned long long a = 6364136223846793005ull, c = 1442695040888963407ull, s = 0x9E3779B97F4A7C15ull;
+  for (unsigned long long k = i0; k; k >>= 1) {
+    if (k & 1) s = s * a + c;
+    c = c * (a + 1);
+    a = a * a;
+  }
+  for (size_t i = i0; i < i0 + kLcgRun && i < len; ++i) {
+    s = s * 6364136223846793005ull + 1442695040888963407ull;
+    x[i] = (float)((double)(s >> 11) / 9007199254740992.0 - 0.5);
+  }
+}
+
+// y = x / |.| with the squared norm from device memory (FP64).
+__global__ void k_scale_by(const float* x, float* y, size_t len,
+                           const double* __restrict__ norm_sq) {
+  const float sf = (float)(1.0 / sqrt(*norm_sq));
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (size_t)gridDim.x * blockDim.x)
+    y[i] = x[i] * sf;
+}
+
+cudaError_t lanczos_start(Handle* h, float* v, size_t len, double* scratch) {
+  const size_t runs = (len + kLcgRun - 1) / kLcgRun;
+  k_lanczos_start<<<(unsigned)((runs + 255) / 256), 256, 0, h->stream>>>(v, len);
+  const cudaError_t e = reduce_dot(h, v, v, len, scratch);
+  return e == cudaSuccess ? lanczos_scale(h, v, v, len, scratch) : e;
+}
+
+cudaError_t lanczos_scale(Handle* h, const float* w, float* u, size_t len, const double* norm_sq) {
+  k_scale_by<<<1024, 256, 0, h->stream>>>(w, u, len, norm_sq);
+  return cudaGetLastError();
+}
+
+// Lanczos three-term recurrence w = w - alpha v - beta u (FP32 vectors, FP64 coefficients from
+// device memory: coef[0] = alpha, *last = beta^2 of the step before, null for the first), and
+// coef[1] = |w|^2 of the result.
+__global__ void k_lanczos_update(float* __restrict__ w, const float* __restrict__ v, const float* __restrict__ u,
+                                 size_t len, double* coef, const double* last, double* part, int* done) {
+  __shared__ double sh[32];
+  const float a = (float)coef[0], b = last ? (float)sqrt(*last) : 0.f;
+  double s = 0.0;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (size_t)gridDim.x * blockDim.x) {
+    const float q = fmaf(-b, u[i], fmaf(-a, v[i], w[i]));
+    w[i] = q;
+    s += (double)q * (double)q;
+  }
+  s = cta_sum(s, sh);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  if (!last_cta(done)) return;
+  s = threadIdx.x < gridDim.x ? __ldcg(&part[threadIdx.x]) : 0.0;
+  s = cta_sum(s, sh);
+  if (threadIdx.x == 0) coef[1] = s;
+}
+
+cudaError_t lanczos_update(Handle* h, float* w, const float* v, const float* u, size_t len, double* coef,
+                           const double* last) {
+  k_lanczos_update<<<kRedBlocks, kRedBlocks, 0, h->stream>>>(w, v, u, len, coef, last, red_partials(h, 2),
+                                                             h->dev_flags + 1);
   return cudaGetLastError();
 }
 
