@@ -293,13 +293,62 @@ __device__ __forceinline__ bool last_cta(int* done) {   // after the partials ar
   return last;
 }
 
-__global__ void k_dot(const float* __restrict__ a, const float* __restrict__ b, size_t len, double* part, int* done,
+// Sums of products for FP64 reductions: the FP64 pipe takes a conversion per operand and an FMA per
+// product, at a sixty-fourth of the FP32 rate (the weighted norm of 1024^2, 38 M products: 345 us, 54 with
+// this). Eight products at a time are therefore summed in FP32 pairs without loss: the product
+// with its rounding error (fma), the sum with its (Knuth's two-sum); the errors add up in the low
+// part, so a group carries about 46 bits, and goes into the FP64 sum as two numbers.
+struct PairSum {
+  float h = 0.f, l = 0.f;
+  __device__ __forceinline__ void add(float a, float b) {
+    const float p = a * b, e = fmaf(a, b, -p);
+    const float s = h + p, q = s - h;
+    l += ((h - (s - q)) + (p - q)) + e;
+    h = s;
+  }
+  __device__ __forceinline__ void add(float4 a, float4 b) {
+    add(a.x, b.x);
+    add(a.y, b.y);
+    add(a.z, b.z);
+    add(a.w, b.w);
+  }
+  __device__ __forceinline__ double take() {
+    const double r = (double)h + (double)l;
+    h = l = 0.f;
+    return r;
+  }
+};
+// Whether a thread's sum is one in which FP32 products have neither overflowed nor lost anything
+// below the smallest normal number that counts; outside (zero, tiny or huge data) it is formed again
+// in FP64.
+__device__ __forceinline__ bool pair_range(double s) { return fabs(s) >= 1e-20 && fabs(s) <= 1e30; }
+// Sum over this thread's share of len products f(a[i]) b[i] (len a multiple of 4, 16-byte aligned).
+template <typename F>
+__device__ __forceinline__ double pair_sums(const float4* __restrict__ a, const float4* __restrict__ b, size_t len, F f) {
+  const size_t n4 = len >> 2, step = (size_t)gridDim.x * blockDim.x;
+  double s = 0.0;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += 2 * step) {
+    PairSum t;
+    const bool two = i + step < n4;
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 a0 = a[i], b0 = b[i], a1 = two ? a[i + step] : z, b1 = two ? b[i + step] : z;
+    t.add(f(a0), b0);
+    t.add(f(a1), b1);
+    s += t.take();
+  }
+  if (pair_range(s)) return s;
+  s = 0.0;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += step) {
+    const float4 x = f(a[i]), y = b[i];
+    s += (double)x.x * y.x + (double)x.y * y.y + (double)x.z * y.z + (double)x.w * y.w;
+  }
+  return s;
+}
+
+__global__ void k_dot(const float4* __restrict__ a, const float4* __restrict__ b, size_t len, double* part, int* done,
                       double* out) {
   __shared__ double sh[32];
-  double s = 0.0;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (size_t)gridDim.x * blockDim.x)
-    s += (double)a[i] * (double)b[i];
-  s = cta_sum(s, sh);
+  double s = cta_sum(pair_sums(a, b, len, [](float4 v) { return v; }), sh);
   if (threadIdx.x == 0) part[blockIdx.x] = s;
   if (!last_cta(done)) return;
   s = threadIdx.x < gridDim.x ? __ldcg(&part[threadIdx.x]) : 0.0;   // at most blockDim CTAs
@@ -316,6 +365,7 @@ __global__ void k_relc_sums(const double* __restrict__ part, int nb, const int* 
   __shared__ double sh[8][8];   // [warp][column]
   const int c = threadIdx.x & 7;
   double s = 0.0;
+#pragma unroll 8
   for (int b = threadIdx.x >> 3; b < nb; b += blockDim.x >> 3) s += part[8 * (size_t)b + c];
   s += __shfl_xor_sync(0xffffffffu, s, 8);    // lanes c, c + 8, c + 16, c + 24 hold column c
   s += __shfl_xor_sync(0xffffffffu, s, 16);
@@ -343,7 +393,8 @@ static constexpr int kRedBlocks = 256;
 static double* red_partials(Handle* h, int back) { return h->red + (size_t)h->red_cap - back * kRedBlocks; }
 
 cudaError_t reduce_dot(Handle* h, const float* a, const float* b, size_t len, double* dev_out) {
-  k_dot<<<kRedBlocks, kRedBlocks, 0, h->stream>>>(a, b, len, red_partials(h, 2), h->dev_flags + 1, dev_out);
+  k_dot<<<kRedBlocks, kRedBlocks, 0, h->stream>>>(reinterpret_cast<const float4*>(a), reinterpret_cast<const float4*>(b),
+                                                  len, red_partials(h, 2), h->dev_flags + 1, dev_out);
   return cudaGetLastError();
 }
 
@@ -356,15 +407,27 @@ __global__ void k_violations(int N, const float* __restrict__ S, const double* r
   __shared__ double sh[32];
   const double q = rms_sum ? *rms_sum : 0.0;
   const double zeta = psf_peak > 0.0 ? zeta_sigma * sqrt(q / (double)N) / psf_peak : 0.0;
-  double c0 = 0.0, c1 = 0.0;
+  const float zhi = __double2float_ru(zeta), zlo = __double2float_rd(zeta);   // zeta >= 0
+  int n0 = 0, n1 = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-    const double I = S[i], Q = S[(size_t)N + i], U = S[2 * (size_t)N + i], V = S[3 * (size_t)N + i];
-    const double p = -I + sqrt(Q * Q + U * U + V * V);
-    c0 += (p > zeta) ? 1.0 : 0.0;
-    c1 += (p > 0.0) ? 1.0 : 0.0;
+    // In FP32 where its error cannot change either comparison (a few roundings of 6e-8 each of the
+    // norm and of I, taken as 1e-6 of both), else in FP64.
+    const float i32 = S[i], q32 = S[(size_t)N + i], u32 = S[2 * (size_t)N + i], v32 = S[3 * (size_t)N + i];
+    const float nr = sqrtf(fmaf(q32, q32, fmaf(u32, u32, v32 * v32))), p32 = nr - i32;
+    const float off = 1e-6f * (nr + fabsf(i32)) + 1e-18f;
+    if (p32 - off > zhi) {
+      n0 += 1;
+      n1 += 1;
+    } else if (p32 + off < zlo && (p32 - off > 0.f || p32 + off < 0.f)) {
+      n1 += p32 > 0.f;
+    } else {
+      const double I = i32, Q = q32, U = u32, V = v32;
+      const double p = -I + sqrt(Q * Q + U * U + V * V);
+      n0 += p > zeta;
+      n1 += p > 0.0;
+    }
   }
-  c0 = cta_sum(c0, sh);
-  c1 = cta_sum(c1, sh);
+  double c0 = cta_sum((double)n0, sh), c1 = cta_sum((double)n1, sh);
   if (threadIdx.x == 0) {
     part[2 * blockIdx.x] = c0;
     part[2 * blockIdx.x + 1] = c1;
@@ -389,13 +452,11 @@ cudaError_t violation_count(Handle* h, const float* S, const double* rms_sum, do
   return cudaGetLastError();
 }
 
-__global__ void k_wl1(const float* __restrict__ c, const float* __restrict__ t, size_t len, double* part, int* done,
+__global__ void k_wl1(const float4* __restrict__ c, const float4* __restrict__ t, size_t len, double* part, int* done,
                       double* out) {
   __shared__ double sh[32];
-  double s = 0.0;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (size_t)gridDim.x * blockDim.x)
-    s += (double)t[i] * fabs((double)c[i]);
-  s = cta_sum(s, sh);
+  double s = cta_sum(pair_sums(c, t, len, [](float4 v) { return make_float4(fabsf(v.x), fabsf(v.y), fabsf(v.z), fabsf(v.w)); }),
+                     sh);
   if (threadIdx.x == 0) part[blockIdx.x] = s;
   if (!last_cta(done)) return;
   s = threadIdx.x < gridDim.x ? __ldcg(&part[threadIdx.x]) : 0.0;
@@ -407,7 +468,8 @@ __global__ void k_wl1(const float* __restrict__ c, const float* __restrict__ t, 
 }
 
 cudaError_t weighted_l1(Handle* h, const float* coef, const float* thr, double* out) {
-  k_wl1<<<kRedBlocks, kRedBlocks, 0, h->stream>>>(coef, thr, (size_t)36 * h->N, red_partials(h, 3), h->dev_flags + 2, out);
+  k_wl1<<<kRedBlocks, kRedBlocks, 0, h->stream>>>(reinterpret_cast<const float4*>(coef), reinterpret_cast<const float4*>(thr),
+                                                  (size_t)36 * h->N, red_partials(h, 3), h->dev_flags + 2, out);
   return cudaGetLastError();
 }
 
@@ -503,15 +565,26 @@ cudaError_t lanczos_scale(Handle* h, const float* w, float* u, size_t len, const
 // Lanczos three-term recurrence w = w - alpha v - beta u (FP32 vectors, FP64 coefficients from
 // device memory: coef[0] = alpha, *last = beta^2 of the step before, null for the first), and
 // coef[1] = |w|^2 of the result.
-__global__ void k_lanczos_update(float* __restrict__ w, const float* __restrict__ v, const float* __restrict__ u,
+__global__ void k_lanczos_update(float4* __restrict__ w, const float4* __restrict__ v, const float4* __restrict__ u,
                                  size_t len, double* coef, const double* last, double* part, int* done) {
   __shared__ double sh[32];
   const float a = (float)coef[0], b = last ? (float)sqrt(*last) : 0.f;
   double s = 0.0;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (size_t)gridDim.x * blockDim.x) {
-    const float q = fmaf(-b, u[i], fmaf(-a, v[i], w[i]));
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < len >> 2; i += (size_t)gridDim.x * blockDim.x) {
+    const float4 x = u[i], y = v[i], z = w[i];
+    const float4 q = make_float4(fmaf(-b, x.x, fmaf(-a, y.x, z.x)), fmaf(-b, x.y, fmaf(-a, y.y, z.y)),
+                                 fmaf(-b, x.z, fmaf(-a, y.z, z.z)), fmaf(-b, x.w, fmaf(-a, y.w, z.w)));
     w[i] = q;
-    s += (double)q * (double)q;
+    PairSum t;
+    t.add(q, q);
+    s += t.take();
+  }
+  if (!pair_range(s)) {
+    s = 0.0;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < len >> 2; i += (size_t)gridDim.x * blockDim.x) {
+      const float4 q = w[i];
+      s += (double)q.x * q.x + (double)q.y * q.y + (double)q.z * q.z + (double)q.w * q.w;
+    }
   }
   s = cta_sum(s, sh);
   if (threadIdx.x == 0) part[blockIdx.x] = s;
@@ -523,8 +596,9 @@ __global__ void k_lanczos_update(float* __restrict__ w, const float* __restrict_
 
 cudaError_t lanczos_update(Handle* h, float* w, const float* v, const float* u, size_t len, double* coef,
                            const double* last) {
-  k_lanczos_update<<<kRedBlocks, kRedBlocks, 0, h->stream>>>(w, v, u, len, coef, last, red_partials(h, 2),
-                                                             h->dev_flags + 1);
+  k_lanczos_update<<<kRedBlocks, kRedBlocks, 0, h->stream>>>(
+      reinterpret_cast<float4*>(w), reinterpret_cast<const float4*>(v), reinterpret_cast<const float4*>(u), len, coef, last,
+      red_partials(h, 2), h->dev_flags + 1);
   return cudaGetLastError();
 }
 
