@@ -49,13 +49,13 @@ __device__ __forceinline__ int bitrev(int i, int logK) { return (int)(__brev((un
 // a linear (GF(2)) function of the higher bits chosen so that the eight lanes of a
 // quarter-warp hit eight different groups in every access pattern of the
 // transforms: the bit-reversed scatter (lanes differ in the top three index bits),
-// the radix-4 passes of stages (0,1) and (2,3) (lanes differ in bits 2-4, resp. 0,
-// 1 and 4), the later passes and the natural-order reads (bits 0-2). Being linear,
+// the passes from stages 0, 1 and 2 on (lanes differ in the lowest three bits that the
+// pass leaves alone), the later ones and the natural-order reads (bits 0-2). Being linear,
 // fsw(a ^ d) = fsw(a) ^ fsw(d).
 __device__ __forceinline__ int fsw(int i) {
   const int h = i >> 5;
   const int r = (h ^ (h >> 3) ^ (h >> 6)) & 7;   // bit t: XOR of index bits 5+t, 8+t, 11+t
-  return i ^ ((i >> 3) & 1) ^ (((i >> 4) & 1) * 6) ^ ((r & 1) << 1) ^ ((r & 2) << 1) ^ ((r >> 2) & 1);
+  return i ^ ((i >> 3) & 1) ^ (((i >> 4) & 1) * 6) ^ ((r & 1) << 2) ^ (r >> 1);
 }
 
 // Twiddle p of radix-2 stage t (span 2^(t+1)): tw[2^t - 1 + p] = exp(-2 pi i p / 2^(t+1));
@@ -67,53 +67,73 @@ __device__ __forceinline__ float2 twid(const float2* __restrict__ tw, int idx) {
   return w;
 }
 
-// In-place decimation-in-time FFT of K = 2^logK float4 (two complex sequences) held
-// in shared memory (swizzled by fsw) in bit-reversed order; output in natural
-// order. INV selects exp(+2 pi i jk/K) (no 1/K normalisation). Radix-2 stages s
-// and s+1 are done together by one thread on the four elements a, a+h, a+2h, a+3h
-// (h = 2^s, bits s and s+1 of a clear), so there is one shared-memory pass and one
-// barrier per two stages; an odd stage count ends with a plain radix-2 stage.
+// N radix-2 stages s .. s + N - 1 on the 2^N elements x (natural offsets j 2^s, j < 2^N) of one group in
+// registers; pos: the group's position below bit s.
+template <bool INV, int N>
+__device__ __forceinline__ void fft_group(float4 (&x)[1 << N], const float2* __restrict__ tw, int s, int pos) {
+#pragma unroll
+  for (int t = 0; t < N; ++t) {
+    // Stage s + t pairs offsets that differ in bit t; its twiddles depend on the bits below.
+#pragma unroll
+    for (int q = 0; q < (1 << t); ++q) {
+      const float2 w = twid<INV>(tw, (1 << (s + t)) - 1 + pos + (q << s));
+#pragma unroll
+      for (int k = q; k < (1 << N); k += 2 << t) {
+        const float4 u = x[k], v = cmul2(x[k + (1 << t)], w);
+        x[k] = f4add(u, v);
+        x[k + (1 << t)] = f4sub(u, v);
+      }
+    }
+  }
+}
+
+// One pass over the nbuf buffers of K elements: stages s .. s + N - 1, a group per thread and turn.
+template <bool INV, int N>
+__device__ __forceinline__ void fft_pass(float4* buf, int nbuf, const float2* __restrict__ tw, int logK, int s) {
+  int c[N];   // fsw is linear: the offset of element k is the XOR of those of its bits
+#pragma unroll
+  for (int k = 0; k < N; ++k) c[k] = fsw(1 << (s + k));
+  auto at = [&](int a, int k) {
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (k >> q & 1) a ^= c[q];
+    return a;
+  };
+  const int groups = 1 << (logK - N);
+  for (int i = threadIdx.x; i < nbuf * groups; i += blockDim.x) {
+    const int g = i & (groups - 1), pos = g & ((1 << s) - 1);
+    float4* b = buf + ((i >> (logK - N)) << logK);
+    const int a = fsw(((g >> s) << (s + N)) + pos);
+    float4 x[1 << N];
+#pragma unroll
+    for (int k = 0; k < (1 << N); ++k) x[k] = b[at(a, k)];
+    fft_group<INV, N>(x, tw, s, pos);
+#pragma unroll
+    for (int k = 0; k < (1 << N); ++k) b[at(a, k)] = x[k];
+  }
+  __syncthreads();
+}
+
+// In-place decimation-in-time FFT of nbuf sequences of K = 2^logK float4 (two complex sequences
+// each) held in shared memory (swizzled by fsw) in bit-reversed order; output in natural
+// order. INV selects exp(+2 pi i jk/K) (no 1/K normalisation). Shared-memory passes and their
+// barriers bound these kernels, so three radix-2 stages go together: a thread takes 8 elements
+// through them in registers, and the eight lanes of a quarter-warp fall into eight bank groups of
+// fsw. What three does not divide ends in a pass of two stages or one. Forward and adjoint
+// transforms (both kernels of each), radix-4 passes -> these: 117 -> 92 and 111 -> 90 us at 2048^2
+// (K = 4096), 34.5 -> 30.7 and 34.8 -> 31.0 at 1024^2, 16.4 -> 14.5 and 17.3 -> 15.8 at 512^2, equal
+// below. Passes of four stages need 140 registers a thread: 110 and 94 us at 2048^2 but 23 and 18 at 512^2.
 // Stages below s0 are taken as done (the caller wrote their output); stages from
 // s_end on are left to the caller (fft_out).
 template <bool INV>
-__device__ void fft_smem(float4* buf, const float2* __restrict__ tw, int logK, int s0 = 0, int s_end = -1) {
-  const int K = 1 << logK;
-  if (s_end < 0) s_end = logK;
+__device__ void fft_smem(float4* buf, int nbuf, const float2* __restrict__ tw, int logK, int s0, int s_end) {
   int s = s0;
-  for (; s + 1 < s_end; s += 2) {
-    const int hs = 1 << s;
-    const int c1 = fsw(hs), c2 = fsw(2 * hs);
-    for (int g = threadIdx.x; g < (K >> 2); g += blockDim.x) {
-      const int pos = g & (hs - 1);
-      const int a = fsw(((g >> s) << (s + 2)) + pos);
-      const float2 w0 = twid<INV>(tw, hs - 1 + pos);          // stage s
-      const float2 w1 = twid<INV>(tw, 2 * hs - 1 + pos);      // stage s+1, pair (a, a+2h)
-      const float2 w2 = twid<INV>(tw, 3 * hs - 1 + pos);      // stage s+1, pair (a+h, a+3h)
-      const float4 x0 = buf[a], x1 = buf[a ^ c1], x2 = buf[a ^ c2], x3 = buf[a ^ c1 ^ c2];
-      const float4 t1 = cmul2(x1, w0), t3 = cmul2(x3, w0);
-      const float4 y0 = f4add(x0, t1), y1 = f4sub(x0, t1), y2 = f4add(x2, t3), y3 = f4sub(x2, t3);
-      const float4 u2 = cmul2(y2, w1), u3 = cmul2(y3, w2);
-      buf[a] = f4add(y0, u2);
-      buf[a ^ c2] = f4sub(y0, u2);
-      buf[a ^ c1] = f4add(y1, u3);
-      buf[a ^ c1 ^ c2] = f4sub(y1, u3);
-    }
-    __syncthreads();
+  for (; s + 3 <= s_end; s += 3) fft_pass<INV, 3>(buf, nbuf, tw, logK, s);
+  if (s + 2 <= s_end) {
+    fft_pass<INV, 2>(buf, nbuf, tw, logK, s);
+    s += 2;
   }
-  if (s < s_end) {
-    const int hs = 1 << s;
-    const int c1 = fsw(hs);
-    for (int b = threadIdx.x; b < (K >> 1); b += blockDim.x) {
-      const int pos = b & (hs - 1);
-      const int i0 = fsw(((b >> s) << (s + 1)) + pos);
-      const float2 w = twid<INV>(tw, hs - 1 + pos);
-      const float4 u = buf[i0];
-      const float4 v = cmul2(buf[i0 ^ c1], w);
-      buf[i0] = f4add(u, v);
-      buf[i0 ^ c1] = f4sub(u, v);
-    }
-    __syncthreads();
-  }
+  if (s < s_end) fft_pass<INV, 1>(buf, nbuf, tw, logK, s);
 }
 
 // Input of a K-point transform whose nonzero samples fill exactly one of each pair of
@@ -128,34 +148,39 @@ __device__ __forceinline__ void scatter_stage0(float4* buf, int idx, int logK, f
   buf[fsw(r | 1)] = (idx < (1 << (logK - 1))) ? v : make_float4(-v.x, -v.y, -v.z, -v.w);
 }
 
-// First stage fft_out finishes when the passes start at s0: the last radix-4 pass, or
-// the last radix-2 stage when the stage count from s0 is odd.
+// First of the stages fft_out finishes when the passes start at s0: one or two, such that whole passes
+// of three remain; two where nothing would be left over (three cost 32.8 us for two's 30.7 in the adjoint
+// transforms at 1024^2).
 __device__ __forceinline__ int fft_tail_start(int logK, int s0) {
-  return ((logK - s0) & 1) ? logK - 1 : logK - 2;
+  const int rem = (logK - s0) % 3;
+  return logK - (rem ? rem : 2);
 }
 
 // Natural-order output k of the transform whose stages below s_last are done in buf;
-// its remaining one (s_last = logK - 1) or two (s_last = logK - 2) stages are applied
-// here for this output alone (the same arithmetic as the last pass of fft_smem), so
-// a caller that needs few outputs skips that pass, its barrier and a buffer rewrite.
+// its remaining one or two stages are applied here for this output alone (the same arithmetic as a
+// pass), so a caller that needs few outputs skips that pass, its barrier and a buffer rewrite.
+template <bool INV, int T>
+__device__ __forceinline__ float4 fft_out_t(const float4* buf, const float2* __restrict__ tw, int s, int k) {
+  const int hs = 1 << s, g = k & (hs - 1), a = fsw(g);
+  float4 x[1 << T];
+#pragma unroll
+  for (int i = 0; i < (1 << T); ++i) x[i] = buf[a ^ fsw(i << s)];
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    const float2 w = twid<INV>(tw, (hs << t) - 1 + (k & ((hs << t) - 1)));
+    const bool minus = (k >> (s + t)) & 1;
+#pragma unroll
+    for (int i = 0; i < (1 << T) >> (t + 1); ++i) {
+      const float4 v = cmul2(x[2 * i + 1], w);
+      x[i] = minus ? f4sub(x[2 * i], v) : f4add(x[2 * i], v);
+    }
+  }
+  return x[0];
+}
 template <bool INV>
 __device__ __forceinline__ float4 fft_out(const float4* buf, const float2* __restrict__ tw, int logK, int s_last,
                                           int k) {
-  const int hs = 1 << s_last;
-  const int g = k & (hs - 1);
-  if (s_last == logK - 2) {
-    const float2 w0 = twid<INV>(tw, hs - 1 + g), w1 = twid<INV>(tw, 2 * hs - 1 + g), w2 = twid<INV>(tw, 3 * hs - 1 + g);
-    const float4 x0 = buf[fsw(g)], x1 = buf[fsw(g + hs)], x2 = buf[fsw(g + 2 * hs)], x3 = buf[fsw(g + 3 * hs)];
-    const float4 t1 = cmul2(x1, w0), t3 = cmul2(x3, w0);
-    const int j = k >> s_last;
-    if (j == 0) return f4add(f4add(x0, t1), cmul2(f4add(x2, t3), w1));
-    if (j == 2) return f4sub(f4add(x0, t1), cmul2(f4add(x2, t3), w1));
-    if (j == 1) return f4add(f4sub(x0, t1), cmul2(f4sub(x2, t3), w2));
-    return f4sub(f4sub(x0, t1), cmul2(f4sub(x2, t3), w2));
-  }
-  const float2 w = twid<INV>(tw, hs - 1 + g);
-  const float4 u = buf[fsw(g)], v = cmul2(buf[fsw(g + hs)], w);
-  return k < hs ? f4add(u, v) : f4sub(u, v);
+  return logK - s_last == 1 ? fft_out_t<INV, 1>(buf, tw, s_last, k) : fft_out_t<INV, 2>(buf, tw, s_last, k);
 }
 
 __device__ __forceinline__ int gidx(int k, int off, int full, int K) {
@@ -163,9 +188,17 @@ __device__ __forceinline__ int gidx(int k, int off, int full, int K) {
 }
 
 // ---------------------------------------------------------------- forward
-__global__ void k_fwd_rows(const float* __restrict__ X, int n, int N, const float* __restrict__ corr,
-                           const float2* __restrict__ tw, int K, int logK, float4* __restrict__ T1,
-                           int Wd, int off, int full, float4* __restrict__ clear, int nclear) {
+// CTAS: resident CTAs per SM that the registers leave room for. At K = 4096 a row's 64 KB of shared memory
+// allows three, and the registers that more of them would cost are worth more (1084 us per iteration with five
+// at 2048^2, 1056 with three). Up to K = 2048 the kernel runs beside the SARA branch: five (48 registers)
+// leave that branch room, 425 us per iteration at 1024^2 where four give 431, although the transform alone
+// is slower (30.7 us for 28.7).
+template <int CTAS>
+__global__ void __launch_bounds__(256, CTAS) k_fwd_rows(const float* __restrict__ X, int n, int N,
+                                                  const float* __restrict__ corr,
+                                                  const float2* __restrict__ tw, int K, int logK,
+                                                  float4* __restrict__ T1, int Wd, int off, int full,
+                                                  float4* __restrict__ clear, int nclear) {
   extern __shared__ float4 sm[];
   pdl_wait();
   // The accumulator of the gridding that follows in the chain (none: nclear = 0).
@@ -185,15 +218,16 @@ __global__ void k_fwd_rows(const float* __restrict__ X, int n, int N, const floa
   }
   __syncthreads();
   const int st = fft_tail_start(logK, 1);
-  fft_smem<false>(buf, tw, logK, 1, st);
+  fft_smem<false>(buf, 1, tw, logK, 1, st);
   for (int gx = threadIdx.x; gx < Wd; gx += blockDim.x) {
     const int k = full ? gx : gx - off;
     T1[(size_t)p * Wd + gx] = fft_out<false>(buf, tw, logK, st, (k + K) & (K - 1));
   }
 }
 
-__global__ void k_fwd_cols(const float4* __restrict__ T1, int n, const float2* __restrict__ tw, int K,
-                           int logK, float4* __restrict__ G, int Wd, int off, int full) {
+__global__ void __launch_bounds__(512) k_fwd_cols(const float4* __restrict__ T1, int n,
+                                                  const float2* __restrict__ tw, int K, int logK,
+                                                  float4* __restrict__ G, int Wd, int off, int full) {
   extern __shared__ float4 sm[];
   pdl_wait();
   float4* buf = sm;
@@ -204,7 +238,7 @@ __global__ void k_fwd_cols(const float4* __restrict__ T1, int n, const float2* _
   }
   __syncthreads();
   const int st = fft_tail_start(logK, 1);
-  fft_smem<false>(buf, tw, logK, 1, st);
+  fft_smem<false>(buf, 1, tw, logK, 1, st);
   for (int gy = threadIdx.x; gy < Wd; gy += blockDim.x) {
     const int k = full ? gy : gy - off;
     G[(size_t)gy * Wd + gx] = fft_out<false>(buf, tw, logK, st, (k + K) & (K - 1));
@@ -746,8 +780,9 @@ __global__ void __launch_bounds__(32 * kGridWarps) k_grid(
 // Hermitian symmetrisation + inverse column FFTs for the column pair (kx, -kx).
 // H1(k) = P1(k) + i Q1(k), P1(k) = aI(k) + conj aI(-k), Q1(k) = aQ(k) + conj aQ(-k);
 // H2 likewise from aU, aV. H(-k) = conj P(k) + i conj Q(k).
-__global__ void k_adj_cols(const float4* __restrict__ Acc, int n, const float2* __restrict__ tw, int K,
-                           int logK, float4* __restrict__ T2, int Wd, int off, int full) {
+__global__ void __launch_bounds__(512) k_adj_cols(const float4* __restrict__ Acc, int n,
+                                                  const float2* __restrict__ tw, int K, int logK,
+                                                  float4* __restrict__ T2, int Wd, int off, int full) {
   extern __shared__ float4 sm[];
   pdl_wait();
   float4* bp = sm;
@@ -797,8 +832,7 @@ __global__ void k_adj_cols(const float4* __restrict__ Acc, int n, const float2* 
     }
     __syncthreads();
     st = fft_tail_start(logK, 2);
-    fft_smem<true>(bp, tw, logK, 2, st);
-    if (!self) fft_smem<true>(bm, tw, logK, 2, st);
+    fft_smem<true>(bp, self ? 1 : 2, tw, logK, 2, st);
   } else {
     for (int i = threadIdx.x; i < 2 * K; i += blockDim.x) sm[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
@@ -818,8 +852,7 @@ __global__ void k_adj_cols(const float4* __restrict__ Acc, int n, const float2* 
     }
     __syncthreads();
     st = fft_tail_start(logK, 0);
-    fft_smem<true>(bp, tw, logK, 0, st);
-    if (!self) fft_smem<true>(bm, tw, logK, 0, st);
+    fft_smem<true>(bp, self ? 1 : 2, tw, logK, 0, st);
   }
   for (int p = threadIdx.x; p < n; p += blockDim.x) {
     const int k = (p - n / 2 + K) & (K - 1);
@@ -828,9 +861,10 @@ __global__ void k_adj_cols(const float4* __restrict__ Acc, int n, const float2* 
   }
 }
 
-__global__ void k_adj_rows(const float4* __restrict__ T2, int n, int N, const float* __restrict__ corr,
-                           const float2* __restrict__ tw, int K, int logK, int Wd, int off, int full,
-                           float* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_adj_rows(const float4* __restrict__ T2, int n, int N,
+                                                  const float* __restrict__ corr,
+                                                  const float2* __restrict__ tw, int K, int logK, int Wd,
+                                                  int off, int full, float* __restrict__ out) {
   extern __shared__ float4 sm[];
   pdl_wait();
   float4* buf = sm;
@@ -862,7 +896,7 @@ __global__ void k_adj_rows(const float4* __restrict__ T2, int n, int N, const fl
     }
     __syncthreads();
     st = fft_tail_start(logK, 2);
-    fft_smem<true>(buf, tw, logK, 2, st);
+    fft_smem<true>(buf, 1, tw, logK, 2, st);
   } else {
     for (int i = threadIdx.x; i < K; i += blockDim.x) buf[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
@@ -872,7 +906,7 @@ __global__ void k_adj_rows(const float4* __restrict__ T2, int n, int N, const fl
     }
     __syncthreads();
     st = fft_tail_start(logK, 0);
-    fft_smem<true>(buf, tw, logK, 0, st);
+    fft_smem<true>(buf, 1, tw, logK, 0, st);
   }
   const float cy = 0.5f * corr[p];
   for (int q = threadIdx.x; q < n; q += blockDim.x) {
@@ -896,7 +930,8 @@ cudaError_t configure_nufft_kernels() {
   // Largest grid: n = 2048, K = 4096.
   const size_t sm1 = fft_smem_bytes(4096, 1), sm2 = fft_smem_bytes(4096, 2);
   cudaError_t e;
-  if ((e = set_smem((const void*)k_fwd_rows, sm1)) != cudaSuccess) return e;
+  if ((e = set_smem((const void*)k_fwd_rows<3>, sm1)) != cudaSuccess) return e;
+  if ((e = set_smem((const void*)k_fwd_rows<5>, sm1)) != cudaSuccess) return e;
   if ((e = set_smem((const void*)k_fwd_cols, sm1)) != cudaSuccess) return e;
   if ((e = set_smem((const void*)k_adj_rows, sm1)) != cudaSuccess) return e;
   // Per-block FP64 accumulators of the degridding kernels (up to 2047 blocks).
@@ -908,11 +943,14 @@ cudaError_t configure_nufft_kernels() {
   return set_smem((const void*)k_adj_cols, sm2);
 }
 
+// Threads of a transform's CTA: one group of 16 per thread and pass for the rows (many CTAs), two
+// threads per group for the columns (few CTAs, whose loads and outputs set the time).
 cudaError_t nufft_forward_grid(Handle* h, const float* X, bool clear_acc) {
   const GridGeom& g = h->g;
   const size_t sm1 = fft_smem_bytes(g.K, 1);
-  cudaError_t e = launch_after(h->early, k_fwd_rows, h->n, 256, sm1, h->stream, X, h->n, h->N, h->corr, h->tw, g.K, g.logK, h->T1,
-                               g.Wd, g.off, g.full, h->Acc, clear_acc ? 2 * g.Wd * g.Wd : 0);
+  cudaError_t e = launch_after(h->early, g.K > 2048 ? k_fwd_rows<3> : k_fwd_rows<5>, h->n, 256, sm1, h->stream, X,
+                               h->n, h->N, h->corr, h->tw, g.K, g.logK, h->T1, g.Wd,
+                               g.off, g.full, h->Acc, clear_acc ? 2 * g.Wd * g.Wd : 0);
   if (e != cudaSuccess) return e;
   return launch_after(h->early, k_fwd_cols, g.Wd, 512, sm1, h->stream, h->T1, h->n, h->tw, g.K, g.logK, h->G, g.Wd, g.off, g.full);
 }

@@ -94,3 +94,25 @@ def test_phi_and_adjoint_match_fp64_interpolation(kind, n, M, blocks, width):
     # The per-block norms of the same rows.
     want = [np.linalg.norm(Y[off[b]:off[b + 1]] - ref[off[b]:off[b + 1]]) for b in range(blocks)]
     assert rel_err(res, np.array(want)) <= OP_TOL
+
+
+# Transform lengths of every remainder modulo the stages that one pass takes, on the full grid and on a window
+# of it: no stage left over, one or two, and the shortest and the longest.
+@pytest.mark.parametrize("kind", ["spread", "window"])
+@pytest.mark.parametrize("n", [16, 64, 128, 256, 512, 1024, 2048])
+def test_every_transform_length_matches_fp64(kind, n):
+    M = 60
+    uv = _uv(kind, M, n)
+    rng = np.random.default_rng(n)
+    w = np.ones(M, np.float32)
+    S = rng.normal(size=(4, n, n)).astype(np.float32)
+    Y = (rng.normal(size=(M, 4)) + 1j * rng.normal(size=(M, 4))).astype(np.complex64)
+    with PolarizedSARA(n, 2) as s:
+        s.set_measurements(uv, Y, w, np.array([0, M], np.int64), np.ones(1))
+        out = np.empty((M, 4), np.complex64)
+        B.ps_apply_phi(s.h, S, out)
+        img = np.empty((4, n, n), np.float32)
+        B.ps_apply_phi_adjoint(s.h, Y, img)
+    op = Nufft64(n, uv, w, 7)
+    assert rel_err(out, op.phi(S.astype(np.float64))) <= OP_TOL
+    assert rel_err(img, op.adjoint(Y.astype(np.complex128))) <= OP_TOL
