@@ -71,6 +71,13 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
+// The same tile brought to the L2 alone.
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(reinterpret_cast<uint64_t>(map)),
+               "r"(x), "r"(y)
+               : "memory");
+}
+
 // ---- programmatic dependent launch. A kernel launched by launch_after (below) may start while the
 // kernel before it in the stream still runs; pdl_wait returns when that kernel has completed and
 // its writes are visible (at once if it already has, or the launch was an ordinary one). Every

@@ -170,11 +170,12 @@ __device__ __forceinline__ void sara_epilogue4(int mode, float4 v, size_t idx, f
 // columns (two packed pairs) of two output rows, whose 2 LF taps reach over LF + 2 input rows, so
 // it reads 18 rows of 16 bytes for db8 where one output row of all four subbands took 32. The
 // epilogue reads and writes A and gamma W as float4 (staged before the filtering).
+template <typename Ready>
 __device__ __forceinline__ void ana_cols(const float* __restrict__ lo_s, const float* __restrict__ hi_s, int bi,
                                          int map, int n, int hm, int oy0, int ox0, int last, float* __restrict__ coef,
                                          float* __restrict__ thr, float* __restrict__ approx_out, int mode,
-                                         float scale, float gamma, float delta, const float* __restrict__ st_a,
-                                         const float* __restrict__ st_t) {
+                                         float scale, float gamma, float delta, const float* st_a, const float* st_t,
+                                         Ready&& ready) {
   const size_t base = ((size_t)map * kBases + (bi + 1)) * (size_t)n * n;
   const bool high = threadIdx.x >= 128;   // warp-uniform
   const int kx0 = (threadIdx.x & 7) * 4, ky0 = 2 * ((threadIdx.x >> 3) & 15);
@@ -202,6 +203,7 @@ __device__ __forceinline__ void ana_cols(const float* __restrict__ lo_s, const f
   }
   x0 = row(2 * bi + 2), x1 = row(2 * bi + 3);
   step(1, x0, x1, th, tg);
+  if (!ready()) return;
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const int ky = ky0 + r, Y = oy0 + ky, X = ox0 + kx0, so = ky * kTO + kx0;
@@ -291,7 +293,7 @@ __device__ __forceinline__ void ana_issue_input_t(const SaraTma& tm, int in_row0
 constexpr int kStage = 3 * kTO * kTO;
 // Staged epilogue operands start on a 128-byte boundary (tensor-map copy destinations).
 constexpr int kAnaPre = (kA2In + 2 * kRSmax * kPlo + 31) / 32 * 32;
-constexpr int kAnaFloats = kAnaPre + 2 * kStage;
+static_assert(2 * kStage <= kA2In, "the staged operands fit the input tile");
 static_assert(kA2In % 4 == 0 && (kRSmax * kPlo) % 4 == 0 && kStage % 32 == 0, "aligned stage buffers");
 
 // The first 3 * 32 * 2 threads each start one bulk copy of this tile's A and gamma W
@@ -339,14 +341,16 @@ struct AnaSmem {
   float *in_s, *lo_s, *hi_s, *st_a, *st_t;
   uint64_t* bar;   // [0] input tile, [1] staged epilogue operands
 };
+// OVERLAY: the staged operands take the place of the input tile, once the rows have read it.
+template <bool OVERLAY>
 __device__ __forceinline__ AnaSmem ana_smem(float4* sma) {
   AnaSmem a;
   a.in_s = reinterpret_cast<float*>(sma);
   a.lo_s = a.in_s + kA2In;
   a.hi_s = a.lo_s + kRSmax * kPlo;
-  a.st_a = a.in_s + kAnaPre;
+  a.st_a = a.in_s + (OVERLAY ? 0 : kAnaPre);
   a.st_t = a.st_a + kStage;
-  a.bar = reinterpret_cast<uint64_t*>(a.st_t + kStage);
+  a.bar = reinterpret_cast<uint64_t*>(a.in_s + kAnaPre + (OVERLAY ? 0 : 2 * kStage));
   return a;
 }
 
@@ -360,39 +364,54 @@ __device__ __forceinline__ void ana_abort(const AnaSmem& S, int staged, int* err
   }
 }
 
-// One basis of one tile: input copies (issued first), staged epilogue operands (dual
-// mode), rows, columns + epilogue.
+// One basis of one tile: input copies, rows, columns + epilogue, whose operands (dual mode) are staged
+// beside the input, or (OVERLAY) over the input tile once the rows have read it, while the columns
+// are filtered: then a CTA takes 49 KB instead of 73, and an SM holds four instead of three. PREFETCH brings the
+// operands to the L2 beforehand: level 2 on of 2048^2 138 -> 132 us, of 1024^2 56 -> 55; not at level 1, where
+// one basis per CTA means a small map whose coefficients are in the L2 (512^2 107.1 without, 108.9 with).
+template <bool OVERLAY, bool PREFETCH>
 __device__ __forceinline__ void ana_basis(const SaraTma& tm, int in_row0, const float* src, int m, const AnaSmem& S,
                                           int bi, int map, int n, int hm, int oy0, int ox0, int last, float* coef,
                                           float* thr, float* approx_out, int mode, float scale, float gamma,
                                           float delta, int* err) {
   ana_issue_input_t(tm, in_row0, src, m, oy0, ox0, 2 * kTO + 2 * bi, S.in_s, &S.bar[0]);
-  if (mode == SARA_DUAL)
-    stage_epilogue_t(tm, coef, thr, ((size_t)map * kBases + bi + 1) * (size_t)n * n, (map * kBases + bi + 1) * n, n,
-                     hm, oy0, ox0, S.st_a, S.st_t, &S.bar[1]);
+  const int prow = (map * kBases + bi + 1) * n;
+  if (PREFETCH && mode == SARA_DUAL && tm.use_stage && threadIdx.x < 6) {
+    const int sb = threadIdx.x % 3;
+    tma_prefetch_2d(threadIdx.x < 3 ? &tm.coef : &tm.thr, sb == 1 ? ox0 : hm + ox0, prow + (sb == 0 ? oy0 : hm + oy0));
+  }
+  auto stage = [&] {
+    if (mode == SARA_DUAL)
+      stage_epilogue_t(tm, coef, thr, ((size_t)map * kBases + bi + 1) * (size_t)n * n, prow, n, hm, oy0, ox0, S.st_a,
+                       S.st_t, &S.bar[1]);
+  };
+  if (!OVERLAY) stage();
   const bool ok = mbar_wait(&S.bar[0], 0);
   if (__syncthreads_or(!ok)) {
-    ana_abort(S, mode == SARA_DUAL, err);
+    ana_abort(S, !OVERLAY && mode == SARA_DUAL, err);
     return;   // this tile is left unchanged (the host reports PS_ETIMEOUT)
   }
   ana_rows(bi, S.in_s, S.lo_s, S.hi_s);
   __syncthreads();
-  if (mode == SARA_DUAL && !mbar_wait(&S.bar[1], 0)) {
-    atomicExch(err, 1);
-    (void)mbar_drain(&S.bar[1], 0);
-    return;
-  }
-  ana_cols(S.lo_s, S.hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta,
-               S.st_a, S.st_t);
+  if (OVERLAY) stage();
+  ana_cols(S.lo_s, S.hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta, S.st_a,
+           S.st_t, [&] {
+             if (mode != SARA_DUAL || mbar_wait(&S.bar[1], 0)) return true;
+             atomicExch(err, 1);
+             (void)mbar_drain(&S.bar[1], 0);
+             return false;
+           });
 }
 
 // Level-1 analysis: input is the map itself; one basis per CTA (grid.y).
-__global__ void __launch_bounds__(256, 3) k_ana_l1(const float* __restrict__ X, int n, int last, float* __restrict__ coef,
+template <bool OVERLAY>
+__global__ void __launch_bounds__(256, OVERLAY ? 4 : 3) k_ana_l1(const float* __restrict__ X, int n, int last,
+                                                                 float* __restrict__ coef,
                                                    float* __restrict__ thr, float* __restrict__ approx_out, int mode,
                                                    float scale, float gamma, float delta, int* err,
                                                    const __grid_constant__ SaraTma tm) {
   extern __shared__ __align__(128) float4 sma[];
-  const AnaSmem S = ana_smem(sma);
+  const AnaSmem S = ana_smem<OVERLAY>(sma);
   const int bi = blockIdx.y, map = blockIdx.z;
   const int hm = n >> 1, tilesx = hm / kTO;
   const int oy0 = (blockIdx.x / tilesx) * kTO, ox0 = (blockIdx.x % tilesx) * kTO;
@@ -401,19 +420,20 @@ __global__ void __launch_bounds__(256, 3) k_ana_l1(const float* __restrict__ X, 
     mbar_init(&S.bar[1], 1);
   }
   __syncthreads();
-  ana_basis(tm, map * n, X + (size_t)map * n * n, n, S, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode,
-            scale, gamma, delta, err);
+  ana_basis<OVERLAY, false>(tm, map * n, X + (size_t)map * n * n, n, S, bi, map, n, hm, oy0, ox0, last, coef, thr,
+                            approx_out, mode, scale, gamma, delta, err);
 }
 
 // Levels >= 2 with half size >= 32: one basis per CTA (grid.y). (A basis-slowest grid, which
 // keeps the co-resident CTAs on one filter's code, measured 5 us slower at 1024^2.)
-__global__ void __launch_bounds__(256, 3) k_ana_lv(const float* __restrict__ approx_in, int m, int n, int last,
-                                                   float* __restrict__ coef, float* __restrict__ thr,
+template <bool OVERLAY>
+__global__ void __launch_bounds__(256, OVERLAY ? 4 : 3) k_ana_lv(const float* __restrict__ approx_in, int m, int n,
+                                                                 int last, float* __restrict__ coef, float* __restrict__ thr,
                                                    float* __restrict__ approx_out, int mode, float scale, float gamma,
                                                    float delta, int* err, const __grid_constant__ SaraTma tm) {
   extern __shared__ __align__(128) float4 sma[];
   pdl_wait();
-  const AnaSmem S = ana_smem(sma);
+  const AnaSmem S = ana_smem<OVERLAY>(sma);
   const int bi = blockIdx.y, map = blockIdx.z;
   const int hm = m >> 1, tilesx = hm / kTO;
   const int oy0 = (blockIdx.x / tilesx) * kTO, ox0 = (blockIdx.x % tilesx) * kTO;
@@ -422,8 +442,8 @@ __global__ void __launch_bounds__(256, 3) k_ana_lv(const float* __restrict__ app
     mbar_init(&S.bar[1], 1);
   }
   __syncthreads();
-  ana_basis(tm, (map * kDb + bi) * m, approx_in + ((size_t)map * kDb + bi) * (size_t)m * m, m, S, bi, map, n, hm, oy0,
-            ox0, last, coef, thr, approx_out, mode, scale, gamma, delta, err);
+  ana_basis<OVERLAY, OVERLAY>(tm, (map * kDb + bi) * m, approx_in + ((size_t)map * kDb + bi) * (size_t)m * m, m, S, bi,
+                              map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta, err);
 }
 
 // Level-1 analysis with the input tile shared by four bases: one CTA per (tile, half of the bases,
@@ -434,7 +454,9 @@ __global__ void __launch_bounds__(256, 3) k_ana_lv(const float* __restrict__ app
 // (Two sets at 2 CTAs/SM, eight bases per CTA, 512 threads and a persistent form over all
 // units were slower: 85-88, 94 and 139 us at 1024^2 against 82.)
 constexpr int kL1Bases = 4;
-static size_t multi_analysis_smem() { return (size_t)(kAnaPre + 2 * kStage) * sizeof(float) + 32; }
+static size_t analysis_smem(bool overlay) {
+  return (size_t)(kAnaPre + (overlay ? 0 : 2 * kStage)) * sizeof(float) + 16;
+}
 
 __global__ void __launch_bounds__(256, 3) k_ana_l1m(const float* __restrict__ X, int n, int last,
                                                     float* __restrict__ coef, float* __restrict__ thr,
@@ -442,7 +464,7 @@ __global__ void __launch_bounds__(256, 3) k_ana_l1m(const float* __restrict__ X,
                                                     float gamma, float delta, int* err,
                                                     const __grid_constant__ SaraTma tm) {
   extern __shared__ __align__(128) float4 smm[];
-  const AnaSmem S = ana_smem(smm);
+  const AnaSmem S = ana_smem<false>(smm);
   const int map = blockIdx.z, b0 = blockIdx.y * kL1Bases;
   const int hm = n >> 1, tilesx = hm / kTO;
   const int oy0 = (blockIdx.x / tilesx) * kTO, ox0 = (blockIdx.x % tilesx) * kTO;
@@ -479,7 +501,7 @@ __global__ void __launch_bounds__(256, 3) k_ana_l1m(const float* __restrict__ X,
       __syncthreads();
     }
     ana_cols(S.lo_s, S.hi_s, bi, map, n, hm, oy0, ox0, last, coef, thr, approx_out, mode, scale, gamma, delta, S.st_a,
-             S.st_t);
+             S.st_t, [] { return true; });
     __syncthreads();   // lo/hi and the stage set consumed before the next basis
     if (staged && i + 1 < kL1Bases) stage(bi + 1);
   }
@@ -764,7 +786,6 @@ __global__ void __launch_bounds__(256, 3) k_syn2_lv(const float* __restrict__ co
     *reinterpret_cast<float4*>(dst + (size_t)(oy0 + 4 * rq + rr) * m + ox0 + 4 * cg) = syn2_row(acc, rr);
 }
 
-static size_t fast_analysis_smem() { return (size_t)kAnaFloats * sizeof(float) + 16; }
 
 
 // ---------------------------------------------------------------------------
@@ -1256,8 +1277,9 @@ cudaError_t configure_nufft_kernels();
 
 cudaError_t configure_kernels() {
   cudaError_t e;
-  for (const void* f : {(const void*)k_ana_l1, (const void*)k_ana_lv}) {
-    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fast_analysis_smem());
+  for (const void* f : {(const void*)k_ana_l1<false>, (const void*)k_ana_l1<true>, (const void*)k_ana_lv<false>,
+                        (const void*)k_ana_lv<true>}) {
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)analysis_smem(false));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
@@ -1268,7 +1290,8 @@ cudaError_t configure_kernels() {
     e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
   }
-  e = cudaFuncSetAttribute((const void*)k_ana_l1m, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)multi_analysis_smem());
+  e = cudaFuncSetAttribute((const void*)k_ana_l1m, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)analysis_smem(false));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute((const void*)k_ana_l1m, cudaFuncAttributePreferredSharedMemoryCarveout,
                            cudaSharedmemCarveoutMaxShared);
@@ -1287,10 +1310,19 @@ cudaError_t configure_kernels() {
 }
 
 // (Tile, map) units of the first analysis level from which its tiles serve four bases per CTA; with
-// fewer, one basis per CTA keeps more of the chip busy. us, one basis / four: 256^2 (64 units) 14.8 /
-// 21, 512^2 (256) 28 / 34, 1024^2 (1024) 87 / 80, 2048^2 (4096) 317 / 283;
-// a batch whose 512^2 class has 512 units 415 / 411 per iteration.
+// fewer, one basis per CTA keeps more of the chip busy. us, one basis / four: 256^2 (64 units) 15 /
+// 21, 512^2 (256) 27 / 34, 1024^2 (1024) 79 / 81 alone but 433 / 423 for the iteration, 2048^2 (4096) 286 / 283
+// and 1063 / 1055; a batch whose 512^2 class has 512 units 415 / 411 per iteration (one basis with three
+// CTAs per SM).
 constexpr int kSharedTiles = 512;
+
+// Levels of one basis per CTA with more CTAs than this per SM overlay the staged operands on the input
+// tile: the waits of the warps in flight bound them, and a fourth CTA per SM hides more of them. Fewer
+// CTAs are all resident (or nearly) as they are, and loading the operands early is the better use. us per
+// iteration, beside / overlaid: 256^2 56.9 / 57.6 (level 1: 512 CTAs), 512^2 111.6 / 108.6 (2048), 1024^2 426.1 /
+// 423.2 and 2048^2 (cone dual) 1057 / 1049 (levels 2 on: 2048 and 8192), a batch of 16 412 / 408.
+// Without a dual update nothing is staged and the smaller CTA always serves (512^2, 5 levels 25.1 -> 24.4 us).
+constexpr int kOverlayWaves = 4;
 
 cudaError_t sara_analysis(Handle* h, const float* X, float* coef, float* thr, int mode, float scale, float gamma,
                           float delta, cudaEvent_t fine_done) {
@@ -1309,17 +1341,19 @@ cudaError_t sara_analysis(Handle* h, const float* X, float* coef, float* thr, in
     const dim3 grid((hm / kTO) * (hm / kTO), kDb, nmaps);
     const SaraTma tm = analysis_maps(l == 1 ? X : buf[(l - 2) & 1], m, l == 1 ? nmaps : kDb * nmaps, coef, thr, n, nmaps,
                                      mode);
+    const bool over = mode != SARA_DUAL || (int)(grid.x * grid.y * grid.z) > kOverlayWaves * h->num_sms;
+    const size_t smem = analysis_smem(over);
     if (l > 1) {
-      launch_after(true, k_ana_lv, grid, 256, fast_analysis_smem(), h->stream, buf[(l - 2) & 1], m, n, l == L, coef, thr,
-                   buf[(l - 1) & 1], mode, scale, gamma, delta, h->dev_flags, tm);
+      launch_after(true, over ? k_ana_lv<true> : k_ana_lv<false>, grid, 256, smem, h->stream, buf[(l - 2) & 1], m, n,
+                   l == L, coef, thr, buf[(l - 1) & 1], mode, scale, gamma, delta, h->dev_flags, tm);
       continue;
     }
     if ((int)(grid.x * grid.z) >= kSharedTiles)
-      k_ana_l1m<<<dim3(grid.x, kDb / kL1Bases, nmaps), 256, multi_analysis_smem(), h->stream>>>(
+      k_ana_l1m<<<dim3(grid.x, kDb / kL1Bases, nmaps), 256, analysis_smem(false), h->stream>>>(
           X, n, l == L, coef, thr, buf[0], mode, scale, gamma, delta, h->dev_flags, tm);
     else
-      k_ana_l1<<<grid, 256, fast_analysis_smem(), h->stream>>>(X, n, l == L, coef, thr, buf[0], mode, scale, gamma, delta,
-                                                              h->dev_flags, tm);
+      (over ? k_ana_l1<true> : k_ana_l1<false>)<<<grid, 256, smem, h->stream>>>(
+          X, n, l == L, coef, thr, buf[0], mode, scale, gamma, delta, h->dev_flags, tm);
     if (fine_done) {
       const cudaError_t e = cudaEventRecord(fine_done, h->stream);
       if (e != cudaSuccess) return e;

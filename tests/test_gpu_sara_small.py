@@ -65,11 +65,12 @@ def test_dual_update_and_reweight_match_oracle(n, levels):
     assert rel_err(T, 0.02 * 0.01 / (0.01 + np.abs(coef))) <= 1e-5
 
 
-def test_dual_update_of_shared_tiles_and_its_bounded_wait():
-    """1024^2: the first analysis level with its input tiles shared by four bases. One iteration without
-    data from a random state, A of one map against clamp(A + rho1 Psi^dagger (2 S' - S), +-gamma W); then
+@pytest.mark.parametrize("n,levels", [(256, 2), (512, 3), (1024, 2)])
+def test_dual_update_of_tiles_and_its_bounded_wait(n, levels):
+    """256^2 and 512^2: one basis per CTA, the operands of the epilogue staged beside and over its input tile; 1024^2:
+    the first analysis level with its input tiles shared by four bases. One iteration without data from
+    a random state, A of one map against clamp(A + rho1 Psi^dagger (2 S' - S), +-gamma W); then
     a launch whose waits give up at once is reported and the handle goes on."""
-    n, levels = 1024, 2
     rng = np.random.default_rng(41)
     st = {k: (0.05 * rng.normal(size=s)).astype(np.float32)
           for k, s in (("S", (4, n, n)), ("Z", (2, n, n)), ("A", (4, 9, n, n)), ("C", (4, n, n)), ("D", (2, n, n)))}
