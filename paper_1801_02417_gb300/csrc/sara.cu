@@ -582,6 +582,15 @@ __device__ __forceinline__ void syn2_issue_t(const SaraTma& tm, int prow, int ap
   }
 }
 
+// The same tiles brought to the L2 ahead of their staging.
+__device__ __forceinline__ void syn2_prefetch_t(const SaraTma& tm, int prow, int aprow, int half, int coarsest, int hm,
+                                                int oy0, int ox0) {
+  if (!(tm.use_scoef && ox0 > 0 && oy0 > 0 && (coarsest || tm.use_apx)) || threadIdx.x >= 4) return;
+  const int ky0 = oy0 / 2 - half, kxa = ox0 / 2 - 8, sb = threadIdx.x;
+  if (sb == 0 && !coarsest) tma_prefetch_2d(&tm.apx, kxa, aprow + ky0);
+  else tma_prefetch_2d(&tm.scoef, (sb & 2 ? hm : 0) + kxa, prow + (sb & 1 ? hm : 0) + ky0);
+}
+
 // Along y for basis LF: lo/hi at output rows 4 rg + t (t = 0..3) and staged columns
 // c, c + 1, from coefficient rows 2 rg + i (i = 0 .. half + 1) through tap
 // j = t - 2 (i - half). Columns start at the even column at or left of 8 - half. The 256 threads take
@@ -700,7 +709,9 @@ __device__ __forceinline__ void syn2_abort(uint64_t* bar, uint32_t parity, int* 
 // Finest level: the eight bases plus the Dirac part summed in registers -> Psi A. One staging set,
 // refilled with basis b+1 as soon as the y-pass of basis b has read it, so the copy overlaps the
 // x-pass (4 CTAs per SM hide the rest; two sets at 3 CTAs per SM and a persistent form whose
-// staging runs on across tiles were slower: 78 and 80 us at 1024^2 against 72).
+// staging runs on across tiles were slower: 78 and 80 us at 1024^2 against 72). The basis after the one being
+// staged is on its way to the L2 meanwhile (us per iteration: 2048^2 1046 -> 1042, 1024^2 421.3 -> 420.5; the same
+// in the shared analysis tiles cost 2, and ahead of the dependency in the coarser synthesis 0.7 at 512^2).
 __global__ void __launch_bounds__(256, 4)
     k_syn2_fine(const float* __restrict__ coef, const float* __restrict__ approx_in, int coarsest, int n,
                 float* __restrict__ out, int* err, const __grid_constant__ SaraTma tm) {
@@ -717,6 +728,8 @@ __global__ void __launch_bounds__(256, 4)
   auto issue = [&](int bi) {
     syn2_issue_t(tm, (map * kBases + bi + 1) * n, (map * kDb + bi) * hm, bi, cmap + (size_t)(bi + 1) * n * n,
                  coarsest ? nullptr : approx_in + ((size_t)map * kDb + bi) * (size_t)hm * hm, n, hm, oy0, ox0, s4, bar);
+    if (bi + 1 < kDb)
+      syn2_prefetch_t(tm, (map * kBases + bi + 2) * n, (map * kDb + bi + 1) * hm, bi + 1, coarsest, hm, oy0, ox0);
   };
   if (threadIdx.x == 0) mbar_init(bar, 1);
   __syncthreads();
