@@ -153,14 +153,10 @@ SINGLE_KERNEL_STAGES = {"primal": "k_primal", "analysis": "k_ana_l1", "synthesis
                         "degrid": "k_degrid", "grid": "k_grid"}
 
 
-def stage_kernel(stage: str, tuning: list) -> str:
-    """Name of the kernel a single-kernel stage launches under the handle's launch choices."""
-    if stage == "analysis" and tuning[3] == 1:
-        return "k_ana_pers"
-    if stage == "analysis" and tuning[3] >= 2:
+def stage_kernel(stage: str, n: int) -> str:
+    """Name of the kernel a single-kernel stage launches for one n x n problem (four maps)."""
+    if stage == "analysis" and 4 * (n // 64) ** 2 >= 512:
         return "k_ana_l1m"
-    if stage == "synthesis" and tuning[0] == 2:
-        return "k_syn2_fine_pers"
     return SINGLE_KERNEL_STAGES[stage]
 
 
@@ -624,7 +620,7 @@ def run_own(args) -> None:
     peak_src = "measured" if "hbm_gbs" in peaks else "fallback"
     dom_bytes = mbytes.get(dom, sbytes[dom])
     achieved = dom_bytes / (stages[dom] * 1e-3) / 1e9
-    dom_kernel = stage_kernel(dom, B.ps_get_tuning(s.h))
+    dom_kernel = stage_kernel(dom, wl.n)
     traffic, traffic_src = dram_traffic(dom_kernel, wl.name)
     total_bytes = sum(sbytes.values())
     fp32 = {"packed_flops": B.ps_fp32_peak(True), "scalar_flops": B.ps_fp32_peak(False)}

@@ -608,8 +608,8 @@ static constexpr size_t degrid_smem_tiles() {
 // Nothing is shared between warps: no barrier, no uneven end of a work item, no list of work,
 // and no FP32 atomic on shared memory (a compare-and-swap loop), which the form before it
 // paid (one CTA per tile of cells, blocks added to a shared tile, weights from a table of 64
-// bytes per row: in this form the table measured 91 us against 87). Grid stage, us: 1024^2 / 2,000,000 rows (34 per cell) 101 -> 87 with 232 -> 106 MB
-// of DRAM traffic, 256^2 / 50,000 17 -> 14; phi^dagger as a whole: 1024^2 / 200,001 scattered rows
+// bytes per row: in this form the table measured 91 us against 87). Grid stage, us: 1024^2 /
+// 2,000,000 rows (34 per cell) 101 -> 87 with 232 -> 106 MB of DRAM traffic, 256^2 / 50,000 17 -> 14; phi^dagger as a whole: 1024^2 / 200,001 scattered rows
 // (1 per cell) 397 -> 193, 512^2 / 2,000,001 scattered 389 -> 333. Bound by issue (62% of the slots
 // busy), the split and the products before the tensor pipe.
 constexpr int kGridWarps = 4;   // warps of a CTA
@@ -978,11 +978,6 @@ cudaError_t nufft_degrid(Handle* h, int mode, float2* out, bool keep_cb, const i
 template <int W>
 static cudaError_t launch_grid(Handle* h, const float2* in, int use_scale, const int32_t* perm) {
   const GridGeom& g = h->g;
-  // Rows per warp: 64 where that leaves two warps for every scheduler of the chip and a cell
-  // holds enough rows that cutting its run at a warp's end costs more than parallelism gives,
-  // else 32. phi^dagger, us at 32 / 64 / 128 rows: 1024^2 / 2,000,000 rows (34 per cell) 147 / 143 /
-  // 144, 64^2 / 100,000 (73 per cell) 35 / 30 / 30; 256^2 / 50,000 29 / 31 / 35, 2048^2 / 700,001
-  // (4 per cell) 215 / 222 / 243, 1024^2 / 200,001 scattered (1 per cell) 193 / 200 / 219.
   // Rows per warp. Few rows: 8, for more warps with fewer cells each. Many rows in dense cells:
   // 64, where that leaves two warps for every scheduler of the chip and a cell holds enough
   // rows that cutting its run at a warp's end costs more than parallelism gives. Else 32.
