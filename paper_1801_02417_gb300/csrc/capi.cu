@@ -3,8 +3,8 @@
 // One handle = one imaging problem resident on the device. ps_pd_iterate replays
 // a CUDA graph of one iteration of Algorithm 1:
 //   k_primal                    steps 3, 4, 9-12 and the Dirac part of 5-6
-//   k_analysis x levels         steps 5-6 (Psi^dagger of 2S'-S, soft-threshold dual)
-//   k_synthesis x levels        Psi A^(k+1) for the next step 3
+//   k_ana_* per level           steps 5-6 (Psi^dagger of 2S'-S, soft-threshold dual)
+//   k_syn* per level            Psi A^(k+1) for the next step 3
 //   k_fwd_rows, k_fwd_cols      F Z of phi(2S'-S)                  (step 7)
 //   k_degrid                    G, mixing by L, B~ and ||B~/rho2 - Y||^2; step 8 (l2-ball factor per block)
 //   k_grid, k_adj_cols, k_adj_rows   phi^dagger B^(k+1) for the next step 3
