@@ -609,8 +609,9 @@ static constexpr size_t degrid_smem_tiles() {
 // and no FP32 atomic on shared memory (a compare-and-swap loop), which the form before it
 // paid (one CTA per tile of cells, blocks added to a shared tile, weights from a table of 64
 // bytes per row: in this form the table measured 91 us against 87). Grid stage, us: 1024^2 /
-// 2,000,000 rows (34 per cell) 101 -> 87 with 232 -> 106 MB of DRAM traffic, 256^2 / 50,000 17 -> 14; phi^dagger as a whole: 1024^2 / 200,001 scattered rows
-// (1 per cell) 397 -> 193, 512^2 / 2,000,001 scattered 389 -> 333. Bound by issue (62% of the slots
+// 2,000,000 rows (34 per cell) 101 -> 85 with 232 -> 105 MB of DRAM traffic, 256^2 / 50,000 17 ->
+// 14; phi^dagger as a whole: 1024^2 / 200,001 scattered rows
+// (1 per cell) 397 -> 193, 512^2 / 2,000,001 scattered 389 -> 333. Bound by issue (70% of the slots
 // busy), the split and the products before the tensor pipe.
 constexpr int kGridWarps = 4;   // warps of a CTA
 template <int W>
