@@ -98,7 +98,8 @@ __device__ __forceinline__ int wrap1(int v, int m) { return v < 0 ? v + m : (v >
 // Rows: lo/hi[r][k] = sum_j h/g[j] in[r][2k + j], k in [0, TO), RS rows. Each thread makes
 // four outputs of one row from 16-byte reads; the taps go in pairs,
 // {c[2p], c[2p+1]} x {in[2k+2p], in[2k+2p+1]}, and the two halves are added at the end. Two pairs per
-// step (an odd count ends with a pair of zero taps); x0 .. x3 are the sample pairs p .. p + 3.
+// step and the last of an odd count on its own: a pair of zero taps in its place would turn an infinity
+// that the filter does not reach into a NaN. x0 .. x3 are the sample pairs p .. p + 3.
 __device__ __forceinline__ void ana_rows(int b, const float* __restrict__ in_s, float* __restrict__ lo_s,
                                          float* __restrict__ hi_s) {
   const int RS = 2 * kTO + 2 * b;
@@ -108,7 +109,7 @@ __device__ __forceinline__ void ana_rows(int b, const float* __restrict__ in_s, 
     const ulonglong2 q0 = row[0], q1 = row[1];
     u64 x0 = q0.x, x1 = q0.y, x2 = q1.x, x3 = q1.y;
     u64 a[4] = {0ull, 0ull, 0ull, 0ull}, c[4] = {0ull, 0ull, 0ull, 0ull};
-    for (int p = 0; p <= b; p += 2) {
+    for (int p = 0; p < b; p += 2) {
       const ulonglong2 n = row[2 + (p >> 1)];
       const ulonglong2 h = *reinterpret_cast<const ulonglong2*>(&c_h[b][2 * p]);
       const ulonglong2 g = *reinterpret_cast<const ulonglong2*>(&c_g[b][2 * p]);
@@ -121,6 +122,17 @@ __device__ __forceinline__ void ana_rows(int b, const float* __restrict__ in_s, 
       c[2] = ffma2(g.y, x3, ffma2(g.x, x2, c[2]));
       c[3] = ffma2(g.y, n.x, ffma2(g.x, x3, c[3]));
       x0 = x2, x1 = x3, x2 = n.x, x3 = n.y;
+    }
+    if (!(b & 1)) {   // b + 1 pairs: the last one
+      const u64 h = *reinterpret_cast<const u64*>(&c_h[b][2 * b]), g = *reinterpret_cast<const u64*>(&c_g[b][2 * b]);
+      a[0] = ffma2(h, x0, a[0]);
+      a[1] = ffma2(h, x1, a[1]);
+      a[2] = ffma2(h, x2, a[2]);
+      a[3] = ffma2(h, x3, a[3]);
+      c[0] = ffma2(g, x0, c[0]);
+      c[1] = ffma2(g, x1, c[1]);
+      c[2] = ffma2(g, x2, c[2]);
+      c[3] = ffma2(g, x3, c[3]);
     }
     float lo[4], hi[4];
 #pragma unroll
@@ -840,10 +852,11 @@ __device__ __forceinline__ void small_ana_level(int b, float* __restrict__ img, 
       float4 x0 = row[0], x1 = row[1];   // samples j .. j + 7 of the step's first tap j
       // One chain per output, in the order of the taps: a scalar FMA does as much per clock
       // as a packed one, and the coarse coefficients are the ones whose rounding shows most.
-      // Four taps per step, zero ones at the end of the shorter filters.
+      // Four taps per step, and two at the end of every second filter (no zero taps, as in ana_rows).
       float l[4] = {0.f, 0.f, 0.f, 0.f}, h[4] = {0.f, 0.f, 0.f, 0.f};
+      const int whole = LF & ~3;
 #pragma unroll U4
-      for (int j = 0; j < LF; j += 4) {
+      for (int j = 0; j < whole; j += 4) {
         const float4 x2 = row[2 + (j >> 2)];
         const float4 ch = *reinterpret_cast<const float4*>(&c_h[b][j]), cg = *reinterpret_cast<const float4*>(&c_g[b][j]);
         const float x[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
@@ -852,11 +865,19 @@ __device__ __forceinline__ void small_ana_level(int b, float* __restrict__ img, 
         for (int i = 0; i < 4; ++i)
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            if (LFT && j + i >= LFT) continue;
             l[q] = fmaf(th[i], x[2 * q + i], l[q]);
             h[q] = fmaf(tg[i], x[2 * q + i], h[q]);
           }
         x0 = x1, x1 = x2;
+      }
+      if (LF & 2) {
+        const float2 ch = *reinterpret_cast<const float2*>(&c_h[b][whole]), cg = *reinterpret_cast<const float2*>(&c_g[b][whole]);
+        const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          l[q] = fmaf(ch.y, x[2 * q + 1], fmaf(ch.x, x[2 * q], l[q]));
+          h[q] = fmaf(cg.y, x[2 * q + 1], fmaf(cg.x, x[2 * q], h[q]));
+        }
       }
       *reinterpret_cast<float4*>(lo + r * Q + k0) = make_float4(l[0], l[1], l[2], l[3]);
       *reinterpret_cast<float4*>(hi + r * Q + k0) = make_float4(h[0], h[1], h[2], h[3]);
