@@ -122,6 +122,7 @@ static bool misaligned(const void* p, int device_ptrs) { return device_ptrs && p
     if (misaligned((p), (dp))) return fail((h), PS_EINVAL, std::string(what) + ": device pointer not 16-byte aligned"); \
   } while (0)
 
+constexpr int kMaxBlocks = 2047;   // l2 blocks of one problem, at most
 
 static void free_vis(Handle* h) {
   const size_t M = h->M;
@@ -382,7 +383,11 @@ int64_t ps_estimate_bytes(int32_t n, int32_t levels, int64_t M) {
   if (n < 16 || n > 2048 || !is_pow2(n) || levels < 1 || (n % (1 << levels)) != 0 || M < 0) return 0;
   const int64_t N = (int64_t)n * n, K = 2 * (int64_t)n;
   const int64_t img = (28 + 72 + 16) * N * 4 + (8 * (int64_t)ps::sweep_blocks((int)N) + 1024) * 8;
-  const int64_t vis = M * (3 * 32 + 16 + 4 + 2) + (M / 64 + 64) * 16;   // rows and work items
+  // Rows; work items, of which every occupied grid tile has one and every 64 rows at most one more; the
+  // four arrays of 28 bytes per block, at their most.
+  const int64_t tiles = ((K + ps::kGridTile - 1) / ps::kGridTile) * ((K + ps::kGridTile - 1) / ps::kGridTile);
+  const int64_t vis = M * (3 * 32 + 16 + 4 + 2) + (M / 64 + std::min(M, tiles)) * (int64_t)sizeof(ps::GridItem) +
+                      (M > 0 ? kMaxBlocks * 28 : 0);
   const int64_t grid = 2 * (int64_t)n * K * 16 + 48 * K * K + K * 12 + (int64_t)n * 4;
   return img + vis + grid;
 }
@@ -581,7 +586,7 @@ ps_status ps_set_measurements(ps_handle* h, int64_t M64, const double* uv, const
   CHECK_ALIGN(h, uv, device_ptrs, "set_measurements");
   CHECK_ALIGN(h, vis, device_ptrs, "set_measurements");
   CHECK_ALIGN(h, weights, device_ptrs, "set_measurements");
-  if (M > 0 && (!uv || !vis || !block_offsets || nblocks < 1 || nblocks > 2047))
+  if (M > 0 && (!uv || !vis || !block_offsets || nblocks < 1 || nblocks > kMaxBlocks))
     return fail(h, PS_EINVAL, "set_measurements: need uv, vis, block_offsets and 1 <= nblocks <= 2047");
   std::vector<double> eps_chi2;
   if (M > 0) {
