@@ -473,7 +473,7 @@ ps_status ps_create(const ps_config* cfg, void* cuda_stream, ps_handle** out) {
   }
   double filt[ps::kDb][ps::kMaxTaps];
   ps::daubechies_filters(filt);
-  if ((e = ps::upload_filters(filt, h->stream)) != cudaSuccess || (e = ps::upload_es_polys(h->stream)) != cudaSuccess) {
+  if ((e = ps::upload_es_polys(h->stream)) != cudaSuccess || (e = ps::upload_filters(filt, h->stream)) != cudaSuccess) {   // waits
     h->err = std::string("upload filters: ") + cudaGetErrorString(e);
     return bail(PS_ECUDA);
   }

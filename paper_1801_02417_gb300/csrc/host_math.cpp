@@ -142,7 +142,7 @@ std::vector<double> es_fourier(double step, int count, int W) {
 // Tap j (offset f + W/2 - j, |f| <= 1/2) as a polynomial of degree 2 kEsTerms - 1 in f: the
 // Chebyshev series of the kernel on 64 nodes, cut at that degree and written out in powers;
 // c holds the even coefficients (of f^0, f^2, ..), then the odd ones (of f, f^3, ..).
-void es_poly(int W, int j, double c[2 * kEsTerms]) {
+static void es_poly(int W, int j, double c[2 * kEsTerms]) {
   constexpr int D = 2 * kEsTerms, NN = 64;
   double a[D];   // Chebyshev coefficients in x = 2 f
   for (int k = 0; k < D; ++k) {
@@ -164,6 +164,24 @@ void es_poly(int W, int j, double c[2 * kEsTerms]) {
     c[k] = p[2 * k] * std::pow(2.0, 2 * k);
     c[kEsTerms + k] = p[2 * k + 1] * std::pow(2.0, 2 * k + 1);
   }
+}
+
+// The polynomials of every tap and width, fitted once per process (thread-safe static initialisation:
+// handles may be created concurrently; a fit of all twelve takes about 0.3 ms).
+const EsTable& es_table() {
+  struct Built {
+    EsTable t{};
+    Built() {
+      for (int q = 0; q < 3; ++q)
+        for (int j = 0; j <= (5 + 2 * q) / 2; ++j) {
+          double c[2 * kEsTerms];
+          es_poly(5 + 2 * q, j, c);
+          for (int k = 0; k < 2 * kEsTerms; ++k) t.c[q][j][k][0] = t.c[q][j][k][1] = (float)c[k];
+        }
+    }
+  };
+  static const Built built;
+  return built.t;
 }
 
 }  // namespace ps

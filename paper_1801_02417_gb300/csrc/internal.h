@@ -137,11 +137,16 @@ void daubechies_filters(double h[kDb][kMaxTaps]);          // db1..db8 scaling f
 double es_beta(int W);
 double es_kernel(double t, int W, double beta);            // ES kernel value at offset t (cells)
 std::vector<double> es_fourier(double step, int count, int W);   // its Fourier transform at k step, k < count (beta = es_beta)
-void es_poly(int W, int j, double c[2 * kEsTerms]);        // tap j as a polynomial of its offset: E then O coefficients
+// Taps 0 .. W/2 of width W = 5 + 2 q as polynomials of their offset: c[q][j] holds the even coefficients, then
+// the odd ones, each in both halves of a 64-bit word. Made once.
+struct EsTable {
+  alignas(16) float c[3][5][2 * kEsTerms][2];
+};
+const EsTable& es_table();
 
 // Kernel launchers (return cudaGetLastError()).
 cudaError_t upload_filters(const double h[kDb][kMaxTaps], cudaStream_t stream);
-cudaError_t upload_es_polys(cudaStream_t stream);
+cudaError_t upload_es_polys(cudaStream_t stream);   // queued on stream, not waited for
 
 // NUFFT pieces (nufft.cu).
 // X (4 planes) -> G; clear_acc: the gridding accumulator too, for the nufft_grid(.., cleared) that follows.

@@ -258,21 +258,14 @@ __device__ __forceinline__ void es_weights(float f, float beta, float* wt) {
   }
 }
 
-// Polynomials of the kernel taps in f (|f| <= 1/2), fitted on the host in FP64 (es_poly):
+// Polynomials of the kernel taps in f (|f| <= 1/2), fitted on the host in FP64 (es_table):
 // tap j = E_j(f^2) + f O_j(f^2) and, the kernel being even, tap W-1-j = E_j(f^2) - f O_j(f^2).
 // Coefficients duplicated in both halves of a 64-bit word, one table per width.
 __constant__ __align__(16) float2 c_es[3][5][2 * kEsTerms];
 
 cudaError_t upload_es_polys(cudaStream_t stream) {
-  float2 t[3][5][2 * kEsTerms] = {};
-  for (int q = 0; q < 3; ++q)
-    for (int j = 0; j <= (5 + 2 * q) / 2; ++j) {
-      double c[2 * kEsTerms];
-      es_poly(5 + 2 * q, j, c);
-      for (int k = 0; k < 2 * kEsTerms; ++k) t[q][j][k] = make_float2((float)c[k], (float)c[k]);
-    }
-  cudaError_t e = cudaMemcpyToSymbolAsync(c_es, t, sizeof(t), 0, cudaMemcpyHostToDevice, stream);
-  return e == cudaSuccess ? cudaStreamSynchronize(stream) : e;
+  static_assert(sizeof(EsTable) == sizeof(c_es), "the table has the layout of c_es");
+  return cudaMemcpyToSymbolAsync(c_es, es_table().c, sizeof(c_es), 0, cudaMemcpyHostToDevice, stream);
 }
 
 // The W x- and W y-weights of a row at once, two polynomials per packed FMA (lanes x, y):
