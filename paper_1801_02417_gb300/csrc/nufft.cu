@@ -245,17 +245,11 @@ __global__ void __launch_bounds__(512) k_fwd_cols(const float4* __restrict__ T1,
   }
 }
 
+// The kernel at offset t (cells).
 template <int W>
-__device__ __forceinline__ void es_weights(float f, float beta, float* wt) {
-  // wt[j] = phi(f + hw - j), tap j at frequency c - hw + j.
-  constexpr int hw = W / 2;
-  const float inv = 2.0f / W;
-#pragma unroll
-  for (int j = 0; j < W; ++j) {
-    const float z = (f + (float)(hw - j)) * inv;
-    const float s = 1.0f - z * z;
-    wt[j] = s > 0.f ? __expf(beta * (s * rsqrtf(s) - 1.0f)) : 0.f;
-  }
+__device__ __forceinline__ float es_weight(float t, float beta) {
+  const float z = t * (2.0f / W), s = 1.0f - z * z;
+  return s > 0.f ? __expf(beta * (s * rsqrtf(s) - 1.0f)) : 0.f;
 }
 
 // Polynomials of the kernel taps in f (|f| <= 1/2), fitted on the host in FP64 (es_table):
@@ -271,32 +265,31 @@ cudaError_t upload_es_polys(cudaStream_t stream) {
 // The W x- and W y-weights of a row at once, two polynomials per packed FMA (lanes x, y):
 // 34 packed FMAs for W = 7 in place of 14 square roots and exponentials, and closer to the
 // kernel: at most 1e-7 of its peak off in FP32 (1.4e-7 at the very end of the outermost tap),
-// the exponential form 7e-7. W = 5 keeps the exponentials: the square-root end of its kernel
-// (height 1e-5) is not a polynomial.
+// the exponential form 7e-7. The outermost taps of W = 5 keep the exponentials: the square-root end of that kernel
+// (height 1e-5) is not a polynomial, and below a tenth of the peak their error is as small.
 template <int W>
 __device__ __forceinline__ void es_weights_xy(float fx, float fy, float beta, float* wx, float* wy) {
-  if constexpr (W == 5) {
-    es_weights<W>(fx, beta, wx);
-    es_weights<W>(fy, beta, wy);
-  } else {
-    constexpr int q = (W - 5) / 2, hw = W / 2;
-    const u64 f = f2pack(fx, fy), nf = f2pack(-fx, -fy), x = ffma2(f, f, 0ull);
-    auto co = [&](int j, int k) { return *reinterpret_cast<const u64*>(&c_es[q][j][k]); };
+  constexpr int q = (W - 5) / 2, hw = W / 2, j0 = W == 5 ? 1 : 0;
+  const u64 f = f2pack(fx, fy), nf = f2pack(-fx, -fy), x = ffma2(f, f, 0ull);
+  auto co = [&](int j, int k) { return *reinterpret_cast<const u64*>(&c_es[q][j][k]); };
 #pragma unroll
-    for (int j = 0; j <= hw; ++j) {
-      u64 e = co(j, kEsTerms - 1);
+  for (int j = j0; j <= hw; ++j) {
+    u64 e = co(j, kEsTerms - 1);
 #pragma unroll
-      for (int k = kEsTerms - 2; k >= 0; --k) e = ffma2(e, x, co(j, k));
-      if (j == hw) {   // the centre tap is even in f
-        f2unpack(e, wx[j], wy[j]);
-      } else {
-        u64 o = co(j, 2 * kEsTerms - 1);
+    for (int k = kEsTerms - 2; k >= 0; --k) e = ffma2(e, x, co(j, k));
+    if (j == hw) {   // the centre tap is even in f
+      f2unpack(e, wx[j], wy[j]);
+    } else {
+      u64 o = co(j, 2 * kEsTerms - 1);
 #pragma unroll
-        for (int k = kEsTerms - 2; k >= 0; --k) o = ffma2(o, x, co(j, kEsTerms + k));
-        f2unpack(ffma2(o, f, e), wx[j], wy[j]);
-        f2unpack(ffma2(o, nf, e), wx[W - 1 - j], wy[W - 1 - j]);
-      }
+      for (int k = kEsTerms - 2; k >= 0; --k) o = ffma2(o, x, co(j, kEsTerms + k));
+      f2unpack(ffma2(o, f, e), wx[j], wy[j]);
+      f2unpack(ffma2(o, nf, e), wx[W - 1 - j], wy[W - 1 - j]);
     }
+  }
+  if constexpr (W == 5) {
+    wx[0] = es_weight<W>(fx + hw, beta), wy[0] = es_weight<W>(fy + hw, beta);
+    wx[W - 1] = es_weight<W>(fx - hw, beta), wy[W - 1] = es_weight<W>(fy - hw, beta);
   }
 }
 
@@ -307,27 +300,6 @@ __device__ __forceinline__ void unpack_rec(float4 r, float& fx, float& fy, float
   const int pk = __float_as_int(r.w);
   cx = (int)(short)(pk & 0xFFFF);
   cy = pk >> 16;
-}
-
-// FP32 -> TF32 hi part (round to nearest, ties away) and the TF32 rounding of the
-// remainder; hi + lo carries the operand to about 2^-21 of its value.
-__device__ __forceinline__ void tf32_split(float a, uint32_t& hi, uint32_t& lo) {
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hi) : "f"(a));
-  const float r = a - __uint_as_float(hi);
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lo) : "f"(r));
-}
-// The same split with integer rounding of the hi part (round half up on the magnitude) and
-// the remainder left for the tensor core to truncate to TF32: |a - hi - lo_tf32| <= 2^-21 |a|.
-__device__ __forceinline__ void tf32_split_fast(float a, uint32_t& hi, uint32_t& lo) {
-  hi = (__float_as_uint(a) + 0x1000u) & 0xFFFFE000u;
-  lo = __float_as_uint(a - __uint_as_float(hi));
-}
-// d += A B for one m16n8k8 TF32 tile: A (16 x 8) fragment a[4], B (8 x 8) fragment b[2].
-__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-  asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-      "{%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
 // Second half of a degridding row m: from the interpolated packed spectra sp (at +u) and sn
@@ -587,65 +559,70 @@ static constexpr size_t degrid_smem_tiles() {
 //  1. lane = row: the row is read, mixed by conj(L) (x_I = RR + LL, x_Q = RR - LL, x_U = RL + LR,
 //     x_V = i (LR - RL)), scaled by c_b w_m, and left in the warp's shared-memory buffer with its
 //     W y- and x-weights (es_weights_xy); the next 32 rows are read meanwhile.
-//  2. Per run of rows of one cell, the cell's W x W x 8 block is accumulated in registers as a
-//     product of two small matrices on the tensor cores: G = P^T Y, P[v][(jx, c)] = w_x[v][jx]
-//     x_c[v] (MT m-tiles of 16 rows (jx, c)) and Y[v][jy] = w_y[v][jy] (NT n-tiles of 8), 8 rows v
-//     per mma.m16n8k8 (TF32). Each FP32 operand is split into TF32 hi + lo parts and the
-//     products hi hi, hi lo, lo hi accumulate in FP32 (lo lo is below FP32 rounding). Rows of
-//     a product that are not the run's enter as zeros.
+//  2. Per run of rows of one cell, the cell's W x W x 8 block is accumulated in registers in FP32: a lane
+//     owns one channel and NY stencil rows, all their columns as packed pairs; per row it forms x_c w_y
+//     and adds its products with the w_x pairs (fma.rn.f32x2).
 //  3. Where the cell ends, the block goes to shared memory and from there to the accumulator
 //     by W bulk reductions (one per stencil row, W cells of 32 bytes; two where the row wraps
 //     around a full grid), which run while the warp goes on with its next cell.
+//  4. MERGE: the last blocks of neighbouring warps that belong to one cell are added up in shared
+//     memory first, so that a cell of many rows is few partial sums (launch_grid says when).
 // Channels are gridded at +u only; k_adj_cols forms the -u half by Hermitian symmetrisation.
 //
-// Nothing is shared between warps: no barrier, no uneven end of a work item, no list of work,
-// and no FP32 atomic on shared memory (a compare-and-swap loop), which the form before it
-// paid (one CTA per tile of cells, blocks added to a shared tile, weights from a table of 64
-// bytes per row: in this form the table measured 91 us against 87). Grid stage, us: 1024^2 /
-// 2,000,000 rows (34 per cell) 101 -> 85 with 232 -> 105 MB of DRAM traffic, 256^2 / 50,000 17 ->
-// 14; phi^dagger as a whole: 1024^2 / 200,001 scattered rows
-// (1 per cell) 397 -> 193, 512^2 / 2,000,001 scattered 389 -> 333. Bound by issue (70% of the slots
-// busy), the split and the products before the tensor pipe.
-constexpr int kGridWarps = 4;   // warps of a CTA
+// But for that merge nothing is shared between warps: no barrier, no uneven end of a work item, no list of
+// work, and no FP32 atomic on shared memory (a compare-and-swap loop). Products and sums are FP32 FMAs: per
+// row a lane issues four shared loads, NY products and NY NX packed FMAs, about 17 instructions for the warp's
+// 392 products at W = 7. As TF32 tensor-core products (m16n8k8, operands split in two) the splits and the
+// fragments' loads took more than that, a lone row cost as much as eight, and 22 bits per operand showed in
+// the result. phi^dagger, us, tensor cores / this: 1024^2 / 2,000,000 rows (34 per cell) 114 / 112, 2048^2 / 700,001
+// (4 per cell) 184 / 161, 1024^2 / 200,001 scattered rows (1 per cell) 173 / 163, 1024^2 / 2,000,001 scattered 602 /
+// 471, W = 9 there 910 / 705; error against the same interpolation in FP64, 128^2 / 165,337 rows, W = 5 2.8e-7 /
+// 1.6e-7, W = 9 at 32^2 / 200,001 1.1e-6 / 2.6e-7. Grid stage: 1024^2 / 2,000,000 86 / 82 us, 2048^2 / 700,001 94 / 73.
+// Bound by issue.
+constexpr int kGridWarps = 4;     // warps of a CTA
+constexpr int kMergeWarps = 8;   // warps of a CTA that merges its warps' last blocks
 template <int W>
 struct GridWarp {
-  static constexpr int MT = (W + 1) / 2, NT = (W + 7) / 8;
-  static constexpr int XP = 2 * MT <= 8 ? 8 : 12;    // x-weights per row (2 MT used)
-  static constexpr int SP = 8 * W + 4;               // stage pitch of a stencil row (2 SP = 24 mod 32 banks for W = 7)
-  static constexpr int kRow = 32 * (8 + 8 * NT + XP);            // floats of the row buffer
+  static constexpr int NY = W == 9 ? 3 : 2, NX = (W + 1) / 2;   // stencil rows of a lane, pairs of columns
+  static constexpr int YP = W == 9 ? 12 : 8;        // y-weights per row: NY (W = 9: and one unused) per lane quarter
+  static constexpr int XP = 2 * NX <= 8 ? 8 : 12;   // x-weights per row (2 NX used)
+  static constexpr int SP = W == 9 ? 88 : 8 * W + 4;   // stage pitch of a stencil row (NY SP = 8 or 24 mod 32 banks)
+  static constexpr int kRow = 32 * (8 + YP + XP);              // floats of the row buffer
   static constexpr int kFloats = kRow + 2 * ((W * SP + 3) / 4 * 4);   // + two staged blocks
 };
-// Six CTAs per SM by registers (W = 9 holds too much for it): 418.0 us per iteration at 1024^2, 420.5 without.
-template <int W, bool PERM>
-__global__ void __launch_bounds__(32 * kGridWarps, W == 9 ? 1 : 6) k_grid(
+// No bound on the registers (64 to 102): 64 a thread (eight CTAs per SM) gives 84.6 us per grid stage at 1024^2 for 82,
+// a bound so loose that the loop takes 154 gives 429 us per iteration for 418. Eight rows of the loop
+// unrolled: 82 us, two 88.
+template <int W, bool PERM, bool MERGE>
+__global__ void __launch_bounds__(32 * (MERGE ? kMergeWarps : kGridWarps)) k_grid(
     int M, int rows, const uint16_t* __restrict__ vblk, const float4* __restrict__ rec, const float2* __restrict__ vin,
     const int32_t* __restrict__ perm,
     const float* __restrict__ cb, int use_scale, int Wd, int off, int full, int K, float beta,
     float* __restrict__ Acc) {
   using T = GridWarp<W>;
-  constexpr int MT = T::MT, NT = T::NT, hw = W / 2;
+  constexpr int NY = T::NY, NX = T::NX, hw = W / 2;
   extern __shared__ __align__(16) float4 smw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* xs = reinterpret_cast<float*>(smw) + warp * T::kFloats;   // 8 channels per row
   float* wyb = xs + 32 * 8;
-  float* wxb = wyb + 32 * 8 * NT;
+  float* wxb = wyb + 32 * T::YP;
   float* stage = xs + T::kRow;
   constexpr int kStageF = (T::kFloats - T::kRow) / 2;
-  const long long first = (long long)(blockIdx.x * kGridWarps + warp) * rows;
+  const long long first = (long long)(blockIdx.x * (MERGE ? kMergeWarps : kGridWarps) + warp) * rows;
   pdl_wait();
-  if (first >= M) return;
-  const int m0 = (int)first, m1 = (int)min((long long)M, first + rows);
+  if (!MERGE && first >= M) return;
+  const int m0 = (int)min((long long)M, first), m1 = (int)min((long long)M, first + rows);
   const float4* v4 = reinterpret_cast<const float4*>(vin);
-  const int g = lane >> 2, tig = lane & 3;
-  float d[MT][NT][4];
+  const int g = lane >> 2, jy0 = NY * (W == 9 ? min(lane & 3, 2) : lane & 3);   // channel, first stencil row
+  u64 d[NY][NX];   // cells (jy0 + y, 2 t) and (jy0 + y, 2 t + 1) of channel g
 #pragma unroll
-  for (int t = 0; t < MT; ++t)
+  for (int y = 0; y < NY; ++y)
 #pragma unroll
-    for (int q = 0; q < NT; ++q) d[t][q][0] = d[t][q][1] = d[t][q][2] = d[t][q][3] = 0.f;
+    for (int t = 0; t < NX; ++t) d[y][t] = 0ull;
   float4 r, b0, b1;
   int blk = 0, buf = 0, cell = -1;   // cell: the accumulated block's (grid row << 12 | column), -1: none
   // vin in stored order, or (PERM) in the caller's; the index of a row is read one step ahead of it.
-  int next = PERM ? perm[min(m0 + lane, m1 - 1)] : 0;
+  int next = PERM && m0 < m1 ? perm[min(m0 + lane, m1 - 1)] : 0;
   auto fetch = [&](int m) {
     const size_t i = min(m + lane, m1 - 1), v = PERM ? next : i;
     r = rec[i];
@@ -654,24 +631,24 @@ __global__ void __launch_bounds__(32 * kGridWarps, W == 9 ? 1 : 6) k_grid(
     if (PERM) next = perm[min(m + 32 + lane, m1 - 1)];
     if (use_scale) blk = vblk[i];
   };
-  // The block to the accumulator: d[t][q][i] is cell (jy = 8 q + 2 tig + (i & 1), jx = 2 t + (i >> 1)),
-  // channel g.
-  auto flush = [&]() {
-    float* st = stage + buf * kStageF;
+  // The block to a stage buffer; from there to the accumulator.
+  auto store = [&](float* st) {
     bulk_wait_read<1>();   // this lane's reductions of two cells ago have read their buffer
     __syncwarp();
 #pragma unroll
-    for (int t = 0; t < MT; ++t)
+    for (int y = 0; y < NY; ++y)
 #pragma unroll
-      for (int q = 0; q < NT; ++q)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int jy = 8 * q + 2 * tig + (i & 1), jx = 2 * t + (i >> 1);
-          if (jy < W && jx < W) st[jy * T::SP + jx * 8 + g] = d[t][q][i];
-          d[t][q][i] = 0.f;
-        }
-    fence_proxy_async();
-    __syncwarp();
+      for (int t = 0; t < NX; ++t) {
+        float v0, v1;
+        f2unpack(d[y][t], v0, v1);
+        d[y][t] = 0ull;
+        if (jy0 + y >= W) continue;
+        float* o = st + (jy0 + y) * T::SP + 16 * t + g;
+        o[0] = v0;
+        if (2 * t + 1 < W) o[8] = v1;
+      }
+  };
+  auto reduce = [&](const float* st) {
     if (lane < W) {
       const int gy = (cell >> 12) - hw + lane, gx = (cell & 4095) - hw;
       const float* src = st + lane * T::SP;
@@ -685,9 +662,16 @@ __global__ void __launch_bounds__(32 * kGridWarps, W == 9 ? 1 : 6) k_grid(
       }
     }
     bulk_commit();
+  };
+  auto flush = [&]() {
+    float* st = stage + buf * kStageF;
+    store(st);
+    fence_proxy_async();
+    __syncwarp();
+    reduce(st);
     buf ^= 1;
   };
-  fetch(m0);
+  if (!MERGE || m0 < m1) fetch(m0);
   for (int m = m0; m < m1; m += 32) {
     const int cnt = min(32, m1 - m);
     int key;
@@ -700,14 +684,15 @@ __global__ void __launch_bounds__(32 * kGridWarps, W == 9 ? 1 : 6) k_grid(
       float4* xo = reinterpret_cast<float4*>(xs) + 2 * lane;
       xo[0] = make_float4(sc * (b0.x + b1.z), sc * (b0.y + b1.w), sc * (b0.x - b1.z), sc * (b0.y - b1.w));
       xo[1] = make_float4(sc * (b0.z + b1.x), sc * (b0.w + b1.y), -sc * (b1.y - b0.w), sc * (b1.x - b0.z));
-      float4* yo = reinterpret_cast<float4*>(wyb + 8 * NT * lane);
+      float4* yo = reinterpret_cast<float4*>(wyb + T::YP * lane);
       float4* po = reinterpret_cast<float4*>(wxb + T::XP * lane);
       float wx[W], wy[W];
       es_weights_xy<W>(fx, fy, beta, wx, wy);
       auto at = [](const float* v, int k) { return k < W ? v[k < W ? k : 0] : 0.f; };
 #pragma unroll
-      for (int q = 0; q < 2 * NT; ++q)
-        yo[q] = make_float4(at(wy, 4 * q), at(wy, 4 * q + 1), at(wy, 4 * q + 2), at(wy, 4 * q + 3));
+      for (int q = 0; q < T::YP / 4; ++q)
+        yo[q] = W == 9 ? make_float4(at(wy, 3 * q), at(wy, 3 * q + 1), at(wy, 3 * q + 2), 0.f)
+                       : make_float4(at(wy, 4 * q), at(wy, 4 * q + 1), at(wy, 4 * q + 2), at(wy, 4 * q + 3));
 #pragma unroll
       for (int q = 0; q < T::XP / 4; ++q)
         po[q] = make_float4(at(wx, 4 * q), at(wx, 4 * q + 1), at(wx, 4 * q + 2), at(wx, 4 * q + 3));
@@ -723,63 +708,69 @@ __global__ void __launch_bounds__(32 * kGridWarps, W == 9 ? 1 : 6) k_grid(
       const int k = __shfl_sync(0xffffffffu, key, a);
       if (cell >= 0 && k != cell) flush();
       cell = k;
-      for (int k0 = a; k0 < end; k0 += 8) {
-        const int va = k0 + tig, vb = va + 4;
-        const int ra = min(va, 31), rb = min(vb, 31);
-        const float xa = xs[8 * ra + g], xb = xs[8 * rb + g];
-        uint32_t bh[NT][2], bl[NT][2];
-#pragma unroll
-        for (int q = 0; q < NT; ++q) {
-          tf32_split(va < end ? wyb[8 * NT * ra + 8 * q + g] : 0.f, bh[q][0], bl[q][0]);
-          tf32_split(vb < end ? wyb[8 * NT * rb + 8 * q + g] : 0.f, bh[q][1], bl[q][1]);
+#pragma unroll 8
+      for (int v = a; v < end; ++v) {
+        const float x = xs[8 * v + g];
+        float wy[4];
+        if constexpr (NY == 2) {
+          const float2 w2 = *reinterpret_cast<const float2*>(wyb + T::YP * v + jy0);
+          wy[0] = w2.x, wy[1] = w2.y;
+        } else {
+          const float4 w4 = *reinterpret_cast<const float4*>(wyb + T::YP * v + jy0 / 3 * 4);
+          wy[0] = w4.x, wy[1] = w4.y, wy[2] = w4.z;
         }
-        float pa[T::XP], pb[T::XP];
+        u64 wx[T::XP / 2];
 #pragma unroll
-        for (int q = 0; q < T::XP / 4; ++q) {
-          const float4 wa = reinterpret_cast<const float4*>(wxb + T::XP * ra)[q];
-          const float4 wb = reinterpret_cast<const float4*>(wxb + T::XP * rb)[q];
-          pa[4 * q] = wa.x, pa[4 * q + 1] = wa.y, pa[4 * q + 2] = wa.z, pa[4 * q + 3] = wa.w;
-          pb[4 * q] = wb.x, pb[4 * q + 1] = wb.y, pb[4 * q + 2] = wb.z, pb[4 * q + 3] = wb.w;
+        for (int q = 0; q < (NX + 1) / 2; ++q) {
+          const ulonglong2 w4 = reinterpret_cast<const ulonglong2*>(wxb + T::XP * v)[q];
+          wx[2 * q] = w4.x, wx[2 * q + 1] = w4.y;
         }
-        uint32_t ah[MT][4], al[MT][4];
 #pragma unroll
-        for (int t = 0; t < MT; ++t) {
-          tf32_split_fast(pa[2 * t] * xa, ah[t][0], al[t][0]);
-          tf32_split_fast(pb[2 * t] * xb, ah[t][2], al[t][2]);
-          if (2 * t + 1 < W) {
-            tf32_split_fast(pa[2 * t + 1] * xa, ah[t][1], al[t][1]);
-            tf32_split_fast(pb[2 * t + 1] * xb, ah[t][3], al[t][3]);
-          } else {
-            ah[t][1] = al[t][1] = ah[t][3] = al[t][3] = 0u;
-          }
-        }
-        // Each step's products start from zero, small terms first (consecutive ones go to different tiles:
-        // independent), and are added to the run's sum by an FP32 addition: the tensor core truncates
-        // what it adds to, which over a run of 64 rows is a bias. Error of phi^dagger against FP64, the products
-        // added to the run's sum there / here: 64^2 / 100,001 rows (73 per cell) 5.5e-7 / 3.4e-7, 128^2 / 165,337
-        // 5.1e-7 / 2.5e-7, 512^2 / 600,001 4.4e-7 / 2.0e-7.
+        for (int y = 0; y < NY; ++y) {
+          const u64 p = fdup(x * wy[y]);
 #pragma unroll
-        for (int q = 0; q < NT; ++q) {
-          float c[MT][4];
-#pragma unroll
-          for (int t = 0; t < MT; ++t) c[t][0] = c[t][1] = c[t][2] = c[t][3] = 0.f;
-#pragma unroll
-          for (int t = 0; t < MT; ++t) mma_tf32(c[t], al[t], bh[q]);
-#pragma unroll
-          for (int t = 0; t < MT; ++t) mma_tf32(c[t], ah[t], bl[q]);
-#pragma unroll
-          for (int t = 0; t < MT; ++t) mma_tf32(c[t], ah[t], bh[q]);
-#pragma unroll
-          for (int t = 0; t < MT; ++t)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) d[t][q][i] += c[t][i];
+          for (int t = 0; t < NX; ++t) d[y][t] = ffma2(p, wx[t], d[y][t]);
         }
       }
       a = end;
     }
     __syncwarp();   // the row buffer is read before the next rows replace it
   }
-  flush();
+  if constexpr (MERGE) {
+    // Neighbouring warps whose last blocks belong to one cell: the first of them takes the sum.
+    __shared__ int s_cell[kMergeWarps], s_buf[kMergeWarps];   // a warp without rows comes after all others (cell -1)
+    if (cell >= 0) store(stage + buf * kStageF);
+    if (lane == 0) s_cell[warp] = cell, s_buf[warp] = buf;
+    __syncthreads();
+    float* base = reinterpret_cast<float*>(smw) + T::kRow;
+    int c[kMergeWarps], at[kMergeWarps];   // the cells and where their blocks are
+#pragma unroll
+    for (int v = 0; v < kMergeWarps; ++v) c[v] = s_cell[v], at[v] = v * T::kFloats + s_buf[v] * kStageF;
+    for (int i = threadIdx.x; i < W * T::SP; i += blockDim.x) {
+      if (i % T::SP >= 8 * W) continue;   // the pitch's unused floats
+      float x[kMergeWarps];
+#pragma unroll
+      for (int v = 0; v < kMergeWarps; ++v) x[v] = c[v] >= 0 ? base[at[v] + i] : 0.f;
+      int lead = at[0];
+      float sum = x[0];
+#pragma unroll
+      for (int v = 1; v < kMergeWarps; ++v) {
+        if (c[v] == c[v - 1]) {
+          sum += x[v];
+        } else {
+          base[lead + i] = sum;
+          lead = at[v];
+          sum = x[v];
+        }
+      }
+      if (c[kMergeWarps - 1] >= 0) base[lead + i] = sum;
+    }
+    fence_proxy_async();
+    __syncthreads();
+    if (cell >= 0 && (warp == 0 || s_cell[warp - 1] != cell)) reduce(stage + buf * kStageF);
+  } else {
+    flush();
+  }
   bulk_wait_all();   // the reductions are done before the CTA's shared memory goes
 }
 
@@ -932,6 +923,15 @@ static cudaError_t set_smem(const void* fn, size_t bytes) {
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+template <int W>
+static constexpr size_t grid_smem(int warps) { return (size_t)warps * GridWarp<W>::kFloats * sizeof(float); }
+
+template <int W>
+static cudaError_t configure_grid() {
+  const cudaError_t e = set_smem((const void*)k_grid<W, false, true>, grid_smem<W>(kMergeWarps));
+  return e == cudaSuccess ? set_smem((const void*)k_grid<W, true, true>, grid_smem<W>(kMergeWarps)) : e;
+}
+
 cudaError_t configure_nufft_kernels() {
   // Largest grid: n = 2048, K = 4096.
   const size_t sm1 = fft_smem_bytes(4096, 1), sm2 = fft_smem_bytes(4096, 2);
@@ -946,6 +946,9 @@ cudaError_t configure_nufft_kernels() {
   const size_t degrid_smem[] = {degrid_smem_tiles<5>(), degrid_smem_tiles<7>(), degrid_smem_tiles<9>()};
   for (int i = 0; i < 6; ++i)
     if ((e = set_smem(degrids[i], degrid_smem[i % 3] + 2048 * sizeof(double))) != cudaSuccess) return e;
+  if ((e = configure_grid<5>()) != cudaSuccess || (e = configure_grid<7>()) != cudaSuccess ||
+      (e = configure_grid<9>()) != cudaSuccess)
+    return e;
   return set_smem((const void*)k_adj_cols, sm2);
 }
 
@@ -989,14 +992,24 @@ static cudaError_t launch_grid(Handle* h, const float2* in, int use_scale, const
   // rows that cutting its run at a warp's end costs more than parallelism gives. Else 32.
   // phi^dagger, us at 8 / 32 / 64 rows: 64^2 / 2,000 rows 27 / 29 / 31, 128^2 / 6,001 scattered
   // (1 per cell) 31 / 43 / 60, 64^2 / 25,153 33 / 27 / 29, 256^2 / 50,000 31 / 29 / 31, 2048^2 /
-  // 700,001 (4 per cell) - / 215 / 222; 64^2 / 100,000 (73 per cell) - / 35 / 30, 1024^2 / 2,000,000
+  // 700,001 (4 per cell) - / 215 / 222; 64^2 / 100,000 (529 per cell) - / 35 / 30, 1024^2 / 2,000,000
   // (34 per cell) - / 147 / 143.
-  const int warps = 8 * std::max(1, h->num_sms);
-  const int rows = h->M <= 12 * warps ? 8 : (h->M >= 64 * warps && h->M / std::max(1, h->ncells) >= 16 ? 64 : 32);
-  const int ctas = (int)(((int64_t)h->M + (int64_t)rows * kGridWarps - 1) / ((int64_t)rows * kGridWarps));
-  return launch_after(h->early, perm ? k_grid<W, true> : k_grid<W, false>, ctas, 32 * kGridWarps, kGridWarps * GridWarp<W>::kFloats * sizeof(float),
-                      h->stream, h->M, rows, h->vblk, h->rec, in, perm, h->cb, use_scale, g.Wd, g.off, g.full, g.K, g.beta,
-                      reinterpret_cast<float*>(h->Acc));
+  // A cell of the accumulator is the FP32 sum, one reduction after another, of all runs of W^2 cells, and its
+  // rounding grows as the root of their number. Where a cell's rows make more than 16 runs (W = 9, which adds up
+  // 81 cells where W = 7 adds 49: 4), CTAs of eight warps merge theirs before the reduction. Error of
+  // phi^dagger, 32^2 / 200,001 rows (about 2,000 per cell), as separate runs / merged: W = 5 3.9e-7 / 1.7e-7, W = 7 5.7e-7 /
+  // 2.2e-7, W = 9 9.7e-7 / 2.6e-7; us 22.5 / 18.4, 28.7 / 20.5, 38 / 25. With fewer runs the merge's barrier costs more
+  // than it saves: 64^2 / 100,000 (529 per cell, 8 runs) grid stage 11.5 separate, 13.2 merged, 64^2 / 200,000 (17 runs) 18.9
+  // and 15.3; a batch of 16 problems with merges from 8 runs on 8288 us for 8247.
+  const int warps = 8 * std::max(1, h->num_sms), per_cell = h->M / std::max(1, h->ncells);
+  const int rows = h->M <= 12 * warps ? 8 : (h->M >= 64 * warps && per_cell >= 16 ? 64 : 32);
+  const bool merge = per_cell > (W == 9 ? 4 : 16) * rows;
+  const int nw = merge ? kMergeWarps : kGridWarps;
+  const int ctas = (int)(((int64_t)h->M + (int64_t)rows * nw - 1) / ((int64_t)rows * nw));
+  auto kern = merge ? (perm ? k_grid<W, true, true> : k_grid<W, false, true>)
+                    : (perm ? k_grid<W, true, false> : k_grid<W, false, false>);
+  return launch_after(h->early, kern, ctas, 32 * nw, grid_smem<W>(nw), h->stream, h->M, rows, h->vblk, h->rec, in, perm, h->cb,
+                      use_scale, g.Wd, g.off, g.full, g.K, g.beta, reinterpret_cast<float*>(h->Acc));
 }
 
 cudaError_t nufft_grid(Handle* h, const float2* in, int use_scale, bool cleared, const int32_t* perm) {
