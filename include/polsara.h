@@ -387,7 +387,7 @@ enum {
 ps_status ps_autotune(ps_handle* h, int32_t reps, int32_t* choices, double* ms);
 
 /* Read / force the launch choices (PS_TUNE_COUNT int32; PS_EINVAL for a value
- * outside a slot's candidates). The defaults are 0. */
+ * outside a slot's accepted values). The defaults are 0. */
 ps_status ps_get_tuning(const ps_handle* h, int32_t* choices);
 ps_status ps_set_tuning(ps_handle* h, const int32_t* choices);
 

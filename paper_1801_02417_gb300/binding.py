@@ -428,7 +428,7 @@ TUNE_SLOTS = ("synthesis", "degrid", "grid", "analysis")
 
 
 def ps_autotune(h, reps: int = 5) -> dict:
-    """Time every launch candidate on the handle's data and keep the fastest; returns
+    """Time the launch form of every slot on the handle's data and select it; returns
     {slot: (choice, ms)}."""
     ch = np.zeros(len(TUNE_SLOTS), dtype=np.int32)
     ms = np.zeros(len(TUNE_SLOTS), dtype=np.float64)

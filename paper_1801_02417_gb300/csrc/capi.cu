@@ -1343,8 +1343,8 @@ ps_status ps_autotune(ps_handle* h, int32_t reps, int32_t* choices, double* ms) 
   ps_status st = pick(PS_TUNE_SYNTHESIS, [&] { return ps::sara_synthesis(h, h->A, h->PsiA); });
   if (st != PS_OK) return st;
   // Degridding as the iteration runs it (the dual update of steps 7-8 with its block sums),
-  // from the spectrum of the current S, on a scratch copy of the dual: the candidates read and
-  // write the visibility rows as in the iteration, and the state's dual is untouched.
+  // from the spectrum of the current S, on a scratch copy of the dual: the visibility rows are read and
+  // written as in the iteration, and the state's dual is untouched.
   if (h->M > 0) {
     CK(h, ps::nufft_forward_grid(h, h->S, false));
     CK(h, cudaMemcpyAsync(h->vtmp, h->R, 4 * (size_t)h->M * sizeof(float2), cudaMemcpyDeviceToDevice, h->stream));

@@ -120,9 +120,9 @@ __device__ __forceinline__ void fft_pass(float4* buf, int nbuf, const float2* __
 // barriers bound these kernels, so three radix-2 stages go together: a thread takes 8 elements
 // through them in registers, and the eight lanes of a quarter-warp fall into eight bank groups of
 // fsw. What three does not divide ends in a pass of two stages or one. Forward and adjoint
-// transforms (both kernels of each), radix-4 passes -> these: 117 -> 92 and 111 -> 90 us at 2048^2
-// (K = 4096), 34.5 -> 30.7 and 34.8 -> 31.0 at 1024^2, 16.4 -> 14.5 and 17.3 -> 15.8 at 512^2, equal
-// below. Passes of four stages need 140 registers a thread: 110 and 94 us at 2048^2 but 23 and 18 at 512^2.
+// transforms (both kernels of each), radix-4 passes -> these: 117 -> 90 and 111 -> 90 us at 2048^2
+// (K = 4096), 34.5 -> 30.5 and 34.8 -> 31 at 1024^2, equal below. Passes of four stages need 140 registers a thread:
+// 110 and 94 us at 2048^2 but 23 and 18 for 16 at 512^2.
 // Stages below s0 are taken as done (the caller wrote their output); stages from
 // s_end on are left to the caller (fft_out).
 template <bool INV>
@@ -149,7 +149,7 @@ __device__ __forceinline__ void scatter_stage0(float4* buf, int idx, int logK, f
 }
 
 // First of the stages fft_out finishes when the passes start at s0: one or two, such that whole passes
-// of three remain; two where nothing would be left over (three cost 32.8 us for two's 30.7 in the adjoint
+// of three remain; two where nothing would be left over (three cost 32.8 us for two's 31 in the adjoint
 // transforms at 1024^2).
 __device__ __forceinline__ int fft_tail_start(int logK, int s0) {
   const int rem = (logK - s0) % 3;
@@ -578,7 +578,7 @@ static constexpr size_t degrid_smem_tiles() {
 // (4 per cell) 184 / 161, 1024^2 / 200,001 scattered rows (1 per cell) 173 / 163, 1024^2 / 2,000,001 scattered 602 /
 // 471, W = 9 there 910 / 705; error against the same interpolation in FP64, 128^2 / 165,337 rows, W = 5 2.8e-7 /
 // 1.6e-7, W = 9 at 32^2 / 200,001 1.1e-6 / 2.6e-7. Grid stage: 1024^2 / 2,000,000 86 / 82 us, 2048^2 / 700,001 94 / 73.
-// Bound by issue.
+// Bound by the L1 data pipe (83%: the rows' broadcast loads), issue at 64%.
 constexpr int kGridWarps = 4;     // warps of a CTA
 constexpr int kMergeWarps = 8;   // warps of a CTA that merges its warps' last blocks
 template <int W>

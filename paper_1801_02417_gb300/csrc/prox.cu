@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_primal(
 // sweep is a latency: 64^2 10.1 -> 7.3 us, 256^2 10.5 -> 8.7 against four pixels in four CTAs,
 // resp. 64), two above, with all 28 loads of a pixel pair in flight (80 registers): 1024^2 39.7
 // us with four pixels and loads as the steps need them, 37.9 with all of four pixels' loads in
-// flight, 32.4 with two's (0.69 -> 0.84 of the copy bandwidth on 192 B per pixel); 2048^2 (cone
+// flight, 33 with two's (0.75 -> 0.91 of the copy bandwidth on 192 B per pixel); 2048^2 (cone
 // dual) 122 -> 104 us.
 static int sweep_pix(int N) { return N <= 65536 ? 1 : 2; }
 int sweep_blocks(int N) { return (N + kSweepThreads * sweep_pix(N) - 1) / (kSweepThreads * sweep_pix(N)); }

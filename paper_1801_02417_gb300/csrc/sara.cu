@@ -99,7 +99,8 @@ __device__ __forceinline__ int wrap1(int v, int m) { return v < 0 ? v + m : (v >
 // four outputs of one row from 16-byte reads; the taps go in pairs,
 // {c[2p], c[2p+1]} x {in[2k+2p], in[2k+2p+1]}, and the two halves are added at the end. Two pairs per
 // step and the last of an odd count on its own: a pair of zero taps in its place would turn an infinity
-// that the filter does not reach into a NaN. x0 .. x3 are the sample pairs p .. p + 3.
+// that the filter does not reach into a NaN (that step is 1% of the stage: 80.7 -> 81.5 us at level 1 of 1024^2).
+// x0 .. x3 are the sample pairs p .. p + 3.
 __device__ __forceinline__ void ana_rows(int b, const float* __restrict__ in_s, float* __restrict__ lo_s,
                                          float* __restrict__ hi_s) {
   const int RS = 2 * kTO + 2 * b;
